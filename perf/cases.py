@@ -84,9 +84,9 @@ def draw(rng):
         n = rng.choice([1024, 2048, 4096, 8192])
         out = 4 * _log_int(rng, 128, 4096)
         return dict(op=op, n=n, out=out, rows=_log_int(rng, 1, 4096), wbits=bits, abits=rng.choice([0, 4, 8]))
-    if op == "calibrate":  # the dense products take K blocks of 64
+    if op == "calibrate":  # the dense products take K blocks of 64; angles are learned where codes are few
         n = rng.choice([512, 1024, 2048, 4096])
-        return dict(op=op, n=n, out=64 * _log_int(rng, 4, 64), rows=64 * _log_int(rng, 2, 32), dtype=dtype, wbits=bits,
+        return dict(op=op, n=n, out=64 * _log_int(rng, 4, 64), rows=64 * _log_int(rng, 2, 32), dtype=dtype, wbits=min(bits, 4),
                     abits=rng.choice([0, 4, 8]))
     n1, n2 = rng.choice([(40, 128), (40, 128), (12, 256), (7, 1024)])
     case = dict(op=op, n1=n1, n=n2, rows=_log_int(rng, 1 if op == "composite" else 64, _MOST[op] // (n1 * n2)), dtype=dtype)
@@ -221,3 +221,120 @@ def tolerance(case):
             return {"rel": 2e-3, "max": 7e-3, "differ": {2: 2e-4, 4: 3.5e-3, 8: 1e-2}[case["bits"]]}
         return {"rel": 1e-3, "max": 2e-3, "differ": 2e-4}
     return {"rel": 9e-3, "max": 4e-2} if bf16 else {"rel": 7e-6, "max": 2.2e-5}
+
+
+# ---- the same passes in 64 bits, in plain torch ----------------------------------------------------------------------
+_CHUNK = 1 << 26  # elements of the rows that are worked on at a time
+
+
+def _stages(theta):
+    """(cos, sin) of each stage's pairs."""
+    t = theta.double()
+    return list(zip(torch.cos(t), torch.sin(t)))
+
+
+def _turn(x, stage, s, back=False):
+    """Stage s (pairs at distance 2^s) on the last axis of x, or its transpose."""
+    d = 1 << s
+    c, sn = (v.view(-1, d) for v in stage)
+    if back:
+        sn = -sn
+    v = x.reshape(*x.shape[:-1], -1, 2, d)
+    lo, hi = v[..., 0, :], v[..., 1, :]
+    return torch.stack((c * lo - sn * hi, sn * lo + c * hi), dim=-2).reshape(x.shape)
+
+
+def _rotate(theta, x, back=False):
+    stages = _stages(theta)
+    x = x.double()
+    for s in (range(len(stages) - 1, -1, -1) if back else range(len(stages))):
+        x = _turn(x, stages[s], s, back)
+    return x
+
+
+def _gradients(theta, x, g):
+    """(y, dx, dtheta): y = Q x, and the gradients of <g, y>."""
+    stages = _stages(theta)
+    y, g, dth = _rotate(theta, x), g.double(), []
+    z = y
+    for s in range(len(stages) - 1, -1, -1):
+        u, w = (t.reshape(t.shape[0], -1, 2, 1 << s) for t in (z, g))
+        dth.append((w[:, :, 1] * u[:, :, 0] - w[:, :, 0] * u[:, :, 1]).sum(0).reshape(-1))
+        z, g = _turn(z, stages[s], s, True), _turn(g, stages[s], s, True)
+    return y, g, torch.stack(dth[::-1])
+
+
+def _chunks(rows, width):
+    step = max(1, _CHUNK // width)
+    return [slice(r, min(rows, r + step)) for r in range(0, rows, step)]
+
+
+def _scales(y, bits):
+    return y.abs().amax(dim=1) / (2 ** (bits - 1) - 1)
+
+
+def _quantized(y, bits):
+    """Rows through codes and 16-bit scales and back."""
+    s = _scales(y, bits).half().double().unsqueeze(1)
+    q = torch.where(s > 0, y / s, torch.zeros_like(y)).round().clamp(-(2 ** (bits - 1)), 2 ** (bits - 1) - 1)
+    return q * s
+
+
+def _cayley(params, n1):
+    i, j = torch.triu_indices(n1, n1, 1, device=params.device)
+    a = torch.zeros((n1, n1), dtype=torch.float64, device=params.device)
+    a[i, j] = params.double()
+    a = a - a.t()
+    eye = torch.eye(n1, dtype=torch.float64, device=params.device)
+    inv = torch.linalg.inv(eye + a)
+    return (eye - a) @ inv, inv
+
+
+def exact(case, seed):
+    """What run() returns, in 64 bits: scales before their rounding to 16, None in the place of codes."""
+    op, n, rows, dtype = case["op"], case["n"], case["rows"], _dtype(case)
+    seed = 16 * int(seed)
+    theta = synth.angles(n, "normal", seed, DEVICE)
+    if op in ("quant", "inverse"):
+        x = _activations(rows, n, seed + 2, dtype)
+        if op == "quant":
+            return None, torch.cat([_scales(_rotate(theta, x[c]), case["bits"]) for c in _chunks(rows, n)])
+        return torch.cat([_rotate(theta, x[c], back=True) for c in _chunks(rows, n)])
+    if op == "fold":
+        w = _weights(rows, n, seed + 1, dtype)
+        parts = [_rotate(theta, w[c]) for c in _chunks(rows, n)]
+        return None, torch.cat([_scales(y, case["bits"]) for y in parts]), torch.cat(parts) if case["keep"] else None
+    if op == "learn":
+        x, g = _activations(rows, n, seed + 2, dtype), synth.rows(rows, n, "normal", seed + 3, dtype=dtype, device=DEVICE)
+        y, dx = (torch.empty((rows, n), dtype=torch.float64, device=DEVICE) for _ in range(2))
+        dth = 0
+        for c in _chunks(rows, n):
+            y[c], dx[c], part = _gradients(theta, x[c], g[c])
+            dth = dth + part
+        return y, dx, dth
+    if op == "linear":
+        w = _quantized(_rotate(theta, _weights(case["out"], n, seed + 1, torch.bfloat16)), case["wbits"])
+        y = _rotate(theta, _activations(rows, n, seed + 2, torch.bfloat16))
+        return (_quantized(y, case["abits"]) if case["abits"] else y) @ w.t()
+    if op == "calibrate":
+        w, x = _weights(case["out"], n, seed + 1, dtype).double(), _activations(rows, n, seed + 2, dtype).double()
+        wq, y = _quantized(_rotate(theta, w), case["wbits"]), _rotate(theta, x)
+        yq = _quantized(y, case["abits"]) if case["abits"] else y
+        err = yq @ wq.t() - x @ w.t()
+        e = err * (2.0 / err.numel())
+        return (err * err).mean(), _gradients(theta, x, e @ wq)[2] + _gradients(theta, w, e.t() @ yq)[2], theta.double()
+    n1 = case["n1"]
+    params = synth.cayley_params(n1, seed + 1, device=DEVICE)
+    q1, inv = _cayley(params, n1)
+    x = _activations(rows, n1 * n, seed + 2, dtype)
+    if op == "composite":
+        return None, torch.cat([_scales(torch.einsum("ik,rkj->rij", q1, _rotate(theta, x[c].reshape(-1, n1, n))).flatten(1),
+                                        case["bits"]) for c in _chunks(rows, n1 * n)])
+    g = synth.rows(rows, n1 * n, "normal", seed + 3, dtype=dtype, device=DEVICE).double().reshape(rows, n1, n)
+    gp = torch.einsum("ki,rkj->rij", q1, g)
+    xp, dx, dth = _gradients(theta, x.reshape(-1, n), gp.reshape(-1, n))
+    xp = xp.reshape(rows, n1, n)
+    dq1 = torch.einsum("rij,rkj->ik", g, xp)
+    da = -(torch.eye(n1, dtype=torch.float64, device=DEVICE) + q1).t() @ dq1 @ inv.t()
+    i, j = torch.triu_indices(n1, n1, 1, device=DEVICE)
+    return torch.einsum("ik,rkj->rij", q1, xp).flatten(1), dx.reshape(rows, -1), dth, dq1, (da - da.t())[i, j]
