@@ -5,26 +5,31 @@
 // [K][rows].  This covers the three products of the reconstruction loss (paper Sec. 3.4):
 //     Dequant(Quant(B x)) . Dequant(Quant(W B^T))^T,   err . Dequant(Quant(W B^T)),   err^T . Dequant(Quant(B x)).
 //
-// One CTA per 128 x 128 tile of C, K blocks of 64.  An operand tile in shared memory is 128 rows of 128 bytes (64 bf16)
-// with the 128-byte swizzle, and every row is 64 elements that are CONTIGUOUS IN THE STORED OPERAND:
+// Tensor-core side: pairs of CTAs (tcgen05 cta_group::2).  The rows of B are the M side of the MMA (256 per pair, 128 per
+// CTA) and the rows of A its N side (`nt` = 32 .. 256 per pair, half per CTA), so that the lanes of an accumulator are
+// consecutive columns of C and every store of the epilogue is 128 contiguous bytes.  K blocks of 64.  An operand tile in
+// shared memory is up to 128 rows of 128 bytes (64 bf16) with the 128-byte swizzle, and every row is 64 elements that are
+// CONTIGUOUS IN THE STORED OPERAND:
 //   * stored [rows][K]: shared-memory row r = tile row r, 64 consecutive k (the K-major layout of the tensor core);
 //   * stored [K][rows]: shared-memory row 64 h + k = stored row k0 + k, tile rows 64 h .. 64 h + 63 (the MN-major
 //     layout: blocks of 64 tile rows 8192 bytes apart, groups of 8 k 1024 bytes apart).
-// So one producer thread (eight producer warps: threads 0..127 for A, 128..255 for B) always turns 64 contiguous stored
-// elements into one 128-byte row, with 16-byte loads and stores, whatever the orientation; the instruction descriptor
-// tells the tensor core which layout each operand has.  Terms per operand:
+// So one producer thread always turns contiguous stored elements into 16-byte pieces of a 128-byte row, whatever the
+// orientation; the instruction descriptor tells the tensor core which layout each operand has.  bf16 operands need no
+// conversion and come by TMA straight into the same layout.  Terms per operand:
 //   * codes contracted along their stored row: the integer codes are exact in bf16 (one term); the row scale multiplies
 //     the finished row / column of C;
-//   * codes contracted across stored rows: the scale varies along k, so code x scale (at most 15 significant bits) is
-//     stored as hi + lo, exactly;
+//   * codes contracted across stored rows: the scale varies along k.  If the other operand is fp32 the scale multiplies
+//     THAT operand before it is split (one fp32 rounding, 2^-24, in front of a split that keeps 2^-17) and the codes stay
+//     one exact term; otherwise code x scale (at most 15 significant bits) is stored as hi + lo, exactly;
 //   * fp32 numbers: hi + lo = 16 significant bits (relative error 2^-17 per element); bf16 numbers: one term, exact.
-// Codes become bf16 without integer-to-float conversions: a field u = code + 2^(b-1) OR-ed into the mantissa of 128.0
-// is the bf16 number 128 + u, two fields per 32-bit word at a time, and one packed subtraction removes the offset.
-// The global loads of the next K block are issued before the current one is converted.  One thread issues
-// tcgen05.mma (kind::f16, M = N = 128, fp32 accumulators in tensor memory) for every pair of terms and commits to
-// the stage's "empty" mbarrier; the ring has as many stages as fit 192 KB.  The producer warps then read the
-// accumulators back (tcgen05.ld, a lane quarter and half of the columns each), apply alpha and the row / column
-// scales and store fp32 rows of C.  Every wait is bounded and reports through the plan's status word.
+// The MMA thread issues one product per pair of terms (1, 2 or 4 per K step), accumulating all of them in fp32.
+//
+// What bounds it: per K block a CTA's tensor core works 512 cycles on nt = 256 (one term pair) and reads 64 KB of
+// operands from shared memory, while 32 KB are written there: with one CTA per 128 x 128 tile, which this replaces, both
+// figures per product were twice as large and the conversion of an element served half as many products.
+// Measured on a B200, before -> now (bf16 rows x 2-bit codes, 1000 x 28672 x 8192: 0.98 -> 0.389 ms = 1.21 PFLOP/s; 8-bit x
+// 2-bit codes, same size: 0.267 ms; 4-bit x 4-bit codes, 2048 x 4096 x 4096: 0.181 -> 0.059 ms; fp32 x 4-bit codes stored
+// [K][rows]: 0.445 -> 0.173 ms; both stored [K][rows]: 0.400 -> 0.235 ms).
 #include "../../include/bfq.h"
 
 #include <cuda_bf16.h>
@@ -32,6 +37,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include "bfq_n4096.cuh"
 #include "bfq_plan.h"
 #include "bfq_ptx.cuh"
 
@@ -39,13 +45,23 @@ namespace bfq {
 namespace dqg {
 using namespace ptx;
 
-constexpr int kTile = 128;       // rows of A and of B per CTA
+constexpr int kRows = 128;       // shared-memory rows of an operand tile; rows of B per CTA
 constexpr int kKB = 64;          // K block: one 128-byte swizzle atom of bf16
+constexpr int kMaxNt = 256;      // rows of A per pair of CTAs
 constexpr int kMaxStages = 6;
-constexpr int kProducers = 256;  // threads 0..127 build A's tile, 128..255 B's; all run the epilogue; thread 256 issues the MMAs
-constexpr uint32_t kTileBytes = kTile * kKB * 2;  // one bf16 term of one operand: 16 KB
-constexpr uint32_t kRingBytes = 12 * kTileBytes;  // 192 KB of operand tiles
-constexpr int kWaitLimit = 1 << 24;
+constexpr int kEpi = 128;        // threads 0 .. 127: epilogue, one tensor-memory lane each
+constexpr int kProd = 256;       // producers per operand: threads 128 .. 383 build B's tiles, 384 .. 639 A's
+constexpr int kIssuer = kEpi + 2 * kProd;  // thread 640: MMAs (even CTA of a pair) or forwarding (odd CTA)
+constexpr int kLoader = kIssuer + 32;      // thread 672: TMA loads of bf16 operands
+constexpr int kThreads = kLoader + 32;
+constexpr uint32_t kTileBytes = kRows * kKB * 2;  // one bf16 term of one operand: 16 KB
+// shared memory: operand tiles, and raw pieces of converted operands on their way (128 bytes for each of 512 producers)
+constexpr uint32_t kRingTiles = 12, kRingTilesStaged = 9;
+constexpr int kStagedPieces = 8;                        // per producer thread
+constexpr uint32_t kStagingBytes = 512 * kStagedPieces * 16;
+constexpr uint32_t kBarsOff = kRingTilesStaged * kTileBytes + kStagingBytes;  // the larger of the two uses
+static_assert(kRingTiles * kTileBytes <= kBarsOff, "both uses lie below the barriers");
+constexpr int kWaitLimit = 1 << 22;
 
 struct Operand {
     const void* data;
@@ -54,20 +70,22 @@ struct Operand {
     int kind;                // BFQ_OP_*
     int transposed;          // 0: [rows][K], 1: [K][rows]
     int rows;                // M or N
+    int terms;               // bf16 terms an element is stored in
+    int scaled;              // codes times their scales go into shared memory (two terms)
 };
 
-__device__ __forceinline__ bool is_codes(int kind) { return kind >= BFQ_OP_CODES2; }
-__host__ __device__ __forceinline__ int terms_of(int kind, int transposed) {
-    if (kind == BFQ_OP_BF16) return 1;
-    if (kind == BFQ_OP_F32) return 2;
-    return transposed ? 2 : 1;
-}
-__host__ __device__ __forceinline__ int stages_of(int terms_a, int terms_b) {
-    const int fit = 12 / (terms_a + terms_b);
+__host__ __device__ __forceinline__ bool is_codes(int kind) { return kind >= BFQ_OP_CODES2; }
+__host__ __device__ __forceinline__ int stages_of(bool staged, int terms_u, int terms_v) {
+    const int fit = static_cast<int>(staged ? kRingTilesStaged : kRingTiles) / (terms_u + terms_v);
     return fit < kMaxStages ? fit : kMaxStages;
 }
 
 __device__ __forceinline__ void fence_proxy_async() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
+__device__ __forceinline__ bool elect_one() {
+    uint32_t r;
+    asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xFFFFFFFF;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(r));
+    return r != 0;
+}
 __device__ __forceinline__ void mbar_arrive(uint32_t bar) {
     asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
 }
@@ -78,12 +96,25 @@ __device__ __forceinline__ bool wait_bounded(uint32_t bar, uint32_t parity, int*
     atomicExch(status, 3);
     return false;
 }
-__device__ __forceinline__ void tmem_alloc128(uint32_t smem_dst) {
-    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], 128;" ::"r"(smem_dst) : "memory");
-    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+// Arrival on another CTA's barrier.  What it announces is read by the tensor core of the CTA that wrote it (or is an
+// accumulator), never by another CTA's threads, so no fence at cluster scope is needed (one would cost more than the
+// products of a K block).
+__device__ __forceinline__ void mbar_arrive_remote(uint32_t cluster_addr) {
+    asm volatile("mbarrier.arrive.shared::cluster.b64 _, [%0];" ::"r"(cluster_addr) : "memory");
 }
-__device__ __forceinline__ void tmem_dealloc128(uint32_t taddr) {
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 128;" ::"r"(taddr) : "memory");
+// both CTAs of a pair allocate and free together
+__device__ __forceinline__ void tmem_alloc_pair(uint32_t smem_dst) {
+    asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], 512;" ::"r"(smem_dst) : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
+}
+__device__ __forceinline__ void tmem_dealloc_pair(uint32_t taddr) {
+    asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, 512;" ::"r"(taddr) : "memory");
+}
+__device__ __forceinline__ void tma_load_2d(uint32_t dst, const void* tmap, int c0, int c1, uint32_t bar) {
+    asm volatile(
+        "cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];"
+        ::"r"(dst), "l"(reinterpret_cast<uint64_t>(tmap)), "r"(c0), "r"(c1), "r"(bar)
+        : "memory");
 }
 // Shared-memory descriptor of a 128-byte-swizzled tile.  K-major operand: rows of 128 bytes, 8-row groups 1024 bytes
 // apart (stride field), the leading field unused; one K step of 16 elements is 32 bytes further along the row.
@@ -93,21 +124,62 @@ __device__ __forceinline__ uint64_t desc_sw128(uint32_t addr, uint32_t leading_b
     return static_cast<uint64_t>((addr & 0x3FFFFu) >> 4) | (static_cast<uint64_t>(leading_bytes >> 4) << 16) |
            (static_cast<uint64_t>(1024 >> 4) << 32) | (static_cast<uint64_t>(1) << 46) | (static_cast<uint64_t>(2) << 61);
 }
-// bf16 x bf16 -> fp32, M = 128, N = 128; bit 15 / 16: A / B is MN-major
-__device__ __forceinline__ uint32_t make_idesc(int a_mn_major, int b_mn_major) {
-    return (1u << 4) | (1u << 7) | (1u << 10) | (static_cast<uint32_t>(a_mn_major) << 15) |
-           (static_cast<uint32_t>(b_mn_major) << 16) | (uint32_t(kTile >> 3) << 17) | (uint32_t(kTile >> 4) << 24);
+// M = 256 over the pair, N = nt; bf16 x bf16 -> fp32 (bit 15 / 16: the M / N operand is MN-major), or 8-bit x 8-bit -> 32-bit
+// signed integers
+__device__ __forceinline__ uint32_t make_idesc(bool int8, int nt, int u_mn_major, int v_mn_major) {
+    return ((int8 ? 2u : 1u) << 4) | (1u << 7) | (1u << 10) | (static_cast<uint32_t>(u_mn_major) << 15) |
+           (static_cast<uint32_t>(v_mn_major) << 16) | (static_cast<uint32_t>(nt >> 3) << 17) | (uint32_t(2 * kRows >> 4) << 24);
 }
-__device__ __forceinline__ void mma_bf16(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc, uint32_t accumulate) {
+// Issued by the one thread of a converged warp whose `lead` is set: a predicate on the instruction and no branch around it,
+// so that the operands can stay in uniform registers.
+template <bool INT8>
+__device__ __forceinline__ void mma_pair(uint32_t lead, uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc, uint32_t accumulate) {
+    if constexpr (INT8) {
+        asm volatile(
+            "{\n\t.reg .pred p, q;\n\t"
+            "setp.ne.b32 p, %4, 0;\n\t"
+            "setp.ne.b32 q, %5, 0;\n\t"
+            "@q tcgen05.mma.cta_group::2.kind::i8 [%0], %1, %2, %3, p;\n\t}"
+            ::"r"(d_tmem), "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate), "r"(lead)
+            : "memory");
+    } else {
+        asm volatile(
+            "{\n\t.reg .pred p, q;\n\t"
+            "setp.ne.b32 p, %4, 0;\n\t"
+            "setp.ne.b32 q, %5, 0;\n\t"
+            "@q tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n\t}"
+            ::"r"(d_tmem), "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate), "r"(lead)
+            : "memory");
+    }
+}
+// arrives on the barrier at this offset of every CTA in `mask` when the MMAs that this thread has issued so far have finished
+__device__ __forceinline__ void mma_commit(uint32_t lead, uint32_t bar, uint16_t mask) {
     asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "setp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}"
-        ::"r"(d_tmem), "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
+        "{\n\t.reg .pred q;\n\t"
+        "setp.ne.b32 q, %2, 0;\n\t"
+        "@q tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;\n\t}"
+        ::"r"(bar), "h"(mask), "r"(lead)
         : "memory");
 }
-__device__ __forceinline__ void mma_commit(uint32_t bar) {
-    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
+// whether a phase is over, without waiting for it
+__device__ __forceinline__ bool mbar_test(uint32_t bar, uint32_t parity) {
+    uint32_t ok;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(ok)
+        : "r"(bar), "r"(parity)
+        : "memory");
+    return ok != 0;
+}
+// the wait of a converged warp
+__device__ __forceinline__ bool wait_warp(uint32_t bar, uint32_t parity, int* status) {
+    for (int i = 0; i < kWaitLimit; ++i) {
+        if (__all_sync(0xFFFFFFFFu, mbar_try_wait(bar, parity))) return true;
+    }
+    atomicExch(status, 3);
+    return false;
 }
 
 // ---- one shared-memory row: 64 elements that are contiguous in the stored operand -------------------------------
@@ -140,10 +212,20 @@ __device__ __forceinline__ void split2(float a, float b, uint32_t& hi, uint32_t&
     lo = pack_bf16(a - __uint_as_float(hi << 16), b - __uint_as_float(hi & 0xFFFF0000u));
 }
 
-// Raw 16-byte words of a row's 64 elements: fp32 16, bf16 8, 8-bit codes 4, 4-bit codes 2, 2-bit codes 1
-template <int KIND>
-struct RawWords {
-    static constexpr int kCount = KIND == BFQ_OP_F32 ? 16 : (KIND == BFQ_OP_BF16 ? 8 : (KIND * 64) / 128);
+// How the 128 shared-memory rows of an operand tile are cut into 16-byte pieces of the stored operand.  INT8: a row is 128
+// codes as bytes instead of 64 elements as bf16.  A group of kThreads threads builds a whole tile by itself; several groups
+// of an operand work on different K blocks, because one block's chain (wait for the stage, convert, make the writes
+// visible to the tensor core) takes longer than the tensor core takes for the block.
+template <int KIND, bool INT8>
+struct Pieces {
+    static constexpr int kBits = KIND == BFQ_OP_F32 ? 32 : KIND;
+    static constexpr int kRowElems = INT8 ? 2 * kKB : kKB;
+    static constexpr int kPerRow = kRowElems * kBits / 128;
+    static constexpr int kElems = 128 / kBits;
+    static constexpr int kThreads = KIND == BFQ_OP_F32 ? 256 : 128;
+    static constexpr int kPerThread = kRows * kPerRow / kThreads;
+    // of the group's own blocks, how many are on their way
+    static constexpr int kDepth = kStagedPieces / kPerThread < 4 ? kStagedPieces / kPerThread : 4;
 };
 
 // 8 codes of 4 bits (one word, element e in bits 4e..4e+3, two's complement) -> 4 words of bf16 pairs in element order
@@ -178,12 +260,44 @@ __device__ __forceinline__ void codes8_to_bf16(uint32_t w, uint32_t (&o)[2]) {
     o[0] = pack_bf16(f0, f1), o[1] = pack_bf16(f2, f3);
 }
 
+// The same codes as 8-bit integers for the integer tensor path, 16 codes -> one 16-byte chunk.  Codes stay where they are
+// in their bytes, so that a 2-bit code counts 64 times and a 4-bit code 16 times (kShift; taken off in the epilogue,
+// exactly); byte b of word j is code 4 b + j of the 16, the order the 2-bit codes fall into, for every width.
+template <int KIND>
+struct Int8Chunk {
+    static constexpr int kShift = KIND == BFQ_OP_CODES2 ? 6 : (KIND == BFQ_OP_CODES4 ? 4 : 0);
+    // w: the 16 codes' words (1, 2 or 4)
+    __device__ __forceinline__ static void make(const uint32_t* w, uint32_t (&o)[4]) {
+        if constexpr (KIND == BFQ_OP_CODES2) {
+            o[0] = (w[0] << 6) & 0xC0C0C0C0u, o[1] = (w[0] << 4) & 0xC0C0C0C0u;
+            o[2] = (w[0] << 2) & 0xC0C0C0C0u, o[3] = w[0] & 0xC0C0C0C0u;
+        } else if constexpr (KIND == BFQ_OP_CODES4) {
+            const uint32_t al = (w[0] << 4) & 0xF0F0F0F0u, ah = w[0] & 0xF0F0F0F0u;  // codes 0, 2, 4, 6 and 1, 3, 5, 7
+            const uint32_t bl = (w[1] << 4) & 0xF0F0F0F0u, bh = w[1] & 0xF0F0F0F0u;
+            o[0] = prmt(al, bl, 0x6420u), o[1] = prmt(ah, bh, 0x6420u);
+            o[2] = prmt(al, bl, 0x7531u), o[3] = prmt(ah, bh, 0x7531u);
+        } else {
+            const uint32_t a = prmt(w[0], w[1], 0x5140u), b = prmt(w[2], w[3], 0x5140u);
+            const uint32_t c = prmt(w[0], w[1], 0x7362u), d = prmt(w[2], w[3], 0x7362u);
+            o[0] = prmt(a, b, 0x5410u), o[1] = prmt(a, b, 0x7632u);
+            o[2] = prmt(c, d, 0x5410u), o[3] = prmt(c, d, 0x7632u);
+        }
+    }
+};
+
 struct Params {
-    Operand a, b;
+    Operand u, v;  // B (M side of the MMA) and A (N side)
     float* c;
     int64_t ldc;
-    int k;
+    int k;        // length of the contraction
+    int kblocks;  // in blocks of 64, or of 128 on the integer path
+    int int8;     // both operands are codes along K: kind::i8 products of the integer codes
+    float unit;   // integer path: 2^-(the places the codes were left in)
     float alpha;
+    int nt;       // rows of A per tile
+    int tiles_v;  // tiles along A's rows; consecutive tiles share the rows of B
+    int tiles;
+    int split;    // pairs per cluster that share a tile, each with its part of K (1: a cluster is one pair, many tiles)
     int* status;
 };
 
@@ -213,16 +327,16 @@ __device__ __forceinline__ void store_bf16_chunk(uint32_t tile, int srow, int j,
     }
 }
 
-// One raw 16-byte word = piece p of shared-memory row `srow` (the row's 64 elements are 128 / kPerWord pieces).
-// SCALED (codes contracted across their stored rows): times `s`, two terms.  PARTIAL: only the first `valid` elements
-// of the piece exist; the others are stored as zero.
+// Piece p of shared-memory row `srow`.  SCALED (codes contracted across their stored rows): times `s`, two terms; fp32
+// numbers: times the scales `f` of the other operand's codes where those vary along k (1 otherwise).  PARTIAL: only the
+// first `valid` elements of the piece exist; the others are stored as zero.
 template <int KIND, bool SCALED, bool PARTIAL>
-__device__ __forceinline__ void convert_word(const uint4 raw, uint32_t tile, int srow, int p, float s, int valid) {
+__device__ __forceinline__ void convert_piece(const uint4 raw, uint32_t tile, int srow, int p, float s, const float (&f)[4], int valid) {
     if constexpr (KIND == BFQ_OP_F32) {
         // 4 numbers = half of chunk p / 2
         uint32_t hi[2], lo[2];
-        split2(__uint_as_float(raw.x), __uint_as_float(raw.y), hi[0], lo[0]);
-        split2(__uint_as_float(raw.z), __uint_as_float(raw.w), hi[1], lo[1]);
+        split2(__uint_as_float(raw.x) * f[0], __uint_as_float(raw.y) * f[1], hi[0], lo[0]);
+        split2(__uint_as_float(raw.z) * f[2], __uint_as_float(raw.w) * f[3], hi[1], lo[1]);
         if constexpr (PARTIAL) {
 #pragma unroll
             for (int w = 0; w < 2; ++w) {
@@ -233,9 +347,6 @@ __device__ __forceinline__ void convert_word(const uint4 raw, uint32_t tile, int
         const uint32_t at = chunk_addr(tile, srow, p >> 1) + 8u * (p & 1);
         asm volatile("st.shared.v2.u32 [%0], {%1,%2};" ::"r"(at), "r"(hi[0]), "r"(hi[1]) : "memory");
         asm volatile("st.shared.v2.u32 [%0], {%1,%2};" ::"r"(at + kTileBytes), "r"(lo[0]), "r"(lo[1]) : "memory");
-    } else if constexpr (KIND == BFQ_OP_BF16) {
-        uint32_t o[4] = {raw.x, raw.y, raw.z, raw.w};
-        store_bf16_chunk<false, PARTIAL>(tile, srow, p, 0, o, 1.f, valid);
     } else if constexpr (KIND == BFQ_OP_CODES4) {
         const uint32_t ws[4] = {raw.x, raw.y, raw.z, raw.w};
 #pragma unroll
@@ -267,215 +378,581 @@ __device__ __forceinline__ void convert_word(const uint4 raw, uint32_t tile, int
     }
 }
 
+// Piece p of shared-memory row `srow` on the integer path
+template <int KIND>
+__device__ __forceinline__ void convert_piece_int8(const uint4 raw, uint32_t tile, int srow, int p) {
+    constexpr int kWords = KIND / 2;          // of 16 codes
+    constexpr int kChunks = 4 / kWords;       // 16-byte chunks that a 16-byte piece turns into
+    const uint32_t ws[4] = {raw.x, raw.y, raw.z, raw.w};
+#pragma unroll
+    for (int c = 0; c < kChunks; ++c) {
+        uint32_t o[4];
+        Int8Chunk<KIND>::make(ws + c * kWords, o);
+        sts128(chunk_addr(tile, srow, kChunks * p + c), o[0], o[1], o[2], o[3]);
+    }
+}
+
+// What a role of a CTA walks through: tiles first, first + step, ... below `tiles`, K blocks [kb0, kb1) of each.
+struct Walk {
+    int first, step, tiles, kb0, kb1;
+    __device__ __forceinline__ int blocks() const {
+        return first < tiles ? ((tiles - first + step - 1) / step) * (kb1 - kb0) : 0;
+    }
+};
+
 struct Ring {
     uint32_t sbase, stage_bytes, bar_full, bar_empty;
     int stages;
 };
 
-// Producer loop of one thread of the 128 that build one operand's tiles.  A K block of the operand is 128 shared-memory
-// rows of kLpr 16-byte pieces; piece id = i * 128 + r (i = 0 .. kLpr - 1) is piece id % kLpr of row id / kLpr, so the
+// the tile rows of one operand that this CTA holds
+struct Span {
+    int tiles_v, row_tile, lim;  // lim: rows of the operand in this CTA's half of a tile
+    bool is_u;
+    int half;                    // 0 / 1: which CTA of the pair
+    __device__ __forceinline__ int row0(int tile) const {
+        const int t = is_u ? tile / tiles_v : tile % tiles_v;
+        return t * row_tile + half * lim;
+    }
+};
+
+__device__ __forceinline__ void cp_async16(uint32_t dst, const void* src, uint32_t bytes) {  // bytes = 0: sixteen zeros
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(bytes) : "memory");
+}
+__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N>
+__device__ __forceinline__ void cp_async_wait() {
+    asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
+}
+
+// Producer loop of thread r of one of the `groups` groups that build one operand's tiles; group g has blocks g, g + groups,
+// ... of the walk.  Piece id = i * kThreads + r (i = 0 .. kPerThread - 1) is piece id % kPerRow of row id / kPerRow, so the
 // lanes of a warp read consecutive pieces of the same stored row: global loads are coalesced as far as the stored row
-// allows.  ACROSS: the operand is stored [K][rows]; shared-memory row 64 h + k is stored row k0 + k, tile rows
-// 64 h .. 64 h + 63.
-template <int KIND, bool ACROSS>
-__device__ __forceinline__ bool produce(const Operand& op, int r, int tile_row0, uint32_t tile_off, const Ring& ring, int kblocks,
+// allows.  Raw pieces go through shared memory (`staging`, `pitch16` bytes between a thread's slots), each thread reading
+// only what it copied itself: kDepth blocks ahead cost no registers (with the pieces in registers an fp32 block waited
+// most of 3400 cycles for its loads).  ACROSS: the operand is stored [K][rows]; shared-memory row 64 h + k is stored row
+// k0 + k, tile rows 64 h .. 64 h + 63.  SCALED / fold: see convert_piece.
+template <int KIND, bool ACROSS, bool SCALED, bool INT8>
+__device__ __forceinline__ void produce(const Operand& op, int k_len, int g, int groups, int r, uint32_t staging, uint32_t pitch16,
+                                        const Span& span, uint32_t tile_off, const Ring& ring, const Walk& walk, const uint16_t* fold,
                                         int* status) {
-    constexpr int kLpr = RawWords<KIND>::kCount;  // pieces per row = pieces per thread
-    constexpr int kEbits = KIND == BFQ_OP_F32 ? 32 : (KIND == BFQ_OP_BF16 ? 16 : KIND);
-    constexpr int kPerWord = 128 / kEbits;  // elements per piece
-    constexpr bool kScaled = ACROSS && KIND >= BFQ_OP_CODES2;
-    constexpr int kRowStep = kTile / kLpr;  // rows between a thread's consecutive pieces
-    const int p = r % kLpr, row_first = r / kLpr;
+    using PC = Pieces<KIND, INT8>;
+    constexpr int kBits = PC::kBits, kElems = PC::kElems, kPer = PC::kPerThread, kDepth = PC::kDepth;
+    constexpr int kRowStep = PC::kThreads / PC::kPerRow;  // rows between a thread's consecutive pieces
+    constexpr int kBlockBytes = PC::kRowElems * kBits / 8;  // a K block of a row stored along K
+    constexpr bool kFold = KIND == BFQ_OP_F32;
+    const int p = r % PC::kPerRow, row_first = r / PC::kPerRow;
     const uint8_t* const base = static_cast<const uint8_t*>(op.data);
-    const int64_t pitch = op.ld * kEbits / 8;  // bytes of a stored row
-    // per piece: how many of its elements exist (0: nothing is loaded) and where K block 0 of it starts
+    const int64_t pitch = op.ld * kBits / 8;  // bytes of a stored row
     auto srow_of = [&](int i) { return row_first + i * kRowStep; };
-    auto valid_of = [&](int i) -> int {
+    auto active = [&](int i) { return ACROSS ? 64 * (srow_of(i) >> 6) < span.lim : srow_of(i) < span.lim; };
+    // how many of piece i's elements exist (0: zeros are staged)
+    auto valid_of = [&](int i, int row0, int kb) -> int {
         if constexpr (!ACROSS) {
-            return tile_row0 + srow_of(i) < op.rows ? kPerWord : 0;
+            return row0 + srow_of(i) < op.rows && (!INT8 || kb * PC::kRowElems + p * kElems < k_len) ? kElems : 0;
         } else {
-            const int left = op.rows - (tile_row0 + 64 * (srow_of(i) >> 6) + p * kPerWord);
-            return left < 0 ? 0 : (left > kPerWord ? kPerWord : left);
+            const int left = op.rows - (row0 + 64 * (srow_of(i) >> 6) + p * kElems);
+            return left < 0 ? 0 : (left > kElems ? kElems : left);
         }
     };
-    auto src_of = [&](int i, int kb) -> const uint4* {
+    struct At {
+        int tile, kb, row0;
+        const uint8_t* src;  // this thread's first piece of the tile, K block 0
+    };
+    auto enter = [&](At& a) {
+        a.row0 = span.row0(a.tile);
         if constexpr (!ACROSS) {
-            return reinterpret_cast<const uint4*>(base + int64_t(tile_row0 + srow_of(i)) * pitch + int64_t(kb) * (kKB * kEbits / 8) + 16 * p);
+            a.src = base + int64_t(a.row0 + row_first) * pitch + 16 * p;
         } else {
-            const int sr = srow_of(i);
-            return reinterpret_cast<const uint4*>(base + (int64_t(kb) * kKB + (sr & 63)) * pitch +
-                                                  int64_t(tile_row0 + 64 * (sr >> 6)) * kEbits / 8 + 16 * p);
+            a.src = base + int64_t(row_first) * pitch + int64_t(a.row0) * kBits / 8 + 16 * p;
         }
     };
-    auto load = [&](uint4 (&raw)[kLpr], float (&sc)[kLpr], int kb) {
-#pragma unroll
-        for (int i = 0; i < kLpr; ++i) {
-            raw[i] = valid_of(i) > 0 ? __ldg(src_of(i, kb)) : make_uint4(0u, 0u, 0u, 0u);
-            if constexpr (kScaled) sc[i] = __half2float(__ushort_as_half(__ldg(op.scales + kb * kKB + (srow_of(i) & 63))));
+    auto advance = [&](At& a, int by) {
+        a.kb += by;
+        if (a.kb >= walk.kb1) {
+            do {
+                a.kb -= walk.kb1 - walk.kb0, a.tile += walk.step;
+            } while (a.kb >= walk.kb1);
+            enter(a);
         }
     };
-    // the raw words of the next kDepth K blocks are in flight while the current one is converted
-    constexpr int kDepth = kLpr >= 16 ? 1 : (kLpr >= 8 ? 2 : 4);
-    uint4 buf[kDepth + 1][kLpr];
-    float sc[kDepth + 1][kScaled ? kLpr : 1];
-    auto load_slot = [&](int d, int kb) {
-        if constexpr (kScaled) {
-            load(buf[d], sc[d], kb);
-        } else {
-            float none[kLpr];
-            load(buf[d], none, kb);
+    auto stage_in = [&](uint32_t slot, const At& a) {
+        if (a.tile < walk.tiles) {
+#pragma unroll
+            for (int i = 0; i < kPer; ++i) {
+                const uint8_t* src;
+                if constexpr (!ACROSS) {
+                    src = a.src + int64_t(i * kRowStep) * pitch + int64_t(a.kb) * kBlockBytes;
+                } else {
+                    // rows repeat every 64: the next 64 tile rows of the same stored rows
+                    constexpr int kHalfBytes = 64 * kBits / 8;
+                    const int sr = srow_of(i);
+                    src = a.src + (int64_t(a.kb) * kKB + ((sr & 63) - row_first)) * pitch + (sr >> 6) * kHalfBytes;
+                }
+                const bool there = active(i) && valid_of(i, a.row0, a.kb) > 0;
+                cp_async16(staging + (slot * kPer + i) * pitch16, there ? src : base, there ? 16u : 0u);
+            }
+        }
+        cp_async_commit();
+    };
+    constexpr int kScales = SCALED ? kPer : (kFold ? 4 : 1);
+    float sc[kScales];
+    auto half_at = [](const uint16_t* q) { return __half2float(__ushort_as_half(__ldg(q))); };
+    auto load_scales = [&](const At& a) {
+        if constexpr (SCALED) {
+#pragma unroll
+            for (int i = 0; i < kPer; ++i) sc[i] = a.tile < walk.tiles ? half_at(op.scales + a.kb * kKB + (srow_of(i) & 63)) : 0.f;
+        }
+        if constexpr (kFold) {
+            // along k: this thread's four k; across: the stored rows of its pieces, which repeat after four
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+                sc[i] = fold != nullptr && a.tile < walk.tiles ? half_at(fold + a.kb * kKB + (ACROSS ? (srow_of(i) & 63) : 4 * p + i)) : 1.f;
         }
     };
+    At ahead{walk.first, walk.kb0, 0, nullptr};
+    enter(ahead);
+    advance(ahead, g);
+    At now = ahead;
+    load_scales(now);
 #pragma unroll
-    for (int d = 0; d < kDepth; ++d)
-        if (d < kblocks) load_slot(d, d);
-    int s = 0;
-    uint32_t round = 0;  // how many times the ring has wrapped
-    for (int kb = 0; kb < kblocks; ++kb) {
-        if (kb + kDepth < kblocks) load_slot(kDepth, kb + kDepth);
-        if (round > 0 && !wait_bounded(ring.bar_empty + 8 * s, (round - 1) & 1, status)) return false;
-        const uint32_t tile = ring.sbase + s * ring.stage_bytes + tile_off;
+    for (int d = 0; d < kDepth; ++d) {
+        stage_in(d, ahead);
+        advance(ahead, groups);
+    }
+    int s = g % ring.stages;
+    uint32_t round = g / ring.stages;  // how many times the ring has wrapped
+    uint32_t slot = 0;
+    while (now.tile < walk.tiles) {
+        cp_async_wait<kDepth - 1>();
+        uint4 raw[kPer];
 #pragma unroll
-        for (int i = 0; i < kLpr; ++i) {
-            const int v = valid_of(i);
-            const float si = kScaled ? sc[0][kScaled ? i : 0] : 1.f;
-            if (v == kPerWord) {
-                convert_word<KIND, kScaled, false>(buf[0][i], tile, srow_of(i), p, si, v);
+        for (int i = 0; i < kPer; ++i) raw[i] = f4k::lds128(staging + (slot * kPer + i) * pitch16);
+        float si[kScales];
+#pragma unroll
+        for (int i = 0; i < kScales; ++i) si[i] = sc[i];
+        At next = now;
+        advance(next, groups);
+        load_scales(next);
+        stage_in(slot, ahead);
+        advance(ahead, groups);
+        slot = slot + 1 == kDepth ? 0 : slot + 1;
+        if (round > 0) {  // one answer for the warp
+            const bool ok = wait_bounded(ring.bar_empty + 8 * s, (round - 1) & 1, status);
+            if (!__all_sync(0xFFFFFFFFu, ok)) break;
+        }
+        const uint32_t dst = ring.sbase + s * ring.stage_bytes + tile_off;
+#pragma unroll
+        for (int i = 0; i < kPer; ++i) {
+            if (!active(i)) continue;
+            if constexpr (INT8) {
+                convert_piece_int8<KIND>(raw[i], dst, srow_of(i), p);
             } else {
-                convert_word<KIND, kScaled, true>(buf[0][i], tile, srow_of(i), p, si, v);
+                float f[4] = {1.f, 1.f, 1.f, 1.f};
+                if constexpr (kFold) {
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) f[j] = si[ACROSS ? (i & 3) : j];
+                }
+                const float scale = SCALED ? si[SCALED ? i : 0] : 1.f;
+                const int v = ACROSS ? valid_of(i, now.row0, now.kb) : kElems;  // rows that do not exist were staged as zeros
+                if (v == kElems) {
+                    convert_piece<KIND, SCALED, false>(raw[i], dst, srow_of(i), p, scale, f, v);
+                } else {
+                    convert_piece<KIND, SCALED, true>(raw[i], dst, srow_of(i), p, scale, f, v);
+                }
             }
         }
         fence_proxy_async();  // written through the generic proxy, read by the tensor core through the async one
-        mbar_arrive(ring.bar_full + 8 * s);
-#pragma unroll
-        for (int d = 0; d < kDepth; ++d) {
-#pragma unroll
-            for (int i = 0; i < kLpr; ++i) {
-                buf[d][i] = buf[d + 1][i];
-                if constexpr (kScaled) sc[d][i] = sc[d + 1][i];
-            }
+        __syncwarp();
+        if ((threadIdx.x & 31) == 0) mbar_arrive(ring.bar_full + 8 * s);
+        now = next;
+        s += groups;
+        while (s >= ring.stages) s -= ring.stages, ++round;
+    }
+    cp_async_wait<0>();  // no copy of this CTA may be in flight when it leaves
+}
+
+// bf16 operands: one thread has their tiles brought in by TMA (elements outside the operand arrive as zeros)
+__device__ __forceinline__ void load_tiles(const Operand& op, const CUtensorMap* map, const Span& span, int tile, int kb, uint32_t dst, uint32_t bar) {
+    const int row0 = span.row0(tile);
+    if (op.transposed) {
+        const int boxes = (span.lim + 63) / 64;
+        mbar_expect_tx(bar, boxes * 8192u);
+        for (int h = 0; h < boxes; ++h) tma_load_2d(dst + 8192u * h, map, row0 + 64 * h, kb * kKB, bar);
+    } else {
+        mbar_expect_tx(bar, static_cast<uint32_t>(span.lim) * 128u);
+        tma_load_2d(dst, map, kb * kKB, row0, bar);
+    }
+}
+
+// `threads` producers (256, or 512 when the other operand comes by TMA) as groups of one tile each
+template <int KIND, bool ACROSS, bool SCALED, bool INT8 = false>
+__device__ __forceinline__ void produce_groups(const Operand& op, int k_len, int t, int threads, uint32_t staging, const Span& span, uint32_t tile_off,
+                                               const Ring& ring, const Walk& walk, const uint16_t* fold, int* status) {
+    constexpr int kGroup = Pieces<KIND, INT8>::kThreads;
+    // never more groups than stages: a group that skips a whole turn of the ring would meet a barrier two phases behind
+    const int groups = threads / kGroup < ring.stages ? threads / kGroup : ring.stages;
+    if (t / kGroup >= groups) return;
+    produce<KIND, ACROSS, SCALED, INT8>(op, k_len, t / kGroup, groups, t % kGroup, staging + 16u * t, 16u * threads, span, tile_off, ring, walk, fold, status);
+}
+__device__ __forceinline__ void produce_any(const Params& p, const Operand& op, int t, int threads, uint32_t staging, const Span& span, uint32_t tile_off,
+                                            const Ring& ring, const Walk& walk, const uint16_t* fold) {
+    if (p.int8) {
+        switch (op.kind) {
+            case BFQ_OP_CODES2: return produce_groups<BFQ_OP_CODES2, false, false, true>(op, p.k, t, threads, staging, span, tile_off, ring, walk, fold, p.status);
+            case BFQ_OP_CODES4: return produce_groups<BFQ_OP_CODES4, false, false, true>(op, p.k, t, threads, staging, span, tile_off, ring, walk, fold, p.status);
+            default: return produce_groups<BFQ_OP_CODES8, false, false, true>(op, p.k, t, threads, staging, span, tile_off, ring, walk, fold, p.status);
         }
-        if (++s == ring.stages) s = 0, ++round;
     }
-    return true;
-}
-
-template <bool ACROSS>
-__device__ __forceinline__ bool produce_kind(const Operand& op, int r, int tile_row0, uint32_t tile_off, const Ring& ring,
-                                             int kblocks, int* status) {
+    if (op.scaled) {
+        switch (op.kind) {
+            case BFQ_OP_CODES2: return produce_groups<BFQ_OP_CODES2, true, true>(op, p.k, t, threads, staging, span, tile_off, ring, walk, fold, p.status);
+            case BFQ_OP_CODES4: return produce_groups<BFQ_OP_CODES4, true, true>(op, p.k, t, threads, staging, span, tile_off, ring, walk, fold, p.status);
+            default: return produce_groups<BFQ_OP_CODES8, true, true>(op, p.k, t, threads, staging, span, tile_off, ring, walk, fold, p.status);
+        }
+    }
+    if (op.transposed) {
+        switch (op.kind) {
+            case BFQ_OP_F32: return produce_groups<BFQ_OP_F32, true, false>(op, p.k, t, threads, staging, span, tile_off, ring, walk, fold, p.status);
+            case BFQ_OP_CODES2: return produce_groups<BFQ_OP_CODES2, true, false>(op, p.k, t, threads, staging, span, tile_off, ring, walk, fold, p.status);
+            case BFQ_OP_CODES4: return produce_groups<BFQ_OP_CODES4, true, false>(op, p.k, t, threads, staging, span, tile_off, ring, walk, fold, p.status);
+            default: return produce_groups<BFQ_OP_CODES8, true, false>(op, p.k, t, threads, staging, span, tile_off, ring, walk, fold, p.status);
+        }
+    }
     switch (op.kind) {
-        case BFQ_OP_F32: return produce<BFQ_OP_F32, ACROSS>(op, r, tile_row0, tile_off, ring, kblocks, status);
-        case BFQ_OP_BF16: return produce<BFQ_OP_BF16, ACROSS>(op, r, tile_row0, tile_off, ring, kblocks, status);
-        case BFQ_OP_CODES2: return produce<BFQ_OP_CODES2, ACROSS>(op, r, tile_row0, tile_off, ring, kblocks, status);
-        case BFQ_OP_CODES4: return produce<BFQ_OP_CODES4, ACROSS>(op, r, tile_row0, tile_off, ring, kblocks, status);
-        default: return produce<BFQ_OP_CODES8, ACROSS>(op, r, tile_row0, tile_off, ring, kblocks, status);
+        case BFQ_OP_F32: return produce_groups<BFQ_OP_F32, false, false>(op, p.k, t, threads, staging, span, tile_off, ring, walk, fold, p.status);
+        case BFQ_OP_CODES2: return produce_groups<BFQ_OP_CODES2, false, false>(op, p.k, t, threads, staging, span, tile_off, ring, walk, fold, p.status);
+        case BFQ_OP_CODES4: return produce_groups<BFQ_OP_CODES4, false, false>(op, p.k, t, threads, staging, span, tile_off, ring, walk, fold, p.status);
+        default: return produce_groups<BFQ_OP_CODES8, false, false>(op, p.k, t, threads, staging, span, tile_off, ring, walk, fold, p.status);
+    }
+}
+// warps that arrive on a stage's barrier for one operand
+__device__ __forceinline__ uint32_t arrivals_of(const Operand& op) {
+    return op.kind == BFQ_OP_BF16 ? 1u : (op.kind == BFQ_OP_F32 ? 8u : 4u);
+}
+
+// The MMA warp of a pair's even CTA: every pair of terms, four K steps of 32 bytes per block.  The issue of a block must
+// take less than its MMAs (512 cycles at nt = 256 and one term pair): with a branch around one thread's loop, descriptors
+// built per MMA and a blocking wait per block it took 850.  So the warp stays converged, one thread's predicate is on the
+// instructions, the steps between descriptors are constants, and the next block's barrier is tested before this block's
+// products are issued.
+template <bool INT8, bool U_MN, bool V_MN>
+__device__ __forceinline__ void issue_products(const Params& p, const Ring& ring, const Walk& walk, uint32_t tmem_base, uint32_t bar_acc_full,
+                                               uint32_t bar_acc_empty, uint16_t mask) {
+    const uint32_t lead = elect_one() ? 1u : 0u;
+    const uint32_t idesc = make_idesc(INT8, p.nt, U_MN, V_MN);
+    // descriptors: start address in 16-byte units in the low bits, so steps are additions
+    constexpr uint64_t kUStep = (U_MN ? 2048u : 32u) >> 4, kVStep = (V_MN ? 2048u : 32u) >> 4, kTerm = kTileBytes >> 4;
+    const uint64_t u_desc = desc_sw128(ring.sbase, U_MN ? 8192u : 16u);
+    const uint64_t v_desc = desc_sw128(ring.sbase + p.u.terms * kTileBytes, V_MN ? 8192u : 16u);
+    const uint64_t stage_step = ring.stage_bytes >> 4;
+    const int blocks = walk.kb1 - walk.kb0;
+    int s = 0, n = 0;
+    uint32_t parity = 0;
+    bool ready = false;
+    for (int tile = walk.first; tile < walk.tiles; tile += walk.step, ++n) {
+        const int buf = n & 1;
+        if (n >= 2 && !wait_warp(bar_acc_empty + 8 * buf, ((n >> 1) - 1) & 1, p.status)) return;
+        tmem_fence_after();
+        const uint32_t d = tmem_base + buf * kMaxNt;
+        uint32_t accumulate = 0u;
+        for (int kb = 0; kb < blocks; ++kb) {
+            if (!ready && !wait_warp(ring.bar_full + 8 * s, parity, p.status)) return;
+            const int s_next = s + 1 == ring.stages ? 0 : s + 1;
+            const uint32_t parity_next = s_next == 0 ? parity ^ 1u : parity;
+            const bool next = mbar_test(ring.bar_full + 8 * s_next, parity_next);
+            tmem_fence_after();
+            const uint64_t ud = u_desc + s * stage_step, vd = v_desc + s * stage_step;
+            if (INT8 || (p.u.terms == 1 && p.v.terms == 1)) {
+#pragma unroll
+                for (int ks = 0; ks < 4; ++ks) {
+                    mma_pair<INT8>(lead, d, ud + ks * kUStep, vd + ks * kVStep, idesc, accumulate);
+                    accumulate = 1u;
+                }
+            } else {
+                for (int iu = 0; iu < p.u.terms; ++iu)
+                    for (int iv = 0; iv < p.v.terms; ++iv) {
+#pragma unroll
+                        for (int ks = 0; ks < 4; ++ks) {
+                            mma_pair<false>(lead, d, ud + iu * kTerm + ks * kUStep, vd + iv * kTerm + ks * kVStep, idesc, accumulate);
+                            accumulate = 1u;
+                        }
+                    }
+            }
+            mma_commit(lead, ring.bar_empty + 8 * s, mask);  // both CTAs may refill the stage
+            s = s_next, parity = parity_next;
+            ready = __all_sync(0xFFFFFFFFu, next);
+        }
+        mma_commit(lead, bar_acc_full + 8 * buf, mask);
     }
 }
 
-__global__ void __launch_bounds__(kProducers + 32, 1) k_dequant_gemm(const Params p) {
+__global__ void __launch_bounds__(kThreads, 1)
+k_dequant_gemm(const __grid_constant__ Params p, const __grid_constant__ CUtensorMap map_u, const __grid_constant__ CUtensorMap map_v) {
     extern __shared__ uint8_t smem_raw[];
-    const uint32_t sbase = (smem_u32(smem_raw) + 1023u) & ~1023u;
-    const int tid = threadIdx.x, warp = tid >> 5;
-    const int ta = terms_of(p.a.kind, p.a.transposed), tb = terms_of(p.b.kind, p.b.transposed);
+    const uint32_t sbase = (smem_u32(smem_raw) + 1023u) & ~1023u;  // the same offset in both CTAs of a pair
+    const int tid = threadIdx.x, warp = __shfl_sync(0xFFFFFFFFu, tid >> 5, 0);
+    // clusters are consecutive CTAs: the rank in the cluster from the (warp-uniform) block index
+    const uint32_t rank = p.split == 1 ? blockIdx.x & 1u : blockIdx.x % (2u * p.split), leader = rank & ~1u;
+    const int half = static_cast<int>(rank & 1u);
     Ring ring;
     ring.sbase = sbase;
-    ring.stage_bytes = static_cast<uint32_t>(ta + tb) * kTileBytes;
-    ring.stages = stages_of(ta, tb);
-    const uint32_t bars = sbase + kRingBytes;  // full[6], empty[6], done, then the tensor-memory address
+    ring.stage_bytes = static_cast<uint32_t>(p.u.terms + p.v.terms) * kTileBytes;
+    ring.stages = stages_of(!(p.u.kind == BFQ_OP_BF16 && p.v.kind == BFQ_OP_BF16), p.u.terms, p.v.terms);
+    // barriers: full[6] (a stage's operand tiles are in place: this CTA's and, in the even CTA, the odd CTA's too),
+    // empty[6], acc_full[2], acc_empty[2] (even CTA), then the tensor-memory address
+    const uint32_t bars = sbase + kBarsOff;
     ring.bar_full = bars, ring.bar_empty = bars + 8 * kMaxStages;
-    const uint32_t bar_done = bars + 16 * kMaxStages, tmem_slot = bar_done + 8;
+    const uint32_t bar_acc_full = bars + 16 * kMaxStages, bar_acc_empty = bar_acc_full + 16;
+    const uint32_t tmem_slot = bar_acc_empty + 16;
 
-    if (warp == 0) tmem_alloc128(tmem_slot);
-    if (tid == kProducers) {
+    grid_dep_launch();
+    if (warp == 0) tmem_alloc_pair(tmem_slot);
+    if (tid == kIssuer) {
+        const uint32_t arrivals = arrivals_of(p.u) + arrivals_of(p.v) + (half == 0 ? 1u : 0u);
         for (int s = 0; s < kMaxStages; ++s) {
-            mbar_init(ring.bar_full + 8 * s, kProducers);
+            mbar_init(ring.bar_full + 8 * s, arrivals);
             mbar_init(ring.bar_empty + 8 * s, 1);
         }
-        mbar_init(bar_done, 1);
+        for (int b = 0; b < 2; ++b) mbar_init(bar_acc_full + 8 * b, 1), mbar_init(bar_acc_empty + 8 * b, 2 * kEpi / 32);
         mbar_init_fence();
     }
     tmem_fence_before();
     __syncthreads();
+    cluster_sync_all();  // the peers' barriers are initialised
     tmem_fence_after();
     uint32_t tmem_base;
     asm volatile("ld.shared.u32 %0, [%1];" : "=r"(tmem_base) : "r"(tmem_slot));
+    grid_dep_wait();
 
-    const int m0 = blockIdx.x * kTile, n0 = blockIdx.y * kTile;
-    const int kblocks = p.k / kKB;
-    bool ok = true;
+    Walk walk;
+    int slice = 0;
+    if (p.split == 1) {
+        walk.first = blockIdx.x >> 1, walk.step = gridDim.x >> 1, walk.tiles = p.tiles, walk.kb0 = 0, walk.kb1 = p.kblocks;
+    } else {
+        slice = static_cast<int>(rank >> 1);
+        walk.first = blockIdx.x / (2 * p.split), walk.step = p.tiles, walk.tiles = p.tiles;
+        walk.kb0 = p.kblocks * slice / p.split, walk.kb1 = p.kblocks * (slice + 1) / p.split;
+    }
+    const int hv = p.nt >> 1;  // rows of A per CTA
 
-    if (tid < kProducers) {
-        // ---- producers: threads 0..127 build A's tiles, 128..255 B's ----
-        const bool for_a = tid < kTile;
-        const int r = tid & (kTile - 1);
-        const Operand& op = for_a ? p.a : p.b;
-        const uint32_t tile_off = for_a ? 0u : static_cast<uint32_t>(ta) * kTileBytes;
-        ok = op.transposed ? produce_kind<true>(op, r, for_a ? m0 : n0, tile_off, ring, kblocks, p.status)
-                           : produce_kind<false>(op, r, for_a ? m0 : n0, tile_off, ring, kblocks, p.status);
-        // ---- epilogue: accumulators -> alpha * row scale * column scale -> C ----
-        if (ok) ok = wait_bounded(bar_done, 0, p.status);
-        ok = __all_sync(0xFFFFFFFFu, ok);  // the tensor-memory loads below are warp-wide
-        tmem_fence_after();
-        if (ok) {
-            // warp w reads lanes 32 (w & 3) .. +31 (rows of the tile) and columns 64 (w >> 2) .. +63
-            const int ra = m0 + 32 * (warp & 3) + (tid & 31);
-            const bool row_ok = ra < p.a.rows;
-            float rs = p.alpha;
-            if (row_ok && is_codes(p.a.kind) && !p.a.transposed) rs *= __half2float(__ushort_as_half(__ldg(p.a.scales + ra)));
-            const bool col_scaled = is_codes(p.b.kind) && !p.b.transposed;
-            float* crow = p.c + int64_t(row_ok ? ra : 0) * p.ldc + n0;
-            const bool vec = (p.ldc & 3) == 0 && (reinterpret_cast<uintptr_t>(p.c) & 15u) == 0;
-            const uint32_t tlane = tmem_base + (static_cast<uint32_t>((warp & 3) * 32) << 16);
-            const int cbase = 64 * (warp >> 2);
-            for (int c0 = cbase; c0 < cbase + 64; c0 += 32) {
+    // scales that do not vary along k multiply the finished column / row of C
+    const bool u_scales = is_codes(p.u.kind) && !p.u.transposed, v_scales = is_codes(p.v.kind) && !p.v.transposed;
+    auto u_scale = [&](int j) { return u_scales && j < p.u.rows ? p.alpha * __half2float(__ushort_as_half(__ldg(p.u.scales + j))) : p.alpha; };
+    auto v_scale = [&](int i) { return v_scales && i < p.v.rows ? __half2float(__ushort_as_half(__ldg(p.v.scales + i))) : 1.f; };
+
+    auto span_of = [&](bool u) {
+        Span span;
+        span.tiles_v = p.tiles_v, span.is_u = u, span.half = half;
+        span.row_tile = u ? 2 * kRows : p.nt, span.lim = u ? kRows : hv;
+        return span;
+    };
+    // an accumulator as a number: the integer path's come with the places its codes were left in
+    auto number = [&](uint32_t acc) { return p.int8 ? __int2float_rn(static_cast<int>(acc)) * p.unit : __uint_as_float(acc); };
+
+    if (tid < kEpi) {
+        // ---- epilogue: lane = column of C, accumulator column = row of C ----
+        const uint32_t tlane = tmem_base + (static_cast<uint32_t>(warp * 32) << 16);
+        const uint32_t empty_at_leader = map_to_cta(bar_acc_empty, leader);
+        bool ok = true;
+        int n = 0;
+        for (int tile = walk.first; tile < walk.tiles; tile += walk.step, ++n) {
+            const int buf = n & 1;
+            ok = wait_bounded(bar_acc_full + 8 * buf, (n >> 1) & 1, p.status);
+            ok = __all_sync(0xFFFFFFFFu, ok);  // the tensor-memory loads below are warp-wide
+            if (!ok || p.split > 1) break;
+            tmem_fence_after();
+            const int j = (tile / p.tiles_v) * (2 * kRows) + half * kRows + tid, i0 = (tile % p.tiles_v) * p.nt;
+            const bool col_ok = j < p.u.rows;
+            const float us = u_scale(j);
+            float* out = p.c + int64_t(i0) * p.ldc + j;
+            for (int c0 = 0; c0 < p.nt; c0 += 32) {
                 uint32_t acc[32];
-                tmem_ld32(tlane + c0, acc);
+                tmem_ld32(tlane + buf * kMaxNt + c0, acc);
                 tmem_wait_ld32(acc);
-                float out[32];
 #pragma unroll
-                for (int j = 0; j < 32; ++j) {
-                    float cs = rs;
-                    if (col_scaled && n0 + c0 + j < p.b.rows) cs *= __half2float(__ushort_as_half(__ldg(p.b.scales + n0 + c0 + j)));
-                    out[j] = __uint_as_float(acc[j]) * cs;
-                }
-                if (!row_ok) continue;
-                if (vec && n0 + c0 + 32 <= p.b.rows) {
-#pragma unroll
-                    for (int j = 0; j < 32; j += 4)
-                        *reinterpret_cast<float4*>(crow + c0 + j) = make_float4(out[j], out[j + 1], out[j + 2], out[j + 3]);
-                } else {
-#pragma unroll
-                    for (int j = 0; j < 32; ++j)
-                        if (n0 + c0 + j < p.b.rows) crow[c0 + j] = out[j];
+                for (int i = 0; i < 32; ++i) {
+                    const float v = number(acc[i]) * (us * v_scale(i0 + c0 + i));
+                    if (col_ok && i0 + c0 + i < p.v.rows) out[int64_t(c0 + i) * p.ldc] = v;
                 }
             }
+            tmem_fence_before();
+            __syncwarp();
+            if ((tid & 31) == 0) mbar_arrive_remote(empty_at_leader + 8 * buf);
         }
-    } else if (tid == kProducers) {
-        // ---- one thread issues the MMAs: every pair of terms, four K steps of 16 per block ----
-        const uint32_t idesc = make_idesc(p.a.transposed, p.b.transposed);
-        const uint32_t a_step = p.a.transposed ? 2048u : 32u, b_step = p.b.transposed ? 2048u : 32u;
-        const uint32_t a_lead = p.a.transposed ? 8192u : 16u, b_lead = p.b.transposed ? 8192u : 16u;
+    } else if (tid < kIssuer) {
+        // ---- producers ----
+        // both operands converted: 256 threads each; one of them bf16 (TMA): all 512 convert the other
+        const bool u_tma = p.u.kind == BFQ_OP_BF16, v_tma = p.v.kind == BFQ_OP_BF16;
+        const int t = tid - kEpi;
+        // staging: 64 KB above the ring, half of it for each operand when both are converted
+        const uint32_t staging = sbase + kRingTilesStaged * kTileBytes;
+        auto convert = [&](bool u, int tt, int threads) {
+            const Operand& op = u ? p.u : p.v;
+            const Operand& other = u ? p.v : p.u;
+            const uint16_t* fold = is_codes(other.kind) && other.transposed && !other.scaled ? other.scales : nullptr;
+            produce_any(p, op, tt, threads, staging + (u || threads > kProd ? 0u : kStagingBytes / 2), span_of(u), u ? 0u : static_cast<uint32_t>(p.u.terms) * kTileBytes, ring, walk, fold);
+        };
+        if (u_tma != v_tma) {
+            convert(!u_tma, t, 2 * kProd);
+        } else if (!u_tma) {
+            convert(t < kProd, t & (kProd - 1), kProd);
+        }
+    } else if (tid == kLoader) {
+        const bool u_tma = p.u.kind == BFQ_OP_BF16, v_tma = p.v.kind == BFQ_OP_BF16;
+        const Span su = span_of(true), sv = span_of(false);
+        int s = 0, issued = 0;
+        uint32_t round = 0;
+        bool ok = u_tma || v_tma;
+        for (int tile = walk.first; ok && tile < walk.tiles; tile += walk.step) {
+            for (int kb = walk.kb0; kb < walk.kb1; ++kb) {
+                if (round > 0 && !wait_bounded(ring.bar_empty + 8 * s, (round - 1) & 1, p.status)) {
+                    // no copy of this CTA may be in flight when it leaves
+                    for (int i = issued > ring.stages ? issued - ring.stages : 0; i < issued; ++i)
+                        wait_bounded(ring.bar_full + 8 * (i % ring.stages), (i / ring.stages) & 1, p.status);
+                    ok = false;
+                    break;
+                }
+                const uint32_t dst = sbase + s * ring.stage_bytes, bar = ring.bar_full + 8 * s;
+                if (u_tma) load_tiles(p.u, &map_u, su, tile, kb, dst, bar);
+                if (v_tma) load_tiles(p.v, &map_v, sv, tile, kb, dst + p.u.terms * kTileBytes, bar);
+                ++issued;
+                if (++s == ring.stages) s = 0, ++round;
+            }
+        }
+    } else if (warp == kIssuer / 32 && half == 0) {
+        const uint16_t mask = static_cast<uint16_t>(3u << leader);
+        const uint32_t base = __shfl_sync(0xFFFFFFFFu, tmem_base, 0);
+        if (p.int8) {
+            issue_products<true, false, false>(p, ring, walk, base, bar_acc_full, bar_acc_empty, mask);
+        } else if (p.u.transposed) {
+            if (p.v.transposed) issue_products<false, true, true>(p, ring, walk, base, bar_acc_full, bar_acc_empty, mask);
+            else issue_products<false, true, false>(p, ring, walk, base, bar_acc_full, bar_acc_empty, mask);
+        } else {
+            if (p.v.transposed) issue_products<false, false, true>(p, ring, walk, base, bar_acc_full, bar_acc_empty, mask);
+            else issue_products<false, false, false>(p, ring, walk, base, bar_acc_full, bar_acc_empty, mask);
+        }
+    } else if (tid == kIssuer) {
+        // ---- odd CTA: tell the even CTA which stages are in place here ----
+        const uint32_t leader_full = map_to_cta(ring.bar_full, leader);
+        const int total = walk.blocks();
         int s = 0;
         uint32_t round = 0;
-        for (int kb = 0; kb < kblocks; ++kb) {
-            ok = wait_bounded(ring.bar_full + 8 * s, round & 1, p.status);
-            if (!ok) break;
-            tmem_fence_after();
-            const uint32_t at = sbase + s * ring.stage_bytes, bt = at + ta * kTileBytes;
-            for (int ia = 0; ia < ta; ++ia)
-                for (int ib = 0; ib < tb; ++ib)
-#pragma unroll
-                    for (int ks = 0; ks < kKB / 16; ++ks)
-                        mma_bf16(tmem_base, desc_sw128(at + ia * kTileBytes + ks * a_step, a_lead),
-                                 desc_sw128(bt + ib * kTileBytes + ks * b_step, b_lead), idesc, (kb | ia | ib | ks) != 0 ? 1u : 0u);
-            mma_commit(ring.bar_empty + 8 * s);  // arrives when the MMAs issued so far have read their operands and finished
+        for (int at = 0; at < total; ++at) {
+            if (!wait_bounded(ring.bar_full + 8 * s, round & 1, p.status)) break;
+            mbar_arrive_remote(leader_full + 8 * s);
             if (++s == ring.stages) s = 0, ++round;
         }
-        if (ok) mma_commit(bar_done);
+    }
+    __syncwarp();
+
+    if (p.split > 1) {
+        // The pairs of the cluster hold partial sums of one tile.  Every CTA sends accumulator columns [w q, w (q + 1)) to
+        // the CTA of its parity in pair q (w = nt / split), into the ring that no MMA reads any more, and adds what it
+        // gets in the order of the pairs: layout [sending pair][column][lane].
+        cluster_sync_all();
+        const int w = p.nt / p.split;
+        if (tid < kEpi) {
+            tmem_fence_after();
+            const uint32_t tlane = tmem_base + (static_cast<uint32_t>(warp * 32) << 16);
+            for (int c0 = 0; c0 < p.nt; c0 += 8) {
+                uint32_t acc[8];
+                tmem_ld8(tlane + c0, acc);
+                tmem_wait_ld8(acc);
+                const int q = c0 / w;
+                const uint32_t dst = map_to_cta(sbase, static_cast<uint32_t>(2 * q + half)) +
+                                     4u * static_cast<uint32_t>((slice * w + (c0 - q * w)) * kRows + tid);
+#pragma unroll
+                for (int i = 0; i < 8; ++i) st_cluster_b32(dst + 4u * kRows * i, acc[i]);
+            }
+            tmem_fence_before();
+        }
+        cluster_sync_all();
+        const int tile = walk.first, lane = tid & (kRows - 1);
+        const int j = (tile / p.tiles_v) * (2 * kRows) + half * kRows + lane, i0 = (tile % p.tiles_v) * p.nt + slice * w;
+        if (tid < kIssuer && j < p.u.rows) {
+            const float us = u_scale(j);
+            for (int c = tid / kRows; c < w && i0 + c < p.v.rows; c += kIssuer / kRows) {
+                float sum = 0.f;
+                int isum = 0;
+                for (int q = 0; q < p.split; ++q) {
+                    uint32_t bits;
+                    asm volatile("ld.shared.u32 %0, [%1];" : "=r"(bits) : "r"(sbase + 4u * static_cast<uint32_t>((q * w + c) * kRows + lane)));
+                    isum += static_cast<int>(bits), sum += __uint_as_float(bits);
+                }
+                if (p.int8) sum = number(static_cast<uint32_t>(isum));
+                p.c[int64_t(i0 + c) * p.ldc + j] = sum * (us * v_scale(i0 + c));
+            }
+        }
     }
     tmem_fence_before();
-    __syncthreads();
-    if (warp == 0) tmem_dealloc128(tmem_base);
+    cluster_sync_all();  // nobody's barriers or operand tiles are in use by a peer any more
+    if (warp == 0) tmem_dealloc_pair(tmem_base);
+}
+
+// ---- host side ---------------------------------------------------------------------------------------------------
+static Operand make_operand(const void* data, const uint16_t* scales, int64_t ld, int kind, int transposed, int rows, int other_kind) {
+    Operand op{data, scales, ld, kind, transposed, rows, 1, 0};
+    op.scaled = is_codes(kind) && transposed && other_kind != BFQ_OP_F32;  // else the scales go into the fp32 operand
+    op.terms = kind == BFQ_OP_F32 || op.scaled ? 2 : 1;
+    return op;
+}
+
+static int code_shift(int kind) {
+    return kind == BFQ_OP_CODES2 ? Int8Chunk<BFQ_OP_CODES2>::kShift : (kind == BFQ_OP_CODES4 ? Int8Chunk<BFQ_OP_CODES4>::kShift : 0);
+}
+
+static bool encode_operand(CUtensorMap* map, const Operand& op, int64_t k, int box_rows) {
+    // stored [rows][K]: box of 64 k x box_rows rows; stored [K][rows]: box of 64 rows x 64 k
+    const cuuint64_t inner = static_cast<cuuint64_t>(op.transposed ? op.rows : k), outer = static_cast<cuuint64_t>(op.transposed ? k : op.rows);
+    const cuuint64_t dims[2] = {inner, outer};
+    const cuuint64_t strides[1] = {static_cast<cuuint64_t>(op.ld) * 2};
+    const cuuint32_t box[2] = {kKB, static_cast<cuuint32_t>(op.transposed ? kKB : box_rows)};
+    const cuuint32_t estr[2] = {1, 1};
+    return encode_tiled() != nullptr &&
+           encode_tiled()(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(op.data), dims, strides, box, estr,
+                          CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
+                          CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
+struct Shape {
+    int nt, tiles_v, tiles, split;
+};
+// Rows of A per tile and pairs per tile.  Model in SM cycles: a round of a pair is its K blocks at the slower of the
+// tensor core (nt / 2 cycles per K step and term pair) and shared memory (operands written once and read once, 128 bytes
+// a cycle: 64 + nt / 4), plus what a tile costs besides (filling the ring, draining the accumulators); a tile shared by
+// 2 or 4 pairs has that much less of K and an exchange more, and is worth it only while all the pairs run at once.
+// nt_step: 32 (the MMA's N step), or more where A is codes stored [K][rows]: a CTA's half of the tile has to start on a
+// whole 16-byte piece.
+static Shape choose_shape(int64_t m, int64_t n, int kblocks, int term_pairs, int nt_step, int sms) {
+    const int64_t pairs = sms / 2 > 0 ? sms / 2 : 1, tiles_u = (n + 2 * kRows - 1) / (2 * kRows);
+    Shape best{};
+    double best_cost = 0.0;
+    for (int nt = kMaxNt; nt >= nt_step; nt -= nt_step) {
+        const int64_t tiles_v = (m + nt - 1) / nt, tiles = tiles_u * tiles_v;
+        const int step = nt / 2 > 64 + nt / 4 ? nt / 2 : 64 + nt / 4;
+        for (int split = 1; split <= 4; split *= 2) {
+            if (split > 1 && (tiles * split > pairs || kblocks < 4 * split)) break;
+            const int64_t rounds = split > 1 ? 1 : (tiles + pairs - 1) / pairs;
+            const double cost = double(rounds) * ((kblocks + split - 1) / split) * (kKB / 16) * step * term_pairs +
+                                double(rounds) * 500 + 2000 + 16 * nt + (split > 1 ? 2000 : 0);
+            if (best.nt == 0 || cost < best_cost) best_cost = cost, best = Shape{nt, int(tiles_v), int(tiles), split};
+        }
+    }
+    return best;
+}
+
+static cudaError_t launch(const Params& p, const CUtensorMap& map_u, const CUtensorMap& map_v, int sms, size_t smem, cudaStream_t st) {
+    cudaLaunchConfig_t cfg = {};
+    const int pairs = p.split > 1 ? p.tiles * p.split : (p.tiles < sms / 2 ? p.tiles : (sms / 2 > 0 ? sms / 2 : 1));
+    cfg.gridDim = dim3(unsigned(2 * pairs)), cfg.blockDim = dim3(kThreads), cfg.dynamicSmemBytes = smem, cfg.stream = st;
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = unsigned(2 * p.split), attr[0].val.clusterDim.y = 1, attr[0].val.clusterDim.z = 1;
+    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[1].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr, cfg.numAttrs = 2;
+    return cudaLaunchKernelEx(&cfg, k_dequant_gemm, p, map_u, map_v);
 }
 
 }  // namespace dqg
@@ -512,20 +989,30 @@ extern "C" int bfq_dequant_gemm(bfq_plan* plan, int64_t m, int64_t n, int64_t k,
     if (k == 0) {
         e = cudaMemset2DAsync(c, size_t(ldc) * 4, 0, size_t(n) * 4, size_t(m), static_cast<cudaStream_t>(stream));
     } else {
-        constexpr size_t smem = size_t(kRingBytes) + 8 * (2 * kMaxStages + 1) + 16 + 1024;
+        constexpr size_t smem = size_t(kBarsOff) + 8 * (2 * kMaxStages + 4) + 16 + 1024;
         static bool attr_set[bfq::kMaxDevices] = {false};
         if (!attr_set[plan->device]) {
             e = cudaFuncSetAttribute(k_dequant_gemm, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
             attr_set[plan->device] = (e == cudaSuccess);
         }
         if (e == cudaSuccess) {
-            Params p;
-            p.a = Operand{a, a_scales, lda, a_kind, a_transposed, int(m)};
-            p.b = Operand{b, b_scales, ldb, b_kind, b_transposed, int(n)};
+            Params p{};
+            p.u = make_operand(b, b_scales, ldb, b_kind, b_transposed, int(n), a_kind);
+            p.v = make_operand(a, a_scales, lda, a_kind, a_transposed, int(m), b_kind);
             p.c = c, p.ldc = ldc, p.k = int(k), p.alpha = alpha, p.status = plan->status_word;
-            const dim3 grid(unsigned((m + kTile - 1) / kTile), unsigned((n + kTile - 1) / kTile));
-            k_dequant_gemm<<<grid, kProducers + 32, smem, static_cast<cudaStream_t>(stream)>>>(p);
-            e = cudaGetLastError();
+            // Two code operands along K are an integer product: exact in 32 bits up to K = 2^17 - 1 (codes left in place are at
+            // most 128 in size), at twice the rate of the bf16 products.
+            p.int8 = is_codes(a_kind) && is_codes(b_kind) && !a_transposed && !b_transposed && k < (1 << 17);
+            p.unit = 1.f / float(1 << (code_shift(a_kind) + code_shift(b_kind)));
+            p.kblocks = p.int8 ? int((k + 2 * kKB - 1) / (2 * kKB)) : int(k / kKB);
+            const Shape shape = choose_shape(m, n, p.kblocks, p.u.terms * p.v.terms,
+                                             is_codes(a_kind) && a_transposed ? (a_kind == BFQ_OP_CODES8 ? 32 : 256 / a_kind) : 32,
+                                             plan->sm_count);
+            p.nt = shape.nt, p.tiles_v = shape.tiles_v, p.tiles = shape.tiles, p.split = shape.split;
+            CUtensorMap map_u{}, map_v{};
+            bool ok = b_kind != BFQ_OP_BF16 || encode_operand(&map_u, p.u, k, kRows);
+            ok = ok && (a_kind != BFQ_OP_BF16 || encode_operand(&map_v, p.v, k, p.nt / 2));
+            e = ok ? launch(p, map_u, map_v, plan->sm_count, smem, static_cast<cudaStream_t>(stream)) : cudaErrorInvalidValue;
         }
     }
     if (prev != plan->device) cudaSetDevice(prev);

@@ -79,6 +79,26 @@ def test_exact_integer_product_of_two_code_operands():
     assert np.abs(c - ref).max() <= 2.0 ** -22 * np.abs(ref).max()   # two roundings (scales) of an exact sum
 
 
+@pytest.mark.parametrize("ka,kb,ta,tb", [("bf16", "codes2", False, False), ("codes4", "codes8", False, False),
+                                         ("codes2", "codes4", False, False), ("bf16", "bf16", False, False),
+                                         ("bf16", "codes4", True, True), ("f32", "codes8", False, True), ("f32", "codes2", True, True)])
+@pytest.mark.parametrize("m,n,k", [(1, 256, 64),         # one row, one K block
+                                   (32, 257, 1088),      # a tile's K shared by several pairs of CTAs, an odd number of blocks
+                                   (130, 640, 448),      # half a K block left over on the integer path
+                                   (1025, 5120, 192),    # more tiles than pairs, a ragged last one
+                                   (290, 36864, 64)])    # several turns of a short ring per pair
+def test_tile_edges(ka, kb, ta, tb, m, n, k):
+    if ta:
+        m = (m + 15) // 16 * 16                           # stored rows are 16-byte multiples
+    if tb:
+        n = (n + 63) // 64 * 64
+    p = Plan(256, DEV)
+    A, a64, ea = operand(ka, m, k, ta, 920)
+    B, b64, eb = operand(kb, n, k, tb, 921)
+    # scales folded into an fp32 operand: one more rounding to fp32
+    check(p, A, a64, ea, B, b64, eb + (2.0 ** -24 if tb and ka == "f32" else 0.0))
+
+
 def test_argument_validation():
     from paper_2509_09679_b200 import BfqError
     p = Plan(256, DEV)
