@@ -59,6 +59,18 @@ static int check_rows(const void* p, int dt, int64_t rows, int64_t ld, int n) {
     return BFQ_OK;
 }
 
+// Rows of 128 .. 2048 elements on the n = 4096 kernels, several as one.  Measured against the generic kernels from 2^13 to
+// 2^25 elements in all (us; bf16, n = 1024; 2^13 / 2^20 / 2^25 elements): codes 8.1 -> 5.2 / 8.7 -> 6.6 / 144 -> 40, rows
+// 7.0 -> 5.0 / 7.6 -> 6.3 / 166 -> 36: always faster.  Inverse 7.2 -> 5.4 / 7.7 -> 6.9 / 168 -> 43, but for n = 128 in fp32
+// the other way round up to 2^20 (6.7 against 7.5).  Backward: filling the tensor memory takes 27 us whatever the size, against
+// 16 - 18 us and 18 - 21 us of the generic kernel on small batches; they meet at about 2^18 elements for n <= 256 (38 against
+// 31, 27 against 29) and 2^19 above (24 against 29 at 1024, 31 against 29 at 512).
+static bool use_short_rows(const bfq_plan* plan, int64_t rows, int64_t min_elems) {
+    return rows < (int64_t(1) << 31) - 64 && rows * plan->n >= min_elems && !env_flag("BFQ_GENERIC_ONLY") && fwdq_short_available(plan);
+}
+static int64_t short_inverse_from(int n) { return n == 128 ? int64_t(1) << 21 : 0; }
+static int64_t short_backward_from(int n) { return n <= 256 ? int64_t(1) << 18 : int64_t(1) << 20; }
+
 // ---- generic kernel dispatch ------------------------------------------------------------------------
 template <int LOG_N, int R, int MODE>
 static cudaError_t launch_generic_t(const bfq_plan* plan, const GenericParams& p, cudaStream_t st) {
@@ -160,29 +172,11 @@ static int64_t backward_slots(int log_n, int sm_count) {
 
 // frees everything a plan owns (every pointer is null or valid) and the plan itself
 static void release_plan(bfq_plan* plan) {
-    cudaFree(plan->tw);
-    cudaFree(plan->img4096);
-    cudaFree(plan->prep4096);
-    cudaFree(plan->img_b4096);
-    cudaFree(plan->img_i4096);
-    cudaFree(plan->img8192);
-    cudaFree(plan->prep8192);
-    for (int h = 0; h < 2; ++h) {
-        cudaFree(plan->img_b8192[h]);
-        cudaFree(plan->img_i8192[h]);
-        cudaFree(plan->dsign8192[h]);
-        cudaFree(plan->gsign8192[h]);
-    }
-    cudaFree(plan->prep_half8192);
-    cudaFree(plan->dsign4096);
-    cudaFree(plan->gsign4096);
-    cudaFree(plan->partial);
-    cudaFree(plan->status_word);
+    cudaFree(plan->arena);
     if (plan->host_in != nullptr) cudaStreamDestroy(plan->host_in);
     if (plan->host_out != nullptr) cudaStreamDestroy(plan->host_out);
     for (int i = 0; i < 8; ++i)
         if (plan->host_ev[i] != nullptr) cudaEventDestroy(plan->host_ev[i]);
-    cudaFree(plan->dense128);
     if (plan->theta_host != nullptr) cudaFreeHost(plan->theta_host);
     if (plan->theta_event != nullptr) cudaEventDestroy(plan->theta_event);
     std::free(plan->comp5120);
@@ -213,37 +207,58 @@ int bfq_plan_create(bfq_plan** out, int n, int64_t max_rows, int device) {
     plan->n = n;
     plan->log_n = ilog2_exact(n);
     plan->device = device;
-    cudaDeviceProp prop;
-    e = cudaGetDeviceProperties(&prop, device);
+    // the two attributes alone: a full cudaGetDeviceProperties takes milliseconds
+    e = cudaDeviceGetAttribute(&plan->sm_count, cudaDevAttrMultiProcessorCount, device);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&plan->cc_major, cudaDevAttrComputeCapabilityMajor, device);
     if (e != cudaSuccess) {
         delete plan;
         return cuda_fail(nullptr, e);
     }
-    plan->sm_count = prop.multiProcessorCount;
-    plan->cc_major = prop.major;
     const size_t angles = size_t(plan->log_n) * (n / 2);
     plan->partial_slots = backward_slots(plan->log_n, plan->sm_count);
-    e = cudaMalloc(&plan->tw, angles * sizeof(float2));
     plan->partial_floats = size_t(plan->partial_slots) * angles;
     if (n == 8192 && plan->partial_floats < bwd8192_partial_floats(plan->sm_count))
         plan->partial_floats = bwd8192_partial_floats(plan->sm_count);
-    if (e == cudaSuccess) e = cudaMalloc(&plan->partial, plan->partial_floats * sizeof(float));
-    if (e == cudaSuccess && n == 4096) e = cudaMalloc(&plan->img4096, fwdq4096_image_bytes());
-    if (e == cudaSuccess && n == 4096) e = cudaMalloc(&plan->prep4096, fwdq4096_prep_bytes());
-    if (e == cudaSuccess && n == 8192) e = cudaMalloc(&plan->img8192, fwdq8192_image_bytes());
-    if (e == cudaSuccess && n == 8192) e = cudaMalloc(&plan->prep8192, fwdq8192_prep_bytes());
-    for (int h = 0; h < 2 && n == 8192; ++h) {
-        if (e == cudaSuccess) e = cudaMalloc(&plan->img_b8192[h], bwd4096_image_bytes());
-        if (e == cudaSuccess) e = cudaMalloc(&plan->img_i8192[h], inv4096_image_bytes());
-        if (e == cudaSuccess) e = cudaMalloc(&plan->dsign8192[h], bwd4096_dsign_bytes());
-        if (e == cudaSuccess) e = cudaMalloc(&plan->gsign8192[h], bwd4096_gsign_bytes());
+    if (n >= 128 && n < 4096 && plan->partial_floats < bwd_short_partial_floats(plan->sm_count))
+        plan->partial_floats = bwd_short_partial_floats(plan->sm_count);
+    // all device memory in one allocation
+    struct Part {
+        void** at;
+        size_t bytes;
+    };
+    Part parts[24];
+    int n_parts = 0;
+    auto want = [&](auto** at, size_t bytes) { parts[n_parts++] = Part{reinterpret_cast<void**>(at), (bytes + 255) / 256 * 256}; };
+    want(&plan->tw, angles * sizeof(float2));
+    want(&plan->partial, plan->partial_floats * sizeof(float));
+    if (n >= 128 && n <= 4096) {
+        want(&plan->img4096, fwdq4096_image_bytes());
+        want(&plan->prep4096, fwdq4096_prep_bytes());
+        want(&plan->img_b4096, bwd4096_image_bytes());
+        want(&plan->img_i4096, inv4096_image_bytes());
+        want(&plan->dsign4096, bwd4096_dsign_bytes());
+        want(&plan->gsign4096, bwd4096_gsign_bytes());
     }
-    if (e == cudaSuccess && n == 8192) e = cudaMalloc(&plan->prep_half8192, bwd8192_prep_bytes());
-    if (e == cudaSuccess && n == 4096) e = cudaMalloc(&plan->img_b4096, bwd4096_image_bytes());
-    if (e == cudaSuccess && n == 4096) e = cudaMalloc(&plan->img_i4096, inv4096_image_bytes());
-    if (e == cudaSuccess && n == 4096) e = cudaMalloc(&plan->dsign4096, bwd4096_dsign_bytes());
-    if (e == cudaSuccess && n == 4096) e = cudaMalloc(&plan->gsign4096, bwd4096_gsign_bytes());
-    if (e == cudaSuccess && n == 128) e = cudaMalloc(&plan->dense128, comp5120d_image_bytes());
+    if (n == 8192) {
+        want(&plan->img8192, fwdq8192_image_bytes());
+        want(&plan->prep8192, fwdq8192_prep_bytes());
+        for (int h = 0; h < 2; ++h) {
+            want(&plan->img_b8192[h], bwd4096_image_bytes());
+            want(&plan->img_i8192[h], inv4096_image_bytes());
+            want(&plan->dsign8192[h], bwd4096_dsign_bytes());
+            want(&plan->gsign8192[h], bwd4096_gsign_bytes());
+        }
+        want(&plan->prep_half8192, bwd8192_prep_bytes());
+    }
+    if (n == 128) want(&plan->dense128, comp5120d_image_bytes());
+    want(&plan->status_word, 4 * sizeof(int));
+    size_t total = 0;
+    for (int i = 0; i < n_parts; ++i) total += parts[i].bytes;
+    e = cudaMalloc(&plan->arena, total);
+    if (e == cudaSuccess) {
+        uint8_t* at = static_cast<uint8_t*>(plan->arena);
+        for (int i = 0; i < n_parts; ++i) *parts[i].at = at, at += parts[i].bytes;
+    }
     if (e == cudaSuccess && n == 128) {  // the composite kernel's constants are computed on the host from the angles
         e = cudaMallocHost(&plan->theta_host, angles * sizeof(float));
         if (e == cudaSuccess) e = cudaEventCreateWithFlags(&plan->theta_event, cudaEventDisableTiming);
@@ -255,7 +270,6 @@ int bfq_plan_create(bfq_plan** out, int n, int64_t max_rows, int device) {
     if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&plan->host_in, cudaStreamNonBlocking);
     if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&plan->host_out, cudaStreamNonBlocking);
     for (int i = 0; i < 8 && e == cudaSuccess; ++i) e = cudaEventCreateWithFlags(&plan->host_ev[i], cudaEventDisableTiming);
-    if (e == cudaSuccess) e = cudaMalloc(&plan->status_word, 4 * sizeof(int));
     if (e == cudaSuccess) e = cudaMemset(plan->status_word, 0, 4 * sizeof(int));
     if (e == cudaSuccess) plan->form_flag = plan->status_word + 1;
     if (e == cudaSuccess) e = cudaDeviceSynchronize();
@@ -283,6 +297,8 @@ int bfq_set_angles(bfq_plan* plan, const float* theta, void* stream) {
     cudaError_t e;
     if (plan->img4096 != nullptr) {
         e = fwdq4096_set_angles(plan, theta, static_cast<cudaStream_t>(stream));
+        // shorter rows: the reverse tables too, so that later calls on any stream find all tables built here
+        if (e == cudaSuccess && plan->n < 4096) e = bwd4096_build_tables(plan, static_cast<cudaStream_t>(stream));
     } else if (plan->img8192 != nullptr) {
         e = fwdq8192_set_angles(plan, theta, static_cast<cudaStream_t>(stream));
     } else {
@@ -332,6 +348,10 @@ int bfq_forward(bfq_plan* plan, const void* x, bfq_dtype xt, int64_t rows, int64
     if (xt == BFQ_BF16 && yt == BFQ_BF16 && x != y && rows < (int64_t(1) << 31) && !env_flag("BFQ_GENERIC_ONLY") &&
         fwdq8192_available(plan)) {
         cudaError_t e = fwdq8192_launch_bf16(plan, x, rows, ldx, y, ldy, static_cast<cudaStream_t>(stream));
+        return e == cudaSuccess ? BFQ_OK : cuda_fail(plan, e);
+    }
+    if (xt == yt && x != y && ldy == plan->n && use_short_rows(plan, rows, 0)) {
+        cudaError_t e = fwdq_short_launch(plan, x, xt == BFQ_F32, rows, ldx, 0, nullptr, nullptr, y, static_cast<cudaStream_t>(stream));
         return e == cudaSuccess ? BFQ_OK : cuda_fail(plan, e);
     }
     GenericParams p{};
@@ -402,6 +422,10 @@ static int forward_quant_impl(bfq_plan* plan, const void* x, int xt, int64_t row
     if (hist == nullptr && xt == BFQ_BF16 && y == nullptr && rows < (int64_t(1) << 31) &&
         !env_flag("BFQ_GENERIC_ONLY") && fwdq8192_available(plan)) {
         e = fwdq8192_launch(plan, x, rows, ldx, bits, codes, scales, static_cast<cudaStream_t>(stream));
+        return e == cudaSuccess ? BFQ_OK : cuda_fail(plan, e);
+    }
+    if (hist == nullptr && y == nullptr && use_short_rows(plan, rows, 0)) {
+        e = fwdq_short_launch(plan, x, xt == BFQ_F32, rows, ldx, bits, codes, scales, nullptr, static_cast<cudaStream_t>(stream));
         return e == cudaSuccess ? BFQ_OK : cuda_fail(plan, e);
     }
     GenericParams p{};
@@ -604,6 +628,11 @@ int bfq_inverse(bfq_plan* plan, const void* y, bfq_dtype yt, int64_t rows, int64
         if (e == cudaSuccess) e = inv8192_launch(plan, y, rows, ldy, x, xt == BFQ_BF16, ldx, st);
         return e == cudaSuccess ? BFQ_OK : cuda_fail(plan, e);
     }
+    if ((yt == BFQ_BF16 || xt == BFQ_F32) && x != y && ldx == plan->n && use_short_rows(plan, rows, short_inverse_from(plan->n)) &&
+        bwd_short_available(plan)) {
+        cudaError_t e = inv_short_launch(plan, y, yt == BFQ_F32, rows, ldy, x, xt == BFQ_BF16, static_cast<cudaStream_t>(stream));
+        return e == cudaSuccess ? BFQ_OK : cuda_fail(plan, e);
+    }
     GenericParams p{};
     p.tw = plan->tw, p.x = y, p.xt = yt, p.ldx = ldy, p.y = x, p.yt = xt, p.ldy = ldx, p.rows = rows;
     cudaError_t e = launch_generic<kModeInverse>(plan, p, static_cast<cudaStream_t>(stream));
@@ -646,6 +675,11 @@ int bfq_backward(bfq_plan* plan, const void* x, bfq_dtype xt, const void* g, bfq
             plan->bwd_tables_valid = (e == cudaSuccess);
         }
         if (e == cudaSuccess) e = bwd8192_launch_halves(plan, x, g, rows, ld, dx, dtheta, st);
+        return e == cudaSuccess ? BFQ_OK : cuda_fail(plan, e);
+    }
+    if (xt == gt && (dx == nullptr || dxt == xt) && ld == plan->n && use_short_rows(plan, rows, short_backward_from(plan->n)) &&
+        bwd_short_available(plan)) {
+        cudaError_t e = bwd_short_launch(plan, x, g, rows, dx, dtheta, xt == BFQ_F32, st);
         return e == cudaSuccess ? BFQ_OK : cuda_fail(plan, e);
     }
     BackwardParams p{};

@@ -132,18 +132,21 @@ struct Ctx {
     Addr a;
     uint32_t tlane;     // tensor-memory address of this thread's lane, column 0
     uint32_t acc_smem;  // this thread's first float4 of the shared-memory accumulators
+    int stages;         // SHORT: log2 of the row length, stages from there on are the identity and passed over
 };
 
 // ---- forward recompute: 24 chunks of 16 constants (two per stage), both rows ---------------------------
 // Chunk C is in Tcur; the next chunk is requested right after the wait.
-template <int C>
+template <int C, bool SHORT>
 __device__ __forceinline__ void fwd_chunks(u64 (&X0)[16], u64 (&X1)[16], uint32_t (&Tcur)[16], uint32_t (&Tnext)[16],
                                            const Ctx& cx) {
     constexpr int s = C / 2, K = s & 3, U0 = 4 * (C & 1);
     tmem_wait_ld16(Tcur);
     if constexpr (C + 1 < 24) tmem_ld16(cx.tlane + 16 * (C + 1), Tnext);
-    stage_lift<K, U0, 4, 16>(X0, Tcur);
-    stage_lift<K, U0, 4, 16>(X1, Tcur);
+    if (!SHORT || s < cx.stages) {
+        stage_lift<K, U0, 4, 16>(X0, Tcur);
+        stage_lift<K, U0, 4, 16>(X1, Tcur);
+    }
     if constexpr (C == 7) {  // inside each half-warp; the group-wide hand-off barrier of the previous row pair
                              // has put every other warp past its reads of these buffers
         fwd1_store(X0, cx.a.ex + 0 * kExBytes, cx.a);
@@ -160,7 +163,7 @@ __device__ __forceinline__ void fwd_chunks(u64 (&X0)[16], u64 (&X1)[16], uint32_
         fwd2_load(X0, cx.a.ex + 0 * kExBytes, cx.a);
         fwd2_load(X1, cx.a.ex + 1 * kExBytes, cx.a);
     }
-    if constexpr (C + 1 < 24) fwd_chunks<C + 1>(X0, X1, Tnext, Tcur, cx);
+    if constexpr (C + 1 < 24) fwd_chunks<C + 1, SHORT>(X0, X1, Tnext, Tcur, cx);
 }
 
 // ---- reverse walk: step I handles half c = I & 1 of stage s = 11 - I / 2 ---------------------------------
@@ -174,7 +177,7 @@ struct RevStep {
 };
 
 // steps I .. END-1 (END = 24: down to stage 0); hook(integral_constant<I>) runs after step I (regroupings, hand-off)
-template <int I, int END, class F>
+template <int I, int END, bool SHORT, class F>
 __device__ __forceinline__ void rev_steps(u64 (&Y0)[16], u64 (&Y1)[16], u64 (&G0)[16], u64 (&G1)[16],
                                           uint32_t (&Tcur)[16], uint32_t (&Tnext)[16], uint32_t (&Acur)[8],
                                           uint32_t (&Anext)[8], const Ctx& cx, F&& hook) {
@@ -192,7 +195,7 @@ __device__ __forceinline__ void rev_steps(u64 (&Y0)[16], u64 (&Y1)[16], u64 (&G0
         tmem_ld16(cx.tlane + N::kTCol, Tnext);
         if constexpr (N::kAccInTmem) tmem_ld8(cx.tlane + N::kAccCol, Anext);
     }
-    {
+    if (!SHORT || S::s < cx.stages) {
         u64 A[4];
 #pragma unroll
         for (int i = 0; i < 4; ++i) A[i] = pack2u(Acur[2 * i], Acur[2 * i + 1]);
@@ -206,14 +209,16 @@ __device__ __forceinline__ void rev_steps(u64 (&Y0)[16], u64 (&Y1)[16], u64 (&G0
         sts128(cx.acc_smem + S::kAccSmem, make_uint4(Acur[0], Acur[1], Acur[2], Acur[3]));
         sts128(cx.acc_smem + S::kAccSmem + kThreads * 16, make_uint4(Acur[4], Acur[5], Acur[6], Acur[7]));
     }
-    if constexpr (S::s > 0) {  // y below stage 0 is x again: not needed
-        stage_lift<S::K, S::U0, 4, 16>(Y0, Tcur);
-        stage_lift<S::K, S::U0, 4, 16>(Y1, Tcur);
+    if (!SHORT || S::s < cx.stages) {
+        if constexpr (S::s > 0) {  // y below stage 0 is x again: not needed
+            stage_lift<S::K, S::U0, 4, 16>(Y0, Tcur);
+            stage_lift<S::K, S::U0, 4, 16>(Y1, Tcur);
+        }
+        stage_lift<S::K, S::U0, 4, 16>(G0, Tcur);
+        stage_lift<S::K, S::U0, 4, 16>(G1, Tcur);
     }
-    stage_lift<S::K, S::U0, 4, 16>(G0, Tcur);
-    stage_lift<S::K, S::U0, 4, 16>(G1, Tcur);
     hook(std::integral_constant<int, I>());
-    if constexpr (I + 1 < END) rev_steps<I + 1, END>(Y0, Y1, G0, G1, Tnext, Tcur, Anext, Acur, cx, hook);
+    if constexpr (I + 1 < END) rev_steps<I + 1, END, SHORT>(Y0, Y1, G0, G1, Tnext, Tcur, Anext, Acur, cx, hook);
 }
 
 __device__ __forceinline__ uint32_t cvt_bf16x2(float lo, float hi) {
@@ -247,12 +252,21 @@ struct alignas(64) WideHalf {
     const int8_t* dsign;
 };
 
-template <bool IN_F32, bool WIDE = false>
+// rows shorter than 4096 (SHORT): 2^log rows of n = 4096 >> log elements go through the kernel as one row of 4096 whose last
+// stages are the identity (they are passed over, so that no row touches another one's infinities); `rows` counts those, the
+// last one may be short (`elems` elements in all, missing ones arrive as zeros).  x, g and dx contiguous.
+struct ShortRows {
+    int log;
+    int64_t elems;
+};
+
+template <bool IN_F32, bool WIDE = false, bool SHORT = false>
 __global__ void __launch_bounds__(kCtaThreads, 1)
 k_bwd4096(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ CUtensorMap gmap,
           const float* __restrict__ img_lo, const uint32_t* __restrict__ gsign_lo, const int8_t* __restrict__ dsign_lo,
           void* __restrict__ dx_out, int64_t ld, float* __restrict__ partial, int rows, int* __restrict__ status,
-          const float2* __restrict__ tw12, const __grid_constant__ WideHalf upper) {
+          const float2* __restrict__ tw12, const __grid_constant__ WideHalf upper, const ShortRows brief) {
+    static_assert(!(SHORT && WIDE), "one or the other");
     static_assert(!(IN_F32 && WIDE), "the wide mode takes bf16 rows");
     // wide mode: even CTAs work on the lower halves of the rows, odd CTAs on the upper halves (CTAs 2i and 2i + 1 take
     // the same row pairs at about the same time, so the second read of a g row comes from L2)
@@ -286,6 +300,7 @@ k_bwd4096(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ CUte
     Ctx cx;
     cx.tlane = tmem_base + (static_cast<uint32_t>(quarter * 32) << 16);
     cx.acc_smem = sbase + S::kAccOff + t * 16;
+    cx.stages = SHORT ? 12 - brief.log : 12;
     {
         const uint32_t t4 = (t >> 4) & 1, t5 = (t >> 5) & 1, t6 = (t >> 6) & 1;
         cx.a.ex = sbase + (is_fwd ? S::kExFOff : S::kExROff);  // the group's own regrouping buffers
@@ -315,10 +330,11 @@ k_bwd4096(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ CUte
         const int r0 = 2 * (first + k * stride);
         const uint32_t bar = bar_base + 8 * slot;
         mbar_expect_tx(bar, 2 * kInRow + 2 * kGRow);
-        tma_load_3d(xring + slot * kPairBytes, xm, 0, 0, r0, bar);
-        tma_load_3d(xring + slot * kPairBytes + kInRow, xm, 0, 0, r0 + 1, bar);
-        tma_load_3d(gring + slot * kPairBytes, &gmap, 0, 0, r0, bar);
-        tma_load_3d(gring + slot * kPairBytes + kGRow, &gmap, 0, 0, r0 + 1, bar);
+        const int at0 = SHORT ? r0 << brief.log : r0, at1 = SHORT ? (r0 + 1) << brief.log : r0 + 1;
+        tma_load_3d(xring + slot * kPairBytes, xm, 0, 0, at0, bar);
+        tma_load_3d(xring + slot * kPairBytes + kInRow, xm, 0, 0, at1, bar);
+        tma_load_3d(gring + slot * kPairBytes, &gmap, 0, 0, at0, bar);
+        tma_load_3d(gring + slot * kPairBytes + kGRow, &gmap, 0, 0, at1, bar);
     };
     if (is_fwd && t == 0) {
         for (int k = 0; k < kSlotsUsed && k < count; ++k) request(k);
@@ -416,7 +432,7 @@ k_bwd4096(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ CUte
                     }
                 }
             }
-            fwd_chunks<0>(Y0, Y1, T0, T1, cx);
+            fwd_chunks<0, SHORT>(Y0, Y1, T0, T1, cx);
             // y to the parity basis
 #pragma unroll
             for (int m = 0; m < 16; ++m) {
@@ -486,7 +502,7 @@ k_bwd4096(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ CUte
                 bar_sync(cx.a.bar, kThreads);
                 if (t == 0 && k + 1 < count) request(k + 1);
             }
-            rev_steps<0, kUpperSteps>(Y0, Y1, G0, G1, T0, T1, A0, A1, cx, [](auto) {});
+            rev_steps<0, kUpperSteps, SHORT>(Y0, Y1, G0, G1, T0, T1, A0, A1, cx, [](auto) {});
             // phase 3 -> phase 2 regrouping = the hand-over: once the lower group is past its reads of the buffers for
             // the previous pair, store in the layout it reads
             bar_sync(kBarEmpty, kCtaThreads);
@@ -509,7 +525,7 @@ k_bwd4096(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ CUte
             rev2_load(Y1, exr + 1 * kExBytes, cx.a);
             rev2_load(G0, exr + 2 * kExBytes, cx.a);
             rev2_load(G1, exr + 3 * kExBytes, cx.a);
-            rev_steps<kUpperSteps, 24>(Y0, Y1, G0, G1, T0, T1, A0, A1, cx, [&](auto step) {
+            rev_steps<kUpperSteps, 24, SHORT>(Y0, Y1, G0, G1, T0, T1, A0, A1, cx, [&](auto step) {
                 constexpr int I = decltype(step)::value;
                 if constexpr (I == 15) {  // phase 2 -> phase 1, inside each half-warp, but the buffers were read across warps
                     bar_sync(cx.a.bar, kThreads);
@@ -534,6 +550,10 @@ k_bwd4096(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ CUte
                 for (int r = 0; r < 2; ++r) {
                     if (r0 + r < rows) {
                         const u64(&G)[16] = r == 0 ? G0 : G1;
+                        // a run of 16 elements exists or not as a whole
+                        auto there = [&](int h) {
+                            return !SHORT || static_cast<int64_t>(r0 + r) * kN + 16 * (t & 15) + 512 * (t >> 4) + 256 * h < brief.elems;
+                        };
                         if constexpr (IN_F32) {
                             float* row = static_cast<float*>(dx_out) + static_cast<int64_t>(r0 + r) * ld + 16 * (t & 15) + 512 * (t >> 4);
 #pragma unroll
@@ -547,6 +567,7 @@ k_bwd4096(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ CUte
                                     const bool odd_c = ((__builtin_popcount(m) + h) & 1) != 0;
                                     w[m] = (h ? hi : lo) ^ (odd_c ? sgn_b : sgn_a);
                                 }
+                                if (!there(h)) continue;
                                 uint4* dst = reinterpret_cast<uint4*>(row + 256 * h);
 #pragma unroll
                                 for (int c = 0; c < 4; ++c) dst[c] = make_uint4(w[4 * c], w[4 * c + 1], w[4 * c + 2], w[4 * c + 3]);
@@ -569,6 +590,7 @@ k_bwd4096(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ CUte
                                 const uint32_t neg_hi = odd_c ? sgn_a : sgn_b;                  // bit 31: element 2j+1
                                 w[j] = cvt_bf16x2(e0, e1) ^ (neg_lo | neg_hi);
                             }
+                            if (!there(h)) continue;
                             uint4* dst = reinterpret_cast<uint4*>(row + 256 * h);
                             dst[0] = make_uint4(w[0], w[1], w[2], w[3]);
                             dst[1] = make_uint4(w[4], w[5], w[6], w[7]);
@@ -631,10 +653,8 @@ k_bwd4096(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ CUte
 // One thread per angle: the three-shear constants of pair (s, j), negated when its two elements carry
 // opposite signs, at the place the owning role reads them; and the sign that turns the accumulated
 // g_hi*y_lo - g_lo*y_hi of the parity basis into d-theta.
-__global__ void __launch_bounds__(256) k_build_image_bwd4096(const float4* __restrict__ prep,
-                                                              const uint8_t* __restrict__ flip,
-                                                              float* __restrict__ img, int8_t* __restrict__ dsign) {
-    const int k = blockIdx.x * blockDim.x + threadIdx.x;
+__device__ __forceinline__ void build_image_bwd(int k, const float4* __restrict__ prep, const uint8_t* __restrict__ flip,
+                                                float* __restrict__ img, int8_t* __restrict__ dsign) {
     if (k >= 12 * (kN / 2)) return;
     const int s = k / (kN / 2), j = k % (kN / 2);
     const int lo = ((j >> s) << (s + 1)) | (j & ((1 << s) - 1));
@@ -660,8 +680,7 @@ __global__ void __launch_bounds__(256) k_build_image_bwd4096(const float4* __res
 
 // One thread per 32-bit word of a bf16 g row in phase-3 ownership (role t, register m): bit 15 / bit 31 set
 // when element 2t + 256m / its neighbour must be negated to enter the basis sigma(after stage 11) * parity.
-__global__ void __launch_bounds__(256) k_build_gsign4096(const uint8_t* __restrict__ flip, uint32_t* __restrict__ gsign) {
-    const int w = blockIdx.x * blockDim.x + threadIdx.x;
+__device__ __forceinline__ void build_gsign(int w, const uint8_t* __restrict__ flip, uint32_t* __restrict__ gsign) {
     if (w >= 16 * kThreads) return;
     const int m = (w / (4 * kThreads)) * 4 + (w & 3), t = (w >> 2) % kThreads;  // layout [m / 4][t][m % 4]
     const int e = 2 * t + 256 * m;
@@ -677,9 +696,7 @@ __global__ void __launch_bounds__(256) k_build_gsign4096(const uint8_t* __restri
 // both factors are multiplied by cos(theta).  Stage 0 is a general 2x2 that absorbs the factors.  Image layout
 // [column quad][role][4]; stage s >= 1 at columns 32 (s - 1), stage 0 at 352.  *form is raised when a factor leaves
 // [2^-64, 1]: the kernel then walks in the three-shear form.
-__global__ void __launch_bounds__(256) k_build_image_inv4096(const double2* __restrict__ cs, float* __restrict__ img,
-                                                              int* __restrict__ form) {
-    const int k = blockIdx.x * blockDim.x + threadIdx.x;
+__device__ __forceinline__ void build_image_inv(int k, const double2* __restrict__ cs, float* __restrict__ img, int* __restrict__ form) {
     if (k >= 12 * (kN / 2)) return;
     const int s = k / (kN / 2), j = k % (kN / 2);
     const int lo = ((j >> s) << (s + 1)) | (j & ((1 << s) - 1));
@@ -724,6 +741,26 @@ __global__ void __launch_bounds__(256) k_build_image_inv4096(const double2* __re
     }
 }
 
+// All three of the above in one launch (their inputs are the same and none needs another's output): blocks of 256 threads,
+// the image of the backward kernel, then that of the reverse walk, then the sign words.  As three launches and a memset of
+// the range flag they took 11.6 us.  *form must be kFormScaled before.
+constexpr int kAngleBlocks = 12 * (kN / 2) / 256, kSignBlocks = 16 * kThreads / 256;
+constexpr int kTableBlocks = 2 * kAngleBlocks + kSignBlocks;
+__global__ void __launch_bounds__(256) k_build_tables(const float4* __restrict__ prep, const uint8_t* __restrict__ flip,
+                                                       const double2* __restrict__ cs, float* __restrict__ img, int8_t* __restrict__ dsign,
+                                                       float* __restrict__ img_inv, int* __restrict__ form, uint32_t* __restrict__ gsign) {
+    grid_dep_launch();
+    grid_dep_wait();
+    const int b = blockIdx.x;
+    if (b < kAngleBlocks) {
+        build_image_bwd(256 * b + threadIdx.x, prep, flip, img, dsign);
+    } else if (b < 2 * kAngleBlocks) {
+        build_image_inv(256 * (b - kAngleBlocks) + threadIdx.x, cs, img_inv, form);
+    } else {
+        build_gsign(256 * (b - 2 * kAngleBlocks) + threadIdx.x, flip, gsign);
+    }
+}
+
 // =================================================================================================================
 // Inverse / transpose for n = 4096 bf16 rows:  x = Q^T y.  The reverse walk of the backward kernel on one array,
 // organised like the forward kernel: four row groups of 128 threads per CTA, 32 constants per tensor-memory chunk.
@@ -757,17 +794,20 @@ __device__ __forceinline__ void stage_general_k0(u64 (&P)[16], const uint32_t (&
 // stage S (11..0) is in Tcur; the next constants are requested right after the wait.  Three-shear form: stage s at
 // column 32 s, all twelve stages alike.  Scaled form: stages 11..1 are two-FMA stages on values that carry the product of
 // the cosines of the stages above, stage 0 is a general 2x2 (two chunks) that absorbs the factors.
-template <int FORM, int S, class F>
+template <int FORM, int S, bool SHORT, class F>
 __device__ __forceinline__ void inv_stages(u64 (&P)[16], uint32_t (&Tcur)[32], uint32_t (&Tnext)[32], uint32_t tlane,
-                                           const Addr& a, uint32_t buf2, uint32_t buf1, F&& after_phase3) {
+                                           const Addr& a, int stages, uint32_t buf2, uint32_t buf1, F&& after_phase3) {
+    const bool runs = !SHORT || S < stages;  // SHORT: stages from log2 of the row length on are passed over
     tmem_wait_ld32(Tcur);
     if constexpr (FORM == kFormShear) {
         if constexpr (S > 0) tmem_ld32(tlane + 32 * (S - 1), Tnext);
-        stage_lift<S & 3, 0, 8, 32>(P, Tcur);
+        if (runs) stage_lift<S & 3, 0, 8, 32>(P, Tcur);
     } else {
         if constexpr (S > 1) tmem_ld32(tlane + 32 * (S - 2), Tnext);
         if constexpr (S == 1) tmem_ld32(tlane + 352, Tnext);
-        if constexpr (S > 0) stage_scaled<S & 3, 0, 8, 32>(P, Tcur);
+        if constexpr (S > 0) {
+            if (runs) stage_scaled<S & 3, 0, 8, 32>(P, Tcur);
+        }
         if constexpr (S == 0) {
             tmem_ld32(tlane + 384, Tnext);
             stage_general_k0<0, 4>(P, Tcur);
@@ -788,7 +828,7 @@ __device__ __forceinline__ void inv_stages(u64 (&P)[16], uint32_t (&Tcur)[32], u
         __syncwarp();
         rev1_load(P, buf1, a);
     }
-    if constexpr (S > 0) inv_stages<FORM, S - 1>(P, Tnext, Tcur, tlane, a, buf2, buf1, after_phase3);
+    if constexpr (S > 0) inv_stages<FORM, S - 1, SHORT>(P, Tnext, Tcur, tlane, a, stages, buf2, buf1, after_phase3);
 }
 
 // what the CTAs of the upper half use in the wide mode of the inverse kernel instead of img, img_scaled, form, gsign
@@ -804,11 +844,12 @@ struct InvUpper {
 // odd CTAs the upper (CTAs 2i and 2i + 1 work on the same rows at about the same time, so the second read of a row comes
 // from L2).  A y row is 16 KB in one slot; the transposed stage-12 rotation y'_own = c y_own +- s y_other with (cos, sin)
 // from `tw12` is applied as the row is read, then the half's own twelve stages follow from its own tables.
-template <int G, bool OUT_BF16, bool IN_F32 = false, bool WIDE = false>
+template <int G, bool OUT_BF16, bool IN_F32 = false, bool WIDE = false, bool SHORT = false>
 __global__ void __launch_bounds__(G * kThreads, 1)
 k_inv4096(const __grid_constant__ CUtensorMap ymap, const float* __restrict__ img_lo, const float* __restrict__ img_scaled_lo,
           const int* __restrict__ form_lo, const uint32_t* __restrict__ gsign_lo, void* __restrict__ xout, int64_t ldx, int rows,
-          int* __restrict__ status, const float2* __restrict__ tw12, const InvUpper upper) {
+          int* __restrict__ status, const float2* __restrict__ tw12, const InvUpper upper, const ShortRows brief) {
+    static_assert(!(SHORT && WIDE), "one or the other");
     static_assert(!(IN_F32 && WIDE), "the wide mode takes bf16 rows");
     const int half = WIDE ? int(blockIdx.x & 1u) : 0;
     const int cta = WIDE ? int(blockIdx.x >> 1) : int(blockIdx.x);
@@ -847,7 +888,7 @@ k_inv4096(const __grid_constant__ CUtensorMap ymap, const float* __restrict__ im
     if (t == 0) {
         for (int k = 0; k < kSlotsUsed && k < count; ++k) {
             mbar_expect_tx(bar_base + 8 * k, kSlotBytes);
-            tma_load_3d(in_base + k * kSlotBytes, &ymap, 0, 0, first + k * stride, bar_base + 8 * k);
+            tma_load_3d(in_base + k * kSlotBytes, &ymap, 0, 0, SHORT ? (first + k * stride) << brief.log : first + k * stride, bar_base + 8 * k);
         }
     }
     // constants: the scaled-form image ([column quad][role][4], coalesced, all loads in flight) unless the table build
@@ -1008,10 +1049,11 @@ k_inv4096(const __grid_constant__ CUtensorMap ymap, const float* __restrict__ im
                 P[m] = pack2u(bf16_lo(w), w & 0xFFFF0000u);
             }
         }
-        inv_stages<FORM, 11>(P, T0, T1, tlane, a, a.ex, a.ex + kExBytes, [&]() {
+        inv_stages<FORM, 11, SHORT>(P, T0, T1, tlane, a, 12 - brief.log, a.ex, a.ex + kExBytes, [&]() {
             if (t == 0 && k + kSlotsUsed < count) {
                 mbar_expect_tx(bar_base + 8 * slot, kSlotBytes);
-                tma_load_3d(in_base + slot * kSlotBytes, &ymap, 0, 0, first + (k + kSlotsUsed) * stride, bar_base + 8 * slot);
+                const int at = first + (k + kSlotsUsed) * stride;
+                tma_load_3d(in_base + slot * kSlotBytes, &ymap, 0, 0, SHORT ? at << brief.log : at, bar_base + 8 * slot);
             }
         });
         // phase-1 ownership: two runs of 16 consecutive elements; the three-shear form undoes the parity sign here
@@ -1019,6 +1061,7 @@ k_inv4096(const __grid_constant__ CUtensorMap ymap, const float* __restrict__ im
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
             const int64_t off = static_cast<int64_t>(row) * ldx + (WIDE ? kN * half : 0) + 16 * (t & 15) + 512 * (t >> 4) + 256 * h;
+            if (SHORT && off >= brief.elems) continue;  // x is contiguous: past the last row
             if constexpr (OUT_BF16) {
                 uint32_t w[8];
 #pragma unroll
@@ -1129,14 +1172,11 @@ cudaError_t bwd8192_build_tables(const bfq_plan* plan, cudaStream_t st) {
     double2* cs_half = reinterpret_cast<double2*>(flip + count);  // count is a multiple of 16
     for (int h = 0; h < 2; ++h) {
         b4k::k_prep_half8192<<<(count + 255) / 256, 256, 0, st>>>(cs, h, prep, flip, cs_half);
-        b4k::k_build_image_bwd4096<<<(count + 255) / 256, 256, 0, st>>>(prep, flip, plan->img_b8192[h], plan->dsign8192[h]);
-        b4k::k_build_gsign4096<<<(16 * b4k::kThreads + 255) / 256, 256, 0, st>>>(flip, plan->gsign8192[h]);
-        cudaError_t e = cudaGetLastError();
+        // the half's scaled reverse walk has its range flag in words 1 and 2 of the plan's form flags
+        cudaError_t e = cudaMemsetAsync(plan->form_flag + 1 + h, 0, sizeof(int), st);
         if (e != cudaSuccess) return e;
-        // the half's scaled reverse walk (inverse kernel) and its range flag: words 1 and 2 of the plan's form flags
-        e = cudaMemsetAsync(plan->form_flag + 1 + h, 0, sizeof(int), st);
-        if (e != cudaSuccess) return e;
-        b4k::k_build_image_inv4096<<<(count + 255) / 256, 256, 0, st>>>(cs_half, plan->img_i8192[h], plan->form_flag + 1 + h);
+        b4k::k_build_tables<<<b4k::kTableBlocks, 256, 0, st>>>(prep, flip, cs_half, plan->img_b8192[h], plan->dsign8192[h],
+                                                               plan->img_i8192[h], plan->form_flag + 1 + h, plan->gsign8192[h]);
         e = cudaGetLastError();
         if (e != cudaSuccess) return e;
     }
@@ -1175,7 +1215,7 @@ cudaError_t bwd8192_launch_halves(bfq_plan* plan, const void* x, const void* g, 
     upper.img = plan->img_b8192[1], upper.gsign = plan->gsign8192[1], upper.dsign = plan->dsign8192[1];
     kern<<<2 * grid, b4k::kCtaThreads, b4k::Smem::kBytesWide, st>>>(xmap, gmap, plan->img_b8192[0], plan->gsign8192[0],
                                                                   plan->dsign8192[0], dx, ld, plan->partial, int(rows),
-                                                                  plan->status_word, plan->tw + 12 * f4k::kN, upper);
+                                                                  plan->status_word, plan->tw + 12 * f4k::kN, upper, b4k::ShortRows{});
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     b4k::k_reduce_wide<<<13 * f4k::kN / 32, 256, 0, st>>>(plan->partial, grid, dtheta);
@@ -1195,22 +1235,98 @@ bool bwd4096_available(const bfq_plan* plan) {
            plan->partial_slots >= plan->sm_count && encode_tiled() != nullptr;
 }
 
-// Builds the backward tables from the staging area bfq_set_angles filled (two launches).
+// Builds the tables of the backward and inverse kernels from the staging area bfq_set_angles filled (it also resets the
+// range flag, word 1 of the plan's form flags).
 cudaError_t bwd4096_build_tables(const bfq_plan* plan, cudaStream_t st) {
     const int count = 12 * (f4k::kN / 2);
     const float4* prep = reinterpret_cast<const float4*>(plan->prep4096);
-    const uint8_t* flip = reinterpret_cast<const uint8_t*>(reinterpret_cast<const double2*>(prep + count) + count);
-    b4k::k_build_image_bwd4096<<<(count + 255) / 256, 256, 0, st>>>(prep, flip, plan->img_b4096, plan->dsign4096);
+    const double2* cs = reinterpret_cast<const double2*>(prep + count);
+    const uint8_t* flip = reinterpret_cast<const uint8_t*>(cs + count);
+    return launch_overlapped(b4k::k_build_tables, dim3(b4k::kTableBlocks), dim3(256), 0, st, prep, flip, cs, plan->img_b4096,
+                             plan->dsign4096, plan->img_i4096, plan->form_flag + 1, plan->gsign4096);
+}
+
+// ---- rows of 128 .. 2048 elements, several as one of 4096 ----------------------------------------------------------
+namespace b4k {
+// dtheta [levels][half] from the slots' [12][2048]: stage s, angle j = the sum over the slots and the 2048 / half row
+// positions r of entry s * 2048 + r * half + j.  A block = 32 lanes x 32 angles (half is a multiple of 32): lane y adds
+// terms y, y + 32, ... in order (term = slot * positions + r), then the lanes are added in order.
+__global__ void __launch_bounds__(1024) k_reduce_short(const float* __restrict__ partial, int slots, int half_log, float* __restrict__ out) {
+    __shared__ float sh[32][33];
+    const int x = threadIdx.x & 31, y = threadIdx.x >> 5;
+    const int k = blockIdx.x * 32 + x, s = k >> half_log, j = k & ((1 << half_log) - 1);
+    const int pos_log = 11 - half_log, terms = slots << pos_log;
+    const float* src = partial + s * (kN / 2) + j;
+    float acc = 0.f;
+#pragma unroll 4
+    for (int i = y; i < terms; i += 32)
+        acc += src[static_cast<int64_t>(i >> pos_log) * kSlotFloats + ((i & ((1 << pos_log) - 1)) << half_log)];
+    sh[y][x] = acc;
+    __syncthreads();
+    if (y == 0) {
+        float a = sh[0][x];
+#pragma unroll
+        for (int i = 1; i < 32; ++i) a += sh[i][x];
+        out[k] = a;
+    }
+}
+}  // namespace b4k
+
+size_t bwd_short_partial_floats(int sm_count) { return size_t(sm_count) * b4k::kSlotFloats; }
+
+bool bwd_short_available(const bfq_plan* plan) {
+    return plan->n >= 128 && plan->n < f4k::kN && plan->cc_major == 10 && plan->img_b4096 != nullptr && plan->img_i4096 != nullptr &&
+           plan->partial_floats >= bwd_short_partial_floats(plan->sm_count) && encode_tiled() != nullptr;
+}
+
+// x, g, dx contiguous rows, all bf16 or all fp32
+cudaError_t bwd_short_launch(bfq_plan* plan, const void* x, const void* g, int64_t rows, void* dx, float* dtheta, bool f32, cudaStream_t st) {
+    static bool attr_set[kMaxDevices] = {false};
+    if (!attr_set[plan->device]) {
+        cudaError_t e = cudaFuncSetAttribute(b4k::k_bwd4096<false, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(b4k::Smem::kBytes));
+        if (e == cudaSuccess)
+            e = cudaFuncSetAttribute(b4k::k_bwd4096<true, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(b4k::Smem::kBytes));
+        if (e != cudaSuccess) return e;
+        attr_set[plan->device] = true;
+    }
+    const int n = plan->n;
+    CUtensorMap xmap, gmap;
+    const bool maps = f32 ? (encode_row_map_f32(&xmap, x, rows, n, n) && encode_row_map_f32(&gmap, g, rows, n, n))
+                          : (encode_row_map(&xmap, x, rows, n, n) && encode_row_map(&gmap, g, rows, n, n));
+    if (!maps) return cudaErrorInvalidValue;
+    const b4k::ShortRows brief{12 - plan->log_n, rows * n};
+    const int64_t joint = (brief.elems + f4k::kN - 1) / f4k::kN, pairs = (joint + 1) / 2;
+    const int grid = int(pairs < plan->sm_count ? pairs : plan->sm_count);
+    auto kern = f32 ? b4k::k_bwd4096<true, false, true> : b4k::k_bwd4096<false, false, true>;
+    kern<<<grid, b4k::kCtaThreads, b4k::Smem::kBytes, st>>>(xmap, gmap, plan->img_b4096, plan->gsign4096, plan->dsign4096, dx, f4k::kN, plan->partial,
+                                                          int(joint), plan->status_word, nullptr, b4k::WideHalf{}, brief);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    b4k::k_build_gsign4096<<<(16 * b4k::kThreads + 255) / 256, 256, 0, st>>>(flip, plan->gsign4096);
-    e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-    // the scaled reverse walk of the inverse kernel and its range flag (word 1 of the plan's form flags)
-    e = cudaMemsetAsync(plan->form_flag + 1, 0, sizeof(int), st);
-    if (e != cudaSuccess) return e;
-    b4k::k_build_image_inv4096<<<(count + 255) / 256, 256, 0, st>>>(reinterpret_cast<const double2*>(prep + count),
-                                                                   plan->img_i4096, plan->form_flag + 1);
+    b4k::k_reduce_short<<<plan->log_n * (n / 2) / 32, 1024, 0, st>>>(plan->partial, grid, plan->log_n - 1, dtheta);
+    plan->last_backward_partials = grid;
+    return cudaGetLastError();
+}
+
+// y: rows of leading dimension ldy; x contiguous; bf16 -> bf16, bf16 -> fp32 or fp32 -> fp32
+cudaError_t inv_short_launch(bfq_plan* plan, const void* y, bool y_f32, int64_t rows, int64_t ldy, void* x, bool x_bf16, cudaStream_t st) {
+    constexpr int G = 4;
+    using S = b4k::InvSmem<G>;
+    auto kern = y_f32 ? b4k::k_inv4096<G, false, true, false, true> : (x_bf16 ? b4k::k_inv4096<G, true, false, false, true> : b4k::k_inv4096<G, false, false, false, true>);
+    const int which = y_f32 ? 0 : (x_bf16 ? 1 : 2);
+    static bool attr_set[3][kMaxDevices] = {{false}};
+    if (!attr_set[which][plan->device]) {
+        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(S::kBytes));
+        if (e != cudaSuccess) return e;
+        attr_set[which][plan->device] = true;
+    }
+    const int n = plan->n;
+    CUtensorMap ymap;
+    if (!(y_f32 ? encode_row_map_f32(&ymap, y, rows, ldy, n) : encode_row_map(&ymap, y, rows, ldy, n))) return cudaErrorInvalidValue;
+    const b4k::ShortRows brief{12 - plan->log_n, rows * n};
+    const int64_t joint = (brief.elems + f4k::kN - 1) / f4k::kN, want = (joint + G - 1) / G;
+    const int grid = int(want < plan->sm_count ? want : plan->sm_count);
+    kern<<<grid, G * b4k::kThreads, S::kBytes, st>>>(ymap, plan->img_b4096, plan->img_i4096, plan->form_flag + 1, plan->gsign4096, x, f4k::kN,
+                                                    int(joint), plan->status_word, nullptr, b4k::InvUpper{}, brief);
     return cudaGetLastError();
 }
 
@@ -1235,11 +1351,11 @@ cudaError_t bwd4096_launch(bfq_plan* plan, const void* x, const void* g, int64_t
     if (f32) {
         b4k::k_bwd4096<true><<<grid, b4k::kCtaThreads, b4k::Smem::kBytes, st>>>(xmap, gmap, plan->img_b4096, plan->gsign4096,
                                                                               plan->dsign4096, dx, ld, plan->partial,
-                                                                              int(rows), plan->status_word, nullptr, b4k::WideHalf{});
+                                                                              int(rows), plan->status_word, nullptr, b4k::WideHalf{}, b4k::ShortRows{});
     } else {
         b4k::k_bwd4096<false><<<grid, b4k::kCtaThreads, b4k::Smem::kBytes, st>>>(xmap, gmap, plan->img_b4096, plan->gsign4096,
                                                                                plan->dsign4096, dx, ld, plan->partial,
-                                                                               int(rows), plan->status_word, nullptr, b4k::WideHalf{});
+                                                                               int(rows), plan->status_word, nullptr, b4k::WideHalf{}, b4k::ShortRows{});
     }
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
@@ -1267,7 +1383,7 @@ cudaError_t inv4096_launch_f32(bfq_plan* plan, const void* y, int64_t rows, int6
     const int grid = int(want < plan->sm_count ? want : plan->sm_count);
     kern<<<grid, G * b4k::kThreads, S::kBytes, st>>>(ymap, plan->img_b4096, plan->img_i4096, plan->form_flag + 1,
                                                     plan->gsign4096, x, ldx, int(rows), plan->status_word, nullptr,
-                                                    b4k::InvUpper{});
+                                                    b4k::InvUpper{}, b4k::ShortRows{});
     return cudaGetLastError();
 }
 
@@ -1292,12 +1408,12 @@ cudaError_t inv4096_launch(bfq_plan* plan, const void* y, int64_t rows, int64_t 
         b4k::k_inv4096<G, true><<<grid, G * b4k::kThreads, S::kBytes, st>>>(ymap, plan->img_b4096, plan->img_i4096,
                                                                             plan->form_flag + 1, plan->gsign4096, x, ldx,
                                                                             int(rows), plan->status_word, nullptr,
-                                                                            b4k::InvUpper{});
+                                                                            b4k::InvUpper{}, b4k::ShortRows{});
     } else {
         b4k::k_inv4096<G, false><<<grid, G * b4k::kThreads, S::kBytes, st>>>(ymap, plan->img_b4096, plan->img_i4096,
                                                                              plan->form_flag + 1, plan->gsign4096, x, ldx,
                                                                              int(rows), plan->status_word, nullptr,
-                                                                             b4k::InvUpper{});
+                                                                             b4k::InvUpper{}, b4k::ShortRows{});
     }
     return cudaGetLastError();
 }
@@ -1337,11 +1453,11 @@ cudaError_t inv8192_launch(bfq_plan* plan, const void* y, int64_t rows, int64_t 
     if (x_bf16) {
         b4k::k_inv4096<G, true, false, true><<<grid, G * b4k::kThreads, S::kBytes, st>>>(
             ymap, plan->img_b8192[0], plan->img_i8192[0], plan->form_flag + 1, plan->gsign8192[0], x, ldx, int(rows),
-            plan->status_word, tw12, upper);
+            plan->status_word, tw12, upper, b4k::ShortRows{});
     } else {
         b4k::k_inv4096<G, false, false, true><<<grid, G * b4k::kThreads, S::kBytes, st>>>(
             ymap, plan->img_b8192[0], plan->img_i8192[0], plan->form_flag + 1, plan->gsign8192[0], x, ldx, int(rows),
-            plan->status_word, tw12, upper);
+            plan->status_word, tw12, upper, b4k::ShortRows{});
     }
     return cudaGetLastError();
 }

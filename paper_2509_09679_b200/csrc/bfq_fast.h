@@ -29,6 +29,27 @@ cudaError_t fwdq4096_launch_f32(const bfq_plan* plan, const void* x, int64_t row
 cudaError_t fwdq4096_launch_stats(const bfq_plan* plan, const void* x, int64_t rows, int64_t ldx, uint8_t* codes,
                                   uint16_t* scales, unsigned long long* hist, float* rowstats, cudaStream_t st);
 
+// rows of 128 .. 2048 elements: several as one of 4096 on the same kernel.  bits = 2, 4, 8: codes + scales; bits = 0: the
+// rotated rows, contiguous, in the type of x
+bool fwdq_short_available(const bfq_plan* plan);
+cudaError_t fwdq_short_launch(const bfq_plan* plan, const void* x, bool f32, int64_t rows, int64_t ldx, int bits, uint8_t* codes,
+                              uint16_t* scales, void* y, cudaStream_t st);
+cudaError_t fwdq128_launch(const bfq_plan* plan, const void* x, bool f32, int64_t rows, int64_t ldx, int bits, uint8_t* codes, uint16_t* scales,
+                           void* y, cudaStream_t st);
+cudaError_t fwdq256_launch(const bfq_plan* plan, const void* x, bool f32, int64_t rows, int64_t ldx, int bits, uint8_t* codes, uint16_t* scales,
+                           void* y, cudaStream_t st);
+cudaError_t fwdq512_launch(const bfq_plan* plan, const void* x, bool f32, int64_t rows, int64_t ldx, int bits, uint8_t* codes, uint16_t* scales,
+                           void* y, cudaStream_t st);
+cudaError_t fwdq1024_launch(const bfq_plan* plan, const void* x, bool f32, int64_t rows, int64_t ldx, int bits, uint8_t* codes, uint16_t* scales,
+                           void* y, cudaStream_t st);
+cudaError_t fwdq2048_launch(const bfq_plan* plan, const void* x, bool f32, int64_t rows, int64_t ldx, int bits, uint8_t* codes, uint16_t* scales,
+                           void* y, cudaStream_t st);
+// the same rows backward and inverse
+size_t bwd_short_partial_floats(int sm_count);
+bool bwd_short_available(const bfq_plan* plan);
+cudaError_t bwd_short_launch(bfq_plan* plan, const void* x, const void* g, int64_t rows, void* dx, float* dtheta, bool f32, cudaStream_t st);
+cudaError_t inv_short_launch(bfq_plan* plan, const void* y, bool y_f32, int64_t rows, int64_t ldy, void* x, bool x_bf16, cudaStream_t st);
+
 // n = 8192, bf16 rows, INT2 (INT4 / INT8 through another epilogue): two-CTA clusters, one 4096-point half per CTA
 size_t fwdq8192_image_bytes();
 size_t fwdq8192_prep_bytes();

@@ -1,0 +1,11 @@
+// Forward of rows of 256 elements on the n = 4096 kernel.
+#include "bfq_fwdq_short.cuh"
+
+namespace bfq {
+
+cudaError_t fwdq256_launch(const bfq_plan* plan, const void* x, bool f32, int64_t rows, int64_t ldx, int bits, uint8_t* codes, uint16_t* scales,
+                           void* y, cudaStream_t st) {
+    return fwdq_short_launch<4>(plan, x, f32, rows, ldx, bits, codes, scales, y, st);
+}
+
+}  // namespace bfq

@@ -15,13 +15,16 @@ struct bfq_plan {
     int sm_count = 0;
     int cc_major = 0;
     bool angles_set = false;
+    void* arena = nullptr;       // one device allocation; every table below (and `partial`, `status_word`) is a part of it
     float2* tw = nullptr;        // [log_n][n/2] (cos, sin), fp32
-    float* img4096 = nullptr;    // [128][416] tensor-memory image of the rotation constants (n = 4096 only)
-    void* prep4096 = nullptr;    // staging for the image build: per-angle constants and negation flags (n = 4096 only)
-    float* img_b4096 = nullptr;  // [128][384] constants of the backward kernel (n = 4096 only)
-    float* img_i4096 = nullptr;  // [104][128][4] scaled-form constants of the inverse kernel (n = 4096 only)
-    int8_t* dsign4096 = nullptr; // [12][2048] sign applied to the accumulated d-theta (n = 4096 only)
-    uint32_t* gsign4096 = nullptr;  // [16 * 128] sign words applied to bf16 g rows (n = 4096 only)
+    // rows of 128 .. 2048 elements use the n = 4096 tables with 4096 / n copies of their angles side by side; there all of
+    // these are built by bfq_set_angles
+    float* img4096 = nullptr;    // [128][416] tensor-memory image of the rotation constants (n = 128 .. 4096)
+    void* prep4096 = nullptr;    // staging for the image build: per-angle constants and negation flags (n = 128 .. 4096)
+    float* img_b4096 = nullptr;  // [128][384] constants of the backward kernel (n = 128 .. 4096)
+    float* img_i4096 = nullptr;  // [104][128][4] scaled-form constants of the inverse kernel (n = 128 .. 4096)
+    int8_t* dsign4096 = nullptr; // [12][2048] sign applied to the accumulated d-theta (n = 128 .. 4096)
+    uint32_t* gsign4096 = nullptr;  // [16 * 128] sign words applied to bf16 g rows (n = 128 .. 4096)
     bool bwd_tables_valid = false;  // the three above match the current angles
     // n = 8192: backward tables of the two 4096-element halves (stages 0 .. 11), built on first use like the above
     float* img_b8192[2] = {nullptr, nullptr};
