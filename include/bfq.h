@@ -242,6 +242,22 @@ int bfq_test_stuck_wait(bfq_plan* plan, int enable);
 const char* bfq_status_string(int status);
 
 /*
+ * Backward of the composite transform (paper Sec. 3.3, y = Q x with Q = Q1 (x) Q2, rows as n1 x n2 matrices), one pass: for
+ * upstream rows g, dx = Q^T g, dtheta [log2 n][n/2] of Q2 (the plan's butterfly) and dq1 [n1][n1] = dL/dQ1, both summed over
+ * all rows in a fixed order (fp32).  x, g, dx: [rows][ld], 16-byte aligned, dx of type xt or NULL.  Arithmetic fp32.
+ * Needs 128 <= n <= 1024, 2 <= n1 <= 64 and n1 (n + 4) * 12 + n1 * (n1 rounded up to 8) * 4 <= 227 KB, else
+ * BFQ_ERR_UNSUPPORTED_N.  Uses the plan's partial sums, as bfq_backward does: calls on one plan are ordered by the caller.
+ * Returns BFQ_OK or the errors of bfq_backward.
+ */
+int bfq_composite_backward(bfq_plan* plan, const float* q1, int n1, const void* x, bfq_dtype xt, const void* g, bfq_dtype gt,
+                           int64_t rows, int64_t ld, void* dx, float* dtheta, float* dq1, void* stream);
+/*
+ * Gradient of the Cayley parameters (bfq_cayley) from dq1 = dL/dQ1: dparams [n1 (n1 - 1) / 2], fp32; float64 inside.
+ * Device pointers.  Returns BFQ_OK, BFQ_ERR_NULL, BFQ_ERR_UNSUPPORTED_N, BFQ_ERR_ALIGN or BFQ_ERR_CUDA.
+ */
+int bfq_cayley_backward(bfq_plan* plan, const float* params, int n1, const float* dq1, float* dparams, void* stream);
+
+/*
  * Dense product with on-the-fly dequantization, for the reconstruction loss of the calibration step (paper Sec. 3.4:
  * || W x - Dequant(Quant(W B^T)) Dequant(Quant(B x)) ||^2) and its gradients:
  *     C[i][j] = alpha * sum_{k < K} A(i, k) * B(j, k),   i < m, j < n;   C fp32, row-major, leading dimension ldc >= n.

@@ -35,6 +35,8 @@ SIGNATURES = {
     "bfq_hadamard_quant": (_i, [_p, _p, _i, _i64, _i64, _i, _p, _p, _p]),
     "bfq_backward": (_i, [_p, _p, _i, _p, _i, _i64, _i64, _p, _i, _p, _p]),
     "bfq_fold_weights": (_i, [_p, _p, _i, _i64, _i64, _i, _p, _p, _p, _i, _p]),
+    "bfq_composite_backward": (_i, [_p, _p, _i, _p, _i, _p, _i, _i64, _i64, _p, _p, _p, _p]),
+    "bfq_cayley_backward": (_i, [_p, _p, _i, _p, _p, _p]),
     "bfq_device_status": (_i, [_p]),
     "bfq_last_cuda_error": (_i, [_p]),
     "bfq_status_string": (ctypes.c_char_p, [_i]),
@@ -248,6 +250,29 @@ class Plan:
                                                  codes.data_ptr(), scales.data_ptr(), _stream(x)),
                "bfq_composite_forward_quant")
         return codes, scales
+
+    def composite_backward(self, q1: torch.Tensor, x: torch.Tensor, g: torch.Tensor):
+        """x, g: [tokens][n1 * n] contiguous.  Returns (dx in the type of x, dtheta of Q2, dQ1)."""
+        n1 = self._q1(q1)
+        d = n1 * self.n
+        rows, ld = _rows(x, d, self.device, what="x")
+        if _rows(g, d, self.device, rows, "g")[1] != ld or (rows > 1 and ld != d):
+            raise ValueError("x and g must have contiguous rows")
+        dx = torch.empty((rows, d), dtype=x.dtype, device=x.device)
+        dtheta = torch.empty((self.L, self.n // 2), dtype=torch.float32, device=x.device)
+        dq1 = torch.empty((n1, n1), dtype=torch.float32, device=x.device)
+        _check(lib().bfq_composite_backward(self._h, q1.data_ptr(), n1, x.data_ptr(), _dt(x), g.data_ptr(), _dt(g), rows, d, dx.data_ptr(),
+                                            dtheta.data_ptr(), dq1.data_ptr(), _stream(x)), "bfq_composite_backward")
+        return dx, dtheta, dq1
+
+    def cayley_backward(self, params: torch.Tensor, n1: int, dq1: torch.Tensor) -> torch.Tensor:
+        """dL/dparams of cayley() from dL/dQ1 (fp32, on the plan's device)."""
+        _exact(params, torch.float32, (n1 * (n1 - 1) // 2,), self.device, "params")
+        _exact(dq1, torch.float32, (n1, n1), self.device, "dq1")
+        dparams = torch.empty_like(params)
+        _check(lib().bfq_cayley_backward(self._h, params.data_ptr(), int(n1), dq1.data_ptr(), dparams.data_ptr(), _stream(params)),
+               "bfq_cayley_backward")
+        return dparams
 
     def forward_quant_stats(self, x: torch.Tensor, bits: int):
         """-> (codes, scales, hist int64 [2^bits], rowstats fp32 [rows][2] = (sum y^2, sum y^4))."""

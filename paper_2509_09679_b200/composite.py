@@ -10,7 +10,8 @@ With a token row as an n1 x n2 matrix X and Y = Q1 (X Q2^T), for an upstream gra
                  M = (I + A)^-1, dQ1 = -(I + Q1) dA M, so dL/dA = -(I + Q1)^T (dL/dQ1) M^T and the parameter (i < j)
                  receives dL/dA[i][j] - dL/dA[j][i].
 
-Everything that touches the butterfly runs in the bfq kernels; the n1 x n1 algebra is torch in float64.
+bfq_composite_backward computes the first four in one pass for 128 <= n2 <= 1024, bfq_cayley_backward the last; other sizes and
+types are composed from the butterfly's own entry points and torch (the n1 x n1 algebra in float64).
 """
 from __future__ import annotations
 
@@ -33,15 +34,29 @@ def cayley_pullback(params: torch.Tensor, n1: int, dQ1: torch.Tensor) -> torch.T
     return (dA - dA.t())[iu[0], iu[1]].to(params.dtype)
 
 
+def _one_pass(plan: Plan, n1: int) -> bool:
+    """Whether bfq_composite_backward takes these sizes (its limits are in the header)."""
+    return 128 <= plan.n <= 1024 and 2 <= n1 <= 64 and 12 * n1 * (plan.n + 4) + 4 * n1 * (-(-n1 // 8) * 8) <= 227 * 1024
+
+
 def composite_backward(plan: Plan, q1: torch.Tensor, params: torch.Tensor | None, x: torch.Tensor, g: torch.Tensor):
     """x, g: [tokens][n1 * n2] (same dtype).  Returns (dx, dtheta2, dQ1, dparams or None)."""
     n1, n2 = q1.shape[0], plan.n
     tokens = x.shape[0]
-    gp = torch.einsum("ki,rkj->rij", q1, g.reshape(tokens, n1, n2).float())      # G' = Q1^T G
-    runs_x = x.reshape(tokens * n1, n2)
-    runs_g = gp.reshape(tokens * n1, n2).to(x.dtype)
-    dx_runs, dtheta2 = plan.backward(runs_x, runs_g)                             # dx = G' Q2 per run, d-theta summed over runs
-    xp = plan.forward(runs_x, out_dtype=torch.float32).reshape(tokens, n1, n2)   # X' = X Q2^T
-    dQ1 = torch.einsum("rij,rkj->ik", g.reshape(tokens, n1, n2).float(), xp)
-    dparams = cayley_pullback(params, n1, dQ1) if params is not None else None
-    return dx_runs.reshape(tokens, n1 * n2), dtheta2, dQ1, dparams
+    if _one_pass(plan, n1) and q1.dtype == torch.float32:
+        g2 = g.reshape(tokens, n1 * n2).contiguous()
+        dx, dtheta2, dQ1 = plan.composite_backward(q1.contiguous(), x.reshape(tokens, n1 * n2).contiguous(),
+                                                   g2 if g2.dtype in (torch.float32, torch.bfloat16) else g2.float())
+    else:
+        gp = torch.einsum("ki,rkj->rij", q1, g.reshape(tokens, n1, n2).float())      # G' = Q1^T G
+        runs_x = x.reshape(tokens * n1, n2)
+        runs_g = gp.reshape(tokens * n1, n2).to(x.dtype)
+        dx_runs, dtheta2 = plan.backward(runs_x, runs_g)                             # dx = G' Q2 per run, d-theta summed over runs
+        xp = plan.forward(runs_x, out_dtype=torch.float32).reshape(tokens, n1, n2)   # X' = X Q2^T
+        dQ1 = torch.einsum("rij,rkj->ik", g.reshape(tokens, n1, n2).float(), xp)
+        dx = dx_runs.reshape(tokens, n1 * n2)
+    if params is None:
+        return dx, dtheta2, dQ1, None
+    if params.dtype == torch.float32 and params.device == plan.device and params.dim() == 1 and params.is_contiguous() and 2 <= n1 <= 64:
+        return dx, dtheta2, dQ1, plan.cayley_backward(params, n1, dQ1.contiguous())
+    return dx, dtheta2, dQ1, cayley_pullback(params, n1, dQ1)

@@ -757,6 +757,42 @@ int bfq_composite_forward_quant(bfq_plan* plan, const float* q1, int n1, const v
     return composite_impl(plan, q1, n1, x, xt, rows, ldx, nullptr, BFQ_F32, 0, bits, codes, scales_f16, stream);
 }
 
+int bfq_cayley_backward(bfq_plan* plan, const float* params, int n1, const float* dq1, float* dparams, void* stream) {
+    if (plan == nullptr || params == nullptr || dq1 == nullptr || dparams == nullptr) return BFQ_ERR_NULL;
+    if (n1 < 2 || n1 > BFQ_MAX_N1) return BFQ_ERR_UNSUPPORTED_N;
+    for (const void* p : {static_cast<const void*>(params), static_cast<const void*>(dq1), static_cast<const void*>(dparams)})
+        if ((reinterpret_cast<uintptr_t>(p) & 3u) != 0) return BFQ_ERR_ALIGN;
+    DeviceGuard guard(plan->device);
+    if (guard.err != cudaSuccess) return cuda_fail(plan, guard.err);
+    cudaError_t e = cayley_backward_launch(params, n1, dq1, dparams, static_cast<cudaStream_t>(stream));
+    return e == cudaSuccess ? BFQ_OK : cuda_fail(plan, e);
+}
+
+int bfq_composite_backward(bfq_plan* plan, const float* q1, int n1, const void* x, bfq_dtype xt, const void* g, bfq_dtype gt, int64_t rows,
+                           int64_t ld, void* dx, float* dtheta, float* dq1, void* stream) {
+    if (plan == nullptr || q1 == nullptr || dtheta == nullptr || dq1 == nullptr) return BFQ_ERR_NULL;
+    if (n1 < 2 || n1 > BFQ_MAX_N1 || !composite_backward_available(plan, n1)) return BFQ_ERR_UNSUPPORTED_N;
+    const int d = n1 * plan->n;
+    int rc = check_rows(x, xt, rows, ld, d);
+    if (rc == BFQ_OK) rc = check_rows(g, gt, rows, ld, d);
+    if (rc == BFQ_OK && dx != nullptr) rc = check_rows(dx, xt, rows, ld, d);
+    if (rc != BFQ_OK) return rc;
+    for (const void* p : {static_cast<const void*>(q1), static_cast<const void*>(dtheta), static_cast<const void*>(dq1)})
+        if ((reinterpret_cast<uintptr_t>(p) & 3u) != 0) return BFQ_ERR_ALIGN;
+    if (!plan->angles_set) return BFQ_ERR_WORKSPACE;
+    DeviceGuard guard(plan->device);
+    if (guard.err != cudaSuccess) return cuda_fail(plan, guard.err);
+    cudaStream_t st = static_cast<cudaStream_t>(stream);
+    cudaError_t e;
+    if (rows == 0) {
+        e = cudaMemsetAsync(dtheta, 0, sizeof(float) * size_t(plan->log_n) * (plan->n / 2), st);
+        if (e == cudaSuccess) e = cudaMemsetAsync(dq1, 0, sizeof(float) * n1 * n1, st);
+    } else {
+        e = composite_backward_launch(plan, q1, n1, x, xt, g, gt, rows, ld, dx, dtheta, dq1, st);
+    }
+    return e == cudaSuccess ? BFQ_OK : cuda_fail(plan, e);
+}
+
 int bfq_device_status(bfq_plan* plan) {
     if (plan == nullptr) return BFQ_ERR_NULL;
     DeviceGuard guard(plan->device);

@@ -406,35 +406,34 @@ k_comp5120d(const __grid_constant__ Params P, const __grid_constant__ CUtensorMa
     }
 }
 
-// Dense Q2 from the plan's (cos, sin) table: thread c pushes the unit vector e_c through the 7 stages in float64 and
-// writes column c, split into two bf16 terms, at its place in the swizzled K-major operand image:
-// [term][half = c / 64][row j][16-byte chunk ((c mod 64) / 8) xor (j mod 8)][c mod 8].
-// The second image (offset kQ2Bytes) holds Q2^T in the same layout, for the inverse transform.
-__global__ void __launch_bounds__(kN2) k_build_dense128(const float2* __restrict__ tw, __nv_bfloat16* __restrict__ img) {
-    const int c = threadIdx.x;
-    double col[kN2];
-    for (int jj = 0; jj < kN2; ++jj) col[jj] = jj == c ? 1.0 : 0.0;
+// Q2 dense from the (cos, sin) table, split into two bf16 terms at its place in the swizzled K-major operand image:
+// [term][half = c / 64][row j][16-byte chunk ((c mod 64) / 8) xor (j mod 8)][c mod 8].  The second image (offset kQ2Bytes)
+// holds Q2^T in the same layout, for the inverse transform.
+// Between input c and output j there is one path through the butterfly (before stage s the index has the bits of j below s and
+// those of c from s on), so an entry is a product of seven numbers in double: one thread per entry.  (One thread per
+// column applying the stages took 77 us.)
+__global__ void __launch_bounds__(256) k_build_dense128(const float2* __restrict__ tw, __nv_bfloat16* __restrict__ img) {
+    grid_dep_launch();
+    grid_dep_wait();
+    const int k = blockIdx.x * 256 + threadIdx.x, j = k >> 7, c = k & (kN2 - 1);
+    double v = 1.0;
+#pragma unroll
     for (int s = 0; s < 7; ++s) {
-        for (int q = 0; q < kN2 / 2; ++q) {
-            const int lo = ((q >> s) << (s + 1)) | (q & ((1 << s) - 1)), hi = lo + (1 << s);
-            const float2 cs = tw[s * (kN2 / 2) + q];
-            const double x0 = col[lo], x1 = col[hi];
-            col[lo] = double(cs.x) * x0 - double(cs.y) * x1;
-            col[hi] = double(cs.y) * x0 + double(cs.x) * x1;
-        }
+        const int i = (j & ((1 << s) - 1)) | (c & ~((1 << s) - 1));  // the index before stage s; bit s is c's, then j's
+        const float2 cs = __ldg(tw + s * (kN2 / 2) + (((i >> (s + 1)) << s) | (i & ((1 << s) - 1))));
+        const int from = (c >> s) & 1, to = (j >> s) & 1;
+        v *= from == to ? double(cs.x) : (to ? double(cs.y) : -double(cs.y));
     }
-    for (int jj = 0; jj < kN2; ++jj) {
-        const float f = static_cast<float>(col[jj]);
-        const __nv_bfloat16 hi = __float2bfloat16_rn(f);
-        const __nv_bfloat16 lo = __float2bfloat16_rn(f - __bfloat162float(hi));
-        const int idx = (c >> 6) * (kQ2Half / 2) + jj * 64 + ((((c & 63) >> 3) ^ (jj & 7)) << 3) + (c & 7);
-        img[idx] = hi;
-        img[2 * (kQ2Half / 2) + idx] = lo;
-        // transposed: row c, contraction index jj
-        const int idt = (jj >> 6) * (kQ2Half / 2) + c * 64 + ((((jj & 63) >> 3) ^ (c & 7)) << 3) + (jj & 7);
-        img[kQ2Bytes / 2 + idt] = hi;
-        img[kQ2Bytes / 2 + 2 * (kQ2Half / 2) + idt] = lo;
-    }
+    const float f = static_cast<float>(v);
+    const __nv_bfloat16 hi = __float2bfloat16_rn(f);
+    const __nv_bfloat16 lo = __float2bfloat16_rn(f - __bfloat162float(hi));
+    const int idx = (c >> 6) * (kQ2Half / 2) + j * 64 + ((((c & 63) >> 3) ^ (j & 7)) << 3) + (c & 7);
+    img[idx] = hi;
+    img[2 * (kQ2Half / 2) + idx] = lo;
+    // transposed: row c, contraction index j
+    const int idt = (j >> 6) * (kQ2Half / 2) + c * 64 + ((((j & 63) >> 3) ^ (c & 7)) << 3) + (j & 7);
+    img[kQ2Bytes / 2 + idt] = hi;
+    img[kQ2Bytes / 2 + 2 * (kQ2Half / 2) + idt] = lo;
 }
 
 }  // namespace c5d
@@ -447,8 +446,8 @@ bool comp5120d_available(const bfq_plan* plan) {
 }
 
 cudaError_t comp5120d_set_angles(const bfq_plan* plan, cudaStream_t st) {
-    c5d::k_build_dense128<<<1, c5d::kN2, 0, st>>>(plan->tw, static_cast<__nv_bfloat16*>(plan->dense128));
-    return cudaGetLastError();
+    return launch_overlapped(c5d::k_build_dense128, dim3(c5d::kN2 * c5d::kN2 / 256), dim3(256), 0, st, plan->tw,
+                             static_cast<__nv_bfloat16*>(plan->dense128));
 }
 
 cudaError_t comp5120d_launch(bfq_plan* plan, const float* q1, const void* x, int64_t rows, int64_t ldx, int bits,

@@ -6,9 +6,9 @@
 // Seen as an n1 x n2 matrix X (row r = the r-th run of n2 consecutive elements), one token maps to
 //     Y = Q1 (X Q2^T):   the butterfly on every run, then the dense factor across the runs.
 //
-// This file holds the Cayley solve and the kernels that work for every (n1 <= 64, n2 <= 1024, n1 n2 <= 16384);
+// This file holds the kernels that work for every (n1 <= 64, n2 <= 1024, n1 n2 <= 16384);
 // the tensor-core kernels for 40 x 128 live in bfq_comp5120d.cu (both factors as MMAs) and bfq_comp5120.cu (fp32
-// butterfly + MMA dense factor) and must agree with these.
+// butterfly + MMA dense factor) and must agree with these; the Cayley transform in bfq_cayley.cu, the backward in bfq_compbwd.cu.
 #include <cuda_runtime.h>
 
 #include "bfq_fast.h"
@@ -16,63 +16,6 @@
 
 namespace bfq {
 namespace comp {
-
-// ---- Q1 = (I - A)(I + A)^{-1} -------------------------------------------------------------------------------
-// (I - A) and (I + A)^{-1} commute, so Q1 solves (I + A) Q1 = I - A: Gauss-Jordan with partial pivoting on the
-// augmented matrix [I + A | I - A], one CTA, float64 in shared memory (I + A has all singular values >= 1).
-constexpr int kCayleyThreads = 256;
-
-__global__ void __launch_bounds__(kCayleyThreads) k_cayley(const float* __restrict__ params, int n1, float* __restrict__ q1) {
-    extern __shared__ double aug[];  // [n1][2 n1]
-    __shared__ int pivot_row;
-    const int t = threadIdx.x, w = 2 * n1;
-    for (int e = t; e < n1 * n1; e += kCayleyThreads) {
-        const int i = e / n1, j = e % n1;
-        double a = 0.0;
-        if (i < j) a = static_cast<double>(params[i * n1 - i * (i + 1) / 2 + (j - i - 1)]);
-        if (i > j) a = -static_cast<double>(params[j * n1 - j * (j + 1) / 2 + (i - j - 1)]);
-        const double id = (i == j) ? 1.0 : 0.0;
-        aug[i * w + j] = id + a;
-        aug[i * w + n1 + j] = id - a;
-    }
-    __syncthreads();
-    for (int col = 0; col < n1; ++col) {
-        if (t == 0) {
-            int best = col;
-            double bv = fabs(aug[col * w + col]);
-            for (int r = col + 1; r < n1; ++r) {
-                const double v = fabs(aug[r * w + col]);
-                if (v > bv) bv = v, best = r;
-            }
-            pivot_row = best;
-        }
-        __syncthreads();
-        const int pr = pivot_row;
-        if (pr != col) {
-            for (int j = t; j < w; j += kCayleyThreads) {
-                const double tmp = aug[col * w + j];
-                aug[col * w + j] = aug[pr * w + j];
-                aug[pr * w + j] = tmp;
-            }
-        }
-        __syncthreads();
-        const double inv = 1.0 / aug[col * w + col];
-        __syncthreads();
-        for (int j = t; j < w; j += kCayleyThreads) aug[col * w + j] *= inv;
-        __syncthreads();
-        // eliminate the column from every other row; the factors are read before any row changes them
-        for (int e = t; e < n1 * w; e += kCayleyThreads) {
-            const int r = e / w, j = e % w;
-            if (r == col || j == col) continue;
-            aug[r * w + j] -= aug[r * w + col] * aug[col * w + j];
-        }
-        __syncthreads();
-        for (int r = t; r < n1; r += kCayleyThreads)
-            if (r != col) aug[r * w + col] = 0.0;
-        __syncthreads();
-    }
-    for (int e = t; e < n1 * n1; e += kCayleyThreads) q1[e] = static_cast<float>(aug[(e / n1) * w + n1 + (e % n1)]);
-}
 
 // ---- generic composite forward: one token per CTA iteration ----------------------------------------------------
 constexpr int kThreads = 256;
@@ -176,14 +119,6 @@ __global__ void __launch_bounds__(kThreads) k_composite_generic(const CompositeP
 }
 
 }  // namespace comp
-
-cudaError_t cayley_launch(const float* params, int n1, float* q1, cudaStream_t st) {
-    const size_t smem = sizeof(double) * 2 * n1 * n1;
-    cudaError_t e = cudaFuncSetAttribute(comp::k_cayley, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
-    if (e != cudaSuccess) return e;
-    comp::k_cayley<<<1, comp::kCayleyThreads, smem, st>>>(params, n1, q1);
-    return cudaGetLastError();
-}
 
 cudaError_t composite_generic_launch(const bfq_plan* plan, const float* q1, int n1, const void* x, int xt, int64_t rows,
                                      int64_t ldx, void* y, int yt, int64_t ldy, int bits, uint8_t* codes,

@@ -376,6 +376,48 @@ def test_composite_backward_against_float64_and_finite_differences():
     assert np.abs(to_f64(dpar) - fd).max() <= 2e-4 * np.abs(fd).max()
 
 
+@pytest.mark.parametrize("n1,n2,tokens", [(40, 128, 1), (40, 128, 1211), (12, 256, 333), (7, 1024, 150), (16, 1024, 67), (2, 128, 40), (64, 128, 5),
+                                          (9, 512, 700)])
+@pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
+def test_composite_backward_in_one_pass(n1, n2, tokens, dtype):
+    """Every pass structure (log2 n2 = 7 .. 10), one and four slices of dQ1, fewer tokens than CTAs and several per CTA.
+    dQ1: fp32 sums of n2 * tokens products, 1e-5 of the largest; dparams: the same relative error through the solve."""
+    from paper_2509_09679_b200.composite import cayley_pullback, composite_backward
+    from parity import check_dtheta
+    theta2, params = synth.angles(n2, "normal", 3), synth.cayley_params(n1, 3, 0.1)
+    x, g = (synth.rows(tokens, n1 * n2, "normal", s, dtype=dtype) for s in (4, 5))
+    p = Plan(n2, DEV)
+    p.set_angles(theta2.to(DEV))
+    q1 = p.cayley(params.to(DEV), n1)
+    dx, dth2, dQ1, dpar = composite_backward(p, q1, params.to(DEV), x.to(DEV), g.to(DEV))
+    th64, x64, g64, Q1 = to_f64(theta2), to_f64(x), to_f64(g), oracle.cayley(to_f64(params), n1)
+    assert np.abs(to_f64(q1) - Q1).max() <= 2e-7
+    assert dx.dtype == dtype
+    check_rows_close(dx, oracle.composite_inverse(Q1, th64, g64), np.abs(g64).max(axis=1), "dx")
+    gp = np.einsum("ki,rkj->rij", Q1, g64.reshape(tokens, n1, n2)).reshape(-1, n2)
+    check_dtheta(dth2, oracle.backward(th64, x64.reshape(-1, n2), gp)[1], "dtheta2")
+    xp = oracle.forward(th64, x64.reshape(-1, n2)).reshape(tokens, n1, n2)
+    dQ1_ref = np.einsum("rij,rkj->ik", g64.reshape(tokens, n1, n2), xp)
+    assert np.abs(to_f64(dQ1) - dQ1_ref).max() <= 1e-5 * np.abs(dQ1_ref).max()
+    dpar_ref = cayley_pullback(params.double(), n1, torch.from_numpy(dQ1_ref)).numpy()
+    assert np.abs(to_f64(dpar) - dpar_ref).max() <= 1e-5 * np.abs(dQ1_ref).max() * n1 ** 0.5
+    again = composite_backward(p, q1, None, x.to(DEV), g.to(DEV))
+    assert torch.equal(again[1], dth2) and torch.equal(again[2], dQ1) and again[3] is None
+    assert p.device_status() == 0
+
+
+@pytest.mark.parametrize("n1,scale", [(2, 1.0), (3, 50.0), (33, 0.5), (64, 5.0)])
+def test_cayley_and_its_gradient(n1, scale):
+    """Sizes around a warp's width and large parameters (the pivots move)."""
+    from paper_2509_09679_b200.composite import cayley_pullback
+    params = synth.cayley_params(n1, 11, scale)
+    p = Plan(128, DEV)
+    assert np.abs(to_f64(p.cayley(params.to(DEV), n1)) - oracle.cayley(to_f64(params), n1)).max() <= 2e-7
+    dq = synth.rows(n1, n1, "normal", 12)
+    ref = cayley_pullback(params.double(), n1, dq.double()).numpy()
+    assert np.abs(to_f64(p.cayley_backward(params.to(DEV), n1, dq.to(DEV))) - ref).max() <= 2e-7 * np.abs(ref).max()
+
+
 @pytest.mark.parametrize("rows", [1, 3, 5, 593, 2500])
 def test_tensor_core_composite_5120_int8(rows):
     p, q1, x, y_ref, tol = _tf32_setup(rows, seed=17, path="dense")
