@@ -85,31 +85,41 @@ def _check(status: int, where: str):
         raise BfqError(status, where)
 
 
+_DTYPES = {torch.float32: BFQ_F32, torch.bfloat16: BFQ_BF16}
+
+
 def _dt(t: torch.Tensor) -> int:
-    if t.dtype == torch.float32:
-        return BFQ_F32
-    if t.dtype == torch.bfloat16:
-        return BFQ_BF16
-    raise TypeError(f"unsupported dtype {t.dtype}")
+    kind = _DTYPES.get(t.dtype)
+    if kind is None:
+        raise TypeError(f"unsupported dtype {t.dtype}")
+    return kind
 
 
+# A call of a few microseconds on the GPU is bound by what happens here, so each property of a tensor is asked for once,
+# buffers allocated here are not checked again, and the stream is read as the raw handle (the Stream object that
+# torch.cuda.current_stream builds takes longer than the rest of a call).
 def _rows(t: torch.Tensor, n: int, device=None, rows=None, what: str = "rows"):
     """Checks a [rows][n] row tensor (unit inner stride; on `device` when given; `rows` rows when given) and returns
     (rows, leading dimension).  Only this layer knows the buffers' sizes: the C ABI takes bare pointers."""
-    if not isinstance(t, torch.Tensor) or t.dim() != 2 or t.shape[1] != n or t.stride(1) != 1:
-        raise ValueError(f"{what}: expected a [rows][{n}] tensor with unit inner stride, got "
-                         f"{tuple(t.shape) if isinstance(t, torch.Tensor) else type(t)}")
+    if not isinstance(t, torch.Tensor):
+        raise ValueError(f"{what}: expected a [rows][{n}] tensor with unit inner stride, got {type(t)}")
+    shape, stride = t.shape, t.stride()
+    if len(shape) != 2 or shape[1] != n or stride[1] != 1:
+        raise ValueError(f"{what}: expected a [rows][{n}] tensor with unit inner stride, got {tuple(shape)}")
     if device is not None:
         _on(t, device, what)
-    if rows is not None and t.shape[0] != rows:
-        raise ValueError(f"{what}: expected {rows} rows, got {t.shape[0]}")
-    if t.shape[0] > 1 and t.stride(0) < n:
-        raise ValueError(f"{what}: rows overlap (row stride {t.stride(0)} < {n})")
-    return t.shape[0], (t.stride(0) if t.shape[0] > 1 else max(t.stride(0), n))
+    count, ld = shape[0], stride[0]
+    if rows is not None and count != rows:
+        raise ValueError(f"{what}: expected {rows} rows, got {count}")
+    if ld < n:
+        if count > 1:
+            raise ValueError(f"{what}: rows overlap (row stride {ld} < {n})")
+        ld = n
+    return count, ld
 
 
 def _on(t: torch.Tensor, device, what: str):
-    if not t.is_cuda or t.device != device:
+    if t.get_device() != device.index or not t.is_cuda:
         raise ValueError(f"{what}: tensor is on {t.device}, the plan works on {device}")
 
 
@@ -123,7 +133,7 @@ def _exact(t: torch.Tensor, dtype, shape, device, what: str):
 
 
 def _stream(t: torch.Tensor):
-    return ctypes.c_void_p(torch.cuda.current_stream(t.device).cuda_stream)
+    return torch._C._cuda_getCurrentRawStream(t.get_device())
 
 
 class GemmOperand:
@@ -131,7 +141,8 @@ class GemmOperand:
     stored rows; `transposed` = stored [K][rows] instead of [rows][K]."""
 
     def __init__(self, data: torch.Tensor, scales: torch.Tensor | None = None, bits: int = 0, transposed: bool = False):
-        if data.dim() != 2 or data.stride(1) != 1:
+        shape, stride = data.shape, data.stride()
+        if len(shape) != 2 or stride[1] != 1:
             raise ValueError("operand: expected a 2-D tensor with unit inner stride")
         self.data, self.scales, self.transposed = data, scales, bool(transposed)
         if scales is None:
@@ -140,10 +151,10 @@ class GemmOperand:
             if bits not in (2, 4, 8) or data.dtype != torch.uint8:
                 raise ValueError("operand: codes are uint8 with bits in {2, 4, 8}")
             self.kind, per = bits, 8 // bits
-            _exact(scales, torch.float16, (data.shape[0],), data.device, "operand scales")
-        stored_rows, width = data.shape[0], data.shape[1] * per
+            _exact(scales, torch.float16, (shape[0],), data.device, "operand scales")
+        stored_rows, width = shape[0], shape[1] * per
         self.rows, self.k = (width, stored_rows) if transposed else (stored_rows, width)
-        self.ld = (data.stride(0) if stored_rows > 1 else data.shape[1]) * per
+        self.ld = (stride[0] if stored_rows > 1 else shape[1]) * per
 
 
 class Plan:
@@ -157,6 +168,7 @@ class Plan:
         self.L = self.n.bit_length() - 1
         self.device = torch.device("cuda", dev.index if dev.index is not None else torch.cuda.current_device())
         self._h = ctypes.c_void_p()
+        self._c = lib()
         _check(lib().bfq_plan_create(ctypes.byref(self._h), self.n, int(max_rows), self.device.index),
                "bfq_plan_create")
 
@@ -174,32 +186,40 @@ class Plan:
     # -- the C ABI, one method per entry point ------------------------------------------------------
     def set_angles(self, theta: torch.Tensor):
         _exact(theta, torch.float32, (self.L, self.n // 2), self.device, "theta")
-        _check(lib().bfq_set_angles(self._h, theta.data_ptr(), _stream(theta)), "bfq_set_angles")
+        _check(self._c.bfq_set_angles(self._h, theta.data_ptr(), _stream(theta)), "bfq_set_angles")
 
     def forward(self, x: torch.Tensor, out_dtype=None, out: torch.Tensor | None = None) -> torch.Tensor:
-        rows, ldx = _rows(x, self.n, self.device, what="x")
-        y = out if out is not None else torch.empty((rows, self.n), dtype=out_dtype or x.dtype, device=x.device)
-        _, ldy = _rows(y, self.n, self.device, rows, "out")
-        _check(lib().bfq_forward(self._h, x.data_ptr(), _dt(x), rows, ldx, y.data_ptr(), _dt(y), ldy, _stream(x)),
-               "bfq_forward")
+        n = self.n
+        rows, ldx = _rows(x, n, self.device, what="x")
+        y, ldy = self._row_output(x, rows, out_dtype, out)
+        _check(self._c.bfq_forward(self._h, x.data_ptr(), _dt(x), rows, ldx, y.data_ptr(), _dt(y), ldy, _stream(x)), "bfq_forward")
         return y
+
+    def _row_output(self, x: torch.Tensor, rows: int, out_dtype, out):
+        """The caller's [rows][n] buffer, checked, or a new one; and its leading dimension."""
+        n = self.n
+        if out is not None:
+            return out, _rows(out, n, self.device, rows, "out")[1]
+        return torch.empty((rows, n), dtype=out_dtype or x.dtype, device=self.device), n
 
     def _outputs(self, rows: int, width: int, bits: int, codes, scales):
         """Allocates or checks the codes uint8 [rows][width * bits / 8] and scales fp16 [rows] buffers (the bit width
         itself is the C side's to reject, before any launch)."""
-        bits = int(bits)
+        shape = (rows, width * int(bits) // 8)
         if codes is None:
-            codes = torch.empty((rows, width * bits // 8), dtype=torch.uint8, device=self.device)
+            codes = torch.empty(shape, dtype=torch.uint8, device=self.device)
+        else:
+            _exact(codes, torch.uint8, shape, self.device, "codes")
         if scales is None:
-            scales = torch.empty((rows,), dtype=torch.float16, device=self.device)
-        _exact(codes, torch.uint8, (rows, width * bits // 8), self.device, "codes")
-        _exact(scales, torch.float16, (rows,), self.device, "scales")
+            scales = torch.empty(rows, dtype=torch.float16, device=self.device)
+        else:
+            _exact(scales, torch.float16, (rows,), self.device, "scales")
         return codes, scales
 
     def forward_quant(self, x: torch.Tensor, bits: int, codes=None, scales=None):
         rows, ldx = _rows(x, self.n, self.device, what="x")
         codes, scales = self._outputs(rows, self.n, bits, codes, scales)
-        _check(lib().bfq_forward_quant(self._h, x.data_ptr(), _dt(x), rows, ldx, int(bits), codes.data_ptr(),
+        _check(self._c.bfq_forward_quant(self._h, x.data_ptr(), _dt(x), rows, ldx, int(bits), codes.data_ptr(),
                                        scales.data_ptr(), _stream(x)), "bfq_forward_quant")
         return codes, scales
 
@@ -210,7 +230,7 @@ class Plan:
             raise ValueError("params must be a contiguous fp32 tensor of n1 (n1 - 1) / 2 entries")
         _on(params, self.device, "params")
         q1 = torch.empty((n1, n1), dtype=torch.float32, device=params.device)
-        _check(lib().bfq_cayley(self._h, params.data_ptr(), int(n1), q1.data_ptr(), _stream(params)), "bfq_cayley")
+        _check(self._c.bfq_cayley(self._h, params.data_ptr(), int(n1), q1.data_ptr(), _stream(params)), "bfq_cayley")
         return q1
 
     def _q1(self, q1: torch.Tensor) -> int:
@@ -226,7 +246,7 @@ class Plan:
         y = out if out is not None else torch.empty((rows, d), dtype=out_dtype or x.dtype, device=x.device)
         if _rows(y, d, self.device, rows, "out")[1] != d:
             raise ValueError("out: rows must be contiguous")
-        _check(lib().bfq_composite_forward(self._h, q1.data_ptr(), n1, x.data_ptr(), _dt(x), rows, ldx, y.data_ptr(),
+        _check(self._c.bfq_composite_forward(self._h, q1.data_ptr(), n1, x.data_ptr(), _dt(x), rows, ldx, y.data_ptr(),
                                            _dt(y), d, _stream(x)), "bfq_composite_forward")
         return y
 
@@ -237,7 +257,7 @@ class Plan:
         x = out if out is not None else torch.empty((rows, d), dtype=out_dtype or y.dtype, device=y.device)
         if _rows(x, d, self.device, rows, "out")[1] != d:
             raise ValueError("out: rows must be contiguous")
-        _check(lib().bfq_composite_inverse(self._h, q1.data_ptr(), n1, y.data_ptr(), _dt(y), rows, ldy, x.data_ptr(),
+        _check(self._c.bfq_composite_inverse(self._h, q1.data_ptr(), n1, y.data_ptr(), _dt(y), rows, ldy, x.data_ptr(),
                                            _dt(x), d, _stream(y)), "bfq_composite_inverse")
         return x
 
@@ -246,7 +266,7 @@ class Plan:
         d = n1 * self.n
         rows, ldx = _rows(x, d, self.device, what="x")
         codes, scales = self._outputs(rows, d, bits, codes, scales)
-        _check(lib().bfq_composite_forward_quant(self._h, q1.data_ptr(), n1, x.data_ptr(), _dt(x), rows, ldx, int(bits),
+        _check(self._c.bfq_composite_forward_quant(self._h, q1.data_ptr(), n1, x.data_ptr(), _dt(x), rows, ldx, int(bits),
                                                  codes.data_ptr(), scales.data_ptr(), _stream(x)),
                "bfq_composite_forward_quant")
         return codes, scales
@@ -261,7 +281,7 @@ class Plan:
         dx = torch.empty((rows, d), dtype=x.dtype, device=x.device)
         dtheta = torch.empty((self.L, self.n // 2), dtype=torch.float32, device=x.device)
         dq1 = torch.empty((n1, n1), dtype=torch.float32, device=x.device)
-        _check(lib().bfq_composite_backward(self._h, q1.data_ptr(), n1, x.data_ptr(), _dt(x), g.data_ptr(), _dt(g), rows, d, dx.data_ptr(),
+        _check(self._c.bfq_composite_backward(self._h, q1.data_ptr(), n1, x.data_ptr(), _dt(x), g.data_ptr(), _dt(g), rows, d, dx.data_ptr(),
                                             dtheta.data_ptr(), dq1.data_ptr(), _stream(x)), "bfq_composite_backward")
         return dx, dtheta, dq1
 
@@ -270,7 +290,7 @@ class Plan:
         _exact(params, torch.float32, (n1 * (n1 - 1) // 2,), self.device, "params")
         _exact(dq1, torch.float32, (n1, n1), self.device, "dq1")
         dparams = torch.empty_like(params)
-        _check(lib().bfq_cayley_backward(self._h, params.data_ptr(), int(n1), dq1.data_ptr(), dparams.data_ptr(), _stream(params)),
+        _check(self._c.bfq_cayley_backward(self._h, params.data_ptr(), int(n1), dq1.data_ptr(), dparams.data_ptr(), _stream(params)),
                "bfq_cayley_backward")
         return dparams
 
@@ -280,31 +300,29 @@ class Plan:
         codes, scales = self._outputs(rows, self.n, bits, None, None)
         hist = torch.empty((1 << bits,), dtype=torch.int64, device=x.device)
         rowstats = torch.empty((rows, 2), dtype=torch.float32, device=x.device)
-        _check(lib().bfq_forward_quant_stats(self._h, x.data_ptr(), _dt(x), rows, ldx, int(bits), codes.data_ptr(),
+        _check(self._c.bfq_forward_quant_stats(self._h, x.data_ptr(), _dt(x), rows, ldx, int(bits), codes.data_ptr(),
                                              scales.data_ptr(), hist.data_ptr(), rowstats.data_ptr(), _stream(x)),
                "bfq_forward_quant_stats")
         return codes, scales, hist, rowstats
 
     def hadamard(self, x: torch.Tensor, out_dtype=None, out: torch.Tensor | None = None) -> torch.Tensor:
         rows, ldx = _rows(x, self.n, self.device, what="x")
-        y = out if out is not None else torch.empty((rows, self.n), dtype=out_dtype or x.dtype, device=x.device)
-        _, ldy = _rows(y, self.n, self.device, rows, "out")
-        _check(lib().bfq_hadamard(self._h, x.data_ptr(), _dt(x), rows, ldx, y.data_ptr(), _dt(y), ldy, _stream(x)),
+        y, ldy = self._row_output(x, rows, out_dtype, out)
+        _check(self._c.bfq_hadamard(self._h, x.data_ptr(), _dt(x), rows, ldx, y.data_ptr(), _dt(y), ldy, _stream(x)),
                "bfq_hadamard")
         return y
 
     def hadamard_quant(self, x: torch.Tensor, bits: int, codes=None, scales=None):
         rows, ldx = _rows(x, self.n, self.device, what="x")
         codes, scales = self._outputs(rows, self.n, bits, codes, scales)
-        _check(lib().bfq_hadamard_quant(self._h, x.data_ptr(), _dt(x), rows, ldx, int(bits), codes.data_ptr(),
+        _check(self._c.bfq_hadamard_quant(self._h, x.data_ptr(), _dt(x), rows, ldx, int(bits), codes.data_ptr(),
                                         scales.data_ptr(), _stream(x)), "bfq_hadamard_quant")
         return codes, scales
 
     def inverse(self, y: torch.Tensor, out_dtype=None, out: torch.Tensor | None = None) -> torch.Tensor:
         rows, ldy = _rows(y, self.n, self.device, what="y")
-        x = out if out is not None else torch.empty((rows, self.n), dtype=out_dtype or y.dtype, device=y.device)
-        _, ldx = _rows(x, self.n, self.device, rows, "out")
-        _check(lib().bfq_inverse(self._h, y.data_ptr(), _dt(y), rows, ldy, x.data_ptr(), _dt(x), ldx, _stream(y)),
+        x, ldx = self._row_output(y, rows, out_dtype, out)
+        _check(self._c.bfq_inverse(self._h, y.data_ptr(), _dt(y), rows, ldy, x.data_ptr(), _dt(x), ldx, _stream(y)),
                "bfq_inverse")
         return x
 
@@ -314,13 +332,14 @@ class Plan:
         if rows_g != rows or ld_g != ld:
             raise ValueError("x and g must have the same shape and row stride")
         if want_dx and dx is None:
-            dx = torch.empty_strided((rows, self.n), (ld, 1), dtype=dx_dtype or x.dtype, device=x.device)
-        if want_dx and _rows(dx, self.n, self.device, rows, "dx")[1] != ld:
+            dx = torch.empty_strided((rows, self.n), (ld, 1), dtype=dx_dtype or x.dtype, device=self.device)
+        elif want_dx and _rows(dx, self.n, self.device, rows, "dx")[1] != ld:
             raise ValueError("dx must have the row stride of x")
         if dtheta is None:
-            dtheta = torch.empty((self.L, self.n // 2), dtype=torch.float32, device=x.device)
-        _exact(dtheta, torch.float32, (self.L, self.n // 2), self.device, "dtheta")
-        _check(lib().bfq_backward(self._h, x.data_ptr(), _dt(x), g.data_ptr(), _dt(g), rows, ld,
+            dtheta = torch.empty((self.L, self.n // 2), dtype=torch.float32, device=self.device)
+        else:
+            _exact(dtheta, torch.float32, (self.L, self.n // 2), self.device, "dtheta")
+        _check(self._c.bfq_backward(self._h, x.data_ptr(), _dt(x), g.data_ptr(), _dt(g), rows, ld,
                                   dx.data_ptr() if want_dx else None, _dt(dx) if want_dx else BFQ_F32,
                                   dtheta.data_ptr(), _stream(x)), "bfq_backward")
         return (dx if want_dx else None), dtheta
@@ -328,7 +347,7 @@ class Plan:
     def forward_quant_host_workspace(self, dtype, bits: int, chunk_rows: int) -> int:
         """Bytes of device workspace for forward_quant_host in chunks of chunk_rows rows."""
         xt = BFQ_F32 if dtype == torch.float32 else BFQ_BF16
-        return int(lib().bfq_forward_quant_host_workspace(self._h, xt, int(bits), int(chunk_rows)))
+        return int(self._c.bfq_forward_quant_host_workspace(self._h, xt, int(bits), int(chunk_rows)))
 
     def forward_quant_host(self, x_host: torch.Tensor, bits: int, codes_host: torch.Tensor, scales_host: torch.Tensor,
                            workspace: torch.Tensor):
@@ -349,7 +368,7 @@ class Plan:
             raise ValueError("workspace must be a contiguous uint8 tensor on the plan's device")
         with torch.cuda.device(self.device):
             stream = torch.cuda.current_stream(self.device).cuda_stream
-            _check(lib().bfq_forward_quant_host(self._h, x_host.data_ptr(), _dt(x_host), rows, x_host.stride(0), int(bits),
+            _check(self._c.bfq_forward_quant_host(self._h, x_host.data_ptr(), _dt(x_host), rows, x_host.stride(0), int(bits),
                                                 codes_host.data_ptr(), scales_host.data_ptr(), workspace.data_ptr(),
                                                 workspace.numel(), stream), "bfq_forward_quant_host")
 
@@ -357,7 +376,7 @@ class Plan:
         m, ldw = _rows(W, self.n, self.device, what="W")
         codes, scales = self._outputs(m, self.n, bits, None, None)
         rot = torch.empty((m, self.n), dtype=rotated_dtype or W.dtype, device=W.device) if want_rotated else None
-        _check(lib().bfq_fold_weights(self._h, W.data_ptr(), _dt(W), m, ldw, int(bits), codes.data_ptr(),
+        _check(self._c.bfq_fold_weights(self._h, W.data_ptr(), _dt(W), m, ldw, int(bits), codes.data_ptr(),
                                       scales.data_ptr(), rot.data_ptr() if rot is not None else None,
                                       _dt(rot) if rot is not None else BFQ_F32, _stream(W)), "bfq_fold_weights")
         return codes, scales, rot
@@ -368,9 +387,11 @@ class Plan:
             raise ValueError(f"operands disagree on K: {a.k} and {b.k}")
         for op, what in ((a, "A"), (b, "B")):
             _on(op.data, self.device, what)
-        c = out if out is not None else torch.empty((a.rows, b.rows), dtype=torch.float32, device=self.device)
-        _exact(c, torch.float32, (a.rows, b.rows), self.device, "out")
-        _check(lib().bfq_dequant_gemm(self._h, a.rows, b.rows, a.k, float(alpha), a.data.data_ptr(), a.kind,
+        if out is None:
+            c = torch.empty((a.rows, b.rows), dtype=torch.float32, device=self.device)
+        else:
+            c = _exact(out, torch.float32, (a.rows, b.rows), self.device, "out")
+        _check(self._c.bfq_dequant_gemm(self._h, a.rows, b.rows, a.k, float(alpha), a.data.data_ptr(), a.kind,
                                       int(a.transposed), a.ld, a.scales.data_ptr() if a.scales is not None else None,
                                       b.data.data_ptr(), b.kind, int(b.transposed), b.ld,
                                       b.scales.data_ptr() if b.scales is not None else None, c.data_ptr(), b.rows,
@@ -378,20 +399,20 @@ class Plan:
         return c
 
     def device_status(self) -> int:
-        return int(lib().bfq_device_status(self._h))
+        return int(self._c.bfq_device_status(self._h))
 
     def stage_form(self) -> int:
         """bit 0 / bit 1: the forward / inverse tables of the tuned kernels use the three-shear fallback."""
-        r = int(lib().bfq_stage_form(self._h))
+        r = int(self._c.bfq_stage_form(self._h))
         if r < 0:
             raise BfqError(r, "bfq_stage_form")
         return r
 
     def test_stuck_wait(self, enable: bool):
-        _check(lib().bfq_test_stuck_wait(self._h, int(bool(enable))), "bfq_test_stuck_wait")
+        _check(self._c.bfq_test_stuck_wait(self._h, int(bool(enable))), "bfq_test_stuck_wait")
 
     def backward_partials(self) -> int:
-        return int(lib().bfq_backward_partials(self._h))
+        return int(self._c.bfq_backward_partials(self._h))
 
 
 def backward_noalloc(theta: torch.Tensor, x: torch.Tensor, g: torch.Tensor, dx: torch.Tensor | None,
