@@ -890,6 +890,132 @@ k_dequant_gemm(const __grid_constant__ Params p, const __grid_constant__ CUtenso
     if (warp == 0) tmem_dealloc_pair(tmem_base);
 }
 
+// ---- a few rows of A against coded rows of B -----------------------------------------------------------------------
+// A decoded token or a few: the product is a pass over B's codes, and a 256-row tile of the pair kernel keeps 32 to 128
+// CTAs in a chain of K blocks (one token, 4096 x 4096 at 2 bits: 25 us).  Here a CTA of eight warps takes 16 rows of B, each
+// warp every eighth part of K, and the partial sums are added in the order of the warps.  mma.sync m16n8k16 with the codes as
+// the 16-row operand straight from registers: a lane's 16 bytes of a row are its k values, in whatever order they come, as
+// long as the lanes that hold A's rows take the same ones.  Bound by the latency of one pass over the codes, not by the
+// (legacy) tensor path.
+constexpr int kFewWarps = 8;
+
+__device__ __forceinline__ void mma_16816(float (&c)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b0, uint32_t b1) {
+    asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
+                 : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
+                 : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
+}
+// 16 bytes of codes -> 64 / KIND * 2 bf16 pairs in element order
+template <int KIND>
+__device__ __forceinline__ void codes_to_pairs(const uint4& raw, uint32_t (&o)[64 / KIND]) {
+    const uint32_t w[4] = {raw.x, raw.y, raw.z, raw.w};
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        if constexpr (KIND == BFQ_OP_CODES2) {
+            uint32_t t[8];
+            codes2_to_bf16(w[i], t);
+#pragma unroll
+            for (int j = 0; j < 8; ++j) o[8 * i + j] = t[j];
+        } else if constexpr (KIND == BFQ_OP_CODES4) {
+            uint32_t t[4];
+            codes4_to_bf16(w[i], t);
+#pragma unroll
+            for (int j = 0; j < 4; ++j) o[4 * i + j] = t[j];
+        } else {
+            uint32_t t[2];
+            codes8_to_bf16(w[i], t);
+            o[2 * i] = t[0], o[2 * i + 1] = t[1];
+        }
+    }
+}
+// 16 bytes of a row of A -> bf16 pairs in element order
+template <int KIND>
+__device__ __forceinline__ void row_to_pairs(const uint4& raw, uint32_t (&o)[KIND == BFQ_OP_BF16 ? 4 : 64 / KIND]) {
+    if constexpr (KIND == BFQ_OP_BF16) {
+        o[0] = raw.x, o[1] = raw.y, o[2] = raw.z, o[3] = raw.w;
+    } else {
+        codes_to_pairs<KIND>(raw, o);
+    }
+}
+
+// UK: kind of B's codes, VK: kind of A
+template <int UK, int VK>
+__global__ void __launch_bounds__(32 * kFewWarps) k_few_rows(const Operand u, const Operand v, float* __restrict__ c, int64_t ldc, int k, float alpha) {
+    constexpr int kElems = 128 / UK;  // codes of 16 bytes of B
+    constexpr int kVBits = VK == BFQ_OP_BF16 ? 16 : VK;
+    constexpr int kVElems = VK == BFQ_OP_BF16 ? 8 : 128 / VK;           // of 16 bytes of A
+    constexpr int kRound = kElems > kVElems ? kElems : kVElems;          // codes of B and elements of A taken together
+    constexpr int kVLoads = kRound / kVElems, kULoads = kRound / kElems;
+    __shared__ float part[kFewWarps][8][16 + 1];
+    grid_dep_launch();
+    grid_dep_wait();
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, q = lane & 3;
+    const int j0 = blockIdx.x * 16;
+    const uint8_t* urow[2];
+    bool there[2];
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        const int j = j0 + g + 8 * h;
+        there[h] = j < u.rows;
+        urow[h] = static_cast<const uint8_t*>(u.data) + int64_t(there[h] ? j : 0) * (u.ld * UK / 8);
+    }
+    const int i0 = 8 * blockIdx.y;  // the MMA's eight columns
+    const bool has_v = i0 + g < v.rows;
+    const uint8_t* vrow = static_cast<const uint8_t*>(v.data) + int64_t(has_v ? i0 + g : 0) * (v.ld * kVBits / 8);
+    float acc[4] = {0.f, 0.f, 0.f, 0.f};
+    // a lane's kRound elements of each row start at a multiple of kRound: inside K as a whole, or cut at a 16-byte piece
+    auto piece = [&](const uint8_t* row, bool yes, int at, int bits) {
+        return yes && at < k ? __ldg(reinterpret_cast<const uint4*>(row + int64_t(at) * bits / 8)) : make_uint4(0u, 0u, 0u, 0u);
+    };
+    constexpr int kStride = kFewWarps * 4 * kRound;
+    uint4 w[2][kULoads];
+    auto fetch = [&](int k0) {
+#pragma unroll
+        for (int h = 0; h < 2; ++h)
+#pragma unroll
+            for (int i = 0; i < kULoads; ++i) w[h][i] = piece(urow[h], there[h], k0 + i * kElems, UK);
+    };
+    int kl = (4 * warp + q) * kRound;
+    fetch(kl);
+    for (; kl - q * kRound < k; kl += kStride) {
+        uint4 x[kVLoads], now[2][kULoads];
+#pragma unroll
+        for (int i = 0; i < kVLoads; ++i) x[i] = piece(vrow, has_v, kl + i * kVElems, kVBits);
+#pragma unroll
+        for (int h = 0; h < 2; ++h)
+#pragma unroll
+            for (int i = 0; i < kULoads; ++i) now[h][i] = w[h][i];
+        fetch(kl + kStride);
+#pragma unroll
+        for (int part_u = 0; part_u < kULoads; ++part_u) {
+            uint32_t a[64 / UK], b[64 / UK];
+            codes_to_pairs<UK>(now[0][part_u], a);
+            codes_to_pairs<UK>(now[1][part_u], b);
+            constexpr int kVPairs = kVElems / 2;
+            uint32_t xp[kVPairs];
+#pragma unroll
+            for (int s = 0; s < kElems / 4; ++s) {
+                const int e = part_u * kElems + 4 * s;  // element of the round
+                if (e % kVElems == 0) row_to_pairs<VK>(x[e / kVElems], xp);
+                const int xi = (e % kVElems) / 2;
+                mma_16816(acc, a[2 * s], b[2 * s], a[2 * s + 1], b[2 * s + 1], xp[xi], xp[xi + 1]);
+            }
+        }
+    }
+#pragma unroll
+    for (int i = 0; i < 4; ++i) part[warp][2 * q + (i & 1)][g + 8 * (i >> 1)] = acc[i];
+    __syncthreads();
+    for (int e = threadIdx.x; e < 8 * 16; e += 32 * kFewWarps) {
+        const int i = i0 + (e >> 4), j = e & 15;
+        if (i >= v.rows || j0 + j >= u.rows) continue;
+        float sum = 0.f;
+#pragma unroll
+        for (int x = 0; x < kFewWarps; ++x) sum += part[x][e >> 4][j];
+        float scale = alpha * __half2float(__ushort_as_half(__ldg(u.scales + j0 + j)));
+        if (is_codes(VK)) scale *= __half2float(__ushort_as_half(__ldg(v.scales + i)));
+        c[int64_t(i) * ldc + j0 + j] = sum * scale;
+    }
+}
+
 // ---- host side ---------------------------------------------------------------------------------------------------
 static Operand make_operand(const void* data, const uint16_t* scales, int64_t ld, int kind, int transposed, int rows, int other_kind) {
     Operand op{data, scales, ld, kind, transposed, rows, 1, 0};
@@ -942,6 +1068,26 @@ static Shape choose_shape(int64_t m, int64_t n, int kblocks, int term_pairs, int
     return best;
 }
 
+// Up to eight rows of A one pass over the codes is faster than tiles at every size measured (1 row, us, tiles -> pass:
+// 1024 x 1024 at 2 bits 7.7 -> 2.5, 4096 x 4096 25 -> 7.0, 28672 x 8192 104 -> 44; 8 rows 8.1 -> 3.0, 26 -> 9.4, 105 -> 75).  More
+// rows are more passes, worth it while they are small together.
+static bool use_few_rows(const Operand& u, const Operand& v, int64_t k) {
+    if (!is_codes(u.kind) || u.transposed || v.kind == BFQ_OP_F32 || v.transposed) return false;
+    const int64_t passes = (int64_t(v.rows) + 7) / 8;
+    return passes == 1 || (passes <= 8 && passes * u.rows * k <= int64_t(1) << 25);
+}
+template <int UK, int VK>
+static cudaError_t launch_few(const Operand& u, const Operand& v, float* c, int64_t ldc, int k, float alpha, cudaStream_t st) {
+    return launch_overlapped(k_few_rows<UK, VK>, dim3(unsigned((u.rows + 15) / 16), unsigned((v.rows + 7) / 8)), dim3(32 * kFewWarps), 0, st, u, v, c, ldc, k, alpha);
+}
+template <int UK>
+static cudaError_t launch_few(const Operand& u, const Operand& v, float* c, int64_t ldc, int k, float alpha, cudaStream_t st) {
+    if (v.kind == BFQ_OP_BF16) return launch_few<UK, BFQ_OP_BF16>(u, v, c, ldc, k, alpha, st);
+    if (v.kind == BFQ_OP_CODES2) return launch_few<UK, BFQ_OP_CODES2>(u, v, c, ldc, k, alpha, st);
+    if (v.kind == BFQ_OP_CODES4) return launch_few<UK, BFQ_OP_CODES4>(u, v, c, ldc, k, alpha, st);
+    return launch_few<UK, BFQ_OP_CODES8>(u, v, c, ldc, k, alpha, st);
+}
+
 static cudaError_t launch(const Params& p, const CUtensorMap& map_u, const CUtensorMap& map_v, int sms, size_t smem, cudaStream_t st) {
     cudaLaunchConfig_t cfg = {};
     const int pairs = p.split > 1 ? p.tiles * p.split : (p.tiles < sms / 2 ? p.tiles : (sms / 2 > 0 ? sms / 2 : 1));
@@ -986,8 +1132,15 @@ extern "C" int bfq_dequant_gemm(bfq_plan* plan, int64_t m, int64_t n, int64_t k,
     if (cudaGetDevice(&prev) != cudaSuccess) return BFQ_ERR_CUDA;
     if (prev != plan->device && cudaSetDevice(plan->device) != cudaSuccess) return BFQ_ERR_CUDA;
     cudaError_t e = cudaSuccess;
+    const Operand u = make_operand(b, b_scales, ldb, b_kind, b_transposed, int(n), a_kind);
+    const Operand v = make_operand(a, a_scales, lda, a_kind, a_transposed, int(m), b_kind);
     if (k == 0) {
         e = cudaMemset2DAsync(c, size_t(ldc) * 4, 0, size_t(n) * 4, size_t(m), static_cast<cudaStream_t>(stream));
+    } else if (use_few_rows(u, v, k)) {
+        cudaStream_t st = static_cast<cudaStream_t>(stream);
+        e = b_kind == BFQ_OP_CODES2 ? launch_few<BFQ_OP_CODES2>(u, v, c, ldc, int(k), alpha, st)
+            : b_kind == BFQ_OP_CODES4 ? launch_few<BFQ_OP_CODES4>(u, v, c, ldc, int(k), alpha, st)
+                                      : launch_few<BFQ_OP_CODES8>(u, v, c, ldc, int(k), alpha, st);
     } else {
         constexpr size_t smem = size_t(kBarsOff) + 8 * (2 * kMaxStages + 4) + 16 + 1024;
         static bool attr_set[bfq::kMaxDevices] = {false};
@@ -997,8 +1150,7 @@ extern "C" int bfq_dequant_gemm(bfq_plan* plan, int64_t m, int64_t n, int64_t k,
         }
         if (e == cudaSuccess) {
             Params p{};
-            p.u = make_operand(b, b_scales, ldb, b_kind, b_transposed, int(n), a_kind);
-            p.v = make_operand(a, a_scales, lda, a_kind, a_transposed, int(m), b_kind);
+            p.u = u, p.v = v;
             p.c = c, p.ldc = ldc, p.k = int(k), p.alpha = alpha, p.status = plan->status_word;
             // Two code operands along K are an integer product: exact in 32 bits up to K = 2^17 - 1 (codes left in place are at
             // most 128 in size), at twice the rate of the bf16 products.

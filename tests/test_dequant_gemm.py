@@ -99,6 +99,17 @@ def test_tile_edges(ka, kb, ta, tb, m, n, k):
     check(p, A, a64, ea, B, b64, eb + (2.0 ** -24 if tb and ka == "f32" else 0.0))
 
 
+@pytest.mark.parametrize("ka", ["bf16", "codes2", "codes4", "codes8"])
+@pytest.mark.parametrize("kb", ["codes2", "codes4", "codes8"])
+@pytest.mark.parametrize("m,n,k", [(1, 16, 64), (8, 15, 192), (3, 4100, 1088), (9, 100, 4096), (64, 33, 64)])
+def test_a_few_rows_against_codes(ka, kb, m, n, k):
+    """One pass over the codes: one lane's part of K up to several turns of the warps, one to eight tiles of eight rows."""
+    p = Plan(256, DEV)
+    A, a64, ea = operand(ka, m, k, False, 930)
+    B, b64, eb = operand(kb, n, k, False, 931)
+    check(p, A, a64, ea, B, b64, eb, alpha=-1.5)
+
+
 def test_argument_validation():
     from paper_2509_09679_b200 import BfqError
     p = Plan(256, DEV)
