@@ -8,8 +8,9 @@
 //
 // A column step is a chain (find the pivot, divide, update), so its latency is what counts.  Two copies of the matrix take
 // turns: every thread reads the old one (the row exchange is only a matter of where a row is read) and writes the new one,
-// one block barrier per column; every warp finds the pivot by itself.  Four barriers and a serial pivot search per column
-// took 96 us for n1 = 40.
+// one block barrier per column; every warp finds the pivot by itself; a row is 2 n1 + 1 doubles, so that the lanes that read
+// down a column fall into different banks, and a thread's loads are all issued before its stores.  Four barriers and a serial
+// pivot search per column took 96 us for n1 = 40.
 #include <cuda_runtime.h>
 
 #include "bfq_fast.h"
@@ -19,9 +20,12 @@ namespace cay {
 
 constexpr int kThreads = 256;
 
-// Q1 of the parameters, row-major with row stride 2 n1 and the returned offset, in one of the two buffers [n1][2 n1] of `aug`
+constexpr int kMaxRows = 64 / (kThreads / 32);  // rows of a warp
+__host__ __device__ constexpr int pitch(int n1) { return 2 * n1 + 1; }
+
+// Q1 of the parameters, row-major with row stride pitch(n1), in one of the two buffers [n1][pitch] of `aug`
 __device__ __forceinline__ const double* solve(const float* __restrict__ params, int n1, double* aug) {
-    const int t = threadIdx.x, lane = t & 31, w = 2 * n1;
+    const int t = threadIdx.x, lane = t & 31, w = pitch(n1), cols = 2 * n1;
     double* cur = aug;
     double* nxt = aug + n1 * w;
     for (int e = t; e < n1 * n1; e += kThreads) {
@@ -36,26 +40,34 @@ __device__ __forceinline__ const double* solve(const float* __restrict__ params,
     __syncthreads();
     const int tx = t & 31, ty = t >> 5;  // a warp updates consecutive columns of a row
     for (int col = 0; col < n1; ++col) {
-        // the largest entry of the column from row `col` down, the first of equals (n1 <= 64: two rows per lane)
-        double best = -1.0;
-        int at = col;
-        for (int r = col + lane; r < n1; r += 32) {
-            const double v = fabs(cur[r * w + col]);
-            if (v > best) best = v, at = r;
-        }
+        // the largest entry of the column from row `col` down, compared in fp32 to 17 bits (as good a pivot as the largest), the
+        // row in the low bits so that one integer reduction gives both; n1 <= 64: two rows per lane
+        uint32_t key = 0u;
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            const double v = __shfl_xor_sync(0xFFFFFFFFu, best, o);
-            const int r = __shfl_xor_sync(0xFFFFFFFFu, at, o);
-            if (v > best || (v == best && r < at)) best = v, at = r;
+        for (int h = 0; h < 2; ++h) {
+            const int r = lane + 32 * h;
+            if (r >= col && r < n1) key = max(key, (__float_as_uint(fabsf(static_cast<float>(cur[r * w + col]))) & ~63u) | (63u - r));
         }
+        const int at = 63 - static_cast<int>(__reduce_max_sync(0xFFFFFFFFu, key) & 63u);
         const double inv = 1.0 / cur[at * w + col];
         const double* pivot = cur + at * w;
-        for (int j = col + 1 + tx; j < w; j += 32) {  // columns up to `col` are columns of the identity: not read again
+        const double* src[kMaxRows];  // row `col` has changed places with the pivot row
+        double f[kMaxRows];
+#pragma unroll
+        for (int a = 0; a < kMaxRows; ++a) {
+            const int r = ty + a * (kThreads / 32);
+            src[a] = cur + (r == at ? col : min(r, n1 - 1)) * w;
+            f[a] = src[a][col];
+        }
+        for (int j = col + 1 + tx; j < cols; j += 32) {  // columns up to `col` are columns of the identity: not read again
             const double pj = pivot[j] * inv;
-            for (int r = ty; r < n1; r += kThreads / 32) {
-                const double* src = cur + (r == at ? col : r) * w;  // row `col` has changed places with the pivot row
-                nxt[r * w + j] = r == col ? pj : src[j] - src[col] * pj;
+            double v[kMaxRows];
+#pragma unroll
+            for (int a = 0; a < kMaxRows; ++a) v[a] = src[a][j];
+#pragma unroll
+            for (int a = 0; a < kMaxRows; ++a) {
+                const int r = ty + a * (kThreads / 32);
+                if (r < n1) nxt[r * w + j] = r == col ? pj : v[a] - f[a] * pj;
             }
         }
         __syncthreads();
@@ -66,17 +78,38 @@ __device__ __forceinline__ const double* solve(const float* __restrict__ params,
 }
 
 __global__ void __launch_bounds__(kThreads) k_cayley(const float* __restrict__ params, int n1, float* __restrict__ q1) {
-    extern __shared__ double aug[];  // [2][n1][2 n1]
+    extern __shared__ double aug[];  // [2][n1][pitch]
     const double* q = solve(params, n1, aug);
-    for (int e = threadIdx.x; e < n1 * n1; e += kThreads) q1[e] = static_cast<float>(q[(e / n1) * 2 * n1 + e % n1]);
+    for (int e = threadIdx.x; e < n1 * n1; e += kThreads) q1[e] = static_cast<float>(q[(e / n1) * pitch(n1) + e % n1]);
+}
+
+// out = scale a b (n1 x n1, all threads): eight entries of a thread at a time, so that their chains overlap
+__device__ __forceinline__ void product(double* out, const double* a, const double* b, int n1, double scale) {
+    const int nn = n1 * n1;
+    for (int e0 = threadIdx.x; e0 < nn; e0 += 8 * kThreads) {
+        double s[8];
+        int ai[8], bj[8];
+#pragma unroll
+        for (int c = 0; c < 8; ++c) {
+            const int e = min(e0 + c * kThreads, nn - 1);
+            s[c] = 0.0, ai[c] = (e / n1) * n1, bj[c] = e % n1;
+        }
+        for (int k = 0; k < n1; ++k) {
+#pragma unroll
+            for (int c = 0; c < 8; ++c) s[c] = fma(a[ai[c] + k], b[k * n1 + bj[c]], s[c]);
+        }
+#pragma unroll
+        for (int c = 0; c < 8; ++c)
+            if (e0 + c * kThreads < nn) out[e0 + c * kThreads] = scale * s[c];
+    }
 }
 
 __global__ void __launch_bounds__(kThreads) k_cayley_backward(const float* __restrict__ params, int n1, const float* __restrict__ dq1,
                                                               float* __restrict__ dparams) {
-    extern __shared__ double aug[];  // [2][n1][2 n1], then two n1 x n1 matrices
+    extern __shared__ double aug[];  // [2][n1][pitch], then two n1 x n1 matrices
     const double* q = solve(params, n1, aug);
-    const int t = threadIdx.x, w = 2 * n1, nn = n1 * n1;
-    double* m2 = aug + 4 * nn;   // 2 M = I + Q1, transposed: m2[j][i] = 2 M[i][j]
+    const int t = threadIdx.x, w = pitch(n1), nn = n1 * n1;
+    double* m2 = aug + 2 * n1 * w;   // 2 M = I + Q1, transposed: m2[j][i] = 2 M[i][j]
     double* g = m2 + nn;         // dL/dQ1, then (2 M)^T (dL/dQ1)
     for (int e = t; e < nn; e += kThreads) {
         const int i = e / n1, j = e % n1;
@@ -85,19 +118,9 @@ __global__ void __launch_bounds__(kThreads) k_cayley_backward(const float* __res
     }
     __syncthreads();
     double* left = aug;  // the solve is done with its buffers
-    for (int e = t; e < nn; e += kThreads) {  // left = (2 M)^T dQ1
-        const int i = e / n1, j = e % n1;
-        double s = 0.0;
-        for (int k = 0; k < n1; ++k) s = fma(m2[i * n1 + k], g[k * n1 + j], s);
-        left[e] = s;
-    }
+    product(left, m2, g, n1, 1.0);  // (2 M)^T dQ1
     __syncthreads();
-    for (int e = t; e < nn; e += kThreads) {  // g = dL/dA = -left M^T
-        const int i = e / n1, j = e % n1;
-        double s = 0.0;
-        for (int k = 0; k < n1; ++k) s = fma(left[i * n1 + k], m2[k * n1 + j], s);
-        g[e] = -0.5 * s;
-    }
+    product(g, left, m2, n1, -0.5);  // dL/dA
     __syncthreads();
     for (int e = t; e < nn; e += kThreads) {
         const int i = e / n1, j = e % n1;
@@ -113,7 +136,7 @@ static cudaError_t allow_smem(K kern, size_t smem) {
 }
 
 cudaError_t cayley_launch(const float* params, int n1, float* q1, cudaStream_t st) {
-    const size_t smem = sizeof(double) * 4 * n1 * n1;
+    const size_t smem = sizeof(double) * 2 * n1 * cay::pitch(n1);
     cudaError_t e = allow_smem(cay::k_cayley, smem);
     if (e != cudaSuccess) return e;
     cay::k_cayley<<<1, cay::kThreads, smem, st>>>(params, n1, q1);
@@ -121,7 +144,7 @@ cudaError_t cayley_launch(const float* params, int n1, float* q1, cudaStream_t s
 }
 
 cudaError_t cayley_backward_launch(const float* params, int n1, const float* dq1, float* dparams, cudaStream_t st) {
-    const size_t smem = sizeof(double) * 6 * n1 * n1;
+    const size_t smem = sizeof(double) * (2 * n1 * cay::pitch(n1) + 2 * n1 * n1);
     cudaError_t e = allow_smem(cay::k_cayley_backward, smem);
     if (e != cudaSuccess) return e;
     cay::k_cayley_backward<<<1, cay::kThreads, smem, st>>>(params, n1, dq1, dparams);

@@ -9,6 +9,9 @@
 //   * dL/dQ1 += G X'^T: up to 4 x 4 entries per thread, kept over all tokens of the CTA (n1 <= 8: four slices of the
 //     positions, so that all threads have work);
 //   * X' and G' walked down together, d-theta in registers over all tokens, dL/dX straight from the last pass to memory.
+// Multiply-adds are packed two by two (a scalar one with three register operands issues at half rate, profiled in
+// bfq_fma_rates.cu): X' and G' of an element share a rotation, so do two runs on the way up; two positions, or two output runs,
+// in the dense products.
 // The sums of a thread, of the threads that share an angle, of the slices and of the CTAs are each added in a fixed order.
 //
 // All fp32 on the CUDA cores: at 40 x 128 a token takes 410 k multiply-adds for the two dense products and 110 k for the
@@ -19,9 +22,11 @@
 
 #include "bfq_fast.h"
 #include "bfq_generic.cuh"
+#include "bfq_ptx.cuh"
 
 namespace bfq {
 namespace cbw {
+using namespace ptx;
 
 constexpr int kThreads = 256;
 
@@ -110,32 +115,37 @@ __device__ __forceinline__ void load_angles(const float2* __restrict__ tw, int u
     if constexpr (K + 1 < Pass<L, P>::kNs) load_angles<L, P, K + 1>(tw, u, cs);
 }
 
+// two runs at once
 template <int L, int P, int K = 0>
-__device__ __forceinline__ void rotate(float (&v)[8], const float2 (&cs)[3][4]) {
+__device__ __forceinline__ void rotate(u64 (&v)[8], const float2 (&cs)[3][4]) {
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
         constexpr int bit = Pair<L, P, K>::kBit;
         const int lo = Pair<L, P, K>::lo(q), hi = lo | (1 << bit);
-        const float a = v[lo], b = v[hi];
-        v[lo] = fmaf(cs[K][q].x, a, -cs[K][q].y * b);
-        v[hi] = fmaf(cs[K][q].y, a, cs[K][q].x * b);
+        const u64 c = pack2(cs[K][q].x, cs[K][q].x), s = pack2(cs[K][q].y, cs[K][q].y), ns = pack2(-cs[K][q].y, -cs[K][q].y);
+        const u64 a = v[lo], b = v[hi];
+        v[lo] = fma2(ns, b, mul2(c, a));
+        v[hi] = fma2(s, a, mul2(c, b));
     }
     if constexpr (K + 1 < Pass<L, P>::kNs) rotate<L, P, K + 1>(v, cs);
 }
 
+// v: (x', g') of each element
 template <int L, int P, int K>
-__device__ __forceinline__ void walk_down(float (&v)[8], float (&w)[8], const float2 (&cs)[3][4], float (&acc)[3][4]) {
+__device__ __forceinline__ void walk_down(u64 (&v)[8], const float2 (&cs)[3][4], float (&acc)[3][4]) {
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
         constexpr int bit = Pair<L, P, K>::kBit;
         const int lo = Pair<L, P, K>::lo(q), hi = lo | (1 << bit);
-        const float c = cs[K][q].x, s = cs[K][q].y;
-        acc[K][q] += w[hi] * v[lo] - w[lo] * v[hi];  // on the stage's outputs
-        const float a = v[lo], b = v[hi], ga = w[lo], gb = w[hi];
-        v[lo] = fmaf(c, a, s * b), v[hi] = fmaf(c, b, -s * a);
-        w[lo] = fmaf(c, ga, s * gb), w[hi] = fmaf(c, gb, -s * ga);
+        const u64 c = pack2(cs[K][q].x, cs[K][q].x), s = pack2(cs[K][q].y, cs[K][q].y), ns = pack2(-cs[K][q].y, -cs[K][q].y);
+        const u64 a = v[lo], b = v[hi];
+        float xa, ga, xb, gb;
+        unpack2(a, xa, ga), unpack2(b, xb, gb);
+        acc[K][q] = fmaf(gb, xa, fmaf(-ga, xb, acc[K][q]));  // on the stage's outputs
+        v[lo] = fma2(s, b, mul2(c, a));
+        v[hi] = fma2(ns, a, mul2(c, b));
     }
-    if constexpr (K > 0) walk_down<L, P, K - 1>(v, w, cs, acc);
+    if constexpr (K > 0) walk_down<L, P, K - 1>(v, cs, acc);
 }
 
 template <int L>
@@ -150,11 +160,20 @@ __device__ __forceinline__ void passes_up(float* X, const Params& p, int u, int 
     using G = Geo<L>;
     float2 cs[3][4];
     load_angles<L, P>(p.tw, u, cs);
-    for (int r = r0; r < p.n1; r += G::kRuns) {
-        float v[8];
+    for (int r = r0; r < p.n1; r += 2 * G::kRuns) {
+        const bool two = r + G::kRuns < p.n1;
+        float* second = X + (two ? r + G::kRuns : r) * G::kPitch;
+        float v[8], w[8];
         load8<L, P>(X + r * G::kPitch, u, v);
-        rotate<L, P>(v, cs);
+        load8<L, P>(second, u, w);
+        u64 vw[8];
+#pragma unroll
+        for (int e = 0; e < 8; ++e) vw[e] = pack2(v[e], w[e]);
+        rotate<L, P>(vw, cs);
+#pragma unroll
+        for (int e = 0; e < 8; ++e) unpack2(vw[e], v[e], w[e]);
         store8<L, P>(X + r * G::kPitch, u, v);
+        if (two) store8<L, P>(second, u, w);
     }
     __syncthreads();
     if constexpr (P + 1 < G::kPasses) passes_up<L, P + 1>(X, p, u, r0);
@@ -169,7 +188,12 @@ __device__ __forceinline__ void passes_down(float* X, float* W, const Params& p,
         float v[8], w[8];
         load8<L, P>(X + r * G::kPitch, u, v);
         load8<L, P>(W + r * G::kPitch, u, w);
-        walk_down<L, P, Pass<L, P>::kNs - 1>(v, w, cs, acc[P]);
+        u64 vw[8];
+#pragma unroll
+        for (int e = 0; e < 8; ++e) vw[e] = pack2(v[e], w[e]);
+        walk_down<L, P, Pass<L, P>::kNs - 1>(vw, cs, acc[P]);
+#pragma unroll
+        for (int e = 0; e < 8; ++e) unpack2(vw[e], v[e], w[e]);
         if constexpr (P > 0) {
             store8<L, P>(X + r * G::kPitch, u, v);
             store8<L, P>(W + r * G::kPitch, u, w);
@@ -225,7 +249,8 @@ __device__ __forceinline__ void load_token(const void* base, int type, int64_t r
     }
 }
 
-template <int L>
+// TILES x TILES entries of dL/dQ1 per thread
+template <int L, int TILES>
 __global__ void __launch_bounds__(kThreads, 2) k_composite_backward(const Params p) {
     using Ge = Geo<L>;
     extern __shared__ __align__(16) float sm[];
@@ -241,18 +266,20 @@ __global__ void __launch_bounds__(kThreads, 2) k_composite_backward(const Params
     const int u = t % Ge::kU, r0 = t / Ge::kU;
     // dL/dQ1: thread (ti, tk) of a dim x dim grid has entries (ti + a dim, tk + b dim); a slice of the grid takes every
     // slices-th chunk of positions
-    const int dim = n1 <= 8 ? 8 : 16, slices = kThreads / (dim * dim), tiles = (n1 + dim - 1) / dim;
+    const int dim = n1 <= 8 ? 8 : 16, slices = kThreads / (dim * dim);
     const int slice = t / (dim * dim), tk = t % dim, ti = (t / dim) % dim;
-    float acc[4][3][4], dq[4][4];
+    float acc[4][3][4];
+    u64 dq[TILES][TILES];  // sums over even and over odd positions
+#pragma unroll
+    for (int a = 0; a < TILES; ++a)
+#pragma unroll
+        for (int b = 0; b < TILES; ++b) dq[a][b] = 0ull;
 #pragma unroll
     for (int a = 0; a < 4; ++a)
 #pragma unroll
-        for (int b = 0; b < 4; ++b) {
-            dq[a][b] = 0.f;
-            if (b < 3)
+        for (int b = 0; b < 3; ++b)
 #pragma unroll
-                for (int c = 0; c < 4; ++c) acc[a][b][c] = 0.f;
-        }
+            for (int c = 0; c < 4; ++c) acc[a][b][c] = 0.f;
 
     for (int64_t row = blockIdx.x; row < p.rows; row += gridDim.x) {
         __syncthreads();  // the buffers' readers of the token before are done
@@ -263,49 +290,52 @@ __global__ void __launch_bounds__(kThreads, 2) k_composite_backward(const Params
         // G' = Q1^T G
         for (int item = t; item < (n1p / 8) * (Ge::kN2 / 4); item += kThreads) {
             const int j = place(4 * (item % (Ge::kN2 / 4))), k0 = 8 * (item / (Ge::kN2 / 4));
-            float s[8][4];
+            u64 s[4][4];  // output runs k0 + 2a, k0 + 2a + 1 at position b
 #pragma unroll
-            for (int a = 0; a < 8; ++a)
+            for (int a = 0; a < 4; ++a)
 #pragma unroll
-                for (int b = 0; b < 4; ++b) s[a][b] = 0.f;
-#pragma unroll 2
+                for (int b = 0; b < 4; ++b) s[a][b] = 0ull;
+#pragma unroll 4
             for (int i = 0; i < n1; ++i) {
                 const float4 gv = *reinterpret_cast<const float4*>(G + i * Ge::kPitch + j);
-                const float4 qa = *reinterpret_cast<const float4*>(q1s + i * n1p + k0), qb = *reinterpret_cast<const float4*>(q1s + i * n1p + k0 + 4);
-                const float qs[8] = {qa.x, qa.y, qa.z, qa.w, qb.x, qb.y, qb.z, qb.w};
+                const ulonglong2 qa = *reinterpret_cast<const ulonglong2*>(q1s + i * n1p + k0), qb = *reinterpret_cast<const ulonglong2*>(q1s + i * n1p + k0 + 4);
+                const u64 qs[4] = {qa.x, qa.y, qb.x, qb.y};
+                const u64 gs[4] = {pack2(gv.x, gv.x), pack2(gv.y, gv.y), pack2(gv.z, gv.z), pack2(gv.w, gv.w)};
 #pragma unroll
-                for (int a = 0; a < 8; ++a) {
-                    s[a][0] = fmaf(qs[a], gv.x, s[a][0]), s[a][1] = fmaf(qs[a], gv.y, s[a][1]);
-                    s[a][2] = fmaf(qs[a], gv.z, s[a][2]), s[a][3] = fmaf(qs[a], gv.w, s[a][3]);
-                }
+                for (int a = 0; a < 4; ++a)
+#pragma unroll
+                    for (int b = 0; b < 4; ++b) s[a][b] = fma2(qs[a], gs[b], s[a][b]);
             }
 #pragma unroll
-            for (int a = 0; a < 8; ++a)
-                if (k0 + a < n1) *reinterpret_cast<float4*>(W + (k0 + a) * Ge::kPitch + j) = make_float4(s[a][0], s[a][1], s[a][2], s[a][3]);
+            for (int a = 0; a < 4; ++a) {
+                float lo[4], hi[4];
+#pragma unroll
+                for (int b = 0; b < 4; ++b) unpack2(s[a][b], lo[b], hi[b]);
+                if (k0 + 2 * a < n1) *reinterpret_cast<float4*>(W + (k0 + 2 * a) * Ge::kPitch + j) = make_float4(lo[0], lo[1], lo[2], lo[3]);
+                if (k0 + 2 * a + 1 < n1) *reinterpret_cast<float4*>(W + (k0 + 2 * a + 1) * Ge::kPitch + j) = make_float4(hi[0], hi[1], hi[2], hi[3]);
+            }
         }
         // dL/dQ1 += G X'^T
         {
-            const float *gr[4], *xr[4];
+            const float *gr[TILES], *xr[TILES];
 #pragma unroll
-            for (int a = 0; a < 4; ++a) {  // entries past n1 take the last run and are never written
+            for (int a = 0; a < TILES; ++a) {  // entries past n1 take the last run and are never written
                 gr[a] = G + min(ti + a * dim, n1 - 1) * Ge::kPitch;
                 xr[a] = X + min(tk + a * dim, n1 - 1) * Ge::kPitch;
             }
+#pragma unroll 2
             for (int c = slice; c < Ge::kN2 / 4; c += slices) {
-                float4 xv[4];
+                const int at = place(4 * c);
+                ulonglong2 xv[TILES];
 #pragma unroll
-                for (int b = 0; b < 4; ++b)
-                    if (b < tiles) xv[b] = *reinterpret_cast<const float4*>(xr[b] + place(4 * c));
+                for (int b = 0; b < TILES; ++b)
+                    xv[b] = *reinterpret_cast<const ulonglong2*>(xr[b] + at);
 #pragma unroll
-                for (int a = 0; a < 4; ++a) {
-                    if (a >= tiles) break;
-                    const float4 gv = *reinterpret_cast<const float4*>(gr[a] + place(4 * c));
+                for (int a = 0; a < TILES; ++a) {
+                    const ulonglong2 gv = *reinterpret_cast<const ulonglong2*>(gr[a] + at);
 #pragma unroll
-                    for (int b = 0; b < 4; ++b) {
-                        if (b >= tiles) break;
-                        float s = dq[a][b];
-                        s = fmaf(gv.x, xv[b].x, s), s = fmaf(gv.y, xv[b].y, s), s = fmaf(gv.z, xv[b].z, s), s = fmaf(gv.w, xv[b].w, s);
-                        dq[a][b] = s;
+                    for (int b = 0; b < TILES; ++b) {
+                        dq[a][b] = fma2(gv.y, xv[b].y, fma2(gv.x, xv[b].x, dq[a][b]));
                     }
                 }
             }
@@ -325,19 +355,28 @@ __global__ void __launch_bounds__(kThreads, 2) k_composite_backward(const Params
     }
     for (int e = t; e < Ge::kAngles; e += kThreads) out[e] = sm[e];
     __syncthreads();
+    float total[TILES][TILES];
+#pragma unroll
+    for (int a = 0; a < TILES; ++a)
+#pragma unroll
+        for (int b = 0; b < TILES; ++b) {
+            float even, odd;
+            unpack2(dq[a][b], even, odd);
+            total[a][b] = even + odd;
+        }
     if (slices > 1) {  // n1 <= 8: one entry per thread
-        sm[t] = dq[0][0];
+        sm[t] = total[0][0];
         __syncthreads();
         if (slice == 0) {
-            for (int s = 1; s < slices; ++s) dq[0][0] += sm[t + s * dim * dim];
+            for (int s = 1; s < slices; ++s) total[0][0] += sm[t + s * dim * dim];
         }
     }
     if (slice == 0) {
 #pragma unroll
-        for (int a = 0; a < 4; ++a)
+        for (int a = 0; a < TILES; ++a)
 #pragma unroll
-            for (int b = 0; b < 4; ++b)
-                if (ti + a * dim < n1 && tk + b * dim < n1) out[Ge::kAngles + (ti + a * dim) * n1 + tk + b * dim] = dq[a][b];
+            for (int b = 0; b < TILES; ++b)
+                if (ti + a * dim < n1 && tk + b * dim < n1) out[Ge::kAngles + (ti + a * dim) * n1 + tk + b * dim] = total[a][b];
     }
 }
 
@@ -361,7 +400,7 @@ __global__ void __launch_bounds__(1024) k_reduce_composite(const float* __restri
     }
 }
 
-template <int L>
+template <int L, int TILES>
 static cudaError_t launch(const bfq_plan* plan, Params p, float* dtheta, float* dq1, cudaStream_t st) {
     using G = Geo<L>;
     const int n1p = (p.n1 + 7) & ~7;
@@ -369,7 +408,7 @@ static cudaError_t launch(const bfq_plan* plan, Params p, float* dtheta, float* 
     if (floats < size_t(G::kAngles)) floats = G::kAngles;  // the sums at the end
     if (floats < size_t(kThreads)) floats = kThreads;
     const size_t smem = floats * sizeof(float);
-    auto kern = k_composite_backward<L>;
+    auto kern = k_composite_backward<L, TILES>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
     if (e != cudaSuccess) return e;
     int occ = 0;
@@ -385,6 +424,14 @@ static cudaError_t launch(const bfq_plan* plan, Params p, float* dtheta, float* 
     if (e != cudaSuccess) return e;
     k_reduce_composite<<<(count + 31) / 32, 1024, 0, st>>>(p.partial, int(grid), count, G::kAngles, dtheta, dq1);
     return cudaGetLastError();
+}
+
+template <int L>
+static cudaError_t launch(const bfq_plan* plan, const Params& p, float* dtheta, float* dq1, cudaStream_t st) {
+    if (p.n1 <= 16) return launch<L, 1>(plan, p, dtheta, dq1, st);
+    if (p.n1 <= 32) return launch<L, 2>(plan, p, dtheta, dq1, st);
+    if (p.n1 <= 48) return launch<L, 3>(plan, p, dtheta, dq1, st);
+    return launch<L, 4>(plan, p, dtheta, dq1, st);
 }
 
 }  // namespace cbw
