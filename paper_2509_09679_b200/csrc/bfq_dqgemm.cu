@@ -27,9 +27,10 @@
 // What bounds it: per K block a CTA's tensor core works 512 cycles on nt = 256 (one term pair) and reads 64 KB of
 // operands from shared memory, while 32 KB are written there: with one CTA per 128 x 128 tile, which this replaces, both
 // figures per product were twice as large and the conversion of an element served half as many products.
-// Measured on a B200, before -> now (bf16 rows x 2-bit codes, 1000 x 28672 x 8192: 0.98 -> 0.389 ms = 1.21 PFLOP/s; 8-bit x
-// 2-bit codes, same size: 0.267 ms; 4-bit x 4-bit codes, 2048 x 4096 x 4096: 0.181 -> 0.059 ms; fp32 x 4-bit codes stored
-// [K][rows]: 0.445 -> 0.173 ms; both stored [K][rows]: 0.400 -> 0.235 ms).
+// Measured on a B200, before -> now (bf16 rows x 2-bit codes, 1000 x 28672 x 8192: 0.98 -> 0.334 ms = 1.40 PFLOP/s; bf16 x bf16,
+// 4096 x 8192 x 8192: 0.386 ms = 1.42 PFLOP/s; 8-bit x 2-bit codes, 1000 x 28672 x 8192: 0.270 ms; 4-bit x 4-bit codes,
+// 2048 x 4096 x 4096: 0.181 -> 0.057 ms; fp32 x 4-bit codes stored [K][rows]: 0.445 -> 0.175 ms; both stored [K][rows]: 0.400 ->
+// 0.227 ms).
 #include "../../include/bfq.h"
 
 #include <cuda_bf16.h>
@@ -109,12 +110,6 @@ __device__ __forceinline__ void tmem_alloc_pair(uint32_t smem_dst) {
 }
 __device__ __forceinline__ void tmem_dealloc_pair(uint32_t taddr) {
     asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, 512;" ::"r"(taddr) : "memory");
-}
-__device__ __forceinline__ void tma_load_2d(uint32_t dst, const void* tmap, int c0, int c1, uint32_t bar) {
-    asm volatile(
-        "cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];"
-        ::"r"(dst), "l"(reinterpret_cast<uint64_t>(tmap)), "r"(c0), "r"(c1), "r"(bar)
-        : "memory");
 }
 // Shared-memory descriptor of a 128-byte-swizzled tile.  K-major operand: rows of 128 bytes, 8-row groups 1024 bytes
 // apart (stride field), the leading field unused; one K step of 16 elements is 32 bytes further along the row.
@@ -572,16 +567,25 @@ __device__ __forceinline__ void produce(const Operand& op, int k_len, int g, int
     cp_async_wait<0>();  // no copy of this CTA may be in flight when it leaves
 }
 
-// bf16 operands: one thread has their tiles brought in by TMA (elements outside the operand arrive as zeros)
-__device__ __forceinline__ void load_tiles(const Operand& op, const CUtensorMap* map, const Span& span, int tile, int kb, uint32_t dst, uint32_t bar) {
-    const int row0 = span.row0(tile);
+// bf16 operands come by TMA (elements outside the operand arrive as zeros), issued like the products: a converged warp, one
+// thread's predicate on the instructions, the next stage's barrier tested ahead.  (One thread's loop behind a branch took 800
+// cycles per block and was what the whole kernel waited for.)
+__device__ __forceinline__ void expect_if(uint32_t lead, uint32_t bar, uint32_t bytes) {
+    asm volatile("{\n\t.reg .pred q;\n\tsetp.ne.b32 q, %2, 0;\n\t@q mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n\t}" ::"r"(bar), "r"(bytes), "r"(lead)
+                 : "memory");
+}
+__device__ __forceinline__ void tma_if(uint32_t lead, uint32_t dst, const CUtensorMap* tmap, int c0, int c1, uint32_t bar) {
+    asm volatile(
+        "{\n\t.reg .pred q;\n\tsetp.ne.b32 q, %5, 0;\n\t"
+        "@q cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];\n\t}"
+        ::"r"(dst), "l"(reinterpret_cast<uint64_t>(tmap)), "r"(c0), "r"(c1), "r"(bar), "r"(lead)
+        : "memory");
+}
+__device__ __forceinline__ void load_tiles(uint32_t lead, const Operand& op, const CUtensorMap* map, int lim, int row0, int kb, uint32_t dst, uint32_t bar) {
     if (op.transposed) {
-        const int boxes = (span.lim + 63) / 64;
-        mbar_expect_tx(bar, boxes * 8192u);
-        for (int h = 0; h < boxes; ++h) tma_load_2d(dst + 8192u * h, map, row0 + 64 * h, kb * kKB, bar);
+        for (int h = 0; h < lim; h += 64) tma_if(lead, dst + 128u * h, map, row0 + h, kb * kKB, bar);
     } else {
-        mbar_expect_tx(bar, static_cast<uint32_t>(span.lim) * 128u);
-        tma_load_2d(dst, map, kb * kKB, row0, bar);
+        tma_if(lead, dst, map, kb * kKB, row0, bar);
     }
 }
 
@@ -798,26 +802,41 @@ k_dequant_gemm(const __grid_constant__ Params p, const __grid_constant__ CUtenso
         } else if (!u_tma) {
             convert(t < kProd, t & (kProd - 1), kProd);
         }
-    } else if (tid == kLoader) {
+    } else if (warp == kLoader / 32) {
         const bool u_tma = p.u.kind == BFQ_OP_BF16, v_tma = p.v.kind == BFQ_OP_BF16;
-        const Span su = span_of(true), sv = span_of(false);
-        int s = 0, issued = 0;
-        uint32_t round = 0;
-        bool ok = u_tma || v_tma;
-        for (int tile = walk.first; ok && tile < walk.tiles; tile += walk.step) {
-            for (int kb = walk.kb0; kb < walk.kb1; ++kb) {
-                if (round > 0 && !wait_bounded(ring.bar_empty + 8 * s, (round - 1) & 1, p.status)) {
-                    // no copy of this CTA may be in flight when it leaves
-                    for (int i = issued > ring.stages ? issued - ring.stages : 0; i < issued; ++i)
-                        wait_bounded(ring.bar_full + 8 * (i % ring.stages), (i / ring.stages) & 1, p.status);
-                    ok = false;
-                    break;
+        if (u_tma || v_tma) {
+            const uint32_t lead = elect_one() ? 1u : 0u;
+            auto bytes_of = [&](const Operand& op, int lim) { return 128u * static_cast<uint32_t>(op.transposed ? (lim + 63) / 64 * 64 : lim); };
+            const uint32_t u_bytes = bytes_of(p.u, kRows), v_bytes = bytes_of(p.v, hv);
+            int s = 0, issued = 0;
+            uint32_t parity = 1u;  // of the phase before the first: over, as far as a fresh barrier tells
+            bool ok = true, ready = false;
+            for (int tile = walk.first; ok && tile < walk.tiles; tile += walk.step) {
+                const int u0 = (tile / p.tiles_v) * (2 * kRows) + half * kRows, v0 = (tile % p.tiles_v) * p.nt + half * hv;
+                for (int kb = walk.kb0; kb < walk.kb1; ++kb) {
+                    if (!ready && !wait_warp(ring.bar_empty + 8 * s, parity, p.status)) {
+                        // no copy of this CTA may be in flight when it leaves
+                        for (int i = issued > ring.stages ? issued - ring.stages : 0; i < issued; ++i)
+                            wait_bounded(ring.bar_full + 8 * (i % ring.stages), (i / ring.stages) & 1, p.status);
+                        ok = false;
+                        break;
+                    }
+                    const int s_next = s + 1 == ring.stages ? 0 : s + 1;
+                    const uint32_t parity_next = s_next == 0 ? parity ^ 1u : parity;
+                    const bool next = mbar_test(ring.bar_empty + 8 * s_next, parity_next);
+                    const uint32_t dst = sbase + s * ring.stage_bytes, bar = ring.bar_full + 8 * s;
+                    if (u_tma) {
+                        expect_if(lead, bar, u_bytes);
+                        load_tiles(lead, p.u, &map_u, kRows, u0, kb, dst, bar);
+                    }
+                    if (v_tma) {
+                        expect_if(lead, bar, v_bytes);
+                        load_tiles(lead, p.v, &map_v, hv, v0, kb, dst + p.u.terms * kTileBytes, bar);
+                    }
+                    ++issued;
+                    s = s_next, parity = parity_next;
+                    ready = __all_sync(0xFFFFFFFFu, next);
                 }
-                const uint32_t dst = sbase + s * ring.stage_bytes, bar = ring.bar_full + 8 * s;
-                if (u_tma) load_tiles(p.u, &map_u, su, tile, kb, dst, bar);
-                if (v_tma) load_tiles(p.v, &map_v, sv, tile, kb, dst + p.u.terms * kTileBytes, bar);
-                ++issued;
-                if (++s == ring.stages) s = 0, ++round;
             }
         }
     } else if (warp == kIssuer / 32 && half == 0) {
@@ -892,7 +911,7 @@ k_dequant_gemm(const __grid_constant__ Params p, const __grid_constant__ CUtenso
 
 // ---- a few rows of A against coded rows of B -----------------------------------------------------------------------
 // A decoded token or a few: the product is a pass over B's codes, and a 256-row tile of the pair kernel keeps 32 to 128
-// CTAs in a chain of K blocks (one token, 4096 x 4096 at 2 bits: 25 us).  Here a CTA of eight warps takes 16 rows of B, each
+// CTAs in a chain of K blocks (one token, 4096 x 4096 at 2 bits: 17 - 25 us).  Here a CTA of eight warps takes 16 rows of B, each
 // warp every eighth part of K, and the partial sums are added in the order of the warps.  mma.sync m16n8k16 with the codes as
 // the 16-row operand straight from registers: a lane's 16 bytes of a row are its k values, in whatever order they come, as
 // long as the lanes that hold A's rows take the same ones.  Bound by the latency of one pass over the codes, not by the
@@ -1058,7 +1077,9 @@ static Shape choose_shape(int64_t m, int64_t n, int kblocks, int term_pairs, int
         const int64_t tiles_v = (m + nt - 1) / nt, tiles = tiles_u * tiles_v;
         const int step = nt / 2 > 64 + nt / 4 ? nt / 2 : 64 + nt / 4;
         for (int split = 1; split <= 4; split *= 2) {
-            if (split > 1 && (tiles * split > pairs || kblocks < 4 * split)) break;
+            // eight-CTA clusters: only about half of the chip's pairs run at once as such (4096 x 4096, 64 rows: 28 us with four
+            // pairs to a tile against 21 with two)
+            if (split > 1 && (tiles * split > (split == 4 ? pairs / 2 : pairs) || kblocks < 4 * split)) break;
             const int64_t rounds = split > 1 ? 1 : (tiles + pairs - 1) / pairs;
             const double cost = double(rounds) * ((kblocks + split - 1) / split) * (kKB / 16) * step * term_pairs +
                                 double(rounds) * 500 + 2000 + 16 * nt + (split > 1 ? 2000 : 0);
