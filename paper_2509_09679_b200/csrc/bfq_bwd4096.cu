@@ -341,16 +341,27 @@ k_bwd4096(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ CUte
     }
     // constants into tensor memory (each group fills half of the columns), accumulators to zero
     {
-        const float4* src = reinterpret_cast<const float4*>(img + t * kConstCols);
-        for (int c = is_fwd ? 16 : 0; c < kConstCols; c += 32) {
-            uint32_t v[16];
+        // the image is [column quad][role][4], so that a warp's load is 512 contiguous bytes, and four blocks of a thread's
+        // loads are in flight together
+        const float4* src = reinterpret_cast<const float4*>(img) + t;
+        constexpr int kBlocks = kConstCols / 32;  // of 16 columns, for each of the two groups
+        static_assert(kConstCols % 32 == 0 && kBlocks % 4 == 0, "three rounds of four blocks");
+        for (int j0 = 0; j0 < kBlocks; j0 += 4) {
+            float4 fill[4][4];
 #pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                const float4 f = __ldg(src + (c >> 2) + i);
-                v[4 * i + 0] = __float_as_uint(f.x), v[4 * i + 1] = __float_as_uint(f.y);
-                v[4 * i + 2] = __float_as_uint(f.z), v[4 * i + 3] = __float_as_uint(f.w);
+            for (int j = 0; j < 4; ++j)
+#pragma unroll
+                for (int i = 0; i < 4; ++i) fill[j][i] = __ldg(src + (8 * (j0 + j) + (is_fwd ? 4 : 0) + i) * kThreads);
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                uint32_t v[16];
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    v[4 * i + 0] = __float_as_uint(fill[j][i].x), v[4 * i + 1] = __float_as_uint(fill[j][i].y);
+                    v[4 * i + 2] = __float_as_uint(fill[j][i].z), v[4 * i + 3] = __float_as_uint(fill[j][i].w);
+                }
+                tmem_st16(cx.tlane + 32 * (j0 + j) + (is_fwd ? 16 : 0), v);
             }
-            tmem_st16(cx.tlane + c, v);
         }
         if (!is_fwd) {
             uint32_t z[16];
@@ -672,9 +683,10 @@ __device__ __forceinline__ void build_image_bwd(int k, const float4* __restrict_
     const int u = ((m >> (kk + 1)) << kk) | (m & ((1 << kk) - 1));
     const float4 p = prep[k];
     const float sg = (sa == sb) ? 1.f : -1.f;
-    float* strip = img + r * kConstCols;
-    strip[32 * s + 4 * u + h] = sg * p.x;
-    strip[32 * s + 4 * u + h + 2] = sg * p.y;
+    float* strip = img + 4 * r;  // [column quad][role][4]
+    auto at = [](int col) { return (col >> 2) * 512 + (col & 3); };
+    strip[at(32 * s + 4 * u + h)] = sg * p.x;
+    strip[at(32 * s + 4 * u + h + 2)] = sg * p.y;
     dsign[k] = static_cast<int8_t>(-(sa * sb));
 }
 
@@ -892,7 +904,7 @@ k_inv4096(const __grid_constant__ CUtensorMap ymap, const float* __restrict__ im
         }
     }
     // constants: the scaled-form image ([column quad][role][4], coalesced, all loads in flight) unless the table build
-    // flagged it out of range; then the three-shear image ([role][384])
+    // flagged it out of range; then the three-shear image (the same layout)
     const bool shear = __ldg(form) != 0;
     if (!shear) {
         constexpr int kFillBlocks = (kInvCols / 16 + G - 1) / G;
@@ -921,12 +933,12 @@ k_inv4096(const __grid_constant__ CUtensorMap ymap, const float* __restrict__ im
         }
         tmem_wait_st();
     } else {
-        const float4* src = reinterpret_cast<const float4*>(img + (q * 32 + lane) * kConstCols);
+        const float4* src = reinterpret_cast<const float4*>(img) + t;
         for (int c = 16 * g; c < kConstCols; c += 16 * G) {
             uint32_t v[16];
 #pragma unroll
             for (int i = 0; i < 4; ++i) {
-                const float4 f = __ldg(src + (c >> 2) + i);
+                const float4 f = __ldg(src + ((c >> 2) + i) * kThreads);
                 v[4 * i + 0] = __float_as_uint(f.x), v[4 * i + 1] = __float_as_uint(f.y);
                 v[4 * i + 2] = __float_as_uint(f.z), v[4 * i + 3] = __float_as_uint(f.w);
             }
