@@ -281,6 +281,17 @@ int bfq_cayley_backward(bfq_plan* plan, const float* params, int n1, const float
 int bfq_dequant_gemm(bfq_plan* plan, int64_t m, int64_t n, int64_t k, float alpha, const void* a, int a_kind,
                      int a_transposed, int64_t lda, const uint16_t* a_scales, const void* b, int b_kind, int b_transposed,
                      int64_t ldb, const uint16_t* b_scales, float* c, int64_t ldc, void* stream);
+/*
+ * The same product, the same results, with a device workspace (256-byte aligned, the caller's, in use until the call's work on
+ * `stream` is done) in which fp32 operands are split once instead of in every tile.  bfq_dequant_gemm_workspace gives the
+ * bytes it takes for these sizes and operands; 0 (also on bad arguments): it would not help and is not used.  Too small a
+ * workspace is BFQ_ERR_WORKSPACE; a null one is bfq_dequant_gemm.
+ */
+size_t bfq_dequant_gemm_workspace(const bfq_plan* plan, int64_t m, int64_t n, int64_t k, int a_kind, int a_transposed, int b_kind,
+                                  int b_transposed);
+int bfq_dequant_gemm_split(bfq_plan* plan, int64_t m, int64_t n, int64_t k, float alpha, const void* a, int a_kind, int a_transposed,
+                           int64_t lda, const uint16_t* a_scales, const void* b, int b_kind, int b_transposed, int64_t ldb,
+                           const uint16_t* b_scales, float* c, int64_t ldc, void* workspace, size_t workspace_bytes, void* stream);
 
 /*
  * bfq_forward_quant for rows that live in HOST memory (paper Sec. 3.4 quantizer on y = Q x, as bfq_forward_quant): the

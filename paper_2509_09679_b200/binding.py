@@ -46,6 +46,9 @@ SIGNATURES = {
     "bfq_measure_fma_rates": (_i, [_p]),
     "bfq_measure_mma_rates": (_i, [_p]),
     "bfq_dequant_gemm": (_i, [_p, _i64, _i64, _i64, ctypes.c_float, _p, _i, _i, _i64, _p, _p, _i, _i, _i64, _p, _p, _i64, _p]),
+    "bfq_dequant_gemm_workspace": (ctypes.c_size_t, [_p, _i64, _i64, _i64, _i, _i, _i, _i]),
+    "bfq_dequant_gemm_split": (_i, [_p, _i64, _i64, _i64, ctypes.c_float, _p, _i, _i, _i64, _p, _p, _i, _i, _i64, _p, _p, _i64, _p,
+                                    ctypes.c_size_t, _p]),
     "bfq_stage_form": (_i, [_p]),
     "bfq_test_stuck_wait": (_i, [_p, _i]),
     "bfq_backward_noalloc": (_i, [_i, _p, _p, _i, _p, _i, _i64, _i64, _p, _i, _p, _p]),
@@ -391,11 +394,16 @@ class Plan:
             c = torch.empty((a.rows, b.rows), dtype=torch.float32, device=self.device)
         else:
             c = _exact(out, torch.float32, (a.rows, b.rows), self.device, "out")
-        _check(self._c.bfq_dequant_gemm(self._h, a.rows, b.rows, a.k, float(alpha), a.data.data_ptr(), a.kind,
-                                      int(a.transposed), a.ld, a.scales.data_ptr() if a.scales is not None else None,
-                                      b.data.data_ptr(), b.kind, int(b.transposed), b.ld,
-                                      b.scales.data_ptr() if b.scales is not None else None, c.data_ptr(), b.rows,
-                                      _stream(c)), "bfq_dequant_gemm")
+        args = (self._h, a.rows, b.rows, a.k, float(alpha), a.data.data_ptr(), a.kind, int(a.transposed), a.ld,
+                a.scales.data_ptr() if a.scales is not None else None, b.data.data_ptr(), b.kind, int(b.transposed), b.ld,
+                b.scales.data_ptr() if b.scales is not None else None, c.data_ptr(), b.rows)
+        if a.kind == BFQ_F32 or b.kind == BFQ_F32:  # room to split fp32 operands in, where that helps
+            size = self._c.bfq_dequant_gemm_workspace(self._h, a.rows, b.rows, a.k, a.kind, int(a.transposed), b.kind, int(b.transposed))
+            if size:
+                room = torch.empty(size + 256, dtype=torch.uint8, device=self.device)
+                _check(self._c.bfq_dequant_gemm_split(*args, (room.data_ptr() + 255) // 256 * 256, size, _stream(c)), "bfq_dequant_gemm_split")
+                return c
+        _check(self._c.bfq_dequant_gemm(*args, _stream(c)), "bfq_dequant_gemm")
         return c
 
     def device_status(self) -> int:

@@ -21,7 +21,9 @@
 //   * codes contracted across stored rows: the scale varies along k.  If the other operand is fp32 the scale multiplies
 //     THAT operand before it is split (one fp32 rounding, 2^-24, in front of a split that keeps 2^-17) and the codes stay
 //     one exact term; otherwise code x scale (at most 15 significant bits) is stored as hi + lo, exactly;
-//   * fp32 numbers: hi + lo = 16 significant bits (relative error 2^-17 per element); bf16 numbers: one term, exact.
+//   * fp32 numbers: hi + lo = 16 significant bits (relative error 2^-17 per element); bf16 numbers: one term, exact.  Given a
+//     workspace, a pass of its own splits an fp32 operand into two bf16 matrices, which then come by TMA; without one every
+//     tile splits the rows it needs again, which takes three times as long as the products.
 // The MMA thread issues one product per pair of terms (1, 2 or 4 per K step), accumulating all of them in fp32.
 //
 // What bounds it: per K block a CTA's tensor core works 512 cycles on nt = 256 (one term pair) and reads 64 KB of
@@ -29,8 +31,8 @@
 // figures per product were twice as large and the conversion of an element served half as many products.
 // Measured on a B200, before -> now (bf16 rows x 2-bit codes, 1000 x 28672 x 8192: 0.98 -> 0.334 ms = 1.40 PFLOP/s; bf16 x bf16,
 // 4096 x 8192 x 8192: 0.386 ms = 1.42 PFLOP/s; 8-bit x 2-bit codes, 1000 x 28672 x 8192: 0.270 ms; 4-bit x 4-bit codes,
-// 2048 x 4096 x 4096: 0.181 -> 0.057 ms; fp32 x 4-bit codes stored [K][rows]: 0.445 -> 0.175 ms; both stored [K][rows]: 0.400 ->
-// 0.227 ms).
+// 2048 x 4096 x 4096: 0.181 -> 0.057 ms; fp32 x 4-bit codes stored [K][rows]: 0.445 -> 0.175 ms, 0.115 ms split
+// beforehand; both stored [K][rows]: 0.400 -> 0.227 ms, 0.126 ms split beforehand).
 #include "../../include/bfq.h"
 
 #include <cuda_bf16.h>
@@ -73,6 +75,7 @@ struct Operand {
     int rows;                // M or N
     int terms;               // bf16 terms an element is stored in
     int scaled;              // codes times their scales go into shared memory (two terms)
+    const void* lo;          // kind bf16, two terms: the second matrix of an fp32 operand that was split beforehand
 };
 
 __host__ __device__ __forceinline__ bool is_codes(int kind) { return kind >= BFQ_OP_CODES2; }
@@ -692,7 +695,8 @@ __device__ __forceinline__ void issue_products(const Params& p, const Ring& ring
 }
 
 __global__ void __launch_bounds__(kThreads, 1)
-k_dequant_gemm(const __grid_constant__ Params p, const __grid_constant__ CUtensorMap map_u, const __grid_constant__ CUtensorMap map_v) {
+k_dequant_gemm(const __grid_constant__ Params p, const __grid_constant__ CUtensorMap map_u, const __grid_constant__ CUtensorMap map_v,
+               const __grid_constant__ CUtensorMap map_u_lo, const __grid_constant__ CUtensorMap map_v_lo) {
     extern __shared__ uint8_t smem_raw[];
     const uint32_t sbase = (smem_u32(smem_raw) + 1023u) & ~1023u;  // the same offset in both CTAs of a pair
     const int tid = threadIdx.x, warp = __shfl_sync(0xFFFFFFFFu, tid >> 5, 0);
@@ -806,7 +810,7 @@ k_dequant_gemm(const __grid_constant__ Params p, const __grid_constant__ CUtenso
         const bool u_tma = p.u.kind == BFQ_OP_BF16, v_tma = p.v.kind == BFQ_OP_BF16;
         if (u_tma || v_tma) {
             const uint32_t lead = elect_one() ? 1u : 0u;
-            auto bytes_of = [&](const Operand& op, int lim) { return 128u * static_cast<uint32_t>(op.transposed ? (lim + 63) / 64 * 64 : lim); };
+            auto bytes_of = [&](const Operand& op, int lim) { return 128u * static_cast<uint32_t>(op.terms * (op.transposed ? (lim + 63) / 64 * 64 : lim)); };
             const uint32_t u_bytes = bytes_of(p.u, kRows), v_bytes = bytes_of(p.v, hv);
             int s = 0, issued = 0;
             uint32_t parity = 1u;  // of the phase before the first: over, as far as a fresh barrier tells
@@ -828,10 +832,12 @@ k_dequant_gemm(const __grid_constant__ Params p, const __grid_constant__ CUtenso
                     if (u_tma) {
                         expect_if(lead, bar, u_bytes);
                         load_tiles(lead, p.u, &map_u, kRows, u0, kb, dst, bar);
+                        if (p.u.terms == 2) load_tiles(lead, p.u, &map_u_lo, kRows, u0, kb, dst + kTileBytes, bar);
                     }
                     if (v_tma) {
                         expect_if(lead, bar, v_bytes);
                         load_tiles(lead, p.v, &map_v, hv, v0, kb, dst + p.u.terms * kTileBytes, bar);
+                        if (p.v.terms == 2) load_tiles(lead, p.v, &map_v_lo, hv, v0, kb, dst + (p.u.terms + 1) * kTileBytes, bar);
                     }
                     ++issued;
                     s = s_next, parity = parity_next;
@@ -1037,10 +1043,41 @@ __global__ void __launch_bounds__(32 * kFewWarps) k_few_rows(const Operand u, co
 
 // ---- host side ---------------------------------------------------------------------------------------------------
 static Operand make_operand(const void* data, const uint16_t* scales, int64_t ld, int kind, int transposed, int rows, int other_kind) {
-    Operand op{data, scales, ld, kind, transposed, rows, 1, 0};
+    Operand op{data, scales, ld, kind, transposed, rows, 1, 0, nullptr};
     op.scaled = is_codes(kind) && transposed && other_kind != BFQ_OP_F32;  // else the scales go into the fp32 operand
     op.terms = kind == BFQ_OP_F32 || op.scaled ? 2 : 1;
     return op;
+}
+
+// An fp32 operand as two bf16 matrices hi + lo of its stored rows (pitch: the row's length rounded up to 8), times the other
+// operand's scales where those vary along k: `row_scales` per stored row (stored [K][rows]), `col_scales` per element of a row.
+// The same arithmetic as in the tiles, so the products come out the same.  Bound by memory: 8 bytes per element.
+__global__ void __launch_bounds__(256) k_split_rows(const float* __restrict__ x, int64_t ld, int64_t rows, int width, const uint16_t* __restrict__ row_scales,
+                                                    const uint16_t* __restrict__ col_scales, uint16_t* __restrict__ hi, uint16_t* __restrict__ lo) {
+    grid_dep_launch();
+    grid_dep_wait();
+    const int chunks = (width + 7) / 8;
+    const int64_t total = rows * chunks, step = int64_t(gridDim.x) * blockDim.x;
+    auto half_at = [](const uint16_t* q) { return __half2float(__ushort_as_half(__ldg(q))); };
+    for (int64_t e = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; e < total; e += step) {
+        const int64_t r = e / chunks;
+        const int c = 8 * static_cast<int>(e - r * chunks);
+        const float4* src = reinterpret_cast<const float4*>(x + r * ld + c);
+        const float4 none = make_float4(0.f, 0.f, 0.f, 0.f), a = __ldg(src), b = c + 4 < width ? __ldg(src + 1) : none;
+        float v[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
+        const float rs = row_scales != nullptr ? half_at(row_scales + r) : 1.f;
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            v[i] *= rs;
+            if (c + i >= width) v[i] = 0.f;
+            else if (col_scales != nullptr) v[i] *= half_at(col_scales + c + i);
+        }
+        uint32_t h[4], l[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) split2(v[2 * i], v[2 * i + 1], h[i], l[i]);
+        *reinterpret_cast<uint4*>(hi + 8 * e) = make_uint4(h[0], h[1], h[2], h[3]);
+        *reinterpret_cast<uint4*>(lo + 8 * e) = make_uint4(l[0], l[1], l[2], l[3]);
+    }
 }
 
 static int code_shift(int kind) {
@@ -1109,7 +1146,35 @@ static cudaError_t launch_few(const Operand& u, const Operand& v, float* c, int6
     return launch_few<UK, BFQ_OP_CODES8>(u, v, c, ldc, k, alpha, st);
 }
 
-static cudaError_t launch(const Params& p, const CUtensorMap& map_u, const CUtensorMap& map_v, int sms, size_t smem, cudaStream_t st) {
+// Bytes of one of an fp32 operand's two matrices, and whether splitting it beforehand pays: a pair that works on 16 K blocks
+// or more loses 20 us and up in its own tiles (2900 cycles a block against 1000), the pass takes 3 us and 8 bytes per element.
+static size_t plane_bytes(const Operand& op, int64_t k) {
+    const int64_t stored = op.transposed ? k : op.rows, width = op.transposed ? op.rows : k;
+    return (size_t(stored) * ((width + 7) / 8 * 8) * 2 + 255) / 256 * 256;
+}
+static bool split_pays(const Operand& u, const Operand& v, int64_t k, int sms) {
+    if (u.kind != BFQ_OP_F32 && v.kind != BFQ_OP_F32) return false;
+    const Shape shape = choose_shape(v.rows, u.rows, int(k / kKB), u.terms * v.terms, 32, sms);
+    const int64_t pairs = sms / 2 > 0 ? sms / 2 : 1, rounds = shape.split > 1 ? 1 : (shape.tiles + pairs - 1) / pairs;
+    return rounds * (k / kKB) / shape.split >= 16;
+}
+// replaces an fp32 operand by its two matrices at *workspace and moves the pointer on
+static cudaError_t split_operand(Operand& op, const Operand& other, int64_t k, uint8_t** workspace, cudaStream_t st) {
+    if (op.kind != BFQ_OP_F32) return cudaSuccess;
+    const int64_t stored = op.transposed ? k : op.rows, width = op.transposed ? op.rows : k, pitch = (width + 7) / 8 * 8;
+    const size_t bytes = plane_bytes(op, k);
+    uint16_t *hi = reinterpret_cast<uint16_t*>(*workspace), *lo = reinterpret_cast<uint16_t*>(*workspace + bytes);
+    *workspace += 2 * bytes;
+    const uint16_t* fold = is_codes(other.kind) && other.transposed && !other.scaled ? other.scales : nullptr;
+    const int64_t blocks = (stored * (pitch / 8) + 255) / 256;
+    const cudaError_t e = launch_overlapped(k_split_rows, dim3(unsigned(blocks < (1 << 20) ? blocks : (1 << 20))), dim3(256), 0, st, static_cast<const float*>(op.data),
+                                            op.ld, stored, int(width), op.transposed ? fold : nullptr, op.transposed ? nullptr : fold, hi, lo);
+    op.data = hi, op.lo = lo, op.kind = BFQ_OP_BF16, op.ld = pitch;
+    return e;
+}
+
+static cudaError_t launch(const Params& p, const CUtensorMap& map_u, const CUtensorMap& map_v, const CUtensorMap& map_u_lo, const CUtensorMap& map_v_lo, int sms,
+                          size_t smem, cudaStream_t st) {
     cudaLaunchConfig_t cfg = {};
     const int pairs = p.split > 1 ? p.tiles * p.split : (p.tiles < sms / 2 ? p.tiles : (sms / 2 > 0 ? sms / 2 : 1));
     cfg.gridDim = dim3(unsigned(2 * pairs)), cfg.blockDim = dim3(kThreads), cfg.dynamicSmemBytes = smem, cfg.stream = st;
@@ -1119,15 +1184,33 @@ static cudaError_t launch(const Params& p, const CUtensorMap& map_u, const CUten
     attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr, cfg.numAttrs = 2;
-    return cudaLaunchKernelEx(&cfg, k_dequant_gemm, p, map_u, map_v);
+    return cudaLaunchKernelEx(&cfg, k_dequant_gemm, p, map_u, map_v, map_u_lo, map_v_lo);
 }
 
 }  // namespace dqg
 }  // namespace bfq
 
+extern "C" size_t bfq_dequant_gemm_workspace(const bfq_plan* plan, int64_t m, int64_t n, int64_t k, int a_kind, int a_transposed, int b_kind,
+                                            int b_transposed) {
+    using namespace bfq::dqg;
+    if (plan == nullptr || m <= 0 || n <= 0 || k <= 0 || k % kKB != 0 || m >= (int64_t(1) << 31) || n >= (int64_t(1) << 31) || k >= (int64_t(1) << 31)) return 0;
+    const Operand u = make_operand(nullptr, nullptr, 0, b_kind, b_transposed, int(n), a_kind);
+    const Operand v = make_operand(nullptr, nullptr, 0, a_kind, a_transposed, int(m), b_kind);
+    if (!split_pays(u, v, k, plan->sm_count)) return 0;
+    return 2 * ((a_kind == BFQ_OP_F32 ? plane_bytes(v, k) : 0) + (b_kind == BFQ_OP_F32 ? plane_bytes(u, k) : 0));
+}
+
 extern "C" int bfq_dequant_gemm(bfq_plan* plan, int64_t m, int64_t n, int64_t k, float alpha, const void* a, int a_kind,
                                 int a_transposed, int64_t lda, const uint16_t* a_scales, const void* b, int b_kind,
                                 int b_transposed, int64_t ldb, const uint16_t* b_scales, float* c, int64_t ldc, void* stream) {
+    return bfq_dequant_gemm_split(plan, m, n, k, alpha, a, a_kind, a_transposed, lda, a_scales, b, b_kind, b_transposed, ldb, b_scales, c, ldc, nullptr, 0,
+                                  stream);
+}
+
+extern "C" int bfq_dequant_gemm_split(bfq_plan* plan, int64_t m, int64_t n, int64_t k, float alpha, const void* a, int a_kind,
+                                      int a_transposed, int64_t lda, const uint16_t* a_scales, const void* b, int b_kind,
+                                      int b_transposed, int64_t ldb, const uint16_t* b_scales, float* c, int64_t ldc, void* workspace,
+                                      size_t workspace_bytes, void* stream) {
     using namespace bfq::dqg;
     if (plan == nullptr) return BFQ_ERR_NULL;
     if (m < 0 || n < 0 || k < 0 || k % kKB != 0 || m >= (int64_t(1) << 31) || n >= (int64_t(1) << 31) || k >= (int64_t(1) << 31))
@@ -1149,6 +1232,9 @@ extern "C" int bfq_dequant_gemm(bfq_plan* plan, int64_t m, int64_t n, int64_t k,
     if (rc == BFQ_OK) rc = check(b, b_kind, b_transposed, ldb, b_scales, n);
     if (rc != BFQ_OK) return rc;
     if (ldc < n || (reinterpret_cast<uintptr_t>(c) & 3u) != 0) return BFQ_ERR_STRIDE;
+    const size_t wanted = workspace != nullptr ? bfq_dequant_gemm_workspace(plan, m, n, k, a_kind, a_transposed, b_kind, b_transposed) : 0;
+    if (workspace != nullptr && (reinterpret_cast<uintptr_t>(workspace) & 255u) != 0) return BFQ_ERR_ALIGN;
+    if (workspace != nullptr && workspace_bytes < wanted) return BFQ_ERR_WORKSPACE;
     int prev = -1;
     if (cudaGetDevice(&prev) != cudaSuccess) return BFQ_ERR_CUDA;
     if (prev != plan->device && cudaSetDevice(plan->device) != cudaSuccess) return BFQ_ERR_CUDA;
@@ -1172,6 +1258,11 @@ extern "C" int bfq_dequant_gemm(bfq_plan* plan, int64_t m, int64_t n, int64_t k,
         if (e == cudaSuccess) {
             Params p{};
             p.u = u, p.v = v;
+            if (wanted > 0) {
+                uint8_t* at = static_cast<uint8_t*>(workspace);
+                e = split_operand(p.u, v, k, &at, static_cast<cudaStream_t>(stream));
+                if (e == cudaSuccess) e = split_operand(p.v, u, k, &at, static_cast<cudaStream_t>(stream));
+            }
             p.c = c, p.ldc = ldc, p.k = int(k), p.alpha = alpha, p.status = plan->status_word;
             // Two code operands along K are an integer product: exact in 32 bits up to K = 2^17 - 1 (codes left in place are at
             // most 128 in size), at twice the rate of the bf16 products.
@@ -1182,10 +1273,16 @@ extern "C" int bfq_dequant_gemm(bfq_plan* plan, int64_t m, int64_t n, int64_t k,
                                              is_codes(a_kind) && a_transposed ? (a_kind == BFQ_OP_CODES8 ? 32 : 256 / a_kind) : 32,
                                              plan->sm_count);
             p.nt = shape.nt, p.tiles_v = shape.tiles_v, p.tiles = shape.tiles, p.split = shape.split;
-            CUtensorMap map_u{}, map_v{};
-            bool ok = b_kind != BFQ_OP_BF16 || encode_operand(&map_u, p.u, k, kRows);
-            ok = ok && (a_kind != BFQ_OP_BF16 || encode_operand(&map_v, p.v, k, p.nt / 2));
-            e = ok ? launch(p, map_u, map_v, plan->sm_count, smem, static_cast<cudaStream_t>(stream)) : cudaErrorInvalidValue;
+            CUtensorMap map_u{}, map_v{}, map_u_lo{}, map_v_lo{};
+            auto encode = [&](CUtensorMap* map, CUtensorMap* map_lo, Operand op, int box_rows) {
+                if (op.kind != BFQ_OP_BF16) return true;
+                if (!encode_operand(map, op, k, box_rows)) return false;
+                op.data = op.lo;
+                return op.terms == 1 || encode_operand(map_lo, op, k, box_rows);
+            };
+            const bool ok = encode(&map_u, &map_u_lo, p.u, kRows) && encode(&map_v, &map_v_lo, p.v, p.nt / 2);
+            if (e == cudaSuccess)
+                e = ok ? launch(p, map_u, map_v, map_u_lo, map_v_lo, plan->sm_count, smem, static_cast<cudaStream_t>(stream)) : cudaErrorInvalidValue;
         }
     }
     if (prev != plan->device) cudaSetDevice(prev);

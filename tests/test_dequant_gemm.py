@@ -99,6 +99,28 @@ def test_tile_edges(ka, kb, ta, tb, m, n, k):
     check(p, A, a64, ea, B, b64, eb + (2.0 ** -24 if tb and ka == "f32" else 0.0))
 
 
+@pytest.mark.parametrize("ka,kb,ta,tb", [("f32", "codes4", False, True), ("f32", "codes2", True, True), ("f32", "f32", False, False),
+                                         ("bf16", "f32", True, True), ("f32", "bf16", True, False)])
+def test_operands_split_beforehand(ka, kb, ta, tb):
+    """The workspace form (a row length that is no multiple of 8, scales along and across the stored rows) gives the bits of
+    the form without; a workspace that is too small is refused."""
+    from paper_2509_09679_b200.binding import lib, _stream
+    m, n, k = ((212 if ka == "f32" else 208) if ta else 201), (192 if tb and kb.startswith("codes") else 136), 4160
+    p = Plan(256, DEV)
+    A, a64, ea = operand(ka, m, k, ta, 940)
+    B, b64, eb = operand(kb, n, k, tb, 941)
+    check(p, A, a64, ea + 2.0 ** -24, B, b64, eb)
+    size = lib().bfq_dequant_gemm_workspace(p._h, m, n, k, A.kind, int(ta), B.kind, int(tb))
+    assert size > 0
+    ptr = lambda t: t.data_ptr() if t is not None else None
+    out = [torch.full((m, n), float("nan"), device=DEV) for _ in range(2)]
+    room = torch.empty(size, dtype=torch.uint8, device=DEV)
+    for c, ws, bytes_, status in ((out[0], None, 0, 0), (out[1], room.data_ptr(), size, 0), (out[1], room.data_ptr(), size - 1, -7)):
+        assert status == lib().bfq_dequant_gemm_split(p._h, m, n, k, 1.0, ptr(A.data), A.kind, int(ta), A.ld, ptr(A.scales), ptr(B.data), B.kind, int(tb),
+                                                      B.ld, ptr(B.scales), ptr(c), n, ws, bytes_, _stream(c))
+    assert torch.equal(out[0], out[1]) and p.device_status() == 0
+
+
 @pytest.mark.parametrize("ka", ["bf16", "codes2", "codes4", "codes8"])
 @pytest.mark.parametrize("kb", ["codes2", "codes4", "codes8"])
 @pytest.mark.parametrize("m,n,k", [(1, 16, 64), (8, 15, 192), (3, 4100, 1088), (9, 100, 4096), (64, 33, 64)])
