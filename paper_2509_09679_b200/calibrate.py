@@ -5,7 +5,7 @@ learning-rate schedule from the identity initialisation on the reconstruction lo
 
 Everything runs in the bfq kernels: forward, forward + quantize, weight folding, backward for the angle gradient, and
 the dense products (bfq_dequant_gemm: tensor cores, the packed codes dequantized on the fly, fp32 operands split into two
-bf16 terms); only element-wise glue (the error, its square, the scaling of the gradient) is torch.  The
+bf16 terms); only element-wise glue (the error, its square) is torch.  The
 quantizers are not differentiable; as usual their gradient is passed straight through (the paper does not
 say so explicitly: this is the reading taken here).  With act_bits = None activations stay unquantized
 (the paper's W2A16 setting).  Synthetic (W, x) only: the paper's models and calibration set are not here.
@@ -66,11 +66,11 @@ class LayerCalibrator:
             YqT = GemmOperand(a_codes, a_scales, self.act_bits, transposed=True)
         err = p.dequant_gemm(Yq, Wq) - ref                                        # [tokens][out]
         loss = (err * err).mean()
-        e = err * (2.0 / err.numel())
-        # dL/d(B x) = e Wq and dL/d(W B^T) = e^T yq, straight through the two quantizers: the contraction runs across
-        # the stored rows of the codes (their scales vary along it) and of e
-        g_y = p.dequant_gemm(GemmOperand(e), GemmOperand(w_codes, w_scales, wb, transposed=True))
-        g_w = p.dequant_gemm(GemmOperand(e, transposed=True), YqT)
+        unit = 2.0 / err.numel()                                                  # dL/d(product) = unit * err
+        # with e = unit * err: dL/d(B x) = e Wq and dL/d(W B^T) = e^T yq, straight through the two quantizers: the contraction
+        # runs across the stored rows of the codes (their scales vary along it) and of err
+        g_y = p.dequant_gemm(GemmOperand(err), GemmOperand(w_codes, w_scales, wb, transposed=True), unit)
+        g_w = p.dequant_gemm(GemmOperand(err, transposed=True), YqT, unit)
         # row i of W B^T is B w_i: both gradients flow through the same transform, one on the activation rows
         # and one on the weight rows
         _, dth_x = p.backward(x, g_y.to(x.dtype), want_dx=False)
