@@ -252,10 +252,12 @@ const char* bfq_status_string(int status);
 int bfq_composite_backward(bfq_plan* plan, const float* q1, int n1, const void* x, bfq_dtype xt, const void* g, bfq_dtype gt,
                            int64_t rows, int64_t ld, void* dx, float* dtheta, float* dq1, void* stream);
 /*
- * Gradient of the Cayley parameters (bfq_cayley) from dq1 = dL/dQ1: dparams [n1 (n1 - 1) / 2], fp32; float64 inside.
+ * Gradient of the Cayley parameters from dq1 = dL/dQ1: dparams [n1 (n1 - 1) / 2], fp32; float64 inside.  q1: the transform
+ * of these parameters as bfq_cayley gives it (a start for the inverse; one that is not is noticed and only costs time).
  * Device pointers.  Returns BFQ_OK, BFQ_ERR_NULL, BFQ_ERR_UNSUPPORTED_N, BFQ_ERR_ALIGN or BFQ_ERR_CUDA.
  */
-int bfq_cayley_backward(bfq_plan* plan, const float* params, int n1, const float* dq1, float* dparams, void* stream);
+int bfq_cayley_backward(bfq_plan* plan, const float* params, int n1, const float* q1, const float* dq1, float* dparams,
+                        void* stream);
 
 /*
  * Dense product with on-the-fly dequantization, for the reconstruction loss of the calibration step (paper Sec. 3.4:

@@ -36,7 +36,7 @@ SIGNATURES = {
     "bfq_backward": (_i, [_p, _p, _i, _p, _i, _i64, _i64, _p, _i, _p, _p]),
     "bfq_fold_weights": (_i, [_p, _p, _i, _i64, _i64, _i, _p, _p, _p, _i, _p]),
     "bfq_composite_backward": (_i, [_p, _p, _i, _p, _i, _p, _i, _i64, _i64, _p, _p, _p, _p]),
-    "bfq_cayley_backward": (_i, [_p, _p, _i, _p, _p, _p]),
+    "bfq_cayley_backward": (_i, [_p, _p, _i, _p, _p, _p, _p]),
     "bfq_device_status": (_i, [_p]),
     "bfq_last_cuda_error": (_i, [_p]),
     "bfq_status_string": (ctypes.c_char_p, [_i]),
@@ -288,12 +288,13 @@ class Plan:
                                             dtheta.data_ptr(), dq1.data_ptr(), _stream(x)), "bfq_composite_backward")
         return dx, dtheta, dq1
 
-    def cayley_backward(self, params: torch.Tensor, n1: int, dq1: torch.Tensor) -> torch.Tensor:
-        """dL/dparams of cayley() from dL/dQ1 (fp32, on the plan's device)."""
+    def cayley_backward(self, params: torch.Tensor, q1: torch.Tensor, dq1: torch.Tensor) -> torch.Tensor:
+        """dL/dparams of q1 = cayley(params) from dL/dQ1 (fp32, on the plan's device)."""
+        n1 = self._q1(q1)
         _exact(params, torch.float32, (n1 * (n1 - 1) // 2,), self.device, "params")
         _exact(dq1, torch.float32, (n1, n1), self.device, "dq1")
         dparams = torch.empty_like(params)
-        _check(self._c.bfq_cayley_backward(self._h, params.data_ptr(), int(n1), dq1.data_ptr(), dparams.data_ptr(), _stream(params)),
+        _check(self._c.bfq_cayley_backward(self._h, params.data_ptr(), n1, q1.data_ptr(), dq1.data_ptr(), dparams.data_ptr(), _stream(params)),
                "bfq_cayley_backward")
         return dparams
 

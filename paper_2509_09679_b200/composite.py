@@ -57,6 +57,6 @@ def composite_backward(plan: Plan, q1: torch.Tensor, params: torch.Tensor | None
         dx = dx_runs.reshape(tokens, n1 * n2)
     if params is None:
         return dx, dtheta2, dQ1, None
-    if params.dtype == torch.float32 and params.device == plan.device and params.dim() == 1 and params.is_contiguous() and 2 <= n1 <= 64:
-        return dx, dtheta2, dQ1, plan.cayley_backward(params, n1, dQ1.contiguous())
+    if params.dtype == torch.float32 and q1.dtype == torch.float32 and params.device == plan.device and params.dim() == 1 and params.is_contiguous() and 2 <= n1 <= 64:
+        return dx, dtheta2, dQ1, plan.cayley_backward(params, q1.contiguous(), dQ1.contiguous())
     return dx, dtheta2, dQ1, cayley_pullback(params, n1, dQ1)

@@ -757,14 +757,14 @@ int bfq_composite_forward_quant(bfq_plan* plan, const float* q1, int n1, const v
     return composite_impl(plan, q1, n1, x, xt, rows, ldx, nullptr, BFQ_F32, 0, bits, codes, scales_f16, stream);
 }
 
-int bfq_cayley_backward(bfq_plan* plan, const float* params, int n1, const float* dq1, float* dparams, void* stream) {
-    if (plan == nullptr || params == nullptr || dq1 == nullptr || dparams == nullptr) return BFQ_ERR_NULL;
+int bfq_cayley_backward(bfq_plan* plan, const float* params, int n1, const float* q1, const float* dq1, float* dparams, void* stream) {
+    if (plan == nullptr || params == nullptr || q1 == nullptr || dq1 == nullptr || dparams == nullptr) return BFQ_ERR_NULL;
     if (n1 < 2 || n1 > BFQ_MAX_N1) return BFQ_ERR_UNSUPPORTED_N;
-    for (const void* p : {static_cast<const void*>(params), static_cast<const void*>(dq1), static_cast<const void*>(dparams)})
+    for (const void* p : {static_cast<const void*>(params), static_cast<const void*>(q1), static_cast<const void*>(dq1), static_cast<const void*>(dparams)})
         if ((reinterpret_cast<uintptr_t>(p) & 3u) != 0) return BFQ_ERR_ALIGN;
     DeviceGuard guard(plan->device);
     if (guard.err != cudaSuccess) return cuda_fail(plan, guard.err);
-    cudaError_t e = cayley_backward_launch(params, n1, dq1, dparams, static_cast<cudaStream_t>(stream));
+    cudaError_t e = cayley_backward_launch(params, n1, q1, dq1, dparams, static_cast<cudaStream_t>(stream));
     return e == cudaSuccess ? BFQ_OK : cuda_fail(plan, e);
 }
 

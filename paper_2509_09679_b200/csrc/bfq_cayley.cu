@@ -10,7 +10,7 @@
 // turns: every thread reads the old one (the row exchange is only a matter of where a row is read) and writes the new one,
 // one block barrier per column; every warp finds the pivot by itself; a row is 2 n1 + 1 doubles, so that the lanes that read
 // down a column fall into different banks, and a thread's loads are all issued before its stores.  Four barriers and a serial
-// pivot search per column took 96 us for n1 = 40.
+// pivot search per column took 96 us for n1 = 40; now 35 us, and the gradient 24 us (76 with a solve of its own).
 #include <cuda_runtime.h>
 
 #include "bfq_fast.h"
@@ -55,15 +55,15 @@ __device__ __forceinline__ const double* solve(const float* __restrict__ params,
         double f[kMaxRows];
 #pragma unroll
         for (int a = 0; a < kMaxRows; ++a) {
-            const int r = ty + a * (kThreads / 32);
-            src[a] = cur + (r == at ? col : min(r, n1 - 1)) * w;
-            f[a] = src[a][col];
+            const int r = ty + a * (kThreads / 32);  // the same for the whole warp
+            src[a] = cur + (r == at ? col : r) * w;
+            f[a] = r < n1 ? src[a][col] : 0.0;
         }
         for (int j = col + 1 + tx; j < cols; j += 32) {  // columns up to `col` are columns of the identity: not read again
             const double pj = pivot[j] * inv;
             double v[kMaxRows];
 #pragma unroll
-            for (int a = 0; a < kMaxRows; ++a) v[a] = src[a][j];
+            for (int a = 0; a < kMaxRows; ++a) v[a] = ty + a * (kThreads / 32) < n1 ? src[a][j] : 0.0;
 #pragma unroll
             for (int a = 0; a < kMaxRows; ++a) {
                 const int r = ty + a * (kThreads / 32);
@@ -83,44 +83,83 @@ __global__ void __launch_bounds__(kThreads) k_cayley(const float* __restrict__ p
     for (int e = threadIdx.x; e < n1 * n1; e += kThreads) q1[e] = static_cast<float>(q[(e / n1) * pitch(n1) + e % n1]);
 }
 
-// out = scale a b (n1 x n1, all threads): eight entries of a thread at a time, so that their chains overlap
-__device__ __forceinline__ void product(double* out, const double* a, const double* b, int n1, double scale) {
-    const int nn = n1 * n1;
-    for (int e0 = threadIdx.x; e0 < nn; e0 += 8 * kThreads) {
-        double s[8];
-        int ai[8], bj[8];
+// out = scale a b + add I (n1 x n1, row stride n1, all threads): four rows x two columns per thread, so that eight chains
+// overlap and a value that is read serves several of them
+__device__ __forceinline__ void product(double* out, const double* a, const double* b, int n1, double scale, double add) {
+    const int cols = (n1 + 1) / 2, items = ((n1 + 3) / 4) * cols;
+    for (int it = threadIdx.x; it < items; it += kThreads) {
+        const int i0 = 4 * (it / cols), j0 = 2 * (it % cols), j1 = min(j0 + 1, n1 - 1);
+        double s[4][2];
+        const double* row[4];
 #pragma unroll
-        for (int c = 0; c < 8; ++c) {
-            const int e = min(e0 + c * kThreads, nn - 1);
-            s[c] = 0.0, ai[c] = (e / n1) * n1, bj[c] = e % n1;
-        }
+        for (int r = 0; r < 4; ++r) s[r][0] = s[r][1] = 0.0, row[r] = a + min(i0 + r, n1 - 1) * n1;
+#pragma unroll 4
         for (int k = 0; k < n1; ++k) {
+            const double x = b[k * n1 + j0], y = b[k * n1 + j1];
 #pragma unroll
-            for (int c = 0; c < 8; ++c) s[c] = fma(a[ai[c] + k], b[k * n1 + bj[c]], s[c]);
+            for (int r = 0; r < 4; ++r) s[r][0] = fma(row[r][k], x, s[r][0]), s[r][1] = fma(row[r][k], y, s[r][1]);
         }
 #pragma unroll
-        for (int c = 0; c < 8; ++c)
-            if (e0 + c * kThreads < nn) out[e0 + c * kThreads] = scale * s[c];
+        for (int r = 0; r < 4; ++r)
+#pragma unroll
+            for (int c = 0; c < 2; ++c)
+                if (i0 + r < n1 && j0 + c < n1) out[(i0 + r) * n1 + j0 + c] = scale * s[r][c] + (i0 + r == j0 + c ? add : 0.0);
     }
 }
 
-__global__ void __launch_bounds__(kThreads) k_cayley_backward(const float* __restrict__ params, int n1, const float* __restrict__ dq1,
-                                                              float* __restrict__ dparams) {
-    extern __shared__ double aug[];  // [2][n1][pitch], then two n1 x n1 matrices
-    const double* q = solve(params, n1, aug);
-    const int t = threadIdx.x, w = pitch(n1), nn = n1 * n1;
-    double* m2 = aug + 2 * n1 * w;   // 2 M = I + Q1, transposed: m2[j][i] = 2 M[i][j]
-    double* g = m2 + nn;         // dL/dQ1, then (2 M)^T (dL/dQ1)
+// M = (I + A)^{-1} in float64 from the Q1 the caller has: (I + Q1) / 2 is M to fp32 rounding, and each Newton step
+// M (2 I - (I + A) M) squares the error (residual of the first guess up to |A| 2^-24; two steps).  If Q1 is not the transform of
+// these parameters (the first residual is not small) the solve is done after all.  Six small products instead of a solve.
+__global__ void __launch_bounds__(kThreads) k_cayley_backward(const float* __restrict__ params, int n1, const float* __restrict__ q1,
+                                                              const float* __restrict__ dq1, float* __restrict__ dparams) {
+    extern __shared__ double aug[];  // [2][n1][pitch] of the solve = four n1 x n1 matrices and more, then two
+    const int t = threadIdx.x, nn = n1 * n1;
+    double *ia = aug, *m = ia + nn, *r = m + nn, *next = r + nn;  // I + A, M, 2 I - (I + A) M, the next M
+    double* g = aug + 2 * n1 * pitch(n1);
+    double* left = g + nn;
+    __shared__ int far;
+    if (t == 0) far = 0;
     for (int e = t; e < nn; e += kThreads) {
         const int i = e / n1, j = e % n1;
-        m2[j * n1 + i] = q[i * w + j] + (i == j ? 1.0 : 0.0);
+        double a = 0.0;
+        if (i < j) a = static_cast<double>(params[i * n1 - i * (i + 1) / 2 + (j - i - 1)]);
+        if (i > j) a = -static_cast<double>(params[j * n1 - j * (j + 1) / 2 + (i - j - 1)]);
+        const double id = i == j ? 1.0 : 0.0;
+        ia[e] = id + a;
+        m[e] = 0.5 * (id + static_cast<double>(q1[e]));
         g[e] = static_cast<double>(dq1[e]);
     }
     __syncthreads();
-    double* left = aug;  // the solve is done with its buffers
-    product(left, m2, g, n1, 1.0);  // (2 M)^T dQ1
+    for (int step = 0; step < 2; ++step) {
+        product(r, ia, m, n1, -1.0, 2.0);
+        __syncthreads();
+        if (step == 0) {
+            for (int e = t; e < nn; e += kThreads)
+                if (!(fabs(r[e] - (e / n1 == e % n1 ? 1.0 : 0.0)) < 1e-4)) far = 1;
+            __syncthreads();
+            if (far != 0) break;
+        }
+        product(next, m, r, n1, 1.0, 0.0);
+        __syncthreads();
+        double* tmp = m;
+        m = next, next = tmp;
+    }
+    if (far != 0) {  // uniform
+        const double* q = solve(params, n1, aug);
+        // 2 M = I + Q1, kept in `left` while the solve's buffers turn back into matrices
+        for (int e = t; e < nn; e += kThreads) left[e] = 0.5 * (q[(e / n1) * pitch(n1) + e % n1] + (e / n1 == e % n1 ? 1.0 : 0.0));
+        __syncthreads();
+        m = aug;
+        for (int e = t; e < nn; e += kThreads) m[e] = left[e];
+        __syncthreads();
+        r = aug + nn;
+    }
+    // dL/dA = -2 M^T dQ1 M^T; M^T in r
+    for (int e = t; e < nn; e += kThreads) r[(e % n1) * n1 + e / n1] = m[e];
     __syncthreads();
-    product(g, left, m2, n1, -0.5);  // dL/dA
+    product(left, r, g, n1, 1.0, 0.0);
+    __syncthreads();
+    product(g, left, r, n1, -2.0, 0.0);
     __syncthreads();
     for (int e = t; e < nn; e += kThreads) {
         const int i = e / n1, j = e % n1;
@@ -143,11 +182,11 @@ cudaError_t cayley_launch(const float* params, int n1, float* q1, cudaStream_t s
     return cudaGetLastError();
 }
 
-cudaError_t cayley_backward_launch(const float* params, int n1, const float* dq1, float* dparams, cudaStream_t st) {
+cudaError_t cayley_backward_launch(const float* params, int n1, const float* q1, const float* dq1, float* dparams, cudaStream_t st) {
     const size_t smem = sizeof(double) * (2 * n1 * cay::pitch(n1) + 2 * n1 * n1);
     cudaError_t e = allow_smem(cay::k_cayley_backward, smem);
     if (e != cudaSuccess) return e;
-    cay::k_cayley_backward<<<1, cay::kThreads, smem, st>>>(params, n1, dq1, dparams);
+    cay::k_cayley_backward<<<1, cay::kThreads, smem, st>>>(params, n1, q1, dq1, dparams);
     return cudaGetLastError();
 }
 

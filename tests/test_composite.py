@@ -415,7 +415,10 @@ def test_cayley_and_its_gradient(n1, scale):
     assert np.abs(to_f64(p.cayley(params.to(DEV), n1)) - oracle.cayley(to_f64(params), n1)).max() <= 2e-7
     dq = synth.rows(n1, n1, "normal", 12)
     ref = cayley_pullback(params.double(), n1, dq.double()).numpy()
-    assert np.abs(to_f64(p.cayley_backward(params.to(DEV), n1, dq.to(DEV))) - ref).max() <= 2e-7 * np.abs(ref).max()
+    q1 = p.cayley(params.to(DEV), n1)
+    # also from a Q1 that is not the parameters' own
+    for start in (q1, torch.eye(n1, device=DEV), torch.full_like(q1, float("nan"))):
+        assert np.abs(to_f64(p.cayley_backward(params.to(DEV), start, dq.to(DEV))) - ref).max() <= 2e-7 * np.abs(ref).max()
 
 
 @pytest.mark.parametrize("rows", [1, 3, 5, 593, 2500])
