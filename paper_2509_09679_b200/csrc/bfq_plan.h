@@ -21,7 +21,7 @@ struct bfq_plan {
     // these are built by bfq_set_angles
     float* img4096 = nullptr;    // [128][416] tensor-memory image of the rotation constants (n = 128 .. 4096)
     void* prep4096 = nullptr;    // staging for the image build: per-angle constants and negation flags (n = 128 .. 4096)
-    float* img_b4096 = nullptr;  // [96][128][4] constants of the backward kernel (n = 128 .. 4096)
+    float* img_b4096 = nullptr;  // [128][384] (n < 4096: [96][128][4]) constants of the backward kernel (n = 128 .. 4096)
     float* img_i4096 = nullptr;  // [104][128][4] scaled-form constants of the inverse kernel (n = 128 .. 4096)
     int8_t* dsign4096 = nullptr; // [12][2048] sign applied to the accumulated d-theta (n = 128 .. 4096)
     uint32_t* gsign4096 = nullptr;  // [16 * 128] sign words applied to bf16 g rows (n = 128 .. 4096)
