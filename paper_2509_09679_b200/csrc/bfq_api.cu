@@ -69,7 +69,12 @@ static bool use_short_rows(const bfq_plan* plan, int64_t rows, int64_t min_elems
     return rows < (int64_t(1) << 31) - 64 && rows * plan->n >= min_elems && !env_flag("BFQ_GENERIC_ONLY") && fwdq_short_available(plan);
 }
 static int64_t short_inverse_from(int n) { return n == 128 ? int64_t(1) << 21 : 0; }
-static int64_t short_backward_from(int n) { return n <= 256 ? int64_t(1) << 18 : int64_t(1) << 20; }
+// (bf16 rows that bfq_backward_noalloc takes too stay on the kernel it runs, so that the two entry points' dx are the same
+// bits, up to 2^23 elements, where that would cost 60 us and more)
+static int64_t short_backward_from(int n, bool f32) {
+    if (!f32 && n <= BFQ_NOALLOC_MAX_N) return int64_t(1) << 23;
+    return n <= 256 ? int64_t(1) << 18 : int64_t(1) << 20;
+}
 
 // ---- generic kernel dispatch ------------------------------------------------------------------------
 template <int LOG_N, int R, int MODE>
@@ -677,7 +682,7 @@ int bfq_backward(bfq_plan* plan, const void* x, bfq_dtype xt, const void* g, bfq
         if (e == cudaSuccess) e = bwd8192_launch_halves(plan, x, g, rows, ld, dx, dtheta, st);
         return e == cudaSuccess ? BFQ_OK : cuda_fail(plan, e);
     }
-    if (xt == gt && (dx == nullptr || dxt == xt) && ld == plan->n && use_short_rows(plan, rows, short_backward_from(plan->n)) &&
+    if (xt == gt && (dx == nullptr || dxt == xt) && ld == plan->n && use_short_rows(plan, rows, short_backward_from(plan->n, xt == BFQ_F32)) &&
         bwd_short_available(plan)) {
         cudaError_t e = bwd_short_launch(plan, x, g, rows, dx, dtheta, xt == BFQ_F32, st);
         return e == cudaSuccess ? BFQ_OK : cuda_fail(plan, e);
@@ -734,6 +739,10 @@ static int composite_impl(bfq_plan* plan, const float* q1, int n1, const void* x
             e = comp5120_launch(plan, q1, x, rows, ldx, codes, scales, y, ldy, static_cast<cudaStream_t>(stream));
             return e == cudaSuccess ? BFQ_OK : cuda_fail(plan, e);
         }
+    }
+    if (!inverse && composite_forward_available(plan, n1) && !env_flag("BFQ_GENERIC_ONLY")) {
+        e = composite_forward_launch(plan, q1, n1, x, xt, rows, ldx, y, yt, ldy, bits, codes, scales, static_cast<cudaStream_t>(stream));
+        return e == cudaSuccess ? BFQ_OK : cuda_fail(plan, e);
     }
     e = composite_generic_launch(plan, q1, n1, x, xt, rows, ldx, y, yt, ldy, bits, codes, scales, inverse,
                                  static_cast<cudaStream_t>(stream));

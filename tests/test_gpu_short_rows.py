@@ -55,7 +55,7 @@ def test_forward_and_inverse(n, dtype, tail, kind, pad):
 @pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
 @pytest.mark.parametrize("tail,kind", [("one", "normal"), ("lacks one", "uniform")])
 def test_backward(n, dtype, tail, kind):
-    rows = batch(n, tail)
+    rows = batch(n, tail, 1 << 23 if dtype == torch.bfloat16 and n <= 1024 else 1 << 20)
     p, theta, x, xd = inputs(n, rows, dtype, kind)
     g = synth.rows(rows, n, "normal", 5, dtype=dtype)
     dx = Guarded((rows, n), dtype, DEV)
@@ -83,7 +83,7 @@ def test_a_few_rows(n, rows):
 @pytest.mark.parametrize("n", [128, 2048])
 def test_rows_do_not_touch_each_other(n):
     """A row of infinities and a row of NaN among ordinary ones: the others' results are the same bits."""
-    rows = batch(n, "whole", 1 << 21)
+    rows = batch(n, "whole", 1 << 23)
     p, _, x, xd = inputs(n, rows, torch.bfloat16)
     spoilt = xd.clone()
     spoilt[5], spoilt[rows - 2] = float("inf"), float("nan")
