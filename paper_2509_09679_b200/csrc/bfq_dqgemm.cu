@@ -1130,7 +1130,7 @@ static Shape choose_shape(int64_t m, int64_t n, int kblocks, int term_pairs, int
 // 1024 x 1024 at 2 bits 7.7 -> 2.5, 4096 x 4096 25 -> 7.0, 28672 x 8192 104 -> 44; 8 rows 8.1 -> 3.0, 26 -> 9.4, 105 -> 75).  More
 // rows are more passes, worth it while they are small together.
 static bool use_few_rows(const Operand& u, const Operand& v, int64_t k) {
-    if (!is_codes(u.kind) || u.transposed || v.kind == BFQ_OP_F32 || v.transposed) return false;
+    if (!is_codes(u.kind) || u.transposed || v.kind == BFQ_OP_F32 || v.transposed || k >= (1 << 30)) return false;
     const int64_t passes = (int64_t(v.rows) + 7) / 8;
     return passes == 1 || (passes <= 8 && passes * u.rows * k <= int64_t(1) << 25);
 }

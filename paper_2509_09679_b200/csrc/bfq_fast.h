@@ -92,7 +92,11 @@ cudaError_t inv4096_launch_f32(bfq_plan* plan, const void* y, int64_t rows, int6
 cudaError_t inv4096_launch(bfq_plan* plan, const void* y, int64_t rows, int64_t ldy, void* x, bool x_bf16, int64_t ldx,
                            cudaStream_t st);
 
-// composite transform Q1 (x) Q2 (n1 <= 64, n2 = the plan's n): Cayley solve and the kernels for every shape
+// composite transform Q1 (x) Q2 (n1 <= 64, n2 = the plan's n): whole tokens in shared memory (n2 = 128 .. 1024, forward), Cayley
+// solve and the kernels for every shape
+bool composite_forward_available(const bfq_plan* plan, int n1);
+cudaError_t composite_forward_launch(const bfq_plan* plan, const float* q1, int n1, const void* x, int xt, int64_t rows, int64_t ldx, void* y, int yt,
+                                     int64_t ldy, int bits, uint8_t* codes, uint16_t* scales, cudaStream_t st);
 cudaError_t cayley_launch(const float* params, int n1, float* q1, cudaStream_t st);
 cudaError_t cayley_backward_launch(const float* params, int n1, const float* q1, const float* dq1, float* dparams, cudaStream_t st);
 // dx (may be null, type of x), dtheta of Q2 and dQ1 for upstream rows g; ld: row stride of x, g and dx

@@ -58,6 +58,18 @@ def test_composite_forward_quant(n1, n2, rows, bits):
     check_quant(codes, scales, y_ref, bits, "composite quant")
 
 
+@pytest.mark.parametrize("n1,n2,rows", [(9, 512, 901), (2, 128, 700), (16, 1024, 3), (40, 128, 1300)])
+@pytest.mark.parametrize("dtype,bits", [(torch.float32, 4), (torch.bfloat16, 2)])
+def test_composite_forward_several_tokens_per_cta(n1, n2, rows, dtype, bits):
+    from parity import Guarded
+    p, q1, Q1_ref, th2, x = setup(n1, n2, rows, dtype)
+    y_ref = oracle.composite_forward(Q1_ref, th2, to_f64(x))
+    codes, scales = Guarded((rows, n1 * n2 * bits // 8), torch.uint8, DEV), Guarded((rows,), torch.float16, DEV)
+    p.composite_forward_quant(q1, x.to(DEV), bits, codes.view, scales.view)
+    check_quant(codes.view, scales.view, y_ref, bits, "codes")
+    assert codes.intact() and scales.intact()
+
+
 def test_composite_identity_factor_is_the_butterfly_on_every_run():
     n1, n2, rows = 6, 128, 10
     p, _, _, th2, x = setup(n1, n2, rows, torch.float32)
