@@ -387,6 +387,7 @@ k_fwdq4096(const __grid_constant__ CUtensorMap tmap, const float* __restrict__ i
         // each register
         constexpr int kPartLog = SUB < 4 ? SUB : 4, kParts = 1 << kPartLog, kPartShift = 4 - kPartLog;
         bool plain;         // every scale here is a normal, unsaturated fp16 number: nothing needs clipping
+        uint32_t plain_parts = 0u;  // SUB > 0: the same of each part
         uint16_t s16 = 0;
         float inv = 0.f;    // SUB == 0: the row's; else lane s < kParts holds part s's
         if constexpr (SUB == 0) {
@@ -480,12 +481,20 @@ k_fwdq4096(const __grid_constant__ CUtensorMap tmap, const float* __restrict__ i
                                               : (static_cast<int64_t>(row) << SUB) + 2 * part + (q >> 1);
             const bool writes = lane < kParts && (SUB < 5 ? q == 0 : (q & 1) == 0) && (short_row << stages_of_sub(SUB)) < elems;
             stg16_if(writes, scales + short_row, s16);
-            plain = __all_sync(0xFFFFFFFFu, (((s16 >> 10) & 31u) != 0u) && (s16 != 0x7BFFu));
+            plain_parts = __ballot_sync(0xFFFFFFFFu, (((s16 >> 10) & 31u) != 0u) && (s16 != 0x7BFFu));
+            plain = plain_parts == 0xFFFFFFFFu;
         }
         float invp[kParts];
 #pragma unroll
         for (int s = 0; s < kParts; ++s) invp[s] = SUB == 0 ? inv : __shfl_sync(0xFFFFFFFFu, inv, s);
         auto inv_of = [&](int m) { return invp[m >> kPartShift]; };
+        // The code of one value where some scale is not plain.  A part whose own scale is rounds as it does when all are, once
+        // (v * inv + the constant, then the constant off): a row's codes must not depend on the rows beside it.
+        auto code_of = [&](float v, int m) {
+            const bool once = SUB != 0 && ((plain_parts >> (m >> kPartShift)) & 1u) != 0u;
+            const float r = once ? __fmaf_rn(v, inv_of(m), 12582912.f) - 12582912.f : rintf(v * inv_of(m));
+            return static_cast<int>(fminf(fmaxf(r, static_cast<float>(-kQmax - 1)), static_cast<float>(kQmax)));
+        };
 
         if constexpr (OUT == kOutInt8) {
             // |v * inv| <= qmax (1 + 2^-10) < qmax + 1/2 for a normal, unsaturated fp16 scale: no clipping; v * inv +
@@ -507,8 +516,7 @@ k_fwdq4096(const __grid_constant__ CUtensorMap tmap, const float* __restrict__ i
                 for (int m = 0; m < 16; ++m) {
                     float a, b;
                     unpack2(P[m], a, b);
-                    const uint32_t lo = static_cast<uint32_t>(quant1(a, inv_of(m), -kQmax - 1, kQmax));
-                    const uint32_t hi = static_cast<uint32_t>(quant1(b, inv_of(m), -kQmax - 1, kQmax));
+                    const uint32_t lo = static_cast<uint32_t>(code_of(a, m)), hi = static_cast<uint32_t>(code_of(b, m));
                     if (there(m)) out16[128 * m] = static_cast<uint16_t>((lo & 0xFFu) | ((hi & 0xFFu) << 8));
                 }
             }
@@ -541,8 +549,7 @@ k_fwdq4096(const __grid_constant__ CUtensorMap tmap, const float* __restrict__ i
                 for (int m = 0; m < 16; ++m) {
                     float a, b;
                     unpack2(P[m], a, b);
-                    const uint32_t c = (static_cast<uint32_t>(quant1(a, inv_of(m), -2, 1)) & 3u) |
-                                       ((static_cast<uint32_t>(quant1(b, inv_of(m), -2, 1)) & 3u) << 2);
+                    const uint32_t c = (static_cast<uint32_t>(code_of(a, m)) & 3u) | ((static_cast<uint32_t>(code_of(b, m)) & 3u) << 2);
                     w[m >> 2] |= c << (8 * (m & 3));
                 }
             }
@@ -581,8 +588,7 @@ k_fwdq4096(const __grid_constant__ CUtensorMap tmap, const float* __restrict__ i
             for (int m = 0; m < 16; ++m) {
                 float a, b;
                 unpack2(P[m], a, b);
-                const int qa = static_cast<int>(fminf(fmaxf(rintf(a * inv_of(m)), -8.f), 7.f));
-                const int qb = static_cast<int>(fminf(fmaxf(rintf(b * inv_of(m)), -8.f), 7.f));
+                const int qa = code_of(a, m), qb = code_of(b, m);
                 const uint32_t byte = static_cast<uint32_t>((qa & 0xF) | ((qb & 0xF) << 4));
                 if (there(m)) out[128 * m] = static_cast<uint8_t>(byte);
                 if constexpr (kCount) red_shared_inc(hist_g + 4u * (byte ^ 0x88u));

@@ -92,3 +92,37 @@ def test_rows_do_not_touch_each_other(n):
     for a, b in ((p.forward(xd), p.forward(spoilt)), (p.inverse(xd), p.inverse(spoilt)), (p.backward(xd, xd)[0], p.backward(spoilt, spoilt)[0]),
                  *zip(p.forward_quant(xd, 4), p.forward_quant(spoilt, 4))):
         assert torch.equal(a[keep], b[keep])
+
+
+def near_ties(rows, n, bits, seed):
+    """fp32 rows whose elements lie a few units in the last place from (k + 1/2) s, s the row's scale: where rounding once and
+    rounding twice differ."""
+    g = np.random.default_rng(seed)
+    s = g.uniform(0.01, 1.0, (rows, 1)).astype(np.float16).astype(np.float32)
+    qmax = 2 ** (bits - 1) - 1
+    x = ((g.integers(-qmax, qmax, (rows, n)) + np.float32(0.5)) * s).astype(np.float32)
+    for _ in range(3):
+        x = np.where(g.random(x.shape) < 0.5, np.nextafter(x, np.float32(np.inf)), np.nextafter(x, np.float32(-np.inf)))
+    x[:, :1] = qmax * s
+    return torch.from_numpy(x)
+
+
+@pytest.mark.parametrize("n", [128, 512, 2048])
+@pytest.mark.parametrize("bits", [2, 4, 8])
+def test_codes_of_a_row_do_not_depend_on_the_rows_beside_it(n, bits):
+    """A row of zeros in every joint row, a saturated one in some, or a batch whose last joint row lacks a row: the other
+    rows' codes are the same bits."""
+    joint, rows = 4096 // n, (1 << 21) // n
+    p = Plan(n, DEV)
+    p.set_angles(synth.angles(n, "zero", 1).to(DEV))
+    x = near_ties(rows, n, bits, 7).to(DEV)
+    codes, scales = p.forward_quant(x, bits)
+    other = x.clone()
+    other[1::joint] = 0.0
+    other[1::3 * joint] = 1e9
+    keep = torch.ones(rows, dtype=torch.bool, device=DEV)
+    keep[1::joint] = False
+    codes2, scales2 = p.forward_quant(other, bits)
+    assert torch.equal(scales[keep], scales2[keep]) and torch.equal(codes[keep], codes2[keep])
+    codes3, scales3 = p.forward_quant(x[:rows - 1], bits)
+    assert torch.equal(scales[:-1], scales3) and torch.equal(codes[:-1], codes3)
