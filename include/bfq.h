@@ -218,20 +218,21 @@ int bfq_device_status(bfq_plan* plan);
 int bfq_last_cuda_error(const bfq_plan* plan);
 
 /*
- * Which rotation form the tuned kernels (n = 4096, n = 8192) run with the current angles.  They use the scaled two-FMA
+ * Which rotation form the tuned kernels (n = 4096, n = 8192, and n = 128 .. 2048, whose rows go through the n = 4096 kernels
+ * several as one) run with the current angles.  They use the scaled two-FMA
  * form (paper Sec. "Inference Efficiency": two FMAs per pair) in which every element carries the product of the
  * cosines it has been through; when such a product leaves [2^-64, 1] (an angle within ~1e-19 .. of an odd multiple of
  * pi/2 along some path, e.g. angles that are exact multiples of pi/2) the table build selects the three-shear form
  * instead, which has no such limit.  Returns bit 0 = forward tables use the fallback, bit 1 = inverse tables (built by
- * the first bfq_inverse / bfq_backward after bfq_set_angles; at n = 8192 the tables of either half of the row) use the
- * fallback; or a negative bfq_status.  Synchronises
- * the device.  With the scaled form, inputs must stay below about 2^56 in magnitude (intermediate values are the true
- * values divided by the factor).  (No counterpart in the paper; informational.)
+ * the first bfq_inverse / bfq_backward after bfq_set_angles, for n < 4096 by bfq_set_angles; at n = 8192 the tables of either
+ * half of the row) use the fallback; or a negative bfq_status.  Synchronises the device.  With the scaled form at n = 4096 and 8192, inputs must stay below about 2^56 in magnitude (intermediate values
+ * are the true values divided by the factor); rows of up to 2048 elements may hold any fp32 numbers: one whose results are not
+ * finite there is computed again without factors.  (No counterpart in the paper; informational.)
  */
 int bfq_stage_form(bfq_plan* plan);
 
 /*
- * Test hook (no counterpart in the paper): while enabled, the tuned n = 4096 forward kernels of this plan announce 16
+ * Test hook (no counterpart in the paper): while enabled, the tuned forward kernels of a plan with 128 <= n <= 4096 announce 16
  * bytes more per row load than the load delivers and bound their waits at 4096 polls, so that every wait runs out:
  * the kernels return normally with meaningless outputs (inside their buffers) and bfq_device_status reports
  * BFQ_ERR_DEVICE_TIMEOUT once.  Exercises the bounded-wait path without hanging or faulting the GPU.

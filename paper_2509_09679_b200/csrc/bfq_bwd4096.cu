@@ -23,6 +23,7 @@
 #include "bfq_fast.h"
 #include "bfq_generic.cuh"
 #include "bfq_n4096.cuh"
+#include "bfq_row_again.cuh"
 
 namespace bfq {
 namespace b4k {
@@ -258,6 +259,7 @@ struct alignas(64) WideHalf {
 struct ShortRows {
     int log;
     int64_t elems;
+    Again again;  // inverse: for rows that are done again
 };
 
 template <bool IN_F32, bool WIDE = false, bool SHORT = false>
@@ -781,7 +783,8 @@ struct InvSmem {
     static constexpr uint32_t kExOff = kInOff + G * kInSlots * kRowBytes;  // [G][2][kExBytes]
     static constexpr uint32_t kBarOff = kExOff + G * 2 * kExBytes;         // mbarriers [G][kInSlots]
     static constexpr uint32_t kTmemOff = kBarOff + 8 * G * kInSlots;
-    static constexpr uint32_t kUsed = kTmemOff + 16;
+    static constexpr uint32_t kBadOff = kTmemOff + 16;  // [G]: the group has met a result that is not finite (short rows)
+    static constexpr uint32_t kUsed = kBadOff + 4 * G;
     static constexpr uint32_t kBytes = kUsed + 1024;
 };
 
@@ -858,7 +861,7 @@ template <int G, bool OUT_BF16, bool IN_F32 = false, bool WIDE = false, bool SHO
 __global__ void __launch_bounds__(G * kThreads, 1)
 k_inv4096(const __grid_constant__ CUtensorMap ymap, const float* __restrict__ img_lo, const float* __restrict__ img_scaled_lo,
           const int* __restrict__ form_lo, const uint32_t* __restrict__ gsign_lo, void* __restrict__ xout, int64_t ldx, int rows,
-          int* __restrict__ status, const float2* __restrict__ tw12, const InvUpper upper, const ShortRows brief) {
+          int* __restrict__ status, const float2* __restrict__ tw12, const InvUpper upper, const __grid_constant__ ShortRows brief) {
     static_assert(!(SHORT && WIDE), "one or the other");
     static_assert(!(IN_F32 && WIDE), "the wide mode takes bf16 rows");
     const int half = WIDE ? int(blockIdx.x & 1u) : 0;
@@ -879,6 +882,9 @@ k_inv4096(const __grid_constant__ CUtensorMap ymap, const float* __restrict__ im
     if (threadIdx.x < G * kInSlots) {
         mbar_init(sbase + S::kBarOff + 8 * threadIdx.x, 1);
         mbar_init_fence();
+    }
+    if constexpr (SHORT) {
+        if (threadIdx.x < G) sts32(sbase + S::kBadOff + 4 * threadIdx.x, 0u);
     }
     tmem_fence_before();
     __syncthreads();
@@ -987,6 +993,7 @@ k_inv4096(const __grid_constant__ CUtensorMap ymap, const float* __restrict__ im
     const uint32_t sgn_a = par_t ? 0x80000000u : 0u, sgn_b = par_t ? 0u : 0x80000000u;
     const uint4* gsv = reinterpret_cast<const uint4*>(gsign);
 
+    const uint32_t bad_flag = sbase + S::kBadOff + 4 * g;
     // the whole row loop exists once per stage form: the choice is made once per launch, outside the loop
     auto row_loop = [&](auto form_tag) {
     constexpr int FORM = decltype(form_tag)::value;
@@ -1103,12 +1110,17 @@ k_inv4096(const __grid_constant__ CUtensorMap ymap, const float* __restrict__ im
                 for (int c = 0; c < 4; ++c) dst[c] = make_uint4(w[4 * c], w[4 * c + 1], w[4 * c + 2], w[4 * c + 3]);
             }
         }
+        if constexpr (SHORT) sts32_if(__float_as_uint(largest<1>(P)) >= not_finite(OUT_BF16), bad_flag, 1u);
     }
     };
     if (!shear) {
         row_loop(std::integral_constant<int, kFormScaled>());
     } else {
         row_loop(std::integral_constant<int, kFormShear>());
+    }
+    if constexpr (SHORT) {  // rows that are not finite (bfq_row_again.cuh)
+        bar_sync(a.bar, kThreads);  // the group's stores are done
+        if (lds32(bad_flag) != 0u) rows_again(brief.again, first, stride, count, a.ex, a.bar, t);
     }
     tmem_fence_before();
     __syncthreads();
@@ -1305,7 +1317,7 @@ cudaError_t bwd_short_launch(bfq_plan* plan, const void* x, const void* g, int64
     const bool maps = f32 ? (encode_row_map_f32(&xmap, x, rows, n, n) && encode_row_map_f32(&gmap, g, rows, n, n))
                           : (encode_row_map(&xmap, x, rows, n, n) && encode_row_map(&gmap, g, rows, n, n));
     if (!maps) return cudaErrorInvalidValue;
-    const b4k::ShortRows brief{12 - plan->log_n, rows * n};
+    const b4k::ShortRows brief{12 - plan->log_n, rows * n, Again{}};
     const int64_t joint = (brief.elems + f4k::kN - 1) / f4k::kN, pairs = (joint + 1) / 2;
     const int grid = int(pairs < plan->sm_count ? pairs : plan->sm_count);
     auto kern = f32 ? b4k::k_bwd4096<true, false, true> : b4k::k_bwd4096<false, false, true>;
@@ -1333,7 +1345,8 @@ cudaError_t inv_short_launch(bfq_plan* plan, const void* y, bool y_f32, int64_t 
     const int n = plan->n;
     CUtensorMap ymap;
     if (!(y_f32 ? encode_row_map_f32(&ymap, y, rows, ldy, n) : encode_row_map(&ymap, y, rows, ldy, n))) return cudaErrorInvalidValue;
-    const b4k::ShortRows brief{12 - plan->log_n, rows * n};
+    const b4k::ShortRows brief{12 - plan->log_n, rows * n,
+                               Again{y, ldy, y_f32 ? kF32 : kBF16, plan->tw, true, plan->log_n, rows * n, 0, x, x_bf16 ? kBF16 : kF32, nullptr, nullptr}};
     const int64_t joint = (brief.elems + f4k::kN - 1) / f4k::kN, want = (joint + G - 1) / G;
     const int grid = int(want < plan->sm_count ? want : plan->sm_count);
     kern<<<grid, G * b4k::kThreads, S::kBytes, st>>>(ymap, plan->img_b4096, plan->img_i4096, plan->form_flag + 1, plan->gsign4096, x, f4k::kN,

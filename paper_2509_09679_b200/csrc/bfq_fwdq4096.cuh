@@ -5,6 +5,7 @@
 #include "bfq_fast.h"
 #include "bfq_generic.cuh"
 #include "bfq_n4096.cuh"
+#include "bfq_row_again.cuh"
 
 namespace bfq {
 namespace f4k {
@@ -165,13 +166,15 @@ enum : int { kOutInt4 = 0, kOutBf16 = 1, kOutInt4Stats = 2, kOutInt2 = 3, kOutIn
 // log2 n on are the identity, so 2^SUB rows go through the kernel as one ("rows" then counts these; `elems` = all
 // elements, the last one may be short: its missing rows arrive as zeros and are not stored).  The absent stages are passed
 // over, not multiplied by 1 and 0 (no row may touch another one's infinities); the general last stage becomes a diagonal
-// that takes the factors off.  A quantized row's maximum is taken over its own part of the 4096.
+// that takes the factors off.  A quantized row's maximum is taken over its own part of the 4096.  A row whose results are not
+// finite is done again at the end (bfq_row_again.cuh); to know of one takes eight maxima per thread and joint row where rows go
+// out.
 template <int G, int CW, int XB, int TRANSFORM, int OUT, int STEP = 2, bool ROWS = false, bool IN_F32 = false, int SUB = 0>
 __global__ void __launch_bounds__(G * kGroupThreads, 1)
 k_fwdq4096(const __grid_constant__ CUtensorMap tmap, const float* __restrict__ img, const int* __restrict__ form,
            uint8_t* __restrict__ codes,
            uint16_t* __restrict__ scales, __nv_bfloat16* __restrict__ yout, int64_t ldy, int rows,
-           int* __restrict__ status, uint32_t tx_bytes, int wait_limit, unsigned long long* __restrict__ hist, int64_t elems) {
+           int* __restrict__ status, uint32_t tx_bytes, int wait_limit, unsigned long long* __restrict__ hist, int64_t elems, const __grid_constant__ Again again) {
     using S = Smem<G, XB>;
     constexpr bool kTmem = TRANSFORM == kButterfly;
     constexpr bool kCount = OUT == kOutInt4Stats;
@@ -206,6 +209,9 @@ k_fwdq4096(const __grid_constant__ CUtensorMap tmap, const float* __restrict__ i
     }
     if constexpr (kCount) {
         for (uint32_t e = threadIdx.x; e < (128u + 1024u * G) / 4u; e += G * kGroupThreads) sts32(sbase + S::kBinsOff + 4u * e, 0u);
+    }
+    if constexpr (SUB != 0) {
+        if (threadIdx.x < G) sts32(sbase + S::kHistOff + 1024u * threadIdx.x + 256u, 0u);
     }
     // everything above overlaps the end of the kernel before this one; global memory is touched from here on
     grid_dep_wait();
@@ -290,6 +296,7 @@ k_fwdq4096(const __grid_constant__ CUtensorMap tmap, const float* __restrict__ i
     const uint32_t in_x = IN_F32 ? ((((t & 1) << 2) ^ ((t >> 1) & 7)) << 4) : ((((t & 3) << 1) ^ ((t >> 2) & 3)) << 4);
     const uint32_t amax_base = sbase + S::kAmaxOff + g * 32;
     uint8_t* const out_t = codes + t;
+    const uint32_t bad_flag = sbase + S::kHistOff + 1024u * g + 256u;  // SUB > 0: the group has met a result that is not finite
     const uint32_t hist_g = sbase + S::kHistOff + 1024u * g;  // this group's counts of packed code bytes
 
     // the whole row loop exists once per stage form: the choice is made once per launch, outside the loop
@@ -379,6 +386,12 @@ k_fwdq4096(const __grid_constant__ CUtensorMap tmap, const float* __restrict__ i
         }
         if constexpr (OUT == kOutBf16 || OUT == kOutF32) {
             bar_sync(ex.bar, kGroupThreads);  // every warp is past its reads of the second regrouping buffer
+            if constexpr (SUB != 0) {
+                // the last stage's pairs lie in registers 2^(3 - SUB) apart, or (n <= 256) in other warps
+                constexpr int kSkip = SUB < 4 ? 8 >> SUB : 0;
+                if (SUB < 4 || (SUB == 4 ? q < 2 : (q & 1) == 0))
+                    sts32_if(__float_as_uint(largest<kSkip>(P)) >= not_finite(OUT == kOutBf16), bad_flag, 1u);
+            }
             continue;
         }
 
@@ -461,7 +474,7 @@ k_fwdq4096(const __grid_constant__ CUtensorMap tmap, const float* __restrict__ i
             for (int m = 0; m < 16; ++m) {
                 float a, b;
                 unpack2(P[m], a, b);
-                mx[m >> kPartShift] = fmaxf(mx[m >> kPartShift], fmaxf(fabsf(a), fabsf(b)));
+                mx[m >> kPartShift] = max_abs_nan(mx[m >> kPartShift], a, b);
             }
             uint32_t mine = 0u;
 #pragma unroll
@@ -474,14 +487,15 @@ k_fwdq4096(const __grid_constant__ CUtensorMap tmap, const float* __restrict__ i
             sts32_if(lane < kParts, slots + 16 * part + 4 * q, mine);
             bar_sync(ex.bar, kGroupThreads);
             const uint4 o = lds128(slots + 16 * part);
-            const float lower = fmaxf(__uint_as_float(o.x), __uint_as_float(o.y)), upper = fmaxf(__uint_as_float(o.z), __uint_as_float(o.w));
-            const float amax = SUB < 5 ? fmaxf(lower, upper) : (q < 2 ? lower : upper);
-            s16 = row_scale_fast<kQmax>(amax, &inv);
+            const uint32_t lower = max(o.x, o.y), upper = max(o.z, o.w);
+            const uint32_t amax = SUB < 5 ? max(lower, upper) : (q < 2 ? lower : upper);
+            sts32_if(amax >= not_finite(false), bad_flag, 1u);
+            s16 = row_scale_fast<kQmax>(__uint_as_float(amax), &inv);
             const int64_t short_row = SUB < 5 ? (static_cast<int64_t>(row) << SUB) + part
                                               : (static_cast<int64_t>(row) << SUB) + 2 * part + (q >> 1);
             const bool writes = lane < kParts && (SUB < 5 ? q == 0 : (q & 1) == 0) && (short_row << stages_of_sub(SUB)) < elems;
             stg16_if(writes, scales + short_row, s16);
-            plain_parts = __ballot_sync(0xFFFFFFFFu, (((s16 >> 10) & 31u) != 0u) && (s16 != 0x7BFFu));
+            plain_parts = __ballot_sync(0xFFFFFFFFu, (((s16 >> 10) & 31u) != 0u) && (s16 < 0x7BFFu));  // NaN is not
             plain = plain_parts == 0xFFFFFFFFu;
         }
         float invp[kParts];
@@ -608,6 +622,12 @@ k_fwdq4096(const __grid_constant__ CUtensorMap tmap, const float* __restrict__ i
         row_loop(std::integral_constant<int, kFormShear>());
     }
 
+    if constexpr (SUB != 0) {
+        bar_sync(ex.bar, kGroupThreads);  // the group's stores are done
+        if (lds32(bad_flag) != 0u)
+            rows_again(again, first, stride, count, sbase + S::kExOff + g * XB * kExBytes, ex.bar, t);
+    }
+
     if constexpr (kCount) {
         // counts of the G groups per offset-binary byte (two nibbles code + 8) -> the CTA's 16 code counts -> the caller's
         // histogram, indexed by code + 8.  Integer additions: the result does not depend on their order.
@@ -639,7 +659,7 @@ k_fwdq4096(const __grid_constant__ CUtensorMap tmap, const float* __restrict__ i
 template <int G, int CW, int XB, int TRANSFORM, int OUT, bool ROWS = false, bool IN_F32 = false, int SUB = 0>
 static cudaError_t launch_variant(const bfq_plan* plan, const CUtensorMap& tmap, int64_t rows, uint8_t* codes,
                                   uint16_t* scales, void* y, int64_t ldy, cudaStream_t st,
-                                  unsigned long long* hist = nullptr, int64_t elems = 0) {
+                                  unsigned long long* hist = nullptr, int64_t elems = 0, const Again& again = Again{}) {
     using S = f4k::Smem<G, XB>;
     static bool attr_set[kMaxDevices] = {false};
     auto kern = f4k::k_fwdq4096<G, CW, XB, TRANSFORM, OUT, 2, ROWS, IN_F32, SUB>;
@@ -656,7 +676,7 @@ static cudaError_t launch_variant(const bfq_plan* plan, const CUtensorMap& tmap,
     const int wait_limit = plan->test_stuck_wait ? 4096 : (1 << 22);
     return launch_overlapped(kern, dim3(grid), dim3(G * f4k::kGroupThreads), S::kBytes, st, tmap, plan->img4096,
                              plan->form_flag, codes, scales, static_cast<__nv_bfloat16*>(y), ldy, int(rows),
-                             plan->status_word, tx_bytes, wait_limit, hist, elems);
+                             plan->status_word, tx_bytes, wait_limit, hist, elems, again);
 }
 
 }  // namespace bfq

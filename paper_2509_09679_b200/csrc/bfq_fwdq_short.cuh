@@ -16,10 +16,12 @@ static cudaError_t fwdq_short_launch(const bfq_plan* plan, const void* x, bool f
     CUtensorMap tmap;
     if (!(f32 ? encode_row_map_f32(&tmap, x, rows, ldx, n) : encode_row_map(&tmap, x, rows, ldx, n))) return cudaErrorInvalidValue;
     const int64_t elems = rows * n, joint = (elems + f4k::kN - 1) / f4k::kN;
+    const int type = f32 ? kF32 : kBF16;
+    const Again again{x, ldx, type, plan->tw, false, 12 - SUB, elems, bits, y, type, codes, scales};
     using namespace f4k;
     auto go = [&](auto out, auto in_f32) {
         return launch_variant<4, 32, 2, kButterfly, decltype(out)::value, false, decltype(in_f32)::value, SUB>(plan, tmap, joint, codes, scales, y,
-                                                                                                    kN, st, nullptr, elems);
+                                                                                                    kN, st, nullptr, elems, again);
     };
     if (f32) {
         const std::true_type in{};

@@ -1,6 +1,8 @@
 """Rows of 128 .. 2048 elements on the n = 4096 kernels (several rows as one of 4096): against the oracle at sizes where the
 last joint row is whole, holds a single row and lacks a single row, with guard bytes around every output; the rules are
 in parity.py.  The row counts are above the sizes from which every one of these kernels is taken."""
+import math
+
 import numpy as np
 import pytest
 import torch
@@ -126,3 +128,68 @@ def test_codes_of_a_row_do_not_depend_on_the_rows_beside_it(n, bits):
     assert torch.equal(scales[keep], scales2[keep]) and torch.equal(codes[keep], codes2[keep])
     codes3, scales3 = p.forward_quant(x[:rows - 1], bits)
     assert torch.equal(scales[:-1], scales3) and torch.equal(codes[:-1], codes3)
+
+
+@pytest.mark.parametrize("n", [128, 256, 512, 1024, 2048])
+@pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
+def test_rows_of_any_magnitude(n, dtype):
+    """Rows up to 1e36 through angles with small cosines, where values divided by the cosines' product overflow on the way: right
+    all the same, in whole and in short joint rows and several in one, and the rows beside them the same bits as without."""
+    theta = synth.angles(n, "uniform", 3)
+    theta[1:3, ::3] = math.pi / 2 - 1e-5
+    theta[3, ::5] = math.pi / 2 - 1e-3
+    rows = 4096 // n * 700 + 1
+    x = synth.rows(rows, n, "normal", 4, dtype=dtype)
+    large = {0: 1e20, 1: 1e34, 4: 1e30, 9: 1e36, rows // 2: 1e28, rows - 1: 1e35}
+    big = x.clone()
+    for r, m in large.items():
+        big[r] = x[r] * m
+    p = Plan(n, DEV)
+    p.set_angles(theta.to(DEV))
+    assert p.stage_form() & 1 == 0  # the scaled form
+    th64, b64 = to_f64(theta), to_f64(big)
+    amax = np.abs(b64).max(axis=1)
+    y_ref, x_ref = oracle.forward(th64, b64), oracle.inverse(th64, b64)
+    keep = torch.tensor([r not in large for r in range(rows)], device=DEV)
+    y, xr = Guarded((rows, n), dtype, DEV), Guarded((rows, n), dtype, DEV)
+    check_rows_close(p.forward(big.to(DEV), out=y.view), y_ref, amax, "forward")
+    check_rows_close(p.inverse(big.to(DEV), out=xr.view), x_ref, amax, "inverse")
+    assert torch.equal(y.view[keep], p.forward(x.to(DEV))[keep]) and torch.equal(xr.view[keep], p.inverse(x.to(DEV))[keep])
+    if dtype == torch.bfloat16:
+        check_rows_close(p.inverse(big.to(DEV), out_dtype=torch.float32), x_ref, amax, "inverse, fp32 out")
+    for bits in (2, 4, 8):
+        codes, scales = Guarded((rows, n * bits // 8), torch.uint8, DEV), Guarded((rows,), torch.float16, DEV)
+        p.forward_quant(big.to(DEV), bits, codes.view, scales.view)
+        check_quant(codes.view[keep], scales.view[keep], y_ref[keep.cpu().numpy()], bits, f"{bits} bits")
+        for r in large:  # saturated: the lowest or the highest code, wherever the value is more than rounding noise
+            assert scales.view[r] == 65504
+            c = oracle.unpack(codes.view[r:r + 1].cpu().numpy(), bits)[0]
+            sure = np.abs(y_ref[r]) > 1e-5 * amax[r]
+            assert np.array_equal(c[sure], np.where(y_ref[r] > 0, 2 ** (bits - 1) - 1, -(2 ** (bits - 1)))[sure])
+        plain = p.forward_quant(x.to(DEV), bits)
+        assert torch.equal(codes.view[keep], plain[0][keep]) and torch.equal(scales.view[keep], plain[1][keep])
+        assert codes.intact() and scales.intact()
+    assert y.intact() and xr.intact() and p.device_status() == 0
+
+
+@pytest.mark.parametrize("n", [128, 256, 2048])
+def test_infinities_and_nan_as_in_the_kernels_for_every_n(n, monkeypatch):
+    """What the rotation by cos and sin makes of them, with the saturated scale of an infinite row; the rows beside them are the
+    same bits as without."""
+    rows = 4096 // n * 5 + 1
+    p = Plan(n, DEV)
+    p.set_angles(synth.angles(n, "normal", 1).to(DEV))
+    x = synth.rows(rows, n, "normal", 2)
+    clean = x.clone()
+    x[3, 5], x[7, 1], x[rows - 1, 100] = float("inf"), float("nan"), float("-inf")
+    x[9] = float("inf")
+    run = lambda v: (p.forward(v.to(DEV)), p.inverse(v.to(DEV)), *(t for b in (2, 4, 8) for t in p.forward_quant(v.to(DEV), b)))
+    got = run(x)
+    others = [r for r in range(rows) if r not in (3, 7, 9, rows - 1)]
+    for a, b in zip(got, run(clean)):
+        assert torch.equal(a[others], b[others])
+    monkeypatch.setenv("BFQ_GENERIC_ONLY", "1")
+    for a, b in zip(got, run(x)):
+        for r in (3, 7, 9, rows - 1):
+            assert torch.equal(a[r].nan_to_num(), b[r].nan_to_num())
+    assert got[3][3] == 65504
