@@ -62,18 +62,22 @@ static int check_rows(const void* p, int dt, int64_t rows, int64_t ld, int n) {
 // Rows of 128 .. 2048 elements on the n = 4096 kernels, several as one.  Measured against the generic kernels from 2^13 to
 // 2^25 elements in all (us; bf16, n = 1024; 2^13 / 2^20 / 2^25 elements): codes 8.1 -> 5.2 / 8.7 -> 6.6 / 144 -> 40, rows
 // 7.0 -> 5.0 / 7.6 -> 6.3 / 166 -> 36: always faster.  Inverse 7.2 -> 5.4 / 7.7 -> 6.9 / 168 -> 43, but for n = 128 in fp32
-// the other way round up to 2^20 (6.7 against 7.5).  Backward: filling the tensor memory takes 27 us whatever the size, against
-// 16 - 18 us and 18 - 21 us of the generic kernel on small batches; they meet at about 2^18 elements for n <= 256 (38 against
-// 31, 27 against 29) and 2^19 above (24 against 29 at 1024, 31 against 29 at 512).
+// the other way round up to 2^20 (8.3 against 10.3; 12.4 against 10.3 at 2^21).
 static bool use_short_rows(const bfq_plan* plan, int64_t rows, int64_t min_elems) {
     return rows < (int64_t(1) << 31) - 64 && rows * plan->n >= min_elems && !env_flag("BFQ_GENERIC_ONLY") && fwdq_short_available(plan);
 }
 static int64_t short_inverse_from(int n) { return n == 128 ? int64_t(1) << 21 : 0; }
-// (bf16 rows that bfq_backward_noalloc takes too stay on the kernel it runs, so that the two entry points' dx are the same
-// bits, up to 2^23 elements, where that would cost 60 us and more)
-static int64_t short_backward_from(int n, bool f32) {
-    if (!f32 && n <= BFQ_NOALLOC_MAX_N) return int64_t(1) << 23;
-    return n <= 256 ? int64_t(1) << 18 : int64_t(1) << 20;
+// Backward: filling the tensor memory takes 27 - 29 us whatever the size, the generic kernel 22 - 25 us on a small batch.  Where
+// they meet (us, generic against short rows, fp32 / bf16; m = 2^16 elements): n = 128 at 2 m 30.8 : 30.6 / 30.8 : 28.8; n = 256
+// at 4 m 30.5 : 30.8 / 29.9 : 29.4; n = 512 at 5 m 28.8 : 28.7 / 28.7 : 28.2, at 6 m 30.8 : 28.7 / 30.8 : 27.7; n = 1024 at 9 m
+// 28.8 : 30.6 / 29.4 : 29.8, at 10 m 37.0 : 30.8 / 36.9 : 30.0; n = 2048 at 9 m 26.7 : 30.8 / 26.4 : 30.6, at 10 m 34.8 : 30.8 / 33.9 : 30.7.
+static int64_t short_backward_from(int n) {
+    const int64_t m = int64_t(1) << 16;
+    return n == 128 ? 2 * m : (n == 256 ? 4 * m : (n == 512 ? 6 * m : 10 * m));
+}
+bool takes_short_backward(int n, int xt, int gt, bool want_dx, int dxt, int64_t rows, int64_t ld) {
+    return n >= 128 && n < 4096 && xt == gt && (!want_dx || dxt == xt) && ld == n && rows < (int64_t(1) << 31) - 64 && rows * n >= short_backward_from(n) &&
+           !env_flag("BFQ_GENERIC_ONLY");
 }
 
 // ---- generic kernel dispatch ------------------------------------------------------------------------
@@ -682,8 +686,7 @@ int bfq_backward(bfq_plan* plan, const void* x, bfq_dtype xt, const void* g, bfq
         if (e == cudaSuccess) e = bwd8192_launch_halves(plan, x, g, rows, ld, dx, dtheta, st);
         return e == cudaSuccess ? BFQ_OK : cuda_fail(plan, e);
     }
-    if (xt == gt && (dx == nullptr || dxt == xt) && ld == plan->n && use_short_rows(plan, rows, short_backward_from(plan->n, xt == BFQ_F32)) &&
-        bwd_short_available(plan)) {
+    if (takes_short_backward(plan->n, xt, gt, dx != nullptr, dxt, rows, ld) && bwd_short_available(plan)) {
         cudaError_t e = bwd_short_launch(plan, x, g, rows, dx, dtheta, xt == BFQ_F32, st);
         return e == cudaSuccess ? BFQ_OK : cuda_fail(plan, e);
     }

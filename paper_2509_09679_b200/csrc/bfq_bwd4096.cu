@@ -1302,16 +1302,23 @@ bool bwd_short_available(const bfq_plan* plan) {
            plan->partial_floats >= bwd_short_partial_floats(plan->sm_count) && encode_tiled() != nullptr;
 }
 
-// x, g, dx contiguous rows, all bf16 or all fp32
-cudaError_t bwd_short_launch(bfq_plan* plan, const void* x, const void* g, int64_t rows, void* dx, float* dtheta, bool f32, cudaStream_t st) {
+// what the kernels need once per device (a caller that captures does this before)
+cudaError_t bwd_short_prepare(int device) {
     static bool attr_set[kMaxDevices] = {false};
-    if (!attr_set[plan->device]) {
+    if (!attr_set[device]) {
         cudaError_t e = cudaFuncSetAttribute(b4k::k_bwd4096<false, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(b4k::Smem::kBytes));
         if (e == cudaSuccess)
             e = cudaFuncSetAttribute(b4k::k_bwd4096<true, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(b4k::Smem::kBytes));
         if (e != cudaSuccess) return e;
-        attr_set[plan->device] = true;
+        attr_set[device] = true;
     }
+    return cudaSuccess;
+}
+
+// x, g, dx contiguous rows, all bf16 or all fp32
+cudaError_t bwd_short_launch(bfq_plan* plan, const void* x, const void* g, int64_t rows, void* dx, float* dtheta, bool f32, cudaStream_t st) {
+    cudaError_t e = bwd_short_prepare(plan->device);
+    if (e != cudaSuccess) return e;
     const int n = plan->n;
     CUtensorMap xmap, gmap;
     const bool maps = f32 ? (encode_row_map_f32(&xmap, x, rows, n, n) && encode_row_map_f32(&gmap, g, rows, n, n))
@@ -1323,7 +1330,7 @@ cudaError_t bwd_short_launch(bfq_plan* plan, const void* x, const void* g, int64
     auto kern = f32 ? b4k::k_bwd4096<true, false, true> : b4k::k_bwd4096<false, false, true>;
     kern<<<grid, b4k::kCtaThreads, b4k::Smem::kBytes, st>>>(xmap, gmap, plan->img_b4096, plan->gsign4096, plan->dsign4096, dx, f4k::kN, plan->partial,
                                                           int(joint), plan->status_word, nullptr, b4k::WideHalf{}, brief);
-    cudaError_t e = cudaGetLastError();
+    e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     b4k::k_reduce_short<<<plan->log_n * (n / 2) / 32, 1024, 0, st>>>(plan->partial, grid, plan->log_n - 1, dtheta);
     plan->last_backward_partials = grid;

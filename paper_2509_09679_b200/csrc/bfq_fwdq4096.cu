@@ -141,15 +141,23 @@ size_t fwdq4096_image_bytes() { return size_t(2) * 128 * f4k::kCols * sizeof(flo
 // per angle: float4 (three-shear constants, cos, sin), double2 (cos, sin), one negation flag
 size_t fwdq4096_prep_bytes() { return size_t(12) * (f4k::kN / 2) * (sizeof(float4) + sizeof(double2) + 1); }
 
-// Builds the generic (cos, sin) table and the tensor-memory image from the angles (two launches).
-cudaError_t fwdq4096_set_angles(const bfq_plan* plan, const float* theta, cudaStream_t st) {
+// The generic (cos, sin) table and the staging entries of every image (one launch).
+cudaError_t fwdq4096_prep_angles(const bfq_plan* plan, const float* theta, cudaStream_t st) {
     const int count = 12 * (f4k::kN / 2);
     float4* prep = reinterpret_cast<float4*>(plan->prep4096);
     double2* cs = reinterpret_cast<double2*>(prep + count);
     uint8_t* flip = reinterpret_cast<uint8_t*>(cs + count);
-    cudaError_t e = launch_overlapped(f4k::k_prep_angles4096, dim3((count + 255) / 256), dim3(256), 0, st, theta, plan->tw,
-                                      prep, flip, cs, plan->form_flag, plan->log_n);
+    return launch_overlapped(f4k::k_prep_angles4096, dim3((count + 255) / 256), dim3(256), 0, st, theta, plan->tw, prep, flip, cs,
+                             plan->form_flag, plan->log_n);
+}
+
+// That and the tensor-memory image of the forward kernels (two launches).
+cudaError_t fwdq4096_set_angles(const bfq_plan* plan, const float* theta, cudaStream_t st) {
+    const int count = 12 * (f4k::kN / 2);
+    cudaError_t e = fwdq4096_prep_angles(plan, theta, st);
     if (e != cudaSuccess) return e;
+    float4* prep = reinterpret_cast<float4*>(plan->prep4096);
+    double2* cs = reinterpret_cast<double2*>(prep + count);
     return launch_overlapped(f4k::k_build_image4096, dim3((count + 255) / 256), dim3(256), 0, st, prep, cs, plan->img4096,
                              plan->form_flag);
 }

@@ -5,9 +5,13 @@
 // latency-critical loop in which the device-wide synchronisation that cudaMalloc / cudaFree imply is
 // not acceptable.  bfq_plan_create allocates (tables, partial sums), so such callers cannot use the
 // plan-based entry points.  This entry point needs no plan: everything the backward pass needs
-// beyond the caller's own buffers (the cos/sin table and the per-CTA partial sums of d-theta) lives
-// in one fixed array in the library's device data segment, which every GPU that loads the library
-// holds until the process exits.
+// beyond the caller's own buffers (the cos/sin table, the tables of the short-row kernel and the
+// per-CTA partial sums of d-theta) lives in one fixed array in the library's device data segment,
+// which every GPU that loads the library holds until the process exits.
+//
+// The kernel is chosen by the rule of bfq_backward, so that dx is the same bits either way: calls it
+// takes to the n = 4096 kernel come here with the tables built in the array on every call and as many
+// CTAs as the rest of it holds partial sums for (72 at 96 KiB each).
 //
 // Consequences of the shared array: the row length is limited to BFQ_NOALLOC_MAX_N; all calls (from
 // any stream or thread) use the same bytes, so two calls that overlap on one GPU race; the array
@@ -17,6 +21,7 @@
 
 #include <cuda_runtime.h>
 
+#include "bfq_fast.h"
 #include "bfq_generic.cuh"
 #include "bfq_plan.h"
 
@@ -32,6 +37,7 @@ static __device__ __align__(256) unsigned char g_scratch[kScratchBytes];
 struct PerDevice {
     void* base = nullptr;  // device address of g_scratch on this GPU
     int sm_count = 0;
+    int cc_major = 0;
 };
 static PerDevice g_dev[kMaxDevices];
 
@@ -44,8 +50,11 @@ static cudaError_t setup(int device, PerDevice** out) {
         if (e != cudaSuccess) return e;
         int sms = 0;
         e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device);
+        int major = 0;
+        if (e == cudaSuccess) e = cudaDeviceGetAttribute(&major, cudaDevAttrComputeCapabilityMajor, device);
+        if (e == cudaSuccess) e = bwd_short_prepare(device);
         if (e != cudaSuccess) return e;
-        d.sm_count = sms;
+        d.sm_count = sms, d.cc_major = major;
         d.base = p;
     }
     *out = &d;
@@ -89,6 +98,38 @@ static cudaError_t launch(int device, const PerDevice& d, BackwardParams p, cons
     return cudaGetLastError();
 }
 
+// The array as a plan's tables and partial sums, as far as bwd_short_launch uses them.
+static cudaError_t launch_short(int device, const PerDevice& d, int log_n, const float* theta, const void* x, const void* g, int64_t rows, void* dx, bool f32,
+                                float* dtheta, cudaStream_t st, bool* taken) {
+    bfq_plan view;
+    view.n = 1 << log_n, view.log_n = log_n, view.device = device, view.cc_major = d.cc_major;
+    unsigned char* at = static_cast<unsigned char*>(d.base);
+    auto part = [&](size_t bytes) {
+        unsigned char* p = at;
+        at += (bytes + 255) / 256 * 256;
+        return p;
+    };
+    view.tw = reinterpret_cast<float2*>(part(kTableBytes));
+    view.prep4096 = part(fwdq4096_prep_bytes());
+    view.img_b4096 = reinterpret_cast<float*>(part(bwd4096_image_bytes()));
+    view.img_i4096 = reinterpret_cast<float*>(part(inv4096_image_bytes()));
+    view.dsign4096 = reinterpret_cast<int8_t*>(part(bwd4096_dsign_bytes()));
+    view.gsign4096 = reinterpret_cast<uint32_t*>(part(bwd4096_gsign_bytes()));
+    view.status_word = reinterpret_cast<int*>(part(4 * sizeof(int)));
+    view.form_flag = view.status_word + 1;
+    view.partial = reinterpret_cast<float*>(at);
+    const size_t left = kScratchBytes - size_t(at - static_cast<unsigned char*>(d.base));
+    view.partial_floats = left / sizeof(float);
+    const int slots = int(left / bwd_short_partial_floats(1) / sizeof(float));
+    view.sm_count = slots < d.sm_count ? slots : d.sm_count;  // CTAs
+    *taken = view.sm_count > 0 && bwd_short_available(&view);
+    if (!*taken) return cudaSuccess;
+    cudaError_t e = fwdq4096_prep_angles(&view, theta, st);
+    if (e == cudaSuccess) e = bwd4096_build_tables(&view, st);
+    if (e == cudaSuccess) e = bwd_short_launch(&view, x, g, rows, dx, dtheta, f32, st);
+    return e;
+}
+
 }  // namespace noalloc
 }  // namespace bfq
 
@@ -125,6 +166,11 @@ extern "C" int bfq_backward_noalloc(int n, const float* theta, const void* x, bf
     BackwardParams p{};
     p.x = x, p.xt = xt, p.g = g, p.gt = gt, p.ld = ld, p.dx = dx, p.dxt = dxt, p.rows = rows;
     cudaError_t e;
+    if (takes_short_backward(n, xt, gt, dx != nullptr, dxt, rows, ld)) {
+        bool taken = false;
+        e = noalloc::launch_short(device, *d, log_n, theta, x, g, rows, dx, xt == BFQ_F32, dtheta, st, &taken);
+        if (taken || e != cudaSuccess) return e == cudaSuccess ? BFQ_OK : BFQ_ERR_CUDA;
+    }
     switch (log_n) {
         case 4: e = noalloc::launch<4>(device, *d, p, theta, dtheta, st); break;
         case 5: e = noalloc::launch<5>(device, *d, p, theta, dtheta, st); break;

@@ -38,8 +38,8 @@ def _check_against_plan(n, rows, dtype, seed):
     check_rows_close(dx, to_f64(dx_ref), np.abs(to_f64(g)).max(axis=1), f"noalloc dx n={n}")
     # d-theta is summed over a different number of CTAs: the d-theta tolerance of the parity tests
     check_dtheta(dth, to_f64(dth_ref), f"noalloc dtheta n={n}")
-    # and against the oracle itself (at these sizes both paths run the same generic kernel: comparing them with each
-    # other alone would compare the kernel with itself)
+    # and against the oracle itself (both paths run the same kernel at every size: comparing them with each other alone
+    # would compare the kernel with itself)
     dx_o, dth_o = oracle.backward(to_f64(theta), to_f64(x), to_f64(g))
     check_rows_close(dx, dx_o, np.abs(to_f64(g)).max(axis=1), f"noalloc dx vs oracle n={n}")
     check_dtheta(dth, dth_o, f"noalloc dtheta vs oracle n={n}")
@@ -71,3 +71,23 @@ def test_limits_and_empty_batch():
     dth = torch.ones((6, 32), dtype=torch.float32, device=DEV)
     backward_noalloc(theta, x, g, None, dth)
     assert not dth.any()
+
+
+@pytest.mark.parametrize("n", [64, 128, 256, 512, 1024])
+@pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
+@pytest.mark.parametrize("elems", [1 << 16, 1 << 17, 3 << 17, 5 << 18, 9 << 20])
+def test_dx_has_the_bits_of_the_plan_based_backward(n, dtype, elems):
+    """On both sides of the sizes from which short rows go to the n = 4096 kernel, and with more joint rows than CTAs."""
+    rows = elems // n + 3
+    theta = synth.angles(n, "uniform", 310).to(DEV)
+    x, g = (synth.rows(rows, n, "normal", s, dtype=dtype, device=DEV) for s in (311, 312))
+    plan = Plan(n, DEV)
+    plan.set_angles(theta)
+    dx_ref, dth_ref = plan.backward(x, g)
+    dx, dth = torch.full_like(x, float("nan")), torch.empty_like(dth_ref)
+    backward_noalloc(theta, x, g, dx, dth)
+    assert torch.equal(dx, dx_ref)
+    check_dtheta(dth, to_f64(dth_ref), f"noalloc dtheta n={n}")
+    dth2 = torch.empty_like(dth)
+    backward_noalloc(theta, x, g, None, dth2)
+    assert torch.equal(dth, dth2)
