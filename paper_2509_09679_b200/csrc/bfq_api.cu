@@ -62,11 +62,12 @@ static int check_rows(const void* p, int dt, int64_t rows, int64_t ld, int n) {
 // Rows of 128 .. 2048 elements on the n = 4096 kernels, several as one.  Measured against the generic kernels from 2^13 to
 // 2^25 elements in all (us; bf16, n = 1024; 2^13 / 2^20 / 2^25 elements): codes 8.1 -> 5.2 / 8.7 -> 6.6 / 144 -> 40, rows
 // 7.0 -> 5.0 / 7.6 -> 6.3 / 166 -> 36: always faster.  Inverse 7.2 -> 5.4 / 7.7 -> 6.9 / 168 -> 43, but for n = 128 in fp32
-// the other way round up to 2^20 (8.3 against 10.3; 12.4 against 10.3 at 2^21).
+// the other way round up to 2^20 (8.3 against 10.3; 12.4 against 10.3 at 2^21; bf16 n = 128 8.2 -> 6.2 at 2^13, 8.3 : 8.3 up to
+// 2^20, 18.5 -> 10.3 at 2^22).
 static bool use_short_rows(const bfq_plan* plan, int64_t rows, int64_t min_elems) {
     return rows < (int64_t(1) << 31) - 64 && rows * plan->n >= min_elems && !env_flag("BFQ_GENERIC_ONLY") && fwdq_short_available(plan);
 }
-static int64_t short_inverse_from(int n) { return n == 128 ? int64_t(1) << 21 : 0; }
+static int64_t short_inverse_from(int n, bool f32) { return n == 128 && f32 ? int64_t(1) << 21 : 0; }
 // Backward: filling the tensor memory takes 27 - 29 us whatever the size, the generic kernel 22 - 25 us on a small batch.  Where
 // they meet (us, generic against short rows, fp32 / bf16; m = 2^16 elements): n = 128 at 2 m 30.8 : 30.6 / 30.8 : 28.8; n = 256
 // at 4 m 30.5 : 30.8 / 29.9 : 29.4; n = 512 at 5 m 28.8 : 28.7 / 28.7 : 28.2, at 6 m 30.8 : 28.7 / 30.8 : 27.7; n = 1024 at 9 m
@@ -637,7 +638,7 @@ int bfq_inverse(bfq_plan* plan, const void* y, bfq_dtype yt, int64_t rows, int64
         if (e == cudaSuccess) e = inv8192_launch(plan, y, rows, ldy, x, xt == BFQ_BF16, ldx, st);
         return e == cudaSuccess ? BFQ_OK : cuda_fail(plan, e);
     }
-    if ((yt == BFQ_BF16 || xt == BFQ_F32) && x != y && ldx == plan->n && use_short_rows(plan, rows, short_inverse_from(plan->n)) &&
+    if ((yt == BFQ_BF16 || xt == BFQ_F32) && x != y && ldx == plan->n && use_short_rows(plan, rows, short_inverse_from(plan->n, yt == BFQ_F32)) &&
         bwd_short_available(plan)) {
         cudaError_t e = inv_short_launch(plan, y, yt == BFQ_F32, rows, ldy, x, xt == BFQ_BF16, static_cast<cudaStream_t>(stream));
         return e == cudaSuccess ? BFQ_OK : cuda_fail(plan, e);
