@@ -279,7 +279,8 @@ class Plan:
         n1 = self._q1(q1)
         d = n1 * self.n
         rows, ld = _rows(x, d, self.device, what="x")
-        if _rows(g, d, self.device, rows, "g")[1] != ld or (rows > 1 and ld != d):
+        ld_g = _rows(g, d, self.device, rows, "g")[1]
+        if rows > 1 and (ld != d or ld_g != d):  # a single row may come with any row stride
             raise ValueError("x and g must have contiguous rows")
         dx = torch.empty((rows, d), dtype=x.dtype, device=x.device)
         dtheta = torch.empty((self.L, self.n // 2), dtype=torch.float32, device=x.device)

@@ -45,8 +45,10 @@ def composite_backward(plan: Plan, q1: torch.Tensor, params: torch.Tensor | None
     tokens = x.shape[0]
     if _one_pass(plan, n1) and q1.dtype == torch.float32:
         g2 = g.reshape(tokens, n1 * n2).contiguous()
-        dx, dtheta2, dQ1 = plan.composite_backward(q1.contiguous(), x.reshape(tokens, n1 * n2).contiguous(),
-                                                   g2 if g2.dtype in (torch.float32, torch.bfloat16) else g2.float())
+        g2 = g2 if g2.dtype in (torch.float32, torch.bfloat16) else g2.float()
+        if g2.data_ptr() % 16:  # g may lie at any address, the kernel's rows may not
+            g2 = g2.clone()
+        dx, dtheta2, dQ1 = plan.composite_backward(q1.contiguous(), x.reshape(tokens, n1 * n2).contiguous(), g2)
     else:
         gp = torch.einsum("ki,rkj->rij", q1, g.reshape(tokens, n1, n2).float())      # G' = Q1^T G
         runs_x = x.reshape(tokens * n1, n2)

@@ -418,6 +418,26 @@ def test_composite_backward_in_one_pass(n1, n2, tokens, dtype):
     assert p.device_status() == 0
 
 
+@pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
+def test_composite_backward_takes_g_at_any_address_and_one_token_at_any_stride(dtype):
+    from paper_2509_09679_b200.composite import composite_backward
+    n1, n2, tokens = 12, 256, 33
+    d = n1 * n2
+    p = Plan(n2, DEV)
+    p.set_angles(synth.angles(n2, "normal", 3).to(DEV))
+    params = synth.cayley_params(n1, 3, 0.1).to(DEV)
+    q1 = p.cayley(params, n1)
+    x, g = (synth.rows(tokens, d, "normal", s, dtype=dtype).to(DEV) for s in (4, 5))
+    odd = torch.empty(tokens * d + 1, dtype=dtype, device=DEV)[1:].view(tokens, d)
+    odd.copy_(g)
+    for a, b in zip(composite_backward(p, q1, params, x, g), composite_backward(p, q1, params, x, odd)):
+        assert torch.equal(a, b)
+    wide = torch.empty((tokens, d + 64), dtype=dtype, device=DEV)
+    wide[:, :d] = x
+    for a, b in zip(composite_backward(p, q1, params, x[:1], g[:1]), composite_backward(p, q1, params, wide[:1, :d], g[:1])):
+        assert torch.equal(a, b)
+
+
 @pytest.mark.parametrize("n1,scale", [(2, 1.0), (3, 50.0), (33, 0.5), (64, 5.0)])
 def test_cayley_and_its_gradient(n1, scale):
     """Sizes around a warp's width and large parameters (the pivots move)."""
