@@ -401,8 +401,11 @@ class Plan:
                 b.scales.data_ptr() if b.scales is not None else None, c.data_ptr(), b.rows)
         if a.kind == BFQ_F32 or b.kind == BFQ_F32:  # room to split fp32 operands in, where that helps
             size = self._c.bfq_dequant_gemm_workspace(self._h, a.rows, b.rows, a.k, a.kind, int(a.transposed), b.kind, int(b.transposed))
-            if size:
-                room = torch.empty(size + 256, dtype=torch.uint8, device=self.device)
+            try:
+                room = torch.empty(size + 256, dtype=torch.uint8, device=self.device) if size else None
+            except torch.OutOfMemoryError:
+                room = None  # the product does not need it
+            if room is not None:
                 _check(self._c.bfq_dequant_gemm_split(*args, (room.data_ptr() + 255) // 256 * 256, size, _stream(c)), "bfq_dequant_gemm_split")
                 return c
         _check(self._c.bfq_dequant_gemm(*args, _stream(c)), "bfq_dequant_gemm")

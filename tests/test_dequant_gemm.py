@@ -121,6 +121,24 @@ def test_operands_split_beforehand(ka, kb, ta, tb):
     assert torch.equal(out[0], out[1]) and p.device_status() == 0
 
 
+def test_fp32_operands_where_there_is_no_room_to_split_them(monkeypatch):
+    p = Plan(256, DEV)
+    A, a64, ea = operand("f32", 200, 4160, False, 950)
+    B, b64, eb = operand("f32", 136, 4160, False, 951)
+    split = p.dequant_gemm(A, B)
+    real, refused = torch.empty, []
+
+    def empty(*size, dtype=None, **kwargs):
+        if dtype == torch.uint8:
+            refused.append(size)
+            raise torch.OutOfMemoryError("no room")
+        return real(*size, dtype=dtype, **kwargs)
+
+    monkeypatch.setattr(torch, "empty", empty)
+    assert torch.equal(p.dequant_gemm(A, B), split) and len(refused) == 1
+    check(p, A, a64, ea, B, b64, eb)
+
+
 @pytest.mark.parametrize("ka", ["bf16", "codes2", "codes4", "codes8"])
 @pytest.mark.parametrize("kb", ["codes2", "codes4", "codes8"])
 @pytest.mark.parametrize("m,n,k", [(1, 16, 64), (8, 15, 192), (3, 4100, 1088), (9, 100, 4096), (64, 33, 64)])
