@@ -272,7 +272,8 @@ int bfq_cayley_backward(bfq_plan* plan, const float* params, int n1, const float
  *               a multiple of 128 and data 16-byte aligned.
  * K must be a multiple of 64; m, n are arbitrary.  All pointers are device pointers.  The products run on the tensor
  * cores in bf16 with fp32 accumulation: codes are exact, fp32 numbers are split into two bf16 terms (relative error
- * 2^-17 per element), bf16 numbers are exact.  Asynchronous on `stream`; allocates nothing; a bounded device-side
+ * 2^-17 per element), bf16 numbers are exact.  Two code operands that are both stored along K are an exact integer product
+ * times their scales while K < 2^17, whatever m and n.  Asynchronous on `stream`; allocates nothing; a bounded device-side
  * wait that runs out is reported by bfq_device_status.  Returns BFQ_OK, BFQ_ERR_NULL, BFQ_ERR_STRIDE (sizes, leading
  * dimensions, K not a multiple of 64), BFQ_ERR_ALIGN, BFQ_ERR_DTYPE (kind) or BFQ_ERR_CUDA.
  */

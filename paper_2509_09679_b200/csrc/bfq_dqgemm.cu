@@ -40,6 +40,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <type_traits>
+
 #include "bfq_n4096.cuh"
 #include "bfq_plan.h"
 #include "bfq_ptx.cuh"
@@ -920,13 +922,22 @@ k_dequant_gemm(const __grid_constant__ Params p, const __grid_constant__ CUtenso
 // CTAs in a chain of K blocks (one token, 4096 x 4096 at 2 bits: 17 - 25 us).  Here a CTA of eight warps takes 16 rows of B, each
 // warp every eighth part of K, and the partial sums are added in the order of the warps.  mma.sync m16n8k16 with the codes as
 // the 16-row operand straight from registers: a lane's 16 bytes of a row are its k values, in whatever order they come, as
-// long as the lanes that hold A's rows take the same ones.  Bound by the latency of one pass over the codes, not by the
-// (legacy) tensor path.
+// long as the lanes that hold A's rows take the same ones.  Two code operands are multiplied as integers (m16n8k32), so that a
+// row of C is the same exact number here and in the pair kernel's integer products.
+// What bounds it: on a small layer the latency of one pass; on a wide one the instructions that turn codes into bf16 pairs and
+// feed them to the m16n8k16 products, and with eight bf16 rows the reading of all of A for every 16 rows of B.  us, one row /
+// eight: 4096 x 4096 at 2 bits bf16 9.4 / 13.2, INT4 codes 7.7 / 7.8 as bf16 pairs -> 4.5 / 4.5 as integers; 28672 x 8192 bf16
+// 44 / 76, INT4 52 / 52 -> 16 / 16, INT8 53 / 54 -> 18 / 24 (its codes alone take 9).
 constexpr int kFewWarps = 8;
 
 __device__ __forceinline__ void mma_16816(float (&c)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b0, uint32_t b1) {
     asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
                  : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
+                 : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
+}
+__device__ __forceinline__ void mma_16832(int (&c)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b0, uint32_t b1) {
+    asm volatile("mma.sync.aligned.m16n8k32.row.col.s32.s8.s8.s32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
+                 : "+r"(c[0]), "+r"(c[1]), "+r"(c[2]), "+r"(c[3])
                  : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
 }
 // 16 bytes of codes -> 64 / KIND * 2 bf16 pairs in element order
@@ -952,16 +963,6 @@ __device__ __forceinline__ void codes_to_pairs(const uint4& raw, uint32_t (&o)[6
         }
     }
 }
-// 16 bytes of a row of A -> bf16 pairs in element order
-template <int KIND>
-__device__ __forceinline__ void row_to_pairs(const uint4& raw, uint32_t (&o)[KIND == BFQ_OP_BF16 ? 4 : 64 / KIND]) {
-    if constexpr (KIND == BFQ_OP_BF16) {
-        o[0] = raw.x, o[1] = raw.y, o[2] = raw.z, o[3] = raw.w;
-    } else {
-        codes_to_pairs<KIND>(raw, o);
-    }
-}
-
 // UK: kind of B's codes, VK: kind of A
 template <int UK, int VK>
 __global__ void __launch_bounds__(32 * kFewWarps) k_few_rows(const Operand u, const Operand v, float* __restrict__ c, int64_t ldc, int k, float alpha) {
@@ -970,7 +971,9 @@ __global__ void __launch_bounds__(32 * kFewWarps) k_few_rows(const Operand u, co
     constexpr int kVElems = VK == BFQ_OP_BF16 ? 8 : 128 / VK;           // of 16 bytes of A
     constexpr int kRound = kElems > kVElems ? kElems : kVElems;          // codes of B and elements of A taken together
     constexpr int kVLoads = kRound / kVElems, kULoads = kRound / kElems;
-    __shared__ float part[kFewWarps][8][16 + 1];
+    constexpr bool kInts = VK != BFQ_OP_BF16;                            // exact sums: K < 2^17
+    using Sum = typename std::conditional<kInts, int, float>::type;
+    __shared__ Sum part[kFewWarps][8][16 + 1];
     grid_dep_launch();
     grid_dep_wait();
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, q = lane & 3;
@@ -986,7 +989,7 @@ __global__ void __launch_bounds__(32 * kFewWarps) k_few_rows(const Operand u, co
     const int i0 = 8 * blockIdx.y;  // the MMA's eight columns
     const bool has_v = i0 + g < v.rows;
     const uint8_t* vrow = static_cast<const uint8_t*>(v.data) + int64_t(has_v ? i0 + g : 0) * (v.ld * kVBits / 8);
-    float acc[4] = {0.f, 0.f, 0.f, 0.f};
+    Sum acc[4] = {0, 0, 0, 0};
     // a lane's kRound elements of each row start at a multiple of kRound: inside K as a whole, or cut at a 16-byte piece
     auto piece = [&](const uint8_t* row, bool yes, int at, int bits) {
         return yes && at < k ? __ldg(reinterpret_cast<const uint4*>(row + int64_t(at) * bits / 8)) : make_uint4(0u, 0u, 0u, 0u);
@@ -1010,19 +1013,30 @@ __global__ void __launch_bounds__(32 * kFewWarps) k_few_rows(const Operand u, co
 #pragma unroll
             for (int i = 0; i < kULoads; ++i) now[h][i] = w[h][i];
         fetch(kl + kStride);
+        if constexpr (kInts) {
+            auto words = [](const uint4& r) { return reinterpret_cast<const uint32_t*>(&r); };
 #pragma unroll
-        for (int part_u = 0; part_u < kULoads; ++part_u) {
-            uint32_t a[64 / UK], b[64 / UK];
-            codes_to_pairs<UK>(now[0][part_u], a);
-            codes_to_pairs<UK>(now[1][part_u], b);
-            constexpr int kVPairs = kVElems / 2;
-            uint32_t xp[kVPairs];
+            for (int e = 0; e < kRound; e += 16) {  // sixteen codes of each row
+                uint32_t a[4], b[4], xi[4];
+                constexpr int kUWords = UK / 2, kVWords = VK / 2;
+                Int8Chunk<UK>::make(words(now[0][e / kElems]) + (e % kElems) / 16 * kUWords, a);
+                Int8Chunk<UK>::make(words(now[1][e / kElems]) + (e % kElems) / 16 * kUWords, b);
+                Int8Chunk<VK>::make(words(x[e / kVElems]) + (e % kVElems) / 16 * kVWords, xi);
+                mma_16832(acc, a[0], b[0], a[1], b[1], xi[0], xi[1]);
+                mma_16832(acc, a[2], b[2], a[3], b[3], xi[2], xi[3]);
+            }
+        } else {
 #pragma unroll
-            for (int s = 0; s < kElems / 4; ++s) {
-                const int e = part_u * kElems + 4 * s;  // element of the round
-                if (e % kVElems == 0) row_to_pairs<VK>(x[e / kVElems], xp);
-                const int xi = (e % kVElems) / 2;
-                mma_16816(acc, a[2 * s], b[2 * s], a[2 * s + 1], b[2 * s + 1], xp[xi], xp[xi + 1]);
+            for (int part_u = 0; part_u < kULoads; ++part_u) {
+                uint32_t a[64 / UK], b[64 / UK];
+                codes_to_pairs<UK>(now[0][part_u], a);
+                codes_to_pairs<UK>(now[1][part_u], b);
+#pragma unroll
+                for (int s = 0; s < kElems / 4; ++s) {
+                    const int e = part_u * kElems + 4 * s;  // element of the round: half of a 16-byte piece of A
+                    const uint4& xe = x[e / 8];
+                    mma_16816(acc, a[2 * s], b[2 * s], a[2 * s + 1], b[2 * s + 1], e % 8 == 0 ? xe.x : xe.z, e % 8 == 0 ? xe.y : xe.w);
+                }
             }
         }
     }
@@ -1032,12 +1046,14 @@ __global__ void __launch_bounds__(32 * kFewWarps) k_few_rows(const Operand u, co
     for (int e = threadIdx.x; e < 8 * 16; e += 32 * kFewWarps) {
         const int i = i0 + (e >> 4), j = e & 15;
         if (i >= v.rows || j0 + j >= u.rows) continue;
-        float sum = 0.f;
+        Sum sum = 0;
 #pragma unroll
         for (int x = 0; x < kFewWarps; ++x) sum += part[x][e >> 4][j];
         float scale = alpha * __half2float(__ushort_as_half(__ldg(u.scales + j0 + j)));
         if (is_codes(VK)) scale *= __half2float(__ushort_as_half(__ldg(v.scales + i)));
-        c[int64_t(i) * ldc + j0 + j] = sum * scale;
+        float value = sum;
+        if constexpr (kInts) value = __int2float_rn(sum) * (1.f / float(1 << (Int8Chunk<UK>::kShift + Int8Chunk<VK>::kShift)));
+        c[int64_t(i) * ldc + j0 + j] = value * scale;
     }
 }
 
@@ -1130,7 +1146,7 @@ static Shape choose_shape(int64_t m, int64_t n, int kblocks, int term_pairs, int
 // 1024 x 1024 at 2 bits 7.7 -> 2.5, 4096 x 4096 25 -> 7.0, 28672 x 8192 104 -> 44; 8 rows 8.1 -> 3.0, 26 -> 9.4, 105 -> 75).  More
 // rows are more passes, worth it while they are small together.
 static bool use_few_rows(const Operand& u, const Operand& v, int64_t k) {
-    if (!is_codes(u.kind) || u.transposed || v.kind == BFQ_OP_F32 || v.transposed || k >= (1 << 30)) return false;
+    if (!is_codes(u.kind) || u.transposed || v.kind == BFQ_OP_F32 || v.transposed || k >= (is_codes(v.kind) ? 1 << 17 : 1 << 30)) return false;
     const int64_t passes = (int64_t(v.rows) + 7) / 8;
     return passes == 1 || (passes <= 8 && passes * u.rows * k <= int64_t(1) << 25);
 }

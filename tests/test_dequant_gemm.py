@@ -150,6 +150,59 @@ def test_a_few_rows_against_codes(ka, kb, m, n, k):
     check(p, A, a64, ea, B, b64, eb, alpha=-1.5)
 
 
+@pytest.mark.parametrize("abits,bbits", [(8, 8), (8, 2), (4, 4), (2, 8), (4, 8), (2, 2)])
+def test_a_row_of_codes_times_codes_is_the_same_in_any_batch(abits, bbits):
+    """An exact integer product: the same bits whether a few rows or many are multiplied, also where the sums pass 2^24."""
+    k, n, m = 16384, 130, 200
+    g = torch.Generator().manual_seed(5)
+    a, b = (torch.randint(0, 256, (r, k * bits // 8), dtype=torch.uint8, generator=g).to(DEV) for r, bits in ((m, abits), (n, bbits)))
+    if abits == bbits == 8:  # codes of 64 .. 127
+        a, b = (a & 0x3F) | 0x40, (b & 0x3F) | 0x40
+    sa, sb = (torch.rand(r, generator=g).half().to(DEV) for r in (m, n))
+    p = Plan(256, DEV)
+    B = GemmOperand(b, sb, bbits)
+    whole = p.dequant_gemm(GemmOperand(a, sa, abits), B)
+    from paper_2509_09679_b200.calibrate import unpack_codes
+    exact = (unpack_codes(a, abits).double() @ unpack_codes(b, bbits).double().t()) * sa.double().unsqueeze(1) * sb.double()
+    assert ((whole.double() - exact).abs() <= 2.0 ** -22 * exact.abs()).all()  # three roundings of an exact sum
+    for few in (1, 8, 30):
+        assert torch.equal(whole[:few], p.dequant_gemm(GemmOperand(a[:few], sa[:few].contiguous(), abits), B)), few
+
+
+@pytest.mark.parametrize("k", [2 ** 17 - 64, 2 ** 17])
+@pytest.mark.parametrize("m", [3, 70])
+@pytest.mark.parametrize("bits,low", [(8, 0x80), (4, 0x88), (2, 0xAA)])
+def test_lowest_codes_up_to_where_integers_end(k, m, bits, low):
+    """The largest sums the integer path takes, and the first K that it does not take (there the sums are multiples of
+    4^(bits - 1), exact in fp32 up to 2^24 of them)."""
+    a, b = (torch.full((r, k * bits // 8), low, dtype=torch.uint8, device=DEV) for r in (m, 33))
+    one = lambda r: torch.ones(r, dtype=torch.float16, device=DEV)
+    p = Plan(256, DEV)
+    c = p.dequant_gemm(GemmOperand(a, one(m), bits), GemmOperand(b, one(33), bits))
+    assert (c == float(k) * 4.0 ** (bits - 1)).all() and p.device_status() == 0
+
+
+@pytest.mark.parametrize("n", [1024, 1040])
+def test_either_side_of_the_rule_for_a_few_rows(n):
+    """64 rows are eight passes up to 8 n K = 2^25 and tiles above."""
+    p = Plan(256, DEV)
+    A, a64, ea = operand("bf16", 64, 4096, False, 960)
+    B, b64, eb = operand("codes4", n, 4096, False, 961)
+    check(p, A, a64, ea, B, b64, eb)
+
+
+@pytest.mark.parametrize("m,n", [(200, 136), (4096, 2048)])
+def test_either_side_of_the_rule_for_splitting_beforehand(m, n):
+    """The last K at which an fp32 operand is split in the tiles and the first at which it is split by a pass of its own."""
+    from paper_2509_09679_b200.binding import lib
+    p = Plan(256, DEV)
+    first = next(k for k in range(128, 1 << 14, 64) if lib().bfq_dequant_gemm_workspace(p._h, m, n, k, 0, 0, 1, 0) > 0)
+    for k in (first - 64, first):
+        A, a64, ea = operand("f32", m, k, False, 970)
+        B, b64, eb = operand("bf16", n, k, False, 971)
+        check(p, A, a64, ea, B, b64, eb)
+
+
 def test_argument_validation():
     from paper_2509_09679_b200 import BfqError
     p = Plan(256, DEV)
