@@ -703,7 +703,7 @@ int bfq_cayley(bfq_plan* plan, const float* params, int n1, float* q1, void* str
     if ((reinterpret_cast<uintptr_t>(params) & 3u) != 0 || (reinterpret_cast<uintptr_t>(q1) & 3u) != 0) return BFQ_ERR_ALIGN;
     DeviceGuard guard(plan->device);
     if (guard.err != cudaSuccess) return cuda_fail(plan, guard.err);
-    cudaError_t e = cayley_launch(params, n1, q1, static_cast<cudaStream_t>(stream));
+    cudaError_t e = cayley_launch(plan, params, n1, q1, static_cast<cudaStream_t>(stream));
     return e == cudaSuccess ? BFQ_OK : cuda_fail(plan, e);
 }
 
@@ -777,7 +777,7 @@ int bfq_cayley_backward(bfq_plan* plan, const float* params, int n1, const float
         if ((reinterpret_cast<uintptr_t>(p) & 3u) != 0) return BFQ_ERR_ALIGN;
     DeviceGuard guard(plan->device);
     if (guard.err != cudaSuccess) return cuda_fail(plan, guard.err);
-    cudaError_t e = cayley_backward_launch(params, n1, q1, dq1, dparams, static_cast<cudaStream_t>(stream));
+    cudaError_t e = cayley_backward_launch(plan, params, n1, q1, dq1, dparams, static_cast<cudaStream_t>(stream));
     return e == cudaSuccess ? BFQ_OK : cuda_fail(plan, e);
 }
 

@@ -11,6 +11,8 @@
 // one block barrier per column; every warp finds the pivot by itself; a row is 2 n1 + 1 doubles, so that the lanes that read
 // down a column fall into different banks, and a thread's loads are all issued before its stores.  Four barriers and a serial
 // pivot search per column took 96 us for n1 = 40; now 35 us, and the gradient 24 us (76 with a solve of its own).
+#include "../../include/bfq.h"
+
 #include <cuda_runtime.h>
 
 #include "bfq_fast.h"
@@ -169,24 +171,30 @@ __global__ void __launch_bounds__(kThreads) k_cayley_backward(const float* __res
 
 }  // namespace cay
 
-template <class K>
-static cudaError_t allow_smem(K kern, size_t smem) {
-    return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
+// shared memory for n1 rows, and the limit of every n1: set once per device (a limit per call would be pulled away by another
+// thread's call with a smaller n1)
+static constexpr size_t cayley_smem(int n1) { return sizeof(double) * 2 * n1 * cay::pitch(n1); }
+static constexpr size_t cayley_backward_smem(int n1) { return cayley_smem(n1) + sizeof(double) * 2 * n1 * n1; }
+static cudaError_t allow_smem(int device) {
+    static bool allowed[kMaxDevices] = {false};
+    if (allowed[device]) return cudaSuccess;
+    cudaError_t e = cudaFuncSetAttribute(cay::k_cayley, cudaFuncAttributeMaxDynamicSharedMemorySize, int(cayley_smem(BFQ_MAX_N1)));
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(cay::k_cayley_backward, cudaFuncAttributeMaxDynamicSharedMemorySize, int(cayley_backward_smem(BFQ_MAX_N1)));
+    allowed[device] = e == cudaSuccess;
+    return e;
 }
 
-cudaError_t cayley_launch(const float* params, int n1, float* q1, cudaStream_t st) {
-    const size_t smem = sizeof(double) * 2 * n1 * cay::pitch(n1);
-    cudaError_t e = allow_smem(cay::k_cayley, smem);
+cudaError_t cayley_launch(const bfq_plan* plan, const float* params, int n1, float* q1, cudaStream_t st) {
+    cudaError_t e = allow_smem(plan->device);
     if (e != cudaSuccess) return e;
-    cay::k_cayley<<<1, cay::kThreads, smem, st>>>(params, n1, q1);
+    cay::k_cayley<<<1, cay::kThreads, cayley_smem(n1), st>>>(params, n1, q1);
     return cudaGetLastError();
 }
 
-cudaError_t cayley_backward_launch(const float* params, int n1, const float* q1, const float* dq1, float* dparams, cudaStream_t st) {
-    const size_t smem = sizeof(double) * (2 * n1 * cay::pitch(n1) + 2 * n1 * n1);
-    cudaError_t e = allow_smem(cay::k_cayley_backward, smem);
+cudaError_t cayley_backward_launch(const bfq_plan* plan, const float* params, int n1, const float* q1, const float* dq1, float* dparams, cudaStream_t st) {
+    cudaError_t e = allow_smem(plan->device);
     if (e != cudaSuccess) return e;
-    cay::k_cayley_backward<<<1, cay::kThreads, smem, st>>>(params, n1, q1, dq1, dparams);
+    cay::k_cayley_backward<<<1, cay::kThreads, cayley_backward_smem(n1), st>>>(params, n1, q1, dq1, dparams);
     return cudaGetLastError();
 }
 

@@ -19,6 +19,8 @@
 // cycle).  Composed from a dense product on permuted copies, the butterfly backward on 40 rows per token, a forward in fp32
 // and another dense product it took about 1000 us for 2048 tokens, and G' went through bf16 in between; this kernel
 // takes 145 us (191 us with scalar multiply-adds).
+#include "../../include/bfq.h"
+
 #include <cuda_runtime.h>
 
 #include "bfq_fast.h"
@@ -27,6 +29,8 @@
 
 namespace bfq {
 namespace cbw {
+
+constexpr int kBackwardSmem = 227 * 1024;  // dynamic shared memory of a CTA at most
 
 struct Params {
     const float2* tw;
@@ -240,13 +244,20 @@ static cudaError_t launch(const bfq_plan* plan, Params p, float* dtheta, float* 
     if (floats < size_t(kThreads)) floats = kThreads;
     const size_t smem = floats * sizeof(float);
     auto kern = k_composite_backward<L, TILES>;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
-    if (e != cudaSuccess) return e;
-    int occ = 0;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, kThreads, smem);
-    if (e != cudaSuccess) return e;
+    // as for the forward kernel: the limit of every n1, and CTAs per SM for each
+    static int8_t per_sm[kMaxDevices][BFQ_MAX_N1 + 1] = {{0}};
+    int8_t& occ = per_sm[plan->device][p.n1];
+    cudaError_t e = cudaSuccess;
+    if (occ == 0) {
+        e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kBackwardSmem);
+        if (e != cudaSuccess) return e;
+        int o = 0;
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o, kern, kThreads, smem);
+        if (e != cudaSuccess) return e;
+        occ = static_cast<int8_t>(o > 0 ? o : 1);
+    }
     const int count = G::kAngles + p.n1 * p.n1;
-    int64_t grid = int64_t(plan->sm_count) * (occ > 0 ? occ : 1);
+    int64_t grid = int64_t(plan->sm_count) * occ;
     if (grid > p.rows) grid = p.rows;
     if (grid * count > int64_t(plan->partial_floats)) grid = int64_t(plan->partial_floats) / count;
     if (grid < 1) return cudaErrorInvalidValue;
@@ -271,7 +282,7 @@ static cudaError_t launch(const bfq_plan* plan, const Params& p, float* dtheta, 
 bool composite_backward_available(const bfq_plan* plan, int n1) {
     if (plan->n < 128 || plan->n > 1024) return false;
     const size_t n1p = (n1 + 7) & ~7;
-    return (size_t(3) * n1 * (plan->n + 4) + size_t(n1) * n1p) * sizeof(float) <= 227 * 1024;
+    return (size_t(3) * n1 * (plan->n + 4) + size_t(n1) * n1p) * sizeof(float) <= cbw::kBackwardSmem;
 }
 
 cudaError_t composite_backward_launch(bfq_plan* plan, const float* q1, int n1, const void* x, int xt, const void* g, int gt, int64_t rows,

@@ -6,6 +6,8 @@
 // The kernel for every shape does one stage per barrier, element by element: 32768 tokens of 40 x 128 at INT2 took
 // 2.07 ms there and take 0.93 ms here (40000 of 12 x 256: 1.43 -> 0.62 ms, 18000 of 7 x 1024: 1.70 -> 0.47 ms; one token 24 us
 // with the call's host side either way).
+#include "../../include/bfq.h"
+
 #include <cuda_runtime.h>
 
 #include "bfq_comp_walk.cuh"
@@ -14,6 +16,8 @@
 
 namespace bfq {
 namespace cbw {
+
+constexpr int kForwardSmem = 226 * 1024;  // dynamic shared memory of a CTA at most
 
 struct ForwardParams {
     const float2* tw;
@@ -84,12 +88,19 @@ template <int L>
 static cudaError_t launch_forward(const bfq_plan* plan, const ForwardParams& p, cudaStream_t st) {
     const size_t smem = (size_t(2) * p.n1 * Geo<L>::kPitch + size_t(p.n1) * ((p.n1 + 7) & ~7)) * sizeof(float);
     auto kern = k_composite_forward<L>;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
-    if (e != cudaSuccess) return e;
-    int occ = 0;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, kThreads, smem);
-    if (e != cudaSuccess) return e;
-    const int64_t cap = int64_t(plan->sm_count) * (occ > 0 ? occ : 1);
+    // the limit of every n1, set once (a limit per call would be pulled away by another thread's call with a smaller n1); CTAs
+    // per SM for each n1
+    static int8_t per_sm[kMaxDevices][BFQ_MAX_N1 + 1] = {{0}};
+    int8_t& occ = per_sm[plan->device][p.n1];
+    if (occ == 0) {
+        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kForwardSmem);
+        if (e != cudaSuccess) return e;
+        int o = 0;
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o, kern, kThreads, smem);
+        if (e != cudaSuccess) return e;
+        occ = static_cast<int8_t>(o > 0 ? o : 1);
+    }
+    const int64_t cap = int64_t(plan->sm_count) * occ;
     kern<<<int(p.rows < cap ? p.rows : cap), kThreads, smem, st>>>(p);
     return cudaGetLastError();
 }
@@ -98,7 +109,7 @@ static cudaError_t launch_forward(const bfq_plan* plan, const ForwardParams& p, 
 
 bool composite_forward_available(const bfq_plan* plan, int n1) {
     const size_t n1p = (n1 + 7) & ~7;
-    return plan->n >= 128 && plan->n <= 1024 && (size_t(2) * n1 * (plan->n + 4) + size_t(n1) * n1p) * sizeof(float) <= 226 * 1024;
+    return plan->n >= 128 && plan->n <= 1024 && (size_t(2) * n1 * (plan->n + 4) + size_t(n1) * n1p) * sizeof(float) <= cbw::kForwardSmem;
 }
 
 cudaError_t composite_forward_launch(const bfq_plan* plan, const float* q1, int n1, const void* x, int xt, int64_t rows, int64_t ldx, void* y, int yt,

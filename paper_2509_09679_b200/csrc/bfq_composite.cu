@@ -9,6 +9,8 @@
 // This file holds the kernels that work for every (n1 <= 64, n2 <= 1024, n1 n2 <= 16384);
 // the tensor-core kernels for 40 x 128 live in bfq_comp5120d.cu (both factors as MMAs) and bfq_comp5120.cu (fp32
 // butterfly + MMA dense factor) and must agree with these; the Cayley transform in bfq_cayley.cu, the backward in bfq_compbwd.cu.
+#include "../../include/bfq.h"
+
 #include <cuda_runtime.h>
 
 #include "bfq_fast.h"
@@ -129,8 +131,13 @@ cudaError_t composite_generic_launch(const bfq_plan* plan, const float* q1, int 
     p.codes = codes, p.scales = scales, p.bits = bits, p.rows = rows, p.inverse = inverse ? 1 : 0;
     const int d = n1 * plan->n, n1p = (n1 + 7) & ~7;
     const size_t smem = sizeof(float) * (size_t(2) * d + size_t(n1p) * n1);
-    cudaError_t e = cudaFuncSetAttribute(comp::k_composite_generic, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
-    if (e != cudaSuccess) return e;
+    static bool allowed[kMaxDevices] = {false};
+    if (!allowed[plan->device]) {  // the limit of every shape
+        constexpr int most = int(sizeof(float)) * (2 * BFQ_COMPOSITE_MAX_D + BFQ_MAX_N1 * BFQ_MAX_N1);
+        cudaError_t e = cudaFuncSetAttribute(comp::k_composite_generic, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
+        if (e != cudaSuccess) return e;
+        allowed[plan->device] = true;
+    }
     const int64_t cap = int64_t(plan->sm_count) * 4;
     const int grid = int(rows < cap ? rows : cap);
     comp::k_composite_generic<<<grid, comp::kThreads, smem, st>>>(p);

@@ -101,8 +101,8 @@ cudaError_t inv4096_launch(bfq_plan* plan, const void* y, int64_t rows, int64_t 
 bool composite_forward_available(const bfq_plan* plan, int n1);
 cudaError_t composite_forward_launch(const bfq_plan* plan, const float* q1, int n1, const void* x, int xt, int64_t rows, int64_t ldx, void* y, int yt,
                                      int64_t ldy, int bits, uint8_t* codes, uint16_t* scales, cudaStream_t st);
-cudaError_t cayley_launch(const float* params, int n1, float* q1, cudaStream_t st);
-cudaError_t cayley_backward_launch(const float* params, int n1, const float* q1, const float* dq1, float* dparams, cudaStream_t st);
+cudaError_t cayley_launch(const bfq_plan* plan, const float* params, int n1, float* q1, cudaStream_t st);
+cudaError_t cayley_backward_launch(const bfq_plan* plan, const float* params, int n1, const float* q1, const float* dq1, float* dparams, cudaStream_t st);
 // dx (may be null, type of x), dtheta of Q2 and dQ1 for upstream rows g; ld: row stride of x, g and dx
 bool composite_backward_available(const bfq_plan* plan, int n1);
 cudaError_t composite_backward_launch(bfq_plan* plan, const float* q1, int n1, const void* x, int xt, const void* g, int gt, int64_t rows,

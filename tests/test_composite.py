@@ -482,3 +482,34 @@ def test_tensor_core_composite_5120_int8(rows):
     assert p.device_status() == 0 and codes.intact() and scales.intact()
     frac = _check_tf32_quant(codes.view, scales.view, y_ref, tol, "composite int8", bits=8)
     assert frac <= 0.2  # codes are 16 times finer than INT4: the TF32 error moves proportionally more of them by one
+
+
+def test_sizes_from_several_threads():
+    """Each thread with a plan, a stream and an n1 of its own: no call may change what another one may launch with."""
+    import threading
+    from paper_2509_09679_b200.composite import composite_backward
+    failed = []
+
+    def work(n1, n2):
+        try:
+            with torch.cuda.stream(torch.cuda.Stream(DEV)):
+                p = Plan(n2, DEV)
+                p.set_angles(synth.angles(n2, "normal", 3, DEV))
+                params = synth.cayley_params(n1, 3, 0.1, DEV)
+                x, g = (synth.rows(3, n1 * n2, "normal", s, device=DEV) for s in (4, 5))
+                ref = None
+                for _ in range(200):
+                    q1 = p.cayley(params, n1)
+                    out = (p.composite_forward(q1, x), p.composite_inverse(q1, x), *composite_backward(p, q1, params, x, g))
+                    ref = ref or [t.clone() for t in out]
+                    assert all(torch.equal(a, b) for a, b in zip(ref, out))
+        except Exception as e:  # noqa: BLE001
+            failed.append(f"{n1} x {n2}: {e}")
+
+    threads = [threading.Thread(target=work, args=a) for a in ((64, 128), (2, 128), (33, 128), (5, 128))]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    torch.cuda.synchronize()
+    assert not failed, failed
