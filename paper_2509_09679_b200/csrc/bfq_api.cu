@@ -329,6 +329,39 @@ int bfq_set_angles(bfq_plan* plan, const float* theta, void* stream) {
     return BFQ_OK;
 }
 
+// bfq_forward after the checks, on the current device
+static int forward_rows(bfq_plan* plan, const void* x, int xt, int64_t rows, int64_t ldx, void* y, int yt, int64_t ldy, cudaStream_t st) {
+    if (xt == BFQ_BF16 && yt == BFQ_BF16 && x != y && rows < (int64_t(1) << 31) && !env_flag("BFQ_GENERIC_ONLY") &&
+        fwdq4096_available(plan)) {
+        cudaError_t e = fwdq4096_launch(plan, x, rows, ldx, false, nullptr, nullptr, y, ldy,
+                                        st);
+        return e == cudaSuccess ? BFQ_OK : cuda_fail(plan, e);
+    }
+    if (xt == BFQ_F32 && yt == BFQ_F32 && x != y && rows < (int64_t(1) << 31) && !env_flag("BFQ_GENERIC_ONLY") &&
+        fwdq4096_available(plan)) {  // fp32 rows in and out on the tuned kernel
+        cudaError_t e = fwdq4096_launch_f32(plan, x, rows, ldx, 0, nullptr, nullptr, y, ldy, st);
+        return e == cudaSuccess ? BFQ_OK : cuda_fail(plan, e);
+    }
+    if (xt == BFQ_F32 && yt == BFQ_F32 && x != y && rows < (int64_t(1) << 31) && !env_flag("BFQ_GENERIC_ONLY") &&
+        fwdq8192_available(plan)) {
+        cudaError_t e = fwdq8192_launch_f32(plan, x, rows, ldx, 0, nullptr, nullptr, y, ldy, st);
+        return e == cudaSuccess ? BFQ_OK : cuda_fail(plan, e);
+    }
+    if (xt == BFQ_BF16 && yt == BFQ_BF16 && x != y && rows < (int64_t(1) << 31) && !env_flag("BFQ_GENERIC_ONLY") &&
+        fwdq8192_available(plan)) {
+        cudaError_t e = fwdq8192_launch_bf16(plan, x, rows, ldx, y, ldy, st);
+        return e == cudaSuccess ? BFQ_OK : cuda_fail(plan, e);
+    }
+    if (xt == yt && x != y && ldy == plan->n && use_short_rows(plan, rows, 0)) {
+        cudaError_t e = fwdq_short_launch(plan, x, xt == BFQ_F32, rows, ldx, 0, nullptr, nullptr, y, st);
+        return e == cudaSuccess ? BFQ_OK : cuda_fail(plan, e);
+    }
+    GenericParams p{};
+    p.tw = plan->tw, p.x = x, p.xt = xt, p.ldx = ldx, p.y = y, p.yt = yt, p.ldy = ldy, p.rows = rows;
+    cudaError_t e = launch_generic<kModeForward>(plan, p, st);
+    return e == cudaSuccess ? BFQ_OK : cuda_fail(plan, e);
+}
+
 int bfq_forward(bfq_plan* plan, const void* x, bfq_dtype xt, int64_t rows, int64_t ldx, void* y, bfq_dtype yt,
                 int64_t ldy, void* stream) {
     if (plan == nullptr) return BFQ_ERR_NULL;
@@ -339,35 +372,7 @@ int bfq_forward(bfq_plan* plan, const void* x, bfq_dtype xt, int64_t rows, int64
     if (rows == 0) return BFQ_OK;
     DeviceGuard guard(plan->device);
     if (guard.err != cudaSuccess) return cuda_fail(plan, guard.err);
-    if (xt == BFQ_BF16 && yt == BFQ_BF16 && x != y && rows < (int64_t(1) << 31) && !env_flag("BFQ_GENERIC_ONLY") &&
-        fwdq4096_available(plan)) {
-        cudaError_t e = fwdq4096_launch(plan, x, rows, ldx, false, nullptr, nullptr, y, ldy,
-                                        static_cast<cudaStream_t>(stream));
-        return e == cudaSuccess ? BFQ_OK : cuda_fail(plan, e);
-    }
-    if (xt == BFQ_F32 && yt == BFQ_F32 && x != y && rows < (int64_t(1) << 31) && !env_flag("BFQ_GENERIC_ONLY") &&
-        fwdq4096_available(plan)) {  // fp32 rows in and out on the tuned kernel
-        cudaError_t e = fwdq4096_launch_f32(plan, x, rows, ldx, 0, nullptr, nullptr, y, ldy, static_cast<cudaStream_t>(stream));
-        return e == cudaSuccess ? BFQ_OK : cuda_fail(plan, e);
-    }
-    if (xt == BFQ_F32 && yt == BFQ_F32 && x != y && rows < (int64_t(1) << 31) && !env_flag("BFQ_GENERIC_ONLY") &&
-        fwdq8192_available(plan)) {
-        cudaError_t e = fwdq8192_launch_f32(plan, x, rows, ldx, 0, nullptr, nullptr, y, ldy, static_cast<cudaStream_t>(stream));
-        return e == cudaSuccess ? BFQ_OK : cuda_fail(plan, e);
-    }
-    if (xt == BFQ_BF16 && yt == BFQ_BF16 && x != y && rows < (int64_t(1) << 31) && !env_flag("BFQ_GENERIC_ONLY") &&
-        fwdq8192_available(plan)) {
-        cudaError_t e = fwdq8192_launch_bf16(plan, x, rows, ldx, y, ldy, static_cast<cudaStream_t>(stream));
-        return e == cudaSuccess ? BFQ_OK : cuda_fail(plan, e);
-    }
-    if (xt == yt && x != y && ldy == plan->n && use_short_rows(plan, rows, 0)) {
-        cudaError_t e = fwdq_short_launch(plan, x, xt == BFQ_F32, rows, ldx, 0, nullptr, nullptr, y, static_cast<cudaStream_t>(stream));
-        return e == cudaSuccess ? BFQ_OK : cuda_fail(plan, e);
-    }
-    GenericParams p{};
-    p.tw = plan->tw, p.x = x, p.xt = xt, p.ldx = ldx, p.y = y, p.yt = yt, p.ldy = ldy, p.rows = rows;
-    cudaError_t e = launch_generic<kModeForward>(plan, p, static_cast<cudaStream_t>(stream));
-    return e == cudaSuccess ? BFQ_OK : cuda_fail(plan, e);
+    return forward_rows(plan, x, xt, rows, ldx, y, yt, ldy, static_cast<cudaStream_t>(stream));
 }
 
 static int forward_quant_impl(bfq_plan* plan, const void* x, int xt, int64_t rows, int64_t ldx, int bits,
@@ -434,8 +439,12 @@ static int forward_quant_impl(bfq_plan* plan, const void* x, int xt, int64_t row
         e = fwdq8192_launch(plan, x, rows, ldx, bits, codes, scales, static_cast<cudaStream_t>(stream));
         return e == cudaSuccess ? BFQ_OK : cuda_fail(plan, e);
     }
-    if (hist == nullptr && y == nullptr && use_short_rows(plan, rows, 0)) {
-        e = fwdq_short_launch(plan, x, xt == BFQ_F32, rows, ldx, bits, codes, scales, nullptr, static_cast<cudaStream_t>(stream));
+    if (hist == nullptr && use_short_rows(plan, rows, 0)) {
+        // rows kept beside the codes: both the bits of the calls that give one of them alone.  In the input's type they come from
+        // the same pass, else (or over the input) from a second one.
+        const bool one_pass = y != nullptr && yt == xt && y != x;
+        e = fwdq_short_launch(plan, x, xt == BFQ_F32, rows, ldx, bits, codes, scales, one_pass ? y : nullptr, static_cast<cudaStream_t>(stream));
+        if (e == cudaSuccess && y != nullptr && !one_pass) return forward_rows(plan, x, xt, rows, ldx, y, yt, plan->n, static_cast<cudaStream_t>(stream));
         return e == cudaSuccess ? BFQ_OK : cuda_fail(plan, e);
     }
     GenericParams p{};

@@ -30,8 +30,8 @@ cudaError_t fwdq4096_launch_stats(const bfq_plan* plan, const void* x, int64_t r
                                   uint16_t* scales, unsigned long long* hist, float* rowstats, cudaStream_t st);
 
 cudaError_t fwdq4096_prep_angles(const bfq_plan* plan, const float* theta, cudaStream_t st);
-// rows of 128 .. 2048 elements: several as one of 4096 on the same kernel.  bits = 2, 4, 8: codes + scales; bits = 0: the
-// rotated rows, contiguous, in the type of x
+// rows of 128 .. 2048 elements: several as one of 4096 on the same kernel.  bits = 2, 4, 8: codes + scales, and
+// the rows if y is not null; bits = 0: the rows alone.  Rows are contiguous, in the type of x
 bool fwdq_short_available(const bfq_plan* plan);
 cudaError_t fwdq_short_launch(const bfq_plan* plan, const void* x, bool f32, int64_t rows, int64_t ldx, int bits, uint8_t* codes,
                               uint16_t* scales, void* y, cudaStream_t st);

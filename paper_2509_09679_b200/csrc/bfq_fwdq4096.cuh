@@ -159,7 +159,8 @@ enum : int { kOutInt4 = 0, kOutBf16 = 1, kOutInt4Stats = 2, kOutInt2 = 3, kOutIn
 // codes + scales + the second and fourth moment of every rotated row (`yout` then points to float [rows][2]) + the
 // tensor-wide counts of the 16 code values added to `hist`, or INT2 / INT8 codes + scales.
 // STEP: group g passes its token to group (g + STEP) % G, so gcd(STEP, G) groups rotate at a time (0: no tokens).
-// ROWS (code outputs only): the rotated rows are written as well, in bf16, to `yout` (weight folding that keeps W Q^T).
+// ROWS (code outputs only): the rotated rows are written as well, in the type of the input, to `yout` (weight folding that
+// keeps W Q^T).
 // IN_F32: the rows are fp32 (16 KB each): one input slot per group instead of two, re-armed as soon as the group has
 // read it (after the second regrouping's barrier), so the load still has most of a row's time to arrive.
 // SUB: rows of n = 4096 >> SUB elements.  Q on 2^SUB consecutive rows is a transform of 4096 elements whose stages from
@@ -358,12 +359,13 @@ k_fwdq4096(const __grid_constant__ CUtensorMap tmap, const float* __restrict__ i
         }
 
         static_assert(!ROWS || OUT == kOutInt4 || OUT == kOutInt2 || OUT == kOutInt8, "rows beside codes only");
-        static_assert(SUB == 0 || (kTmem && !ROWS && OUT != kOutInt4Stats), "not built for short rows");
+        static_assert(SUB == 0 || (kTmem && OUT != kOutInt4Stats), "not built for short rows");
+        static_assert(!(ROWS && IN_F32 && SUB == 0), "not built for fp32 rows of 4096");
         // elements of this row that exist; thread t's pair of register m is 2t + 256m, +1
         const int64_t left = elems - static_cast<int64_t>(row) * kN;
         const int lim = SUB == 0 || left >= kN ? kN : static_cast<int>(left);
         auto there = [&](int m) { return SUB == 0 || 2 * t + 256 * m < lim; };
-        if constexpr (OUT == kOutBf16 || ROWS) {
+        if constexpr (OUT == kOutBf16 || (ROWS && !IN_F32)) {
             // thread t holds elements 2t + 256m, +1: one 32-bit word of the bf16 row per packed register
             uint32_t* out = reinterpret_cast<uint32_t*>(yout + static_cast<int64_t>(row) * ldy) + t;
 #pragma unroll
@@ -374,7 +376,7 @@ k_fwdq4096(const __grid_constant__ CUtensorMap tmap, const float* __restrict__ i
                 if (there(m)) out[128 * m] = *reinterpret_cast<const uint32_t*>(&v);
             }
         }
-        if constexpr (OUT == kOutF32) {
+        if constexpr (OUT == kOutF32 || (ROWS && IN_F32)) {
             // thread t holds elements 2t + 256m, +1: one 64-bit word of the fp32 row per packed register
             u64* out = reinterpret_cast<u64*>(reinterpret_cast<float*>(yout) + static_cast<int64_t>(row) * ldy) + t;
 #pragma unroll

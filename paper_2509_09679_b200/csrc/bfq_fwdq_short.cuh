@@ -19,22 +19,21 @@ static cudaError_t fwdq_short_launch(const bfq_plan* plan, const void* x, bool f
     const int type = f32 ? kF32 : kBF16;
     const Again again{x, ldx, type, plan->tw, false, 12 - SUB, elems, bits, y, type, codes, scales};
     using namespace f4k;
-    auto go = [&](auto out, auto in_f32) {
-        return launch_variant<4, 32, 2, kButterfly, decltype(out)::value, false, decltype(in_f32)::value, SUB>(plan, tmap, joint, codes, scales, y,
-                                                                                                    kN, st, nullptr, elems, again);
+    auto go = [&](auto out, auto in_f32, auto rows_too) {
+        return launch_variant<4, 32, 2, kButterfly, decltype(out)::value, decltype(rows_too)::value, decltype(in_f32)::value, SUB>(
+            plan, tmap, joint, codes, scales, y, kN, st, nullptr, elems, again);
     };
-    if (f32) {
-        const std::true_type in{};
-        if (bits == 0) return go(std::integral_constant<int, kOutF32>(), in);
-        if (bits == 2) return go(std::integral_constant<int, kOutInt2>(), in);
-        if (bits == 4) return go(std::integral_constant<int, kOutInt4>(), in);
-        return go(std::integral_constant<int, kOutInt8>(), in);
-    }
-    const std::false_type in{};
-    if (bits == 0) return go(std::integral_constant<int, kOutBf16>(), in);
-    if (bits == 2) return go(std::integral_constant<int, kOutInt2>(), in);
-    if (bits == 4) return go(std::integral_constant<int, kOutInt4>(), in);
-    return go(std::integral_constant<int, kOutInt8>(), in);
+    auto of_type = [&](auto in_f32) {
+        constexpr int kRowsOut = decltype(in_f32)::value ? kOutF32 : kOutBf16;
+        if (bits == 0) return go(std::integral_constant<int, kRowsOut>(), in_f32, std::false_type());
+        auto coded = [&](auto rows_too) {
+            if (bits == 2) return go(std::integral_constant<int, kOutInt2>(), in_f32, rows_too);
+            if (bits == 4) return go(std::integral_constant<int, kOutInt4>(), in_f32, rows_too);
+            return go(std::integral_constant<int, kOutInt8>(), in_f32, rows_too);
+        };
+        return y != nullptr ? coded(std::true_type()) : coded(std::false_type());
+    };
+    return f32 ? of_type(std::true_type()) : of_type(std::false_type());
 }
 
 }  // namespace bfq

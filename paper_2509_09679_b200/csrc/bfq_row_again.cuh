@@ -20,8 +20,8 @@ struct Again {
     bool inverse;
     int levels;     // log2 of the row length
     int64_t elems;  // elements of all rows
-    int bits;       // 0: rows of ytype out, contiguous; else codes and scales
-    void* y;
+    int bits;       // 0: rows out only; else codes and scales
+    void* y;        // rows of ytype out, contiguous, or null
     int ytype;
     uint8_t* codes;
     uint16_t* scales;
@@ -88,13 +88,13 @@ __device__ __forceinline__ void row_again(const Again& p, int64_t row, uint32_t 
         bar_sync(bar, kGroupThreads);
     }
     auto value = [&](int e) { return __uint_as_float(lds32(buf + 4 * e)); };
-    if (p.bits == 0) {
+    if (p.y != nullptr) {
         for (int e = t; e < n; e += kGroupThreads) {
             if (p.ytype == kF32) static_cast<float*>(p.y)[row * n + e] = value(e);
             else static_cast<__nv_bfloat16*>(p.y)[row * n + e] = __float2bfloat16_rn(value(e));
         }
-        return;
     }
+    if (p.bits == 0) return;
     float m = 0.f;
     for (int e = t; e < n; e += kGroupThreads) m = fmaxf(m, fabsf(value(e)));  // drops NaN
     const uint32_t wmax = __reduce_max_sync(0xFFFFFFFFu, __float_as_uint(m));

@@ -169,6 +169,8 @@ def test_rows_of_any_magnitude(n, dtype):
         plain = p.forward_quant(x.to(DEV), bits)
         assert torch.equal(codes.view[keep], plain[0][keep]) and torch.equal(scales.view[keep], plain[1][keep])
         assert codes.intact() and scales.intact()
+        kept = p.fold_weights(big.to(DEV), bits, want_rotated=True)
+        assert torch.equal(kept[0], codes.view) and torch.equal(kept[1], scales.view) and torch.equal(kept[2], y.view)
     assert y.intact() and xr.intact() and p.device_status() == 0
 
 
@@ -193,3 +195,20 @@ def test_infinities_and_nan_as_in_the_kernels_for_every_n(n, monkeypatch):
         for r in (3, 7, 9, rows - 1):
             assert torch.equal(a[r].nan_to_num(), b[r].nan_to_num())
     assert got[3][3] == 65504
+
+
+@pytest.mark.parametrize("n", [128, 256, 512, 1024, 2048])
+@pytest.mark.parametrize("dtype,kept", [(torch.float32, torch.float32), (torch.bfloat16, torch.bfloat16), (torch.bfloat16, torch.float32)])
+def test_a_fold_that_keeps_its_rows_gives_the_bits_of_the_calls_that_give_one_of_them(n, dtype, kept):
+    p = Plan(n, DEV)
+    theta = synth.angles(n, "uniform", 3)
+    p.set_angles(theta.to(DEV))
+    W = synth.rows((1 << 20) // n + 1, n, "normal", 4, scale=0.02, dtype=dtype)
+    y_ref = oracle.forward(to_f64(theta), to_f64(W))
+    for bits in (2, 4, 8):
+        codes, scales, rows = p.fold_weights(W.to(DEV), bits, want_rotated=True, rotated_dtype=kept)
+        alone = p.fold_weights(W.to(DEV), bits)
+        assert torch.equal(codes, alone[0]) and torch.equal(scales, alone[1])
+        assert torch.equal(rows, p.forward(W.to(DEV), out_dtype=kept))
+        check_quant(codes, scales, y_ref, bits, f"{bits} bits")
+        check_rows_close(rows, y_ref, np.abs(to_f64(W)).max(axis=1), "rows")
