@@ -352,8 +352,8 @@ static int forward_rows(bfq_plan* plan, const void* x, int xt, int64_t rows, int
         cudaError_t e = fwdq8192_launch_bf16(plan, x, rows, ldx, y, ldy, st);
         return e == cudaSuccess ? BFQ_OK : cuda_fail(plan, e);
     }
-    if (xt == yt && x != y && ldy == plan->n && use_short_rows(plan, rows, 0)) {
-        cudaError_t e = fwdq_short_launch(plan, x, xt == BFQ_F32, rows, ldx, 0, nullptr, nullptr, y, st);
+    if (xt == yt && x != y && use_short_rows(plan, rows, 0)) {
+        cudaError_t e = fwdq_short_launch(plan, x, xt == BFQ_F32, rows, ldx, 0, nullptr, nullptr, y, ldy, st);
         return e == cudaSuccess ? BFQ_OK : cuda_fail(plan, e);
     }
     GenericParams p{};
@@ -443,7 +443,7 @@ static int forward_quant_impl(bfq_plan* plan, const void* x, int xt, int64_t row
         // rows kept beside the codes: both the bits of the calls that give one of them alone.  In the input's type they come from
         // the same pass, else (or over the input) from a second one.
         const bool one_pass = y != nullptr && yt == xt && y != x;
-        e = fwdq_short_launch(plan, x, xt == BFQ_F32, rows, ldx, bits, codes, scales, one_pass ? y : nullptr, static_cast<cudaStream_t>(stream));
+        e = fwdq_short_launch(plan, x, xt == BFQ_F32, rows, ldx, bits, codes, scales, one_pass ? y : nullptr, plan->n, static_cast<cudaStream_t>(stream));
         if (e == cudaSuccess && y != nullptr && !one_pass) return forward_rows(plan, x, xt, rows, ldx, y, yt, plan->n, static_cast<cudaStream_t>(stream));
         return e == cudaSuccess ? BFQ_OK : cuda_fail(plan, e);
     }
@@ -647,9 +647,9 @@ int bfq_inverse(bfq_plan* plan, const void* y, bfq_dtype yt, int64_t rows, int64
         if (e == cudaSuccess) e = inv8192_launch(plan, y, rows, ldy, x, xt == BFQ_BF16, ldx, st);
         return e == cudaSuccess ? BFQ_OK : cuda_fail(plan, e);
     }
-    if ((yt == BFQ_BF16 || xt == BFQ_F32) && x != y && ldx == plan->n && use_short_rows(plan, rows, short_inverse_from(plan->n, yt == BFQ_F32)) &&
+    if ((yt == BFQ_BF16 || xt == BFQ_F32) && x != y && use_short_rows(plan, rows, short_inverse_from(plan->n, yt == BFQ_F32)) &&
         bwd_short_available(plan)) {
-        cudaError_t e = inv_short_launch(plan, y, yt == BFQ_F32, rows, ldy, x, xt == BFQ_BF16, static_cast<cudaStream_t>(stream));
+        cudaError_t e = inv_short_launch(plan, y, yt == BFQ_F32, rows, ldy, x, xt == BFQ_BF16, ldx, static_cast<cudaStream_t>(stream));
         return e == cudaSuccess ? BFQ_OK : cuda_fail(plan, e);
     }
     GenericParams p{};

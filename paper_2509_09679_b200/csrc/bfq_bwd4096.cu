@@ -857,7 +857,8 @@ struct InvUpper {
 // odd CTAs the upper (CTAs 2i and 2i + 1 work on the same rows at about the same time, so the second read of a row comes
 // from L2).  A y row is 16 KB in one slot; the transposed stage-12 rotation y'_own = c y_own +- s y_other with (cos, sin)
 // from `tw12` is applied as the row is read, then the half's own twelve stages follow from its own tables.
-template <int G, bool OUT_BF16, bool IN_F32 = false, bool WIDE = false, bool SHORT = false>
+// STRIDED (SHORT): the short rows of x lie brief.again.ldy apart instead of one after the other.
+template <int G, bool OUT_BF16, bool IN_F32 = false, bool WIDE = false, bool SHORT = false, bool STRIDED = false>
 __global__ void __launch_bounds__(G * kThreads, 1)
 k_inv4096(const __grid_constant__ CUtensorMap ymap, const float* __restrict__ img_lo, const float* __restrict__ img_scaled_lo,
           const int* __restrict__ form_lo, const uint32_t* __restrict__ gsign_lo, void* __restrict__ xout, int64_t ldx, int rows,
@@ -1078,8 +1079,12 @@ k_inv4096(const __grid_constant__ CUtensorMap ymap, const float* __restrict__ im
         const uint32_t sa_ = kSigns ? sgn_a : 0u, sb_ = kSigns ? sgn_b : 0u;
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
-            const int64_t off = static_cast<int64_t>(row) * ldx + (WIDE ? kN * half : 0) + 16 * (t & 15) + 512 * (t >> 4) + 256 * h;
-            if (SHORT && off >= brief.elems) continue;  // x is contiguous: past the last row
+            const int at = 16 * (t & 15) + 512 * (t >> 4) + 256 * h;
+            int64_t off = static_cast<int64_t>(row) * ldx + (WIDE ? kN * half : 0) + at;
+            if constexpr (SHORT) {
+                if (static_cast<int64_t>(row) * kN + at >= brief.elems) continue;  // past the last row
+                if constexpr (STRIDED) off += (at >> (12 - brief.log)) * (brief.again.ldy - (kN >> brief.log));
+            }
             if constexpr (OUT_BF16) {
                 uint32_t w[8];
 #pragma unroll
@@ -1337,13 +1342,18 @@ cudaError_t bwd_short_launch(bfq_plan* plan, const void* x, const void* g, int64
     return cudaGetLastError();
 }
 
-// y: rows of leading dimension ldy; x contiguous; bf16 -> bf16, bf16 -> fp32 or fp32 -> fp32
-cudaError_t inv_short_launch(bfq_plan* plan, const void* y, bool y_f32, int64_t rows, int64_t ldy, void* x, bool x_bf16, cudaStream_t st) {
+// y, x: rows of leading dimension ldy, ldx; bf16 -> bf16, bf16 -> fp32 or fp32 -> fp32
+cudaError_t inv_short_launch(bfq_plan* plan, const void* y, bool y_f32, int64_t rows, int64_t ldy, void* x, bool x_bf16, int64_t ldx, cudaStream_t st) {
     constexpr int G = 4;
     using S = b4k::InvSmem<G>;
-    auto kern = y_f32 ? b4k::k_inv4096<G, false, true, false, true> : (x_bf16 ? b4k::k_inv4096<G, true, false, false, true> : b4k::k_inv4096<G, false, false, false, true>);
-    const int which = y_f32 ? 0 : (x_bf16 ? 1 : 2);
-    static bool attr_set[3][kMaxDevices] = {{false}};
+    auto pick = [&](auto strided) {
+        constexpr bool kStrided = decltype(strided)::value;
+        return y_f32 ? b4k::k_inv4096<G, false, true, false, true, kStrided>
+                     : (x_bf16 ? b4k::k_inv4096<G, true, false, false, true, kStrided> : b4k::k_inv4096<G, false, false, false, true, kStrided>);
+    };
+    auto kern = ldx == plan->n ? pick(std::false_type()) : pick(std::true_type());
+    const int which = (y_f32 ? 0 : (x_bf16 ? 1 : 2)) + (ldx == plan->n ? 0 : 3);
+    static bool attr_set[6][kMaxDevices] = {{false}};
     if (!attr_set[which][plan->device]) {
         cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(S::kBytes));
         if (e != cudaSuccess) return e;
@@ -1353,10 +1363,10 @@ cudaError_t inv_short_launch(bfq_plan* plan, const void* y, bool y_f32, int64_t 
     CUtensorMap ymap;
     if (!(y_f32 ? encode_row_map_f32(&ymap, y, rows, ldy, n) : encode_row_map(&ymap, y, rows, ldy, n))) return cudaErrorInvalidValue;
     const b4k::ShortRows brief{12 - plan->log_n, rows * n,
-                               Again{y, ldy, y_f32 ? kF32 : kBF16, plan->tw, true, plan->log_n, rows * n, 0, x, x_bf16 ? kBF16 : kF32, nullptr, nullptr}};
+                               Again{y, ldy, y_f32 ? kF32 : kBF16, plan->tw, true, plan->log_n, rows * n, 0, x, ldx, x_bf16 ? kBF16 : kF32, nullptr, nullptr}};
     const int64_t joint = (brief.elems + f4k::kN - 1) / f4k::kN, want = (joint + G - 1) / G;
     const int grid = int(want < plan->sm_count ? want : plan->sm_count);
-    kern<<<grid, G * b4k::kThreads, S::kBytes, st>>>(ymap, plan->img_b4096, plan->img_i4096, plan->form_flag + 1, plan->gsign4096, x, f4k::kN,
+    kern<<<grid, G * b4k::kThreads, S::kBytes, st>>>(ymap, plan->img_b4096, plan->img_i4096, plan->form_flag + 1, plan->gsign4096, x, ldx << (12 - plan->log_n),
                                                     int(joint), plan->status_word, nullptr, b4k::InvUpper{}, brief);
     return cudaGetLastError();
 }

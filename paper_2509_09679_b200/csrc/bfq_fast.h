@@ -31,20 +31,20 @@ cudaError_t fwdq4096_launch_stats(const bfq_plan* plan, const void* x, int64_t r
 
 cudaError_t fwdq4096_prep_angles(const bfq_plan* plan, const float* theta, cudaStream_t st);
 // rows of 128 .. 2048 elements: several as one of 4096 on the same kernel.  bits = 2, 4, 8: codes + scales, and
-// the rows if y is not null; bits = 0: the rows alone.  Rows are contiguous, in the type of x
+// the rows if y is not null; bits = 0: the rows alone.  Rows are in the type of x, ldy apart (beside codes: contiguous)
 bool fwdq_short_available(const bfq_plan* plan);
 cudaError_t fwdq_short_launch(const bfq_plan* plan, const void* x, bool f32, int64_t rows, int64_t ldx, int bits, uint8_t* codes,
-                              uint16_t* scales, void* y, cudaStream_t st);
+                              uint16_t* scales, void* y, int64_t ldy, cudaStream_t st);
 cudaError_t fwdq128_launch(const bfq_plan* plan, const void* x, bool f32, int64_t rows, int64_t ldx, int bits, uint8_t* codes, uint16_t* scales,
-                           void* y, cudaStream_t st);
+                           void* y, int64_t ldy, cudaStream_t st);
 cudaError_t fwdq256_launch(const bfq_plan* plan, const void* x, bool f32, int64_t rows, int64_t ldx, int bits, uint8_t* codes, uint16_t* scales,
-                           void* y, cudaStream_t st);
+                           void* y, int64_t ldy, cudaStream_t st);
 cudaError_t fwdq512_launch(const bfq_plan* plan, const void* x, bool f32, int64_t rows, int64_t ldx, int bits, uint8_t* codes, uint16_t* scales,
-                           void* y, cudaStream_t st);
+                           void* y, int64_t ldy, cudaStream_t st);
 cudaError_t fwdq1024_launch(const bfq_plan* plan, const void* x, bool f32, int64_t rows, int64_t ldx, int bits, uint8_t* codes, uint16_t* scales,
-                           void* y, cudaStream_t st);
+                           void* y, int64_t ldy, cudaStream_t st);
 cudaError_t fwdq2048_launch(const bfq_plan* plan, const void* x, bool f32, int64_t rows, int64_t ldx, int bits, uint8_t* codes, uint16_t* scales,
-                           void* y, cudaStream_t st);
+                           void* y, int64_t ldy, cudaStream_t st);
 // the same rows backward and inverse.  takes_short_backward: whether bfq_backward (and bfq_backward_noalloc, whose dx are the
 // same bits) hands a call to bwd_short_launch
 bool takes_short_backward(int n, int xt, int gt, bool want_dx, int dxt, int64_t rows, int64_t ld);
@@ -52,7 +52,7 @@ size_t bwd_short_partial_floats(int sm_count);
 bool bwd_short_available(const bfq_plan* plan);
 cudaError_t bwd_short_prepare(int device);
 cudaError_t bwd_short_launch(bfq_plan* plan, const void* x, const void* g, int64_t rows, void* dx, float* dtheta, bool f32, cudaStream_t st);
-cudaError_t inv_short_launch(bfq_plan* plan, const void* y, bool y_f32, int64_t rows, int64_t ldy, void* x, bool x_bf16, cudaStream_t st);
+cudaError_t inv_short_launch(bfq_plan* plan, const void* y, bool y_f32, int64_t rows, int64_t ldy, void* x, bool x_bf16, int64_t ldx, cudaStream_t st);
 
 // n = 8192, bf16 rows, INT2 (INT4 / INT8 through another epilogue): two-CTA clusters, one 4096-point half per CTA
 size_t fwdq8192_image_bytes();

@@ -4,8 +4,8 @@
 namespace bfq {
 
 cudaError_t fwdq256_launch(const bfq_plan* plan, const void* x, bool f32, int64_t rows, int64_t ldx, int bits, uint8_t* codes, uint16_t* scales,
-                           void* y, cudaStream_t st) {
-    return fwdq_short_launch<4>(plan, x, f32, rows, ldx, bits, codes, scales, y, st);
+                           void* y, int64_t ldy, cudaStream_t st) {
+    return fwdq_short_launch<4>(plan, x, f32, rows, ldx, bits, codes, scales, y, ldy, st);
 }
 
 }  // namespace bfq

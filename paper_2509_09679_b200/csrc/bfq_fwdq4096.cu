@@ -162,18 +162,18 @@ cudaError_t fwdq4096_set_angles(const bfq_plan* plan, const float* theta, cudaSt
                              plan->form_flag);
 }
 
-// rows of 128 .. 2048 elements: several as one of 4096.  bits = 0: the rotated rows, contiguous, in the type of x.
+// rows of 128 .. 2048 elements: several as one of 4096.  bits = 0: the rotated rows, in the type of x.
 bool fwdq_short_available(const bfq_plan* plan) {
     return plan->n >= 128 && plan->n < f4k::kN && plan->cc_major == 10 && plan->img4096 != nullptr && encode_tiled() != nullptr;
 }
 cudaError_t fwdq_short_launch(const bfq_plan* plan, const void* x, bool f32, int64_t rows, int64_t ldx, int bits, uint8_t* codes,
-                              uint16_t* scales, void* y, cudaStream_t st) {
+                              uint16_t* scales, void* y, int64_t ldy, cudaStream_t st) {
     switch (plan->n) {
-        case 128: return fwdq128_launch(plan, x, f32, rows, ldx, bits, codes, scales, y, st);
-        case 256: return fwdq256_launch(plan, x, f32, rows, ldx, bits, codes, scales, y, st);
-        case 512: return fwdq512_launch(plan, x, f32, rows, ldx, bits, codes, scales, y, st);
-        case 1024: return fwdq1024_launch(plan, x, f32, rows, ldx, bits, codes, scales, y, st);
-        case 2048: return fwdq2048_launch(plan, x, f32, rows, ldx, bits, codes, scales, y, st);
+        case 128: return fwdq128_launch(plan, x, f32, rows, ldx, bits, codes, scales, y, ldy, st);
+        case 256: return fwdq256_launch(plan, x, f32, rows, ldx, bits, codes, scales, y, ldy, st);
+        case 512: return fwdq512_launch(plan, x, f32, rows, ldx, bits, codes, scales, y, ldy, st);
+        case 1024: return fwdq1024_launch(plan, x, f32, rows, ldx, bits, codes, scales, y, ldy, st);
+        case 2048: return fwdq2048_launch(plan, x, f32, rows, ldx, bits, codes, scales, y, ldy, st);
         default: return cudaErrorInvalidValue;
     }
 }

@@ -170,7 +170,8 @@ enum : int { kOutInt4 = 0, kOutBf16 = 1, kOutInt4Stats = 2, kOutInt2 = 3, kOutIn
 // that takes the factors off.  A quantized row's maximum is taken over its own part of the 4096.  A row whose results are not
 // finite is done again at the end (bfq_row_again.cuh); to know of one takes eight maxima per thread and joint row where rows go
 // out.
-template <int G, int CW, int XB, int TRANSFORM, int OUT, int STEP = 2, bool ROWS = false, bool IN_F32 = false, int SUB = 0>
+// STRIDED (rows out alone): the short rows of the output lie again.ldy apart instead of one after the other.
+template <int G, int CW, int XB, int TRANSFORM, int OUT, int STEP = 2, bool ROWS = false, bool IN_F32 = false, int SUB = 0, bool STRIDED = false>
 __global__ void __launch_bounds__(G * kGroupThreads, 1)
 k_fwdq4096(const __grid_constant__ CUtensorMap tmap, const float* __restrict__ img, const int* __restrict__ form,
            uint8_t* __restrict__ codes,
@@ -365,6 +366,12 @@ k_fwdq4096(const __grid_constant__ CUtensorMap tmap, const float* __restrict__ i
         const int64_t left = elems - static_cast<int64_t>(row) * kN;
         const int lim = SUB == 0 || left >= kN ? kN : static_cast<int>(left);
         auto there = [&](int m) { return SUB == 0 || 2 * t + 256 * m < lim; };
+        static_assert(!STRIDED || (SUB != 0 && (OUT == kOutBf16 || OUT == kOutF32)), "rows out alone");
+        // pairs of elements between where register m's would lie in contiguous rows and where they lie
+        auto gap = [&](int m) -> int64_t {
+            if constexpr (!STRIDED) return 0;
+            else return (SUB < 5 ? m >> (4 - SUB) : 2 * m + (q >> 1)) * ((again.ldy - (kN >> SUB)) / 2);
+        };
         if constexpr (OUT == kOutBf16 || (ROWS && !IN_F32)) {
             // thread t holds elements 2t + 256m, +1: one 32-bit word of the bf16 row per packed register
             uint32_t* out = reinterpret_cast<uint32_t*>(yout + static_cast<int64_t>(row) * ldy) + t;
@@ -373,7 +380,7 @@ k_fwdq4096(const __grid_constant__ CUtensorMap tmap, const float* __restrict__ i
                 float a, b;
                 unpack2(P[m], a, b);
                 const __nv_bfloat162 v = __floats2bfloat162_rn(a * kPost, b * kPost);
-                if (there(m)) out[128 * m] = *reinterpret_cast<const uint32_t*>(&v);
+                if (there(m)) out[128 * m + gap(m)] = *reinterpret_cast<const uint32_t*>(&v);
             }
         }
         if constexpr (OUT == kOutF32 || (ROWS && IN_F32)) {
@@ -383,7 +390,7 @@ k_fwdq4096(const __grid_constant__ CUtensorMap tmap, const float* __restrict__ i
             for (int m = 0; m < 16; ++m) {
                 float a, b;
                 unpack2(P[m], a, b);
-                if (there(m)) out[128 * m] = pack2(a * kPost, b * kPost);
+                if (there(m)) out[128 * m + gap(m)] = pack2(a * kPost, b * kPost);
             }
         }
         if constexpr (OUT == kOutBf16 || OUT == kOutF32) {
@@ -658,13 +665,13 @@ k_fwdq4096(const __grid_constant__ CUtensorMap tmap, const float* __restrict__ i
 
 }  // namespace f4k
 
-template <int G, int CW, int XB, int TRANSFORM, int OUT, bool ROWS = false, bool IN_F32 = false, int SUB = 0>
+template <int G, int CW, int XB, int TRANSFORM, int OUT, bool ROWS = false, bool IN_F32 = false, int SUB = 0, bool STRIDED = false>
 static cudaError_t launch_variant(const bfq_plan* plan, const CUtensorMap& tmap, int64_t rows, uint8_t* codes,
                                   uint16_t* scales, void* y, int64_t ldy, cudaStream_t st,
                                   unsigned long long* hist = nullptr, int64_t elems = 0, const Again& again = Again{}) {
     using S = f4k::Smem<G, XB>;
     static bool attr_set[kMaxDevices] = {false};
-    auto kern = f4k::k_fwdq4096<G, CW, XB, TRANSFORM, OUT, 2, ROWS, IN_F32, SUB>;
+    auto kern = f4k::k_fwdq4096<G, CW, XB, TRANSFORM, OUT, 2, ROWS, IN_F32, SUB, STRIDED>;
     if (!attr_set[plan->device]) {
         cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(S::kBytes));
         if (e != cudaSuccess) return e;

@@ -11,27 +11,30 @@ namespace bfq {
 
 template <int SUB>
 static cudaError_t fwdq_short_launch(const bfq_plan* plan, const void* x, bool f32, int64_t rows, int64_t ldx, int bits, uint8_t* codes,
-                                     uint16_t* scales, void* y, cudaStream_t st) {
+                                     uint16_t* scales, void* y, int64_t ldy, cudaStream_t st) {
     constexpr int n = f4k::kN >> SUB;
     CUtensorMap tmap;
     if (!(f32 ? encode_row_map_f32(&tmap, x, rows, ldx, n) : encode_row_map(&tmap, x, rows, ldx, n))) return cudaErrorInvalidValue;
     const int64_t elems = rows * n, joint = (elems + f4k::kN - 1) / f4k::kN;
     const int type = f32 ? kF32 : kBF16;
-    const Again again{x, ldx, type, plan->tw, false, 12 - SUB, elems, bits, y, type, codes, scales};
+    const Again again{x, ldx, type, plan->tw, false, 12 - SUB, elems, bits, y, ldy, type, codes, scales};
     using namespace f4k;
-    auto go = [&](auto out, auto in_f32, auto rows_too) {
-        return launch_variant<4, 32, 2, kButterfly, decltype(out)::value, decltype(rows_too)::value, decltype(in_f32)::value, SUB>(
-            plan, tmap, joint, codes, scales, y, kN, st, nullptr, elems, again);
+    auto go = [&](auto out, auto in_f32, auto rows_too, auto strided) {
+        return launch_variant<4, 32, 2, kButterfly, decltype(out)::value, decltype(rows_too)::value, decltype(in_f32)::value, SUB, decltype(strided)::value>(
+            plan, tmap, joint, codes, scales, y, ldy << SUB, st, nullptr, elems, again);
     };
     auto of_type = [&](auto in_f32) {
         constexpr int kRowsOut = decltype(in_f32)::value ? kOutF32 : kOutBf16;
-        if (bits == 0) return go(std::integral_constant<int, kRowsOut>(), in_f32, std::false_type());
+        const std::false_type no{};
+        const std::true_type yes{};
+        if (bits == 0)
+            return ldy == n ? go(std::integral_constant<int, kRowsOut>(), in_f32, no, no) : go(std::integral_constant<int, kRowsOut>(), in_f32, no, yes);
         auto coded = [&](auto rows_too) {
-            if (bits == 2) return go(std::integral_constant<int, kOutInt2>(), in_f32, rows_too);
-            if (bits == 4) return go(std::integral_constant<int, kOutInt4>(), in_f32, rows_too);
-            return go(std::integral_constant<int, kOutInt8>(), in_f32, rows_too);
+            if (bits == 2) return go(std::integral_constant<int, kOutInt2>(), in_f32, rows_too, no);
+            if (bits == 4) return go(std::integral_constant<int, kOutInt4>(), in_f32, rows_too, no);
+            return go(std::integral_constant<int, kOutInt8>(), in_f32, rows_too, no);
         };
-        return y != nullptr ? coded(std::true_type()) : coded(std::false_type());
+        return y != nullptr ? coded(yes) : coded(no);
     };
     return f32 ? of_type(std::true_type()) : of_type(std::false_type());
 }

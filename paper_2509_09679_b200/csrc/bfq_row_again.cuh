@@ -21,7 +21,8 @@ struct Again {
     int levels;     // log2 of the row length
     int64_t elems;  // elements of all rows
     int bits;       // 0: rows out only; else codes and scales
-    void* y;        // rows of ytype out, contiguous, or null
+    void* y;        // rows of ytype out, row stride ldy, or null
+    int64_t ldy;
     int ytype;
     uint8_t* codes;
     uint16_t* scales;
@@ -90,8 +91,8 @@ __device__ __forceinline__ void row_again(const Again& p, int64_t row, uint32_t 
     auto value = [&](int e) { return __uint_as_float(lds32(buf + 4 * e)); };
     if (p.y != nullptr) {
         for (int e = t; e < n; e += kGroupThreads) {
-            if (p.ytype == kF32) static_cast<float*>(p.y)[row * n + e] = value(e);
-            else static_cast<__nv_bfloat16*>(p.y)[row * n + e] = __float2bfloat16_rn(value(e));
+            if (p.ytype == kF32) static_cast<float*>(p.y)[row * p.ldy + e] = value(e);
+            else static_cast<__nv_bfloat16*>(p.y)[row * p.ldy + e] = __float2bfloat16_rn(value(e));
         }
     }
     if (p.bits == 0) return;
@@ -126,8 +127,8 @@ static __device__ __noinline__ void rows_again(const Again& p, int first, int st
             } else {
                 for (int e = t; e < n; e += kGroupThreads) {
                     if ((e & upper) != 0) continue;
-                    if (p.ytype == kF32) bad |= (*reinterpret_cast<volatile const uint32_t*>(static_cast<float*>(p.y) + row * n + e) & 0x7F800000u) == 0x7F800000u;
-                    else bad |= (*reinterpret_cast<volatile const uint16_t*>(static_cast<__nv_bfloat16*>(p.y) + row * n + e) & 0x7F80u) == 0x7F80u;
+                    if (p.ytype == kF32) bad |= (*reinterpret_cast<volatile const uint32_t*>(static_cast<float*>(p.y) + row * p.ldy + e) & 0x7F800000u) == 0x7F800000u;
+                    else bad |= (*reinterpret_cast<volatile const uint16_t*>(static_cast<__nv_bfloat16*>(p.y) + row * p.ldy + e) & 0x7F80u) == 0x7F80u;
                 }
             }
             if (group_any(bar, bad)) row_again(p, row, buf, bar, t);

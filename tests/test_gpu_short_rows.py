@@ -212,3 +212,23 @@ def test_a_fold_that_keeps_its_rows_gives_the_bits_of_the_calls_that_give_one_of
         assert torch.equal(rows, p.forward(W.to(DEV), out_dtype=kept))
         check_quant(codes, scales, y_ref, bits, f"{bits} bits")
         check_rows_close(rows, y_ref, np.abs(to_f64(W)).max(axis=1), "rows")
+
+
+@pytest.mark.parametrize("n", [128, 256, 512, 1024, 2048])
+@pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
+def test_an_output_with_a_row_stride_has_the_bits_of_a_contiguous_one(n, dtype):
+    rows = (1 << 22) // n + 1
+    p = Plan(n, DEV)
+    p.set_angles(synth.angles(n, "uniform", 3).to(DEV))
+    x = synth.rows(rows, n, "normal", 4, dtype=dtype).to(DEV)
+    x[2] *= 1e37  # done again
+    x[rows - 1, 3] = float("inf")
+    for call in (p.forward, p.inverse):
+        ref = call(x)
+        for pad in (8, 4096):
+            wide = Guarded((rows, n + pad), dtype, DEV)
+            untouched = wide.view[:, n:].clone()
+            call(x, out=wide.view[:, :n])
+            same = lambda a, b: torch.equal(a.contiguous().view(torch.uint8), b.contiguous().view(torch.uint8))
+            assert same(wide.view[:, :n], ref) and same(wide.view[:, n:], untouched) and wide.intact()
+    assert p.device_status() == 0
