@@ -232,7 +232,7 @@ static inline EncodeTiledFn encode_tiled() {
 // 3-D map over bf16 rows of n <= 4096: {64 elements, n / 64 lines, rows}, box = 4096 / n rows (4096 elements), 128-byte swizzle
 static inline bool encode_row_map(CUtensorMap* tmap, const void* x, int64_t rows, int64_t ld, int n = f4k::kN) {
     const cuuint64_t dims[3] = {64, static_cast<cuuint64_t>(n / 64), static_cast<cuuint64_t>(rows)};
-    const cuuint64_t strides[2] = {128, static_cast<cuuint64_t>(ld) * 2};
+    const cuuint64_t strides[2] = {128, static_cast<cuuint64_t>(rows == 1 ? n : ld) * 2};  // one row: any ld (a map's are below 2^40)
     const cuuint32_t box[3] = {64, static_cast<cuuint32_t>(n / 64), static_cast<cuuint32_t>(f4k::kN / n)};
     const cuuint32_t estr[3] = {1, 1, 1};
     return encode_tiled()(tmap, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(x), dims, strides, box, estr,
@@ -243,7 +243,7 @@ static inline bool encode_row_map(CUtensorMap* tmap, const void* x, int64_t rows
 // the same for fp32 rows: n / 32 lines of 32 elements per row
 static inline bool encode_row_map_f32(CUtensorMap* tmap, const void* x, int64_t rows, int64_t ld, int n = f4k::kN) {
     const cuuint64_t dims[3] = {32, static_cast<cuuint64_t>(n / 32), static_cast<cuuint64_t>(rows)};
-    const cuuint64_t strides[2] = {128, static_cast<cuuint64_t>(ld) * 4};
+    const cuuint64_t strides[2] = {128, static_cast<cuuint64_t>(rows == 1 ? n : ld) * 4};
     const cuuint32_t box[3] = {32, static_cast<cuuint32_t>(n / 32), static_cast<cuuint32_t>(f4k::kN / n)};
     const cuuint32_t estr[3] = {1, 1, 1};
     return encode_tiled()(tmap, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 3, const_cast<void*>(x), dims, strides, box, estr,

@@ -232,3 +232,17 @@ def test_an_output_with_a_row_stride_has_the_bits_of_a_contiguous_one(n, dtype):
             same = lambda a, b: torch.equal(a.contiguous().view(torch.uint8), b.contiguous().view(torch.uint8))
             assert same(wide.view[:, :n], ref) and same(wide.view[:, n:], untouched) and wide.intact()
     assert p.device_status() == 0
+
+
+@pytest.mark.parametrize("n", [128, 2048, 4096])
+@pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
+def test_a_single_row_may_have_any_row_stride(n, dtype):
+    p = Plan(n, DEV)
+    p.set_angles(synth.angles(n, "normal", 3).to(DEV))
+    x = synth.rows(1, n, "normal", 4, dtype=dtype).to(DEV)
+    far = x.as_strided((1, n), (1 << 41, 1))
+    assert torch.equal(p.forward(far), p.forward(x)) and torch.equal(p.inverse(far), p.inverse(x))
+    out = torch.empty_like(x)
+    p.forward(x, out=out.as_strided((1, n), (1 << 41, 1)))
+    assert torch.equal(out, p.forward(x))
+    assert all(torch.equal(a, b) for a, b in zip(p.forward_quant(far, 4), p.forward_quant(x, 4)))
