@@ -307,8 +307,6 @@ int bfq_set_angles(bfq_plan* plan, const float* theta, void* stream) {
     cudaError_t e;
     if (plan->img4096 != nullptr) {
         e = fwdq4096_set_angles(plan, theta, static_cast<cudaStream_t>(stream));
-        // shorter rows: the reverse tables too, so that later calls on any stream find all tables built here
-        if (e == cudaSuccess && plan->n < 4096) e = bwd4096_build_tables(plan, static_cast<cudaStream_t>(stream));
     } else if (plan->img8192 != nullptr) {
         e = fwdq8192_set_angles(plan, theta, static_cast<cudaStream_t>(stream));
     } else {

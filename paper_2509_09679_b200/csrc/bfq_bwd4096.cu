@@ -40,7 +40,6 @@ constexpr int kUpperSteps = 8;               // half-stage steps of the reverse 
 constexpr uint32_t kPairBytes = 2 * kRowBytes;  // two bf16 rows
 constexpr int kWideCol = 416;  // wide inverse: (cos, +-sin) of the stage that joins the halves, 64 columns behind either table
 constexpr int kInvCols = 416;  // scaled inverse: stages 11..1 (32 columns each, stage s at 32 (s - 1)), then stage 0 (64)
-enum : int { kFormScaled = 0, kFormShear = 1 };
 
 struct Smem {
     static constexpr uint32_t kXOff = 0;                                   // [kSlots][2][kRowBytes]
@@ -754,13 +753,15 @@ __device__ __forceinline__ void build_image_inv(int k, const double2* __restrict
 }
 
 // All three of the above in one launch (their inputs are the same and none needs another's output): blocks of 256 threads,
-// the image of the backward kernel, then that of the reverse walk, then the sign words.  As three launches and a memset of
-// the range flag they took 11.6 us.  *form must be kFormScaled before.
+// the image of the backward kernel, then that of the reverse walk, then the sign words, then (img_fwd not null) that of the
+// forward kernel.  As three launches and a memset of the range flag the first three took 11.6 us.  The range flags *form and
+// *form_fwd must be kFormScaled before.
 constexpr int kAngleBlocks = 12 * (kN / 2) / 256, kSignBlocks = 16 * kThreads / 256;
 constexpr int kTableBlocks = 2 * kAngleBlocks + kSignBlocks;
 __global__ void __launch_bounds__(256) k_build_tables(const float4* __restrict__ prep, const uint8_t* __restrict__ flip,
                                                        const double2* __restrict__ cs, float* __restrict__ img, int8_t* __restrict__ dsign,
-                                                       float* __restrict__ img_inv, int* __restrict__ form, uint32_t* __restrict__ gsign, bool quads) {
+                                                       float* __restrict__ img_inv, int* __restrict__ form, uint32_t* __restrict__ gsign, bool quads,
+                                                       float* __restrict__ img_fwd, int* __restrict__ form_fwd) {
     grid_dep_launch();
     grid_dep_wait();
     const int b = blockIdx.x;
@@ -768,8 +769,10 @@ __global__ void __launch_bounds__(256) k_build_tables(const float4* __restrict__
         build_image_bwd(256 * b + threadIdx.x, quads, prep, flip, img, dsign);
     } else if (b < 2 * kAngleBlocks) {
         build_image_inv(256 * (b - kAngleBlocks) + threadIdx.x, cs, img_inv, form);
-    } else {
+    } else if (b < kTableBlocks) {
         build_gsign(256 * (b - 2 * kAngleBlocks) + threadIdx.x, flip, gsign);
+    } else {
+        build_image_fwd(256 * (b - kTableBlocks) + threadIdx.x, prep, cs, img_fwd, form_fwd);
     }
 }
 
@@ -1204,7 +1207,7 @@ cudaError_t bwd8192_build_tables(const bfq_plan* plan, cudaStream_t st) {
         cudaError_t e = cudaMemsetAsync(plan->form_flag + 1 + h, 0, sizeof(int), st);
         if (e != cudaSuccess) return e;
         b4k::k_build_tables<<<b4k::kTableBlocks, 256, 0, st>>>(prep, flip, cs_half, plan->img_b8192[h], plan->dsign8192[h],
-                                                               plan->img_i8192[h], plan->form_flag + 1 + h, plan->gsign8192[h], false);
+                                                               plan->img_i8192[h], plan->form_flag + 1 + h, plan->gsign8192[h], false, nullptr, nullptr);
         e = cudaGetLastError();
         if (e != cudaSuccess) return e;
     }
@@ -1265,13 +1268,14 @@ bool bwd4096_available(const bfq_plan* plan) {
 
 // Builds the tables of the backward and inverse kernels from the staging area bfq_set_angles filled (it also resets the
 // range flag, word 1 of the plan's form flags).
-cudaError_t bwd4096_build_tables(const bfq_plan* plan, cudaStream_t st) {
+cudaError_t bwd4096_build_tables(const bfq_plan* plan, cudaStream_t st, bool forward_too) {
     const int count = 12 * (f4k::kN / 2);
     const float4* prep = reinterpret_cast<const float4*>(plan->prep4096);
     const double2* cs = reinterpret_cast<const double2*>(prep + count);
     const uint8_t* flip = reinterpret_cast<const uint8_t*>(cs + count);
-    return launch_overlapped(b4k::k_build_tables, dim3(b4k::kTableBlocks), dim3(256), 0, st, prep, flip, cs, plan->img_b4096,
-                             plan->dsign4096, plan->img_i4096, plan->form_flag + 1, plan->gsign4096, plan->n < f4k::kN);
+    return launch_overlapped(b4k::k_build_tables, dim3(b4k::kTableBlocks + (forward_too ? b4k::kAngleBlocks : 0)), dim3(256), 0, st, prep, flip, cs, plan->img_b4096,
+                             plan->dsign4096, plan->img_i4096, plan->form_flag + 1, plan->gsign4096, plan->n < f4k::kN,
+                             plan->img4096, plan->form_flag);
 }
 
 // ---- rows of 128 .. 2048 elements, several as one of 4096 ----------------------------------------------------------

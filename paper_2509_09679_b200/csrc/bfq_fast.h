@@ -86,7 +86,7 @@ cudaError_t inv8192_launch(bfq_plan* plan, const void* y, int64_t rows, int64_t 
                            cudaStream_t st);
 cudaError_t bwd8192_launch_halves(bfq_plan* plan, const void* x, const void* g, int64_t rows, int64_t ld, void* dx,
                                   float* dtheta, cudaStream_t st);
-cudaError_t bwd4096_build_tables(const bfq_plan* plan, cudaStream_t st);
+cudaError_t bwd4096_build_tables(const bfq_plan* plan, cudaStream_t st, bool forward_too = false);  // forward_too: img4096 as well
 cudaError_t bwd4096_launch(bfq_plan* plan, const void* x, const void* g, int64_t rows, int64_t ld, void* dx,
                            float* dtheta, bool f32, cudaStream_t st);
 

@@ -74,8 +74,6 @@ struct Chunks {
     static constexpr int kPhase3 = next(kAfterPhase2);
 };
 
-enum : int { kFormScaled = 0, kFormShear = 1 };  // FORM: how stages 0..10 rotate (the image must match)
-
 template <int FORM, int C, int CW, int SUB>
 __device__ __forceinline__ void run_chunk(u64 (&P)[16], const uint32_t (&T)[CW]) {
     using CH = Chunks<CW>;

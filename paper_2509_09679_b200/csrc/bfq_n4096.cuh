@@ -179,6 +179,73 @@ __device__ __forceinline__ int sign_before(const uint8_t* __restrict__ flip, int
     return f ? -1 : 1;
 }
 
+enum : int { kFormScaled = 0, kFormShear = 1 };  // FORM: how the stages rotate (the image must match)
+
+// factor carried by element i when it enters stage s: the product of the cosines of the pairs it belonged to in
+// stages 0..s-1 (its sign is the tracked sign of the three-shear form)
+__device__ __forceinline__ double factor_before(const double2* __restrict__ cs, int i, int s) {
+    double c[11];
+#pragma unroll
+    for (int sp = 0; sp < 11; ++sp) {  // all loads issued together
+        const int j = ((i >> (sp + 1)) << sp) | (i & ((1 << sp) - 1));
+        c[sp] = sp < s ? cs[sp * (kN / 2) + j].x : 1.0;
+    }
+    double d = 1.0;
+#pragma unroll
+    for (int sp = 0; sp < 11; ++sp) d *= c[sp];
+    return d;
+}
+
+// One thread per angle: place the constants of pair (s, j) in both tensor-memory images
+// img[form][role][column], with the role / register / half of the pair's low element in its phase, and raise *form
+// when an element's factor leaves the range the scaled form is used in.
+__device__ __forceinline__ void build_image_fwd(int k, const float4* __restrict__ prep, const double2* __restrict__ cs, float* __restrict__ img,
+                                                int* __restrict__ form) {
+    if (k >= 12 * (kN / 2)) return;
+    const int s = k / (kN / 2), j = k % (kN / 2);
+    const int lo = ((j >> s) << (s + 1)) | (j & ((1 << s) - 1));
+    const int hi = lo + (1 << s);
+    const double da = factor_before(cs, lo, s), db = factor_before(cs, hi, s);
+    const int sa = da < 0.0 ? -1 : 1, sb = db < 0.0 ? -1 : 1;
+    const int kk = s & 3;
+    int r, m, h;
+    if (s < 4) {
+        r = ((lo >> 4) & 15) | ((lo >> 9) << 4), m = lo & 15, h = (lo >> 8) & 1;
+    } else if (s < 8) {
+        r = (lo & 15) | ((lo >> 9) << 4), m = (lo >> 4) & 15, h = (lo >> 8) & 1;
+    } else {
+        r = (lo >> 1) & 127, m = lo >> 8, h = lo & 1;
+    }
+    const int u = ((m >> (kk + 1)) << kk) | (m & ((1 << kk) - 1));
+    const float4 p = prep[k];
+    const double2 own = cs[k];
+    // image layout [column quad][role][4]: column col of role r is word ((col >> 2) * 128 + r) * 4 + (col & 3)
+    float* scaled = img + kFormScaled * (128 * kCols) + 4 * r;
+    float* shear = img + kFormShear * (128 * kCols) + 4 * r;
+    auto at = [](int col) { return (col >> 2) * 512 + (col & 3); };
+    if (s < 11) {
+        const float sg = (sa == sb) ? 1.f : -1.f;
+        shear[at(32 * s + 4 * u + h)] = sg * p.x;
+        shear[at(32 * s + 4 * u + h + 2)] = sg * p.y;
+        // k1 = -tan(theta) db/da, k2 = tan(theta) da/db, with one division
+        const double w = own.y / (own.x * da * db);
+        scaled[at(32 * s + 4 * u + h)] = static_cast<float>(-w * db * db);
+        scaled[at(32 * s + 4 * u + h + 2)] = static_cast<float>(w * da * da);
+        const double lim = 5.421010862427522e-20;  // 2^-64
+        if (!(fabs(own.x * da) >= lim && fabs(own.x * db) >= lim)) *form = kFormShear;
+    } else {
+        const int col = 352 + 8 * u + h;
+        shear[at(col + 0)] = p.z * sa;
+        shear[at(col + 2)] = -p.w * sb;
+        shear[at(col + 4)] = p.w * sa;
+        shear[at(col + 6)] = p.z * sb;
+        scaled[at(col + 0)] = static_cast<float>(own.x * da);
+        scaled[at(col + 2)] = static_cast<float>(-own.y * db);
+        scaled[at(col + 4)] = static_cast<float>(own.y * da);
+        scaled[at(col + 6)] = static_cast<float>(own.x * db);
+    }
+}
+
 // Walsh-Hadamard local stage K: (a, b) -> (a + b, a - b) on packed registers m and m | 2^K, no constants; the
 // 1/sqrt(n) is applied later, once
 template <int K>
