@@ -81,7 +81,8 @@ int bfq_set_angles(bfq_plan* plan, const float* theta, void* stream);
 /*
  * y = Q x for every row (Sec. 3.2.1: B = prod B_i; stage order as stated at the top).
  * x: [rows][ldx] of xt; y: [rows][ldy] of yt; fp32 arithmetic.  x and y may be the same buffer
- * only if xt == yt and ldx == ldy.
+ * only if xt == yt and ldx == ldy.  A row's result does not depend on the other rows of the call.  Calls
+ * that differ in types, or in place against out of place, may run different kernels and round differently.
  */
 int bfq_forward(bfq_plan* plan, const void* x, bfq_dtype xt, int64_t rows, int64_t ldx,
                 void* y, bfq_dtype yt, int64_t ldy, void* stream);
@@ -105,7 +106,9 @@ int bfq_forward_quant(bfq_plan* plan, const void* x, bfq_dtype xt, int64_t rows,
  *            uniformity regulariser L_uniform = D_KL(P_bins || U) (Sec. 3.4); the caller forms the value.
  *   rowstats [rows][2] fp32: sum_k y_k^2 and sum_k y_k^4 of each row (kurtosis n * s4 / s2^2, sigma^2 = s2 / n,
  *            max|y| / sigma with the row's scale: the diagnostics of the paper's kurtosis / outlier tables).
- * Counts are exact for the codes written; the sums are taken in a fixed order (bit-reproducible).
+ * Counts are exact for the codes written; the sums are taken in a fixed order (bit-reproducible).  Where this call runs another
+ * kernel than bfq_forward_quant (n >= 128, all but bf16 rows of 4096 at 4 bits) a code whose value lies within fp32 rounding of a
+ * boundary may be the neighbouring one.
  */
 int bfq_forward_quant_stats(bfq_plan* plan, const void* x, bfq_dtype xt, int64_t rows, int64_t ldx, int bits,
                             uint8_t* codes, uint16_t* scales_f16, uint64_t* hist, float* rowstats, void* stream);

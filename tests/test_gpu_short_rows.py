@@ -246,3 +246,27 @@ def test_a_single_row_may_have_any_row_stride(n, dtype):
     p.forward(x, out=out.as_strided((1, n), (1 << 41, 1)))
     assert torch.equal(out, p.forward(x))
     assert all(torch.equal(a, b) for a, b in zip(p.forward_quant(far, 4), p.forward_quant(x, 4)))
+
+
+@pytest.mark.parametrize("n", [128, 256, 512, 1024, 2048])
+@pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
+def test_angles_that_need_the_three_shear_form(n, dtype):
+    """Three stages of cosines of 1e-7: the factors leave the scaled form's range, forward and inverse (its own table layout)."""
+    theta = synth.angles(n, "normal", 6)
+    theta[2:5] = math.pi / 2 - 1e-7
+    rows = ((1 << 21) + (1 << 12) if n == 128 else 1 << 19) // n + 3
+    x = synth.rows(rows, n, "student_t3", 5, outliers=4, outlier_scale=20.0, dtype=dtype)
+    x[4] *= 1e-30  # scale 0
+    p = Plan(n, DEV)
+    p.set_angles(theta.to(DEV))
+    th64, x64 = to_f64(theta), to_f64(x)
+    amax = np.abs(x64).max(axis=1)
+    y_ref = oracle.forward(th64, x64)
+    y, xr = Guarded((rows, n + 8), dtype, DEV), Guarded((rows, n), dtype, DEV)
+    check_rows_close(p.forward(x.to(DEV), out=y.view[:, :n]), y_ref, amax, "forward")
+    check_rows_close(p.inverse(x.to(DEV), out=xr.view), oracle.inverse(th64, x64), amax, "inverse")
+    for bits in (2, 4, 8):
+        codes, scales, kept = p.fold_weights(x.to(DEV), bits, want_rotated=True)
+        check_quant(codes, scales, y_ref, bits, f"{bits} bits")
+        assert torch.equal(kept, y.view[:, :n])
+    assert y.intact() and xr.intact() and p.stage_form() == 3 and p.device_status() == 0
