@@ -258,7 +258,8 @@ struct alignas(64) WideHalf {
 struct ShortRows {
     int log;
     int64_t elems;
-    Again again;  // inverse: for rows that are done again
+    RowSource from;  // inverse: for rows that are done again
+    int64_t ldx;     // inverse: row stride of x
 };
 
 template <bool IN_F32, bool WIDE = false, bool SHORT = false>
@@ -860,12 +861,12 @@ struct InvUpper {
 // odd CTAs the upper (CTAs 2i and 2i + 1 work on the same rows at about the same time, so the second read of a row comes
 // from L2).  A y row is 16 KB in one slot; the transposed stage-12 rotation y'_own = c y_own +- s y_other with (cos, sin)
 // from `tw12` is applied as the row is read, then the half's own twelve stages follow from its own tables.
-// STRIDED (SHORT): the short rows of x lie brief.again.ldy apart instead of one after the other.
+// STRIDED (SHORT): the short rows of x lie brief.ldx apart instead of one after the other.
 template <int G, bool OUT_BF16, bool IN_F32 = false, bool WIDE = false, bool SHORT = false, bool STRIDED = false>
 __global__ void __launch_bounds__(G * kThreads, 1)
 k_inv4096(const __grid_constant__ CUtensorMap ymap, const float* __restrict__ img_lo, const float* __restrict__ img_scaled_lo,
           const int* __restrict__ form_lo, const uint32_t* __restrict__ gsign_lo, void* __restrict__ xout, int64_t ldx, int rows,
-          int* __restrict__ status, const float2* __restrict__ tw12, const InvUpper upper, const __grid_constant__ ShortRows brief) {
+          int* __restrict__ status, const float2* __restrict__ tw12, const InvUpper upper, const ShortRows brief) {
     static_assert(!(SHORT && WIDE), "one or the other");
     static_assert(!(IN_F32 && WIDE), "the wide mode takes bf16 rows");
     const int half = WIDE ? int(blockIdx.x & 1u) : 0;
@@ -1086,7 +1087,7 @@ k_inv4096(const __grid_constant__ CUtensorMap ymap, const float* __restrict__ im
             int64_t off = static_cast<int64_t>(row) * ldx + (WIDE ? kN * half : 0) + at;
             if constexpr (SHORT) {
                 if (static_cast<int64_t>(row) * kN + at >= brief.elems) continue;  // past the last row
-                if constexpr (STRIDED) off += (at >> (12 - brief.log)) * (brief.again.ldy - (kN >> brief.log));
+                if constexpr (STRIDED) off += (at >> (12 - brief.log)) * (brief.ldx - (kN >> brief.log));
             }
             if constexpr (OUT_BF16) {
                 uint32_t w[8];
@@ -1128,7 +1129,10 @@ k_inv4096(const __grid_constant__ CUtensorMap ymap, const float* __restrict__ im
     }
     if constexpr (SHORT) {  // rows that are not finite (bfq_row_again.cuh)
         bar_sync(a.bar, kThreads);  // the group's stores are done
-        if (lds32(bad_flag) != 0u) rows_again(brief.again, first, stride, count, a.ex, a.bar, t);
+        if (lds32(bad_flag) != 0u) {
+            const Again again{brief.from, IN_F32 ? kF32 : kBF16, true, 12 - brief.log, brief.elems, 0, xout, brief.ldx, OUT_BF16 ? kBF16 : kF32, nullptr, nullptr};
+            rows_again(again, first, stride, count, a.ex, a.bar, t);
+        }
     }
     tmem_fence_before();
     __syncthreads();
@@ -1333,7 +1337,7 @@ cudaError_t bwd_short_launch(bfq_plan* plan, const void* x, const void* g, int64
     const bool maps = f32 ? (encode_row_map_f32(&xmap, x, rows, n, n) && encode_row_map_f32(&gmap, g, rows, n, n))
                           : (encode_row_map(&xmap, x, rows, n, n) && encode_row_map(&gmap, g, rows, n, n));
     if (!maps) return cudaErrorInvalidValue;
-    const b4k::ShortRows brief{12 - plan->log_n, rows * n, Again{}};
+    const b4k::ShortRows brief{12 - plan->log_n, rows * n, RowSource{}, 0};
     const int64_t joint = (brief.elems + f4k::kN - 1) / f4k::kN, pairs = (joint + 1) / 2;
     const int grid = int(pairs < plan->sm_count ? pairs : plan->sm_count);
     auto kern = f32 ? b4k::k_bwd4096<true, false, true> : b4k::k_bwd4096<false, false, true>;
@@ -1366,8 +1370,7 @@ cudaError_t inv_short_launch(bfq_plan* plan, const void* y, bool y_f32, int64_t 
     const int n = plan->n;
     CUtensorMap ymap;
     if (!(y_f32 ? encode_row_map_f32(&ymap, y, rows, ldy, n) : encode_row_map(&ymap, y, rows, ldy, n))) return cudaErrorInvalidValue;
-    const b4k::ShortRows brief{12 - plan->log_n, rows * n,
-                               Again{y, ldy, y_f32 ? kF32 : kBF16, plan->tw, true, plan->log_n, rows * n, 0, x, ldx, x_bf16 ? kBF16 : kF32, nullptr, nullptr}};
+    const b4k::ShortRows brief{12 - plan->log_n, rows * n, RowSource{y, ldy, plan->tw}, ldx};
     const int64_t joint = (brief.elems + f4k::kN - 1) / f4k::kN, want = (joint + G - 1) / G;
     const int grid = int(want < plan->sm_count ? want : plan->sm_count);
     kern<<<grid, G * b4k::kThreads, S::kBytes, st>>>(ymap, plan->img_b4096, plan->img_i4096, plan->form_flag + 1, plan->gsign4096, x, ldx << (12 - plan->log_n),

@@ -168,13 +168,14 @@ enum : int { kOutInt4 = 0, kOutBf16 = 1, kOutInt4Stats = 2, kOutInt2 = 3, kOutIn
 // that takes the factors off.  A quantized row's maximum is taken over its own part of the 4096.  A row whose results are not
 // finite is done again at the end (bfq_row_again.cuh); to know of one takes eight maxima per thread and joint row where rows go
 // out.
-// STRIDED (rows out alone): the short rows of the output lie again.ldy apart instead of one after the other.
+// STRIDED (rows out alone): the short rows of the output lie ldy >> SUB apart instead of one after the other.
 template <int G, int CW, int XB, int TRANSFORM, int OUT, int STEP = 2, bool ROWS = false, bool IN_F32 = false, int SUB = 0, bool STRIDED = false>
 __global__ void __launch_bounds__(G * kGroupThreads, 1)
 k_fwdq4096(const __grid_constant__ CUtensorMap tmap, const float* __restrict__ img, const int* __restrict__ form,
            uint8_t* __restrict__ codes,
            uint16_t* __restrict__ scales, __nv_bfloat16* __restrict__ yout, int64_t ldy, int rows,
-           int* __restrict__ status, uint32_t tx_bytes, int wait_limit, unsigned long long* __restrict__ hist, int64_t elems, const __grid_constant__ Again again) {
+           int* __restrict__ status, uint32_t tx_bytes, int wait_limit, unsigned long long* __restrict__ hist, int64_t elems,
+           const __grid_constant__ typename std::conditional<SUB != 0, Again, Never>::type again) {
     using S = Smem<G, XB>;
     constexpr bool kTmem = TRANSFORM == kButterfly;
     constexpr bool kCount = OUT == kOutInt4Stats;
@@ -368,7 +369,7 @@ k_fwdq4096(const __grid_constant__ CUtensorMap tmap, const float* __restrict__ i
         // pairs of elements between where register m's would lie in contiguous rows and where they lie
         auto gap = [&](int m) -> int64_t {
             if constexpr (!STRIDED) return 0;
-            else return (SUB < 5 ? m >> (4 - SUB) : 2 * m + (q >> 1)) * ((again.ldy - (kN >> SUB)) / 2);
+            else return (SUB < 5 ? m >> (4 - SUB) : 2 * m + (q >> 1)) * (((ldy >> SUB) - (kN >> SUB)) / 2);
         };
         if constexpr (OUT == kOutBf16 || (ROWS && !IN_F32)) {
             // thread t holds elements 2t + 256m, +1: one 32-bit word of the bf16 row per packed register
@@ -631,8 +632,7 @@ k_fwdq4096(const __grid_constant__ CUtensorMap tmap, const float* __restrict__ i
 
     if constexpr (SUB != 0) {
         bar_sync(ex.bar, kGroupThreads);  // the group's stores are done
-        if (lds32(bad_flag) != 0u)
-            rows_again(again, first, stride, count, sbase + S::kExOff + g * XB * kExBytes, ex.bar, t);
+        if (lds32(bad_flag) != 0u) rows_again(again, first, stride, count, sbase + S::kExOff + g * XB * kExBytes, ex.bar, t);
     }
 
     if constexpr (kCount) {
@@ -666,7 +666,7 @@ k_fwdq4096(const __grid_constant__ CUtensorMap tmap, const float* __restrict__ i
 template <int G, int CW, int XB, int TRANSFORM, int OUT, bool ROWS = false, bool IN_F32 = false, int SUB = 0, bool STRIDED = false>
 static cudaError_t launch_variant(const bfq_plan* plan, const CUtensorMap& tmap, int64_t rows, uint8_t* codes,
                                   uint16_t* scales, void* y, int64_t ldy, cudaStream_t st,
-                                  unsigned long long* hist = nullptr, int64_t elems = 0, const Again& again = Again{}) {
+                                  unsigned long long* hist = nullptr, int64_t elems = 0, const RowSource& source = RowSource{}) {
     using S = f4k::Smem<G, XB>;
     static bool attr_set[kMaxDevices] = {false};
     auto kern = f4k::k_fwdq4096<G, CW, XB, TRANSFORM, OUT, 2, ROWS, IN_F32, SUB, STRIDED>;
@@ -681,6 +681,12 @@ static cudaError_t launch_variant(const bfq_plan* plan, const CUtensorMap& tmap,
     // bytes than arrive, so that every wait runs out (quickly) and reports through the status word
     const uint32_t tx_bytes = (IN_F32 ? 2 : 1) * f4k::kRowBytes + (plan->test_stuck_wait ? 16u : 0u);
     const int wait_limit = plan->test_stuck_wait ? 4096 : (1 << 22);
+    typename std::conditional<SUB != 0, Again, Never>::type again{};
+    if constexpr (SUB != 0) {
+        using namespace f4k;
+        constexpr int kBits = OUT == kOutInt2 ? 2 : (OUT == kOutInt4 ? 4 : (OUT == kOutInt8 ? 8 : 0)), kType = IN_F32 ? kF32 : kBF16;
+        again = Again{source, kType, false, stages_of_sub(SUB), elems, kBits, kBits == 0 || ROWS ? y : nullptr, ldy >> SUB, kType, codes, scales};
+    }
     return launch_overlapped(kern, dim3(grid), dim3(G * f4k::kGroupThreads), S::kBytes, st, tmap, plan->img4096,
                              plan->form_flag, codes, scales, static_cast<__nv_bfloat16*>(y), ldy, int(rows),
                              plan->status_word, tx_bytes, wait_limit, hist, elems, again);

@@ -16,12 +16,10 @@ static cudaError_t fwdq_short_launch(const bfq_plan* plan, const void* x, bool f
     CUtensorMap tmap;
     if (!(f32 ? encode_row_map_f32(&tmap, x, rows, ldx, n) : encode_row_map(&tmap, x, rows, ldx, n))) return cudaErrorInvalidValue;
     const int64_t elems = rows * n, joint = (elems + f4k::kN - 1) / f4k::kN;
-    const int type = f32 ? kF32 : kBF16;
-    const Again again{x, ldx, type, plan->tw, false, 12 - SUB, elems, bits, y, ldy, type, codes, scales};
     using namespace f4k;
     auto go = [&](auto out, auto in_f32, auto rows_too, auto strided) {
         return launch_variant<4, 32, 2, kButterfly, decltype(out)::value, decltype(rows_too)::value, decltype(in_f32)::value, SUB, decltype(strided)::value>(
-            plan, tmap, joint, codes, scales, y, ldy << SUB, st, nullptr, elems, again);
+            plan, tmap, joint, codes, scales, y, ldy << SUB, st, nullptr, elems, RowSource{x, ldx, plan->tw});
     };
     auto of_type = [&](auto in_f32) {
         constexpr int kRowsOut = decltype(in_f32)::value ? kOutF32 : kOutBf16;

@@ -12,11 +12,17 @@
 
 namespace bfq {
 
-struct Again {
-    const void* x;  // the call's input rows, row stride ld
+// the call's input rows, row stride ld, and the plan's (cos, sin): what the kernels do not have anyway
+struct RowSource {
+    const void* x;
     int64_t ld;
+    const float2* tw;
+};
+struct Never {};  // in the place of Again: kernels that never do a row again
+
+struct Again {
+    RowSource from;
     int xtype;
-    const float2* tw;  // the plan's (cos, sin)
     bool inverse;
     int levels;     // log2 of the row length
     int64_t elems;  // elements of all rows
@@ -72,8 +78,8 @@ __device__ __forceinline__ void row_again(const Again& p, int64_t row, uint32_t 
     const int n = 1 << p.levels, half = n >> 1;
     bar_sync(bar, kGroupThreads);  // nobody uses the buffer any more
     for (int e = t; e < n; e += kGroupThreads) {
-        const int64_t at = row * p.ld + e;
-        const float v = p.xtype == kF32 ? static_cast<const float*>(p.x)[at] : __bfloat162float(static_cast<const __nv_bfloat16*>(p.x)[at]);
+        const int64_t at = row * p.from.ld + e;
+        const float v = p.xtype == kF32 ? static_cast<const float*>(p.from.x)[at] : __bfloat162float(static_cast<const __nv_bfloat16*>(p.from.x)[at]);
         sts32(buf + 4 * e, __float_as_uint(v));
     }
     bar_sync(bar, kGroupThreads);
@@ -81,7 +87,7 @@ __device__ __forceinline__ void row_again(const Again& p, int64_t row, uint32_t 
         const int s = p.inverse ? p.levels - 1 - i : i;
         for (int j = t; j < half; j += kGroupThreads) {
             const uint32_t lo = buf + 4 * (((j >> s) << (s + 1)) | (j & ((1 << s) - 1))), hi = lo + (4u << s);
-            const float2 cs = __ldg(p.tw + s * half + j);
+            const float2 cs = __ldg(p.from.tw + s * half + j);
             const float a = __uint_as_float(lds32(lo)), b = __uint_as_float(lds32(hi));
             sts32(lo, __float_as_uint(p.inverse ? cs.x * a + cs.y * b : cs.x * a - cs.y * b));
             sts32(hi, __float_as_uint(p.inverse ? cs.x * b - cs.y * a : cs.y * a + cs.x * b));
