@@ -60,8 +60,8 @@ static int check_rows(const void* p, int dt, int64_t rows, int64_t ld, int n) {
 }
 
 // Rows of 128 .. 2048 elements on the n = 4096 kernels, several as one.  Measured against the generic kernels from 2^13 to
-// 2^25 elements in all (us; bf16, n = 1024; 2^13 / 2^20 / 2^25 elements): codes 8.1 -> 5.2 / 8.7 -> 6.6 / 144 -> 40, rows
-// 7.0 -> 5.0 / 7.6 -> 6.3 / 166 -> 36: always faster.  Inverse 7.2 -> 5.4 / 7.7 -> 6.9 / 168 -> 43, but for n = 128 in fp32
+// 2^25 elements in all (us; bf16, n = 1024; 2^13 / 2^20 / 2^25 elements): codes 8.1 -> 5.2 / 8.7 -> 6.6 / 144 -> 43, rows
+// 7.0 -> 5.0 / 7.6 -> 6.3 / 166 -> 37: always faster.  Inverse 7.2 -> 5.4 / 7.7 -> 6.9 / 168 -> 47, but for n = 128 in fp32
 // the other way round up to 2^20 (8.3 against 10.3; 12.4 against 10.3 at 2^21; bf16 n = 128 8.2 -> 6.2 at 2^13, 8.3 : 8.3 up to
 // 2^20, 18.5 -> 10.3 at 2^22).
 static bool use_short_rows(const bfq_plan* plan, int64_t rows, int64_t min_elems) {

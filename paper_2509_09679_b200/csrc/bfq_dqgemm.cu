@@ -1143,7 +1143,7 @@ static Shape choose_shape(int64_t m, int64_t n, int kblocks, int term_pairs, int
 }
 
 // Up to eight rows of A one pass over the codes is faster than tiles at every size measured (1 row, us, tiles -> pass:
-// 1024 x 1024 at 2 bits 7.7 -> 2.5, 4096 x 4096 25 -> 7.0, 28672 x 8192 104 -> 44; 8 rows 8.1 -> 3.0, 26 -> 9.4, 105 -> 75).  More
+// 1024 x 1024 at 2 bits 7.7 -> 2.8, 4096 x 4096 25 -> 9.4, 28672 x 8192 104 -> 44; 8 rows 8.1 -> 3.2, 26 -> 13, 105 -> 76).  More
 // rows are more passes, worth it while they are small together.
 static bool use_few_rows(const Operand& u, const Operand& v, int64_t k) {
     if (!is_codes(u.kind) || u.transposed || v.kind == BFQ_OP_F32 || v.transposed || k >= (is_codes(v.kind) ? 1 << 17 : 1 << 30)) return false;

@@ -166,8 +166,8 @@ enum : int { kOutInt4 = 0, kOutBf16 = 1, kOutInt4Stats = 2, kOutInt2 = 3, kOutIn
 // elements, the last one may be short: its missing rows arrive as zeros and are not stored).  The absent stages are passed
 // over, not multiplied by 1 and 0 (no row may touch another one's infinities); the general last stage becomes a diagonal
 // that takes the factors off.  A quantized row's maximum is taken over its own part of the 4096.  A row whose results are not
-// finite is done again at the end (bfq_row_again.cuh); to know of one takes eight maxima per thread and joint row where rows go
-// out.
+// finite is done again at the end (bfq_row_again.cuh); to know of one takes sixteen maxima per thread and joint row where
+// rows go out.
 // STRIDED (rows out alone): the short rows of the output lie ldy >> SUB apart instead of one after the other.
 template <int G, int CW, int XB, int TRANSFORM, int OUT, int STEP = 2, bool ROWS = false, bool IN_F32 = false, int SUB = 0, bool STRIDED = false>
 __global__ void __launch_bounds__(G * kGroupThreads, 1)
@@ -394,12 +394,7 @@ k_fwdq4096(const __grid_constant__ CUtensorMap tmap, const float* __restrict__ i
         }
         if constexpr (OUT == kOutBf16 || OUT == kOutF32) {
             bar_sync(ex.bar, kGroupThreads);  // every warp is past its reads of the second regrouping buffer
-            if constexpr (SUB != 0) {
-                // the last stage's pairs lie in registers 2^(3 - SUB) apart, or (n <= 256) in other warps
-                constexpr int kSkip = SUB < 4 ? 8 >> SUB : 0;
-                if (SUB < 4 || (SUB == 4 ? q < 2 : (q & 1) == 0))
-                    sts32_if(__float_as_uint(largest<kSkip>(P)) >= not_finite(OUT == kOutBf16), bad_flag, 1u);
-            }
+            if constexpr (SUB != 0) sts32_if(__float_as_uint(largest<0>(P)) >= not_finite(OUT == kOutBf16), bad_flag, 1u);
             continue;
         }
 

@@ -46,8 +46,9 @@ __device__ __forceinline__ float max_abs_nan(float m, float a, float b) {
     return r;
 }
 
-// The largest magnitude among the thread's elements in registers m with (m & SKIP) == 0, NaN if there is one.  One element of
-// each pair of the last stage tells of both: the results of a rotation with an infinity or NaN in it are not finite.
+// The largest magnitude among the thread's elements in registers m with (m & SKIP) == 0, NaN if there is one.  The inverse's last
+// stage multiplies the factors out, so that an infinity or NaN in either element of a pair is in both results: it looks at one of
+// them.  The forward's last stage may overflow in one element alone.
 template <int SKIP>
 __device__ __forceinline__ float largest(const u64 (&P)[16]) {
     float r[2] = {0.f, 0.f};
@@ -119,11 +120,11 @@ __device__ __forceinline__ void row_again(const Again& p, int64_t row, uint32_t 
     }
 }
 
-// The group's joint rows first, first + stride, ...: those of their rows that are not finite (for rows out, in the elements
-// that `largest` looks at: lower ones of the last stage's pairs).  A quantized row of that kind has a NaN for its scale
+// The group's joint rows first, first + stride, ...: those of their rows that are not finite (in the elements that `largest`
+// looks at: in the inverse the lower ones of the last stage's pairs).  A quantized row of that kind has a NaN for its scale
 // (row_scale_fast of an infinite or NaN maximum; no finite row has).
 static __device__ __noinline__ void rows_again(const Again& p, int first, int stride, int count, uint32_t buf, int bar, int t) {
-    const int n = 1 << p.levels, upper = p.inverse ? 1 : n >> 1;
+    const int n = 1 << p.levels, upper = p.inverse ? 1 : 0;
     for (int k = 0; k < count; ++k) {
         int64_t row = (static_cast<int64_t>(first) + static_cast<int64_t>(k) * stride) << (12 - p.levels);
         for (const int64_t end = row + (4096 >> p.levels); row < end && (row << p.levels) < p.elems; ++row) {

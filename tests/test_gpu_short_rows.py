@@ -270,3 +270,26 @@ def test_angles_that_need_the_three_shear_form(n, dtype):
         check_quant(codes, scales, y_ref, bits, f"{bits} bits")
         assert torch.equal(kept, y.view[:, :n])
     assert y.intact() and xr.intact() and p.stage_form() == 3 and p.device_status() == 0
+
+
+@pytest.mark.parametrize("n", [128, 256, 512, 1024, 2048])
+@pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
+@pytest.mark.parametrize("upper", [True, False])
+def test_an_overflow_in_one_element_of_the_last_stage(n, dtype, upper):
+    """Small factors in one half of the row only: of a pair of the forward's last stage one quotient overflows, the other
+    does not."""
+    theta = synth.angles(n, "zero", 1)
+    half = slice(n // 4, None) if upper else slice(0, n // 4)
+    theta[2:4, half] = math.pi / 2
+    theta[-1] = 0.5
+    x = synth.rows(4096 // n * 3, n, "normal", 4, dtype=dtype)
+    x[1, (slice(0, n // 2) if upper else slice(n // 2, None))] *= 1e30
+    p = Plan(n, DEV)
+    p.set_angles(theta.to(DEV))
+    assert p.stage_form() & 1 == 0
+    th64, x64 = to_f64(theta), to_f64(x)
+    amax = np.abs(x64).max(axis=1)
+    y_ref = oracle.forward(th64, x64)
+    check_rows_close(p.forward(x.to(DEV)), y_ref, amax, "forward")
+    check_rows_close(p.inverse(x.to(DEV)), oracle.inverse(th64, x64), amax, "inverse")
+    assert torch.equal(p.forward_quant(x.to(DEV), 8)[1][1], torch.tensor(65504.0, dtype=torch.float16, device=DEV))
