@@ -4,8 +4,8 @@
 // A CTA keeps a token in shared memory; the butterfly runs in passes of three stages in registers (two runs packed into one
 // instruction), the dense factor with eight output runs x four positions per thread (packed), then one maximum and the codes.
 // The kernel for every shape does one stage per barrier, element by element: 32768 tokens of 40 x 128 at INT2 took
-// 2.07 ms there and take 0.93 ms here (40000 of 12 x 256: 1.43 -> 0.62 ms, 18000 of 7 x 1024: 1.70 -> 0.47 ms; one token 24 us
-// with the call's host side either way).
+// 2.07 ms there and take 0.93 ms here (40000 of 12 x 256: 1.43 -> 0.62 ms, 18000 of 7 x 1024: 1.70 -> 0.47 ms; one token 11.4 us,
+// most of it the call).
 #include "../../include/bfq.h"
 
 #include <cuda_runtime.h>
