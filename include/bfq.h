@@ -107,7 +107,7 @@ int bfq_forward_quant(bfq_plan* plan, const void* x, bfq_dtype xt, int64_t rows,
  *   rowstats [rows][2] fp32: sum_k y_k^2 and sum_k y_k^4 of each row (kurtosis n * s4 / s2^2, sigma^2 = s2 / n,
  *            max|y| / sigma with the row's scale: the diagnostics of the paper's kurtosis / outlier tables).
  * Counts are exact for the codes written; the sums are taken in a fixed order (bit-reproducible).  Where this call runs another
- * kernel than bfq_forward_quant (n >= 128, all but bf16 rows of 4096 at 4 bits) a code whose value lies within fp32 rounding of a
+ * kernel than bfq_forward_quant (n >= 4096, all but bf16 rows of 4096 at 4 bits) a code whose value lies within fp32 rounding of a
  * boundary may be the neighbouring one.
  */
 int bfq_forward_quant_stats(bfq_plan* plan, const void* x, bfq_dtype xt, int64_t rows, int64_t ldx, int bits,

@@ -448,6 +448,11 @@ static int forward_quant_impl(bfq_plan* plan, const void* x, int xt, int64_t row
     GenericParams p{};
     p.tw = plan->tw, p.x = x, p.xt = xt, p.ldx = ldx, p.y = y, p.yt = yt, p.ldy = plan->n;
     p.codes = codes, p.scales = scales, p.bits = bits, p.rows = rows, p.hist = hist, p.rowstats = rowstats;
+    if (hist != nullptr && use_short_rows(plan, rows, 0)) {  // the codes of bfq_forward_quant, then their counts and the moments
+        e = fwdq_short_launch(plan, x, xt == BFQ_F32, rows, ldx, bits, codes, scales, nullptr, plan->n, static_cast<cudaStream_t>(stream));
+        if (e == cudaSuccess) e = launch_generic<kModeForwardCount>(plan, p, static_cast<cudaStream_t>(stream));
+        return e == cudaSuccess ? BFQ_OK : cuda_fail(plan, e);
+    }
     e = launch_generic<kModeForwardQuant>(plan, p, static_cast<cudaStream_t>(stream));
     return e == cudaSuccess ? BFQ_OK : cuda_fail(plan, e);
 }

@@ -18,7 +18,7 @@
 namespace bfq {
 
 enum : int { kF32 = 0, kBF16 = 1 };
-enum : int { kModeForward = 0, kModeForwardQuant = 1, kModeInverse = 2, kModeHadamard = 3, kModeHadamardQuant = 4 };
+enum : int { kModeForward = 0, kModeForwardQuant = 1, kModeInverse = 2, kModeHadamard = 3, kModeHadamardQuant = 4, kModeForwardCount = 5 };
 
 struct GenericParams {
     const float2* tw;  // [L][n/2] (cos, sin)
@@ -328,7 +328,7 @@ __global__ void __launch_bounds__(Geo<LOG_N>::kThreads) k_generic(const GenericP
     extern __shared__ __align__(16) float smem[];
     float* red = smem + G::kGroups * R * G::kN;  // [R][kGroups][warps per row]
     unsigned int* shist = reinterpret_cast<unsigned int*>(red + R * G::kGroups * G::kWarpsPerRow);  // [256], stats only
-    const bool stats = (MODE == kModeForwardQuant || MODE == kModeHadamardQuant) && p.hist != nullptr;
+    const bool stats = MODE == kModeForwardCount || ((MODE == kModeForwardQuant || MODE == kModeHadamardQuant) && p.hist != nullptr);
     if (stats) {
         for (int i = threadIdx.x; i < 256; i += blockDim.x) shist[i] = 0u;
         __syncthreads();
@@ -401,6 +401,47 @@ __global__ void __launch_bounds__(Geo<LOG_N>::kThreads) k_generic(const GenericP
                         const int qmin = -(1 << (p.bits - 1));
 #pragma unroll
                         for (int e = 0; e < 16; ++e) atomicAdd(&shist[quant1(v[r][e], inv, qmin, qmax) - qmin], 1u);
+                    }
+                }
+            }
+            if constexpr (G::kTPR >= 32) __syncthreads();  // red[] is reused by the next tile
+        }
+        if constexpr (MODE == kModeForwardCount) {  // codes and scales are there already: their counts and the rows' moments
+            const int64_t row_bytes = (static_cast<int64_t>(G::kN) * p.bits) >> 3;
+            const uint32_t mask = (1u << p.bits) - 1u, flip = 1u << (p.bits - 1);
+#pragma unroll
+            for (int r = 0; r < R; ++r) {
+                uint32_t w[4] = {0u, 0u, 0u, 0u};  // the thread's 16 codes
+                if (row0 + r < p.rows) {
+                    const uint8_t* mine = p.codes + (row0 + r) * row_bytes + t * 2 * p.bits;
+                    if (p.bits == 2) {
+                        w[0] = *reinterpret_cast<const uint32_t*>(mine);
+                    } else if (p.bits == 4) {
+                        const uint2 u = *reinterpret_cast<const uint2*>(mine);
+                        w[0] = u.x, w[1] = u.y;
+                    } else {
+                        const uint4 u = *reinterpret_cast<const uint4*>(mine);
+                        w[0] = u.x, w[1] = u.y, w[2] = u.z, w[3] = u.w;
+                    }
+                }
+                float s2 = 0.f, s4 = 0.f;
+#pragma unroll
+                for (int e = 0; e < 16; ++e) {
+                    const float sq = v[r][e] * v[r][e];
+                    s2 += sq;
+                    s4 = fmaf(sq, sq, s4);
+                }
+                s2 = row_sum<LOG_N>(s2, red, r, group, t);
+                s4 = row_sum<LOG_N>(s4, red, r, group, t);
+                if (row0 + r < p.rows) {
+                    if (t == 0) {
+                        p.rowstats[2 * (row0 + r)] = s2;
+                        p.rowstats[2 * (row0 + r) + 1] = s4;
+                    }
+#pragma unroll
+                    for (int e = 0; e < 16; ++e) {
+                        const uint32_t word = p.bits == 2 ? w[0] : (p.bits == 4 ? w[e >> 3] : w[e >> 2]);
+                        atomicAdd(&shist[((word >> ((e * p.bits) & 31)) & mask) ^ flip], 1u);
                     }
                 }
             }

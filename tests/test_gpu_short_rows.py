@@ -293,3 +293,19 @@ def test_an_overflow_in_one_element_of_the_last_stage(n, dtype, upper):
     check_rows_close(p.forward(x.to(DEV)), y_ref, amax, "forward")
     check_rows_close(p.inverse(x.to(DEV)), oracle.inverse(th64, x64), amax, "inverse")
     assert torch.equal(p.forward_quant(x.to(DEV), 8)[1][1], torch.tensor(65504.0, dtype=torch.float16, device=DEV))
+
+
+@pytest.mark.parametrize("n", [128, 256, 512, 1024, 2048])
+@pytest.mark.parametrize("dtype,bits", [(torch.float32, 8), (torch.bfloat16, 4), (torch.float32, 2)])
+def test_statistics_count_the_codes_of_the_call_without_them(n, dtype, bits):
+    rows = (1 << 20) // n + 3
+    p = Plan(n, DEV)
+    theta = synth.angles(n, "uniform", 3)
+    p.set_angles(theta.to(DEV))
+    x = synth.rows(rows, n, "student_t3", 4, dtype=dtype)
+    x[5] = 0.0
+    codes, scales, hist, moments = p.forward_quant_stats(x.to(DEV), bits)
+    plain = p.forward_quant(x.to(DEV), bits)
+    assert torch.equal(codes, plain[0]) and torch.equal(scales, plain[1])
+    assert np.array_equal(hist.cpu().numpy(), oracle.code_histogram(oracle.unpack(codes.cpu().numpy(), bits), bits))
+    np.testing.assert_allclose(to_f64(moments), oracle.row_moments(oracle.forward(to_f64(theta), to_f64(x))), rtol=2e-5)
