@@ -229,8 +229,8 @@ int bfq_plan_create(bfq_plan** out, int n, int64_t max_rows, int device) {
     plan->partial_floats = size_t(plan->partial_slots) * angles;
     if (n == 8192 && plan->partial_floats < bwd8192_partial_floats(plan->sm_count))
         plan->partial_floats = bwd8192_partial_floats(plan->sm_count);
-    if (n >= 128 && n < 4096 && plan->partial_floats < bwd_short_partial_floats(plan->sm_count))
-        plan->partial_floats = bwd_short_partial_floats(plan->sm_count);
+    if (n >= 128 && n <= 4096 && plan->partial_floats < grad4096_partial_floats(plan->sm_count))
+        plan->partial_floats = grad4096_partial_floats(plan->sm_count);
     // all device memory in one allocation
     struct Part {
         void** at;
@@ -244,9 +244,10 @@ int bfq_plan_create(bfq_plan** out, int n, int64_t max_rows, int device) {
     if (n >= 128 && n <= 4096) {
         want(&plan->img4096, fwdq4096_image_bytes());
         want(&plan->prep4096, fwdq4096_prep_bytes());
+        want(&plan->weight4096, grad4096_weight_bytes());
+        want(&plan->slot_form, sizeof(int) * plan->sm_count);
         want(&plan->img_b4096, bwd4096_image_bytes());
         want(&plan->img_i4096, inv4096_image_bytes());
-        want(&plan->dsign4096, bwd4096_dsign_bytes());
         want(&plan->gsign4096, bwd4096_gsign_bytes());
     }
     if (n == 8192) {
@@ -261,7 +262,7 @@ int bfq_plan_create(bfq_plan** out, int n, int64_t max_rows, int device) {
         want(&plan->prep_half8192, bwd8192_prep_bytes());
     }
     if (n == 128) want(&plan->dense128, comp5120d_image_bytes());
-    want(&plan->status_word, 4 * sizeof(int));
+    want(&plan->status_word, 5 * sizeof(int));
     size_t total = 0;
     for (int i = 0; i < n_parts; ++i) total += parts[i].bytes;
     e = cudaMalloc(&plan->arena, total);
@@ -280,7 +281,7 @@ int bfq_plan_create(bfq_plan** out, int n, int64_t max_rows, int device) {
     if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&plan->host_in, cudaStreamNonBlocking);
     if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&plan->host_out, cudaStreamNonBlocking);
     for (int i = 0; i < 8 && e == cudaSuccess; ++i) e = cudaEventCreateWithFlags(&plan->host_ev[i], cudaEventDisableTiming);
-    if (e == cudaSuccess) e = cudaMemset(plan->status_word, 0, 4 * sizeof(int));
+    if (e == cudaSuccess) e = cudaMemset(plan->status_word, 0, 5 * sizeof(int));
     if (e == cudaSuccess) plan->form_flag = plan->status_word + 1;
     if (e == cudaSuccess) e = cudaDeviceSynchronize();
     if (e != cudaSuccess) {
@@ -651,7 +652,7 @@ int bfq_inverse(bfq_plan* plan, const void* y, bfq_dtype yt, int64_t rows, int64
         return e == cudaSuccess ? BFQ_OK : cuda_fail(plan, e);
     }
     if ((yt == BFQ_BF16 || xt == BFQ_F32) && x != y && use_short_rows(plan, rows, short_inverse_from(plan->n, yt == BFQ_F32)) &&
-        bwd_short_available(plan)) {
+        inv_short_available(plan)) {
         cudaError_t e = inv_short_launch(plan, y, yt == BFQ_F32, rows, ldy, x, xt == BFQ_BF16, ldx, static_cast<cudaStream_t>(stream));
         return e == cudaSuccess ? BFQ_OK : cuda_fail(plan, e);
     }
@@ -679,13 +680,8 @@ int bfq_backward(bfq_plan* plan, const void* x, bfq_dtype xt, const void* g, bfq
         return e == cudaSuccess ? BFQ_OK : cuda_fail(plan, e);
     }
     if (xt == gt && (dx == nullptr || dxt == xt) && rows < (int64_t(1) << 31) - 1 && !env_flag("BFQ_GENERIC_ONLY") &&
-        bwd4096_available(plan)) {  // all rows bf16, or all fp32
-        cudaError_t e = cudaSuccess;
-        if (!plan->bwd_tables_valid) {  // built on first use after bfq_set_angles, on the caller's stream
-            e = bwd4096_build_tables(plan, st);
-            plan->bwd_tables_valid = (e == cudaSuccess);
-        }
-        if (e == cudaSuccess) e = bwd4096_launch(plan, x, g, rows, ld, dx, dtheta, xt == BFQ_F32, st);
+        plan->n == 4096 && grad4096_available(plan)) {  // all rows bf16, or all fp32
+        cudaError_t e = grad4096_launch(plan, x, g, rows, ld, dx, dtheta, xt == BFQ_F32, st);
         return e == cudaSuccess ? BFQ_OK : cuda_fail(plan, e);
     }
     if (xt == BFQ_BF16 && gt == BFQ_BF16 && (dx == nullptr || dxt == BFQ_BF16) && rows < (int64_t(1) << 31) - 1 &&
@@ -699,8 +695,8 @@ int bfq_backward(bfq_plan* plan, const void* x, bfq_dtype xt, const void* g, bfq
         if (e == cudaSuccess) e = bwd8192_launch_halves(plan, x, g, rows, ld, dx, dtheta, st);
         return e == cudaSuccess ? BFQ_OK : cuda_fail(plan, e);
     }
-    if (takes_short_backward(plan->n, xt, gt, dx != nullptr, dxt, rows, ld) && bwd_short_available(plan)) {
-        cudaError_t e = bwd_short_launch(plan, x, g, rows, dx, dtheta, xt == BFQ_F32, st);
+    if (takes_short_backward(plan->n, xt, gt, dx != nullptr, dxt, rows, ld) && grad4096_available(plan)) {
+        cudaError_t e = grad4096_launch(plan, x, g, rows, ld, dx, dtheta, xt == BFQ_F32, st);
         return e == cudaSuccess ? BFQ_OK : cuda_fail(plan, e);
     }
     BackwardParams p{};

@@ -23,6 +23,7 @@
 #include "bfq_fast.h"
 #include "bfq_generic.cuh"
 #include "bfq_n4096.cuh"
+#include "bfq_regroup.cuh"
 #include "bfq_row_again.cuh"
 
 namespace bfq {
@@ -30,7 +31,6 @@ namespace b4k {
 using namespace ptx;
 using namespace f4k;
 
-constexpr int kThreads = 128;                // one group; the CTA has two (reverse = threads 0..127, forward = 128..255)
 constexpr int kCtaThreads = 2 * kThreads;
 constexpr int kSlots = 2;                    // TMA ring depth (row pairs), x and g rings separately
 constexpr int kBarRev = 1, kBarFwd = 2, kBarFull = 3, kBarEmpty = 4;  // named barriers
@@ -60,58 +60,6 @@ struct Smem {
 static_assert(Smem::kBytesWide <= 232448, "shared memory budget of one CTA");
 constexpr int kSlotFloats = 12 * (kN / 2);            // one CTA's sums of stages 0 .. 11
 constexpr int kSlotFloatsWide = kSlotFloats + kN;     // ... followed by its share of stage 12's (wide mode)
-
-__device__ __forceinline__ void sts128(uint32_t a, uint4 v) {
-    asm volatile("st.shared.v4.u32 [%0], {%1,%2,%3,%4};" ::"r"(a), "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w) : "memory");
-}
-
-struct Addr {
-    uint32_t w1, r1, w2, r2;  // per-thread byte offsets inside a regrouping buffer (forward write / read sides)
-    uint32_t ex;              // base of the group's regrouping buffers
-    int bar;                  // the group's named barrier
-};
-
-// ---- regroupings: forward direction (phase 1 -> 2 -> 3) and back, one row array at a time -------------
-__device__ __forceinline__ void fwd1_store(const u64 (&P)[16], uint32_t buf, const Addr& a) {
-#pragma unroll
-    for (int m = 0; m < 16; ++m) sts64(buf + a.w1 + ex1_wr_local(m), P[m]);
-}
-__device__ __forceinline__ void fwd1_load(u64 (&P)[16], uint32_t buf, const Addr& a) {
-#pragma unroll
-    for (int m = 0; m < 16; ++m) P[m] = lds64(buf + a.r1 + ex1_rd_local(m));
-}
-__device__ __forceinline__ void fwd2_store(const u64 (&P)[16], uint32_t buf, const Addr& a) {
-#pragma unroll
-    for (int m = 0; m < 16; ++m) {
-        uint32_t lo, hi;
-        unpack2u(P[m], lo, hi);
-        sts32(buf + a.w2 + ex2_wr_local(m, 0), lo);
-        sts32(buf + a.w2 + ex2_wr_local(m, 1), hi);
-    }
-}
-__device__ __forceinline__ void fwd2_load(u64 (&P)[16], uint32_t buf, const Addr& a) {
-#pragma unroll
-    for (int m = 0; m < 16; ++m) P[m] = lds64(buf + a.r2 + ex2_rd_local(m));
-}
-// back from phase 3 to phase 2: the phase-3 owner stores whole packed registers where it read them,
-// the phase-2 owner reads scalars where it wrote them
-__device__ __forceinline__ void rev2_store(const u64 (&P)[16], uint32_t buf, const Addr& a) {
-#pragma unroll
-    for (int m = 0; m < 16; ++m) sts64(buf + a.r2 + ex2_rd_local(m), P[m]);
-}
-__device__ __forceinline__ void rev2_load(u64 (&P)[16], uint32_t buf, const Addr& a) {
-#pragma unroll
-    for (int m = 0; m < 16; ++m)
-        P[m] = pack2u(lds32(buf + a.w2 + ex2_wr_local(m, 0)), lds32(buf + a.w2 + ex2_wr_local(m, 1)));
-}
-__device__ __forceinline__ void rev1_store(const u64 (&P)[16], uint32_t buf, const Addr& a) {
-#pragma unroll
-    for (int m = 0; m < 16; ++m) sts64(buf + a.r1 + ex1_rd_local(m), P[m]);
-}
-__device__ __forceinline__ void rev1_load(u64 (&P)[16], uint32_t buf, const Addr& a) {
-#pragma unroll
-    for (int m = 0; m < 16; ++m) P[m] = lds64(buf + a.w1 + ex1_wr_local(m));
-}
 
 // ---- d-theta of four pairs (U0..U0+3) of local stage K, both rows:  A[i] += g_hi*y_lo - g_lo*y_hi ------
 template <int K, int U0>
@@ -221,19 +169,6 @@ __device__ __forceinline__ void rev_steps(u64 (&Y0)[16], u64 (&Y1)[16], u64 (&G0
     if constexpr (I + 1 < END) rev_steps<I + 1, END, SHORT>(Y0, Y1, G0, G1, Tnext, Tcur, Anext, Acur, cx, hook);
 }
 
-__device__ __forceinline__ uint32_t cvt_bf16x2(float lo, float hi) {
-    uint32_t r;
-    asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(r) : "f"(hi), "f"(lo));
-    return r;
-}
-
-// element index of (phase P, role t, packed register m, half h)
-__device__ __forceinline__ int elem_of(int P, int t, int m, int h) {
-    if (P == 0) return m | ((t & 15) << 4) | (h << 8) | ((t >> 4) << 9);
-    if (P == 1) return (t & 15) | (m << 4) | (h << 8) | ((t >> 4) << 9);
-    return h | (t << 1) | (m << 8);
-}
-
 // IN_F32: x, g and dx are fp32.  A row pair of x and of g then fills the whole input ring (one slot of 64 KB instead of
 // two of 32 KB): the next pair is requested as soon as the upper group has read g, behind a barrier of that group.
 // WIDE (bf16 rows): the launch handles half `half` of n = 8192 rows, i.e. stages 0 .. 11 of that half, whose tables it
@@ -250,16 +185,6 @@ struct alignas(64) WideHalf {
     const float* img;
     const uint32_t* gsign;
     const int8_t* dsign;
-};
-
-// rows shorter than 4096 (SHORT): 2^log rows of n = 4096 >> log elements go through the kernel as one row of 4096 whose last
-// stages are the identity (they are passed over, so that no row touches another one's infinities); `rows` counts those, the
-// last one may be short (`elems` elements in all, missing ones arrive as zeros).  x, g and dx contiguous.
-struct ShortRows {
-    int log;
-    int64_t elems;
-    RowSource from;  // inverse: for rows that are done again
-    int64_t ldx;     // inverse: row stride of x
 };
 
 template <bool IN_F32, bool WIDE = false, bool SHORT = false>
@@ -687,7 +612,7 @@ __device__ __forceinline__ void build_image_bwd(int k, bool quads, const float4*
     auto at = [quads](int col) { return quads ? (col >> 2) * 512 + (col & 3) : col; };
     strip[at(32 * s + 4 * u + h)] = sg * p.x;
     strip[at(32 * s + 4 * u + h + 2)] = sg * p.y;
-    dsign[k] = static_cast<int8_t>(-(sa * sb));
+    if (dsign != nullptr) dsign[k] = static_cast<int8_t>(-(sa * sb));
 }
 
 // One thread per 32-bit word of a bf16 g row in phase-3 ownership (role t, register m): bit 15 / bit 31 set
@@ -762,7 +687,7 @@ constexpr int kTableBlocks = 2 * kAngleBlocks + kSignBlocks;
 __global__ void __launch_bounds__(256) k_build_tables(const float4* __restrict__ prep, const uint8_t* __restrict__ flip,
                                                        const double2* __restrict__ cs, float* __restrict__ img, int8_t* __restrict__ dsign,
                                                        float* __restrict__ img_inv, int* __restrict__ form, uint32_t* __restrict__ gsign, bool quads,
-                                                       float* __restrict__ img_fwd, int* __restrict__ form_fwd) {
+                                                       float* __restrict__ img_fwd, int* __restrict__ form_fwd, float* __restrict__ weight) {
     grid_dep_launch();
     grid_dep_wait();
     const int b = blockIdx.x;
@@ -773,7 +698,7 @@ __global__ void __launch_bounds__(256) k_build_tables(const float4* __restrict__
     } else if (b < kTableBlocks) {
         build_gsign(256 * (b - 2 * kAngleBlocks) + threadIdx.x, flip, gsign);
     } else {
-        build_image_fwd(256 * (b - kTableBlocks) + threadIdx.x, prep, cs, img_fwd, form_fwd);
+        build_image_fwd(256 * (b - kTableBlocks) + threadIdx.x, prep, cs, img_fwd, form_fwd, weight);
     }
 }
 
@@ -1211,7 +1136,7 @@ cudaError_t bwd8192_build_tables(const bfq_plan* plan, cudaStream_t st) {
         cudaError_t e = cudaMemsetAsync(plan->form_flag + 1 + h, 0, sizeof(int), st);
         if (e != cudaSuccess) return e;
         b4k::k_build_tables<<<b4k::kTableBlocks, 256, 0, st>>>(prep, flip, cs_half, plan->img_b8192[h], plan->dsign8192[h],
-                                                               plan->img_i8192[h], plan->form_flag + 1 + h, plan->gsign8192[h], false, nullptr, nullptr);
+                                                               plan->img_i8192[h], plan->form_flag + 1 + h, plan->gsign8192[h], false, nullptr, nullptr, nullptr);
         e = cudaGetLastError();
         if (e != cudaSuccess) return e;
     }
@@ -1266,8 +1191,7 @@ size_t bwd4096_dsign_bytes() { return size_t(12) * (f4k::kN / 2); }
 size_t bwd4096_gsign_bytes() { return size_t(16) * b4k::kThreads * sizeof(uint32_t); }
 
 bool bwd4096_available(const bfq_plan* plan) {
-    return plan->n == f4k::kN && plan->cc_major == 10 && plan->img_b4096 != nullptr && plan->prep4096 != nullptr &&
-           plan->partial_slots >= plan->sm_count && encode_tiled() != nullptr;
+    return plan->n == f4k::kN && plan->cc_major == 10 && plan->img_b4096 != nullptr && plan->prep4096 != nullptr && encode_tiled() != nullptr;
 }
 
 // Builds the tables of the backward and inverse kernels from the staging area bfq_set_angles filled (it also resets the
@@ -1278,76 +1202,12 @@ cudaError_t bwd4096_build_tables(const bfq_plan* plan, cudaStream_t st, bool for
     const double2* cs = reinterpret_cast<const double2*>(prep + count);
     const uint8_t* flip = reinterpret_cast<const uint8_t*>(cs + count);
     return launch_overlapped(b4k::k_build_tables, dim3(b4k::kTableBlocks + (forward_too ? b4k::kAngleBlocks : 0)), dim3(256), 0, st, prep, flip, cs, plan->img_b4096,
-                             plan->dsign4096, plan->img_i4096, plan->form_flag + 1, plan->gsign4096, plan->n < f4k::kN,
-                             plan->img4096, plan->form_flag);
+                             static_cast<int8_t*>(nullptr), plan->img_i4096, plan->form_flag + 1, plan->gsign4096, plan->n < f4k::kN,
+                             plan->img4096, plan->form_flag, plan->weight4096);
 }
 
-// ---- rows of 128 .. 2048 elements, several as one of 4096 ----------------------------------------------------------
-namespace b4k {
-// dtheta [levels][half] from the slots' [12][2048]: stage s, angle j = the sum over the slots and the 2048 / half row
-// positions r of entry s * 2048 + r * half + j.  A block = 32 lanes x 32 angles (half is a multiple of 32): lane y adds
-// terms y, y + 32, ... in order (term = slot * positions + r), then the lanes are added in order.
-__global__ void __launch_bounds__(1024) k_reduce_short(const float* __restrict__ partial, int slots, int half_log, float* __restrict__ out) {
-    __shared__ float sh[32][33];
-    const int x = threadIdx.x & 31, y = threadIdx.x >> 5;
-    const int k = blockIdx.x * 32 + x, s = k >> half_log, j = k & ((1 << half_log) - 1);
-    const int pos_log = 11 - half_log, terms = slots << pos_log;
-    const float* src = partial + s * (kN / 2) + j;
-    float acc = 0.f;
-#pragma unroll 4
-    for (int i = y; i < terms; i += 32)
-        acc += src[static_cast<int64_t>(i >> pos_log) * kSlotFloats + ((i & ((1 << pos_log) - 1)) << half_log)];
-    sh[y][x] = acc;
-    __syncthreads();
-    if (y == 0) {
-        float a = sh[0][x];
-#pragma unroll
-        for (int i = 1; i < 32; ++i) a += sh[i][x];
-        out[k] = a;
-    }
-}
-}  // namespace b4k
-
-size_t bwd_short_partial_floats(int sm_count) { return size_t(sm_count) * b4k::kSlotFloats; }
-
-bool bwd_short_available(const bfq_plan* plan) {
-    return plan->n >= 128 && plan->n < f4k::kN && plan->cc_major == 10 && plan->img_b4096 != nullptr && plan->img_i4096 != nullptr &&
-           plan->partial_floats >= bwd_short_partial_floats(plan->sm_count) && encode_tiled() != nullptr;
-}
-
-// what the kernels need once per device (a caller that captures does this before)
-cudaError_t bwd_short_prepare(int device) {
-    static bool attr_set[kMaxDevices] = {false};
-    if (!attr_set[device]) {
-        cudaError_t e = cudaFuncSetAttribute(b4k::k_bwd4096<false, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(b4k::Smem::kBytes));
-        if (e == cudaSuccess)
-            e = cudaFuncSetAttribute(b4k::k_bwd4096<true, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(b4k::Smem::kBytes));
-        if (e != cudaSuccess) return e;
-        attr_set[device] = true;
-    }
-    return cudaSuccess;
-}
-
-// x, g, dx contiguous rows, all bf16 or all fp32
-cudaError_t bwd_short_launch(bfq_plan* plan, const void* x, const void* g, int64_t rows, void* dx, float* dtheta, bool f32, cudaStream_t st) {
-    cudaError_t e = bwd_short_prepare(plan->device);
-    if (e != cudaSuccess) return e;
-    const int n = plan->n;
-    CUtensorMap xmap, gmap;
-    const bool maps = f32 ? (encode_row_map_f32(&xmap, x, rows, n, n) && encode_row_map_f32(&gmap, g, rows, n, n))
-                          : (encode_row_map(&xmap, x, rows, n, n) && encode_row_map(&gmap, g, rows, n, n));
-    if (!maps) return cudaErrorInvalidValue;
-    const b4k::ShortRows brief{12 - plan->log_n, rows * n, RowSource{}, 0};
-    const int64_t joint = (brief.elems + f4k::kN - 1) / f4k::kN, pairs = (joint + 1) / 2;
-    const int grid = int(pairs < plan->sm_count ? pairs : plan->sm_count);
-    auto kern = f32 ? b4k::k_bwd4096<true, false, true> : b4k::k_bwd4096<false, false, true>;
-    kern<<<grid, b4k::kCtaThreads, b4k::Smem::kBytes, st>>>(xmap, gmap, plan->img_b4096, plan->gsign4096, plan->dsign4096, dx, f4k::kN, plan->partial,
-                                                          int(joint), plan->status_word, nullptr, b4k::WideHalf{}, brief);
-    e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-    b4k::k_reduce_short<<<plan->log_n * (n / 2) / 32, 1024, 0, st>>>(plan->partial, grid, plan->log_n - 1, dtheta);
-    plan->last_backward_partials = grid;
-    return cudaGetLastError();
+bool inv_short_available(const bfq_plan* plan) {
+    return plan->n >= 128 && plan->n < f4k::kN && plan->cc_major == 10 && plan->img_b4096 != nullptr && plan->img_i4096 != nullptr && encode_tiled() != nullptr;
 }
 
 // y, x: rows of leading dimension ldy, ldx; bf16 -> bf16, bf16 -> fp32 or fp32 -> fp32
@@ -1375,41 +1235,6 @@ cudaError_t inv_short_launch(bfq_plan* plan, const void* y, bool y_f32, int64_t 
     const int grid = int(want < plan->sm_count ? want : plan->sm_count);
     kern<<<grid, G * b4k::kThreads, S::kBytes, st>>>(ymap, plan->img_b4096, plan->img_i4096, plan->form_flag + 1, plan->gsign4096, x, ldx << (12 - plan->log_n),
                                                     int(joint), plan->status_word, nullptr, b4k::InvUpper{}, brief);
-    return cudaGetLastError();
-}
-
-// f32: x, g and dx are fp32 rows (else bf16)
-cudaError_t bwd4096_launch(bfq_plan* plan, const void* x, const void* g, int64_t rows, int64_t ld, void* dx,
-                           float* dtheta, bool f32, cudaStream_t st) {
-    static bool attr_set[kMaxDevices] = {false};
-    if (!attr_set[plan->device]) {
-        cudaError_t e = cudaFuncSetAttribute(b4k::k_bwd4096<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             int(b4k::Smem::kBytes));
-        if (e == cudaSuccess)
-            e = cudaFuncSetAttribute(b4k::k_bwd4096<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(b4k::Smem::kBytes));
-        if (e != cudaSuccess) return e;
-        attr_set[plan->device] = true;
-    }
-    CUtensorMap xmap, gmap;
-    const bool maps = f32 ? (encode_row_map_f32(&xmap, x, rows, ld) && encode_row_map_f32(&gmap, g, rows, ld))
-                          : (encode_row_map(&xmap, x, rows, ld) && encode_row_map(&gmap, g, rows, ld));
-    if (!maps) return cudaErrorInvalidValue;
-    const int64_t pairs = (rows + 1) / 2;
-    const int grid = int(pairs < plan->sm_count ? pairs : plan->sm_count);
-    if (f32) {
-        b4k::k_bwd4096<true><<<grid, b4k::kCtaThreads, b4k::Smem::kBytes, st>>>(xmap, gmap, plan->img_b4096, plan->gsign4096,
-                                                                              plan->dsign4096, dx, ld, plan->partial,
-                                                                              int(rows), plan->status_word, nullptr, b4k::WideHalf{}, b4k::ShortRows{});
-    } else {
-        b4k::k_bwd4096<false><<<grid, b4k::kCtaThreads, b4k::Smem::kBytes, st>>>(xmap, gmap, plan->img_b4096, plan->gsign4096,
-                                                                               plan->dsign4096, dx, ld, plan->partial,
-                                                                               int(rows), plan->status_word, nullptr, b4k::WideHalf{}, b4k::ShortRows{});
-    }
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-    const int count = 12 * (f4k::kN / 2);
-    k_reduce_partials<<<(count + 31) / 32, 256, 0, st>>>(plan->partial, grid, count, dtheta);
-    plan->last_backward_partials = grid;
     return cudaGetLastError();
 }
 

@@ -29,7 +29,7 @@ cudaError_t fwdq4096_launch_f32(const bfq_plan* plan, const void* x, int64_t row
 cudaError_t fwdq4096_launch_stats(const bfq_plan* plan, const void* x, int64_t rows, int64_t ldx, uint8_t* codes,
                                   uint16_t* scales, unsigned long long* hist, float* rowstats, cudaStream_t st);
 
-cudaError_t fwdq4096_prep_angles(const bfq_plan* plan, const float* theta, cudaStream_t st);
+cudaError_t fwdq4096_build_forward(const bfq_plan* plan, const float* theta, cudaStream_t st);
 // rows of 128 .. 2048 elements: several as one of 4096 on the same kernel.  bits = 2, 4, 8: codes + scales, and
 // the rows if y is not null; bits = 0: the rows alone.  Rows are in the type of x, ldy apart (beside codes: contiguous)
 bool fwdq_short_available(const bfq_plan* plan);
@@ -45,13 +45,8 @@ cudaError_t fwdq1024_launch(const bfq_plan* plan, const void* x, bool f32, int64
                            void* y, int64_t ldy, cudaStream_t st);
 cudaError_t fwdq2048_launch(const bfq_plan* plan, const void* x, bool f32, int64_t rows, int64_t ldx, int bits, uint8_t* codes, uint16_t* scales,
                            void* y, int64_t ldy, cudaStream_t st);
-// the same rows backward and inverse.  takes_short_backward: whether bfq_backward (and bfq_backward_noalloc, whose dx are the
-// same bits) hands a call to bwd_short_launch
-bool takes_short_backward(int n, int xt, int gt, bool want_dx, int dxt, int64_t rows, int64_t ld);
-size_t bwd_short_partial_floats(int sm_count);
-bool bwd_short_available(const bfq_plan* plan);
-cudaError_t bwd_short_prepare(int device);
-cudaError_t bwd_short_launch(bfq_plan* plan, const void* x, const void* g, int64_t rows, void* dx, float* dtheta, bool f32, cudaStream_t st);
+// the same rows inverse
+bool inv_short_available(const bfq_plan* plan);
 cudaError_t inv_short_launch(bfq_plan* plan, const void* y, bool y_f32, int64_t rows, int64_t ldy, void* x, bool x_bf16, int64_t ldx, cudaStream_t st);
 
 // n = 8192, bf16 rows, INT2 (INT4 / INT8 through another epilogue): two-CTA clusters, one 4096-point half per CTA
@@ -70,7 +65,17 @@ cudaError_t fwdq8192_launch_hadamard(const bfq_plan* plan, const void* x, int64_
 cudaError_t fwdq8192_launch_bf16(const bfq_plan* plan, const void* x, int64_t rows, int64_t ldx, void* y, int64_t ldy,
                                  cudaStream_t st);
 
-// n = 4096, bf16 x / g / dx: backward with tensor-memory constants and accumulators
+// rows of 128 .. 4096 elements (below 4096: contiguous, several as one row), x, g and dx all bf16 or all fp32: backward with
+// tensor-memory constants and accumulators, from the tables of the forward kernel.  takes_short_backward: whether bfq_backward
+// (and bfq_backward_noalloc, whose dx are the same bits) hands a call with n < 4096 to grad4096_launch
+bool takes_short_backward(int n, int xt, int gt, bool want_dx, int dxt, int64_t rows, int64_t ld);
+size_t grad4096_weight_bytes();
+size_t grad4096_partial_floats(int ctas);
+bool grad4096_available(const bfq_plan* plan);
+cudaError_t grad4096_prepare(int device);
+cudaError_t grad4096_launch(bfq_plan* plan, const void* x, const void* g, int64_t rows, int64_t ld, void* dx, float* dtheta, bool f32, cudaStream_t st);
+
+// tables of the inverse, and (dsign) of the backward of the halves of n = 8192
 size_t bwd4096_image_bytes();
 size_t inv4096_image_bytes();
 size_t bwd4096_dsign_bytes();
@@ -87,8 +92,6 @@ cudaError_t inv8192_launch(bfq_plan* plan, const void* y, int64_t rows, int64_t 
 cudaError_t bwd8192_launch_halves(bfq_plan* plan, const void* x, const void* g, int64_t rows, int64_t ld, void* dx,
                                   float* dtheta, cudaStream_t st);
 cudaError_t bwd4096_build_tables(const bfq_plan* plan, cudaStream_t st, bool forward_too = false);  // forward_too: img4096 as well
-cudaError_t bwd4096_launch(bfq_plan* plan, const void* x, const void* g, int64_t rows, int64_t ld, void* dx,
-                           float* dtheta, bool f32, cudaStream_t st);
 
 // n = 4096, bf16 y -> bf16 / fp32 x: inverse (uses the backward tables)
 cudaError_t inv4096_launch_f32(bfq_plan* plan, const void* y, int64_t rows, int64_t ldy, void* x, int64_t ldx,

@@ -46,8 +46,9 @@ __global__ void __launch_bounds__(256) k_prep_angles4096(const float* __restrict
     const int k = blockIdx.x * blockDim.x + threadIdx.x;
     grid_dep_launch();
     grid_dep_wait();
-    // step 2 raises the first word when the scaled form is out of range, the build of the reverse walk the second
-    if (k == 0) form[0] = kFormScaled, form[1] = kFormScaled;
+    // step 2 raises the first word when the scaled form is out of range, and the fourth (backward); the build of the reverse
+    // walk the second
+    if (k == 0) form[0] = kFormScaled, form[1] = kFormScaled, form[3] = kFormScaled;
     if (k >= 12 * (kN / 2)) return;
     const int s = k / (kN / 2), j = k % (kN / 2), half = 1 << (levels - 1);
     const int src = s * half + (j & (half - 1));
@@ -67,10 +68,10 @@ __global__ void __launch_bounds__(256) k_prep_angles4096(const float* __restrict
 
 // Step 2 (one thread per angle): build_image_fwd in bfq_n4096.cuh
 __global__ void __launch_bounds__(256) k_build_image4096(const float4* __restrict__ prep, const double2* __restrict__ cs,
-                                                          float* __restrict__ img, int* __restrict__ form) {
+                                                          float* __restrict__ img, int* __restrict__ form, float* __restrict__ weight) {
     grid_dep_launch();
     grid_dep_wait();
-    build_image_fwd(blockIdx.x * blockDim.x + threadIdx.x, prep, cs, img, form);
+    build_image_fwd(blockIdx.x * blockDim.x + threadIdx.x, prep, cs, img, form, weight);
 }
 
 }  // namespace f4k
@@ -82,7 +83,7 @@ size_t fwdq4096_image_bytes() { return size_t(2) * 128 * f4k::kCols * sizeof(flo
 size_t fwdq4096_prep_bytes() { return size_t(12) * (f4k::kN / 2) * (sizeof(float4) + sizeof(double2) + 1); }
 
 // The generic (cos, sin) table and the staging entries of every image (one launch).
-cudaError_t fwdq4096_prep_angles(const bfq_plan* plan, const float* theta, cudaStream_t st) {
+static cudaError_t fwdq4096_prep_angles(const bfq_plan* plan, const float* theta, cudaStream_t st) {
     const int count = 12 * (f4k::kN / 2);
     float4* prep = reinterpret_cast<float4*>(plan->prep4096);
     double2* cs = reinterpret_cast<double2*>(prep + count);
@@ -96,14 +97,20 @@ cudaError_t fwdq4096_prep_angles(const bfq_plan* plan, const float* theta, cudaS
 // 7.7 us on the GPU, now 5.4; the table of the kernels for every n
 // alone takes 3.1 - 3.6).
 cudaError_t fwdq4096_set_angles(const bfq_plan* plan, const float* theta, cudaStream_t st) {
+    if (plan->n == f4k::kN) return fwdq4096_build_forward(plan, theta, st);
+    const cudaError_t e = fwdq4096_prep_angles(plan, theta, st);
+    return e == cudaSuccess ? bwd4096_build_tables(plan, st, true) : e;
+}
+
+// the forward tables alone, which are the backward kernel's too
+cudaError_t fwdq4096_build_forward(const bfq_plan* plan, const float* theta, cudaStream_t st) {
     const int count = 12 * (f4k::kN / 2);
-    cudaError_t e = fwdq4096_prep_angles(plan, theta, st);
+    const cudaError_t e = fwdq4096_prep_angles(plan, theta, st);
     if (e != cudaSuccess) return e;
-    if (plan->n < f4k::kN) return bwd4096_build_tables(plan, st, true);
     float4* prep = reinterpret_cast<float4*>(plan->prep4096);
     double2* cs = reinterpret_cast<double2*>(prep + count);
     return launch_overlapped(f4k::k_build_image4096, dim3((count + 255) / 256), dim3(256), 0, st, prep, cs, plan->img4096,
-                             plan->form_flag);
+                             plan->form_flag, plan->weight4096);
 }
 
 // rows of 128 .. 2048 elements: several as one of 4096.  bits = 0: the rotated rows, in the type of x.

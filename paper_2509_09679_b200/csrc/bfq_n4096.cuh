@@ -197,10 +197,11 @@ __device__ __forceinline__ double factor_before(const double2* __restrict__ cs, 
 }
 
 // One thread per angle: place the constants of pair (s, j) in both tensor-memory images
-// img[form][role][column], with the role / register / half of the pair's low element in its phase, and raise *form
-// when an element's factor leaves the range the scaled form is used in.
+// img[form][role][column], with the role / register / half of the pair's low element in its phase, and raise form[0]
+// when an element's factor leaves the range the scaled form is used in, form[3] when it leaves that of the backward kernel;
+// weight[form][angle] = the product of the factors with which the pair's elements enter the stage.
 __device__ __forceinline__ void build_image_fwd(int k, const float4* __restrict__ prep, const double2* __restrict__ cs, float* __restrict__ img,
-                                                int* __restrict__ form) {
+                                                int* __restrict__ form, float* __restrict__ weight) {
     if (k >= 12 * (kN / 2)) return;
     const int s = k / (kN / 2), j = k % (kN / 2);
     const int lo = ((j >> s) << (s + 1)) | (j & ((1 << s) - 1));
@@ -219,6 +220,8 @@ __device__ __forceinline__ void build_image_fwd(int k, const float4* __restrict_
     const int u = ((m >> (kk + 1)) << kk) | (m & ((1 << kk) - 1));
     const float4 p = prep[k];
     const double2 own = cs[k];
+    weight[k] = static_cast<float>(da * db);
+    weight[12 * (kN / 2) + k] = sa == sb ? 1.f : -1.f;
     // image layout [column quad][role][4]: column col of role r is word ((col >> 2) * 128 + r) * 4 + (col & 3)
     float* scaled = img + kFormScaled * (128 * kCols) + 4 * r;
     float* shear = img + kFormShear * (128 * kCols) + 4 * r;
@@ -232,7 +235,10 @@ __device__ __forceinline__ void build_image_fwd(int k, const float4* __restrict_
         scaled[at(32 * s + 4 * u + h)] = static_cast<float>(-w * db * db);
         scaled[at(32 * s + 4 * u + h + 2)] = static_cast<float>(w * da * da);
         const double lim = 5.421010862427522e-20;  // 2^-64
-        if (!(fabs(own.x * da) >= lim && fabs(own.x * db) >= lim)) *form = kFormShear;
+        const double lim_grad = 9.094947017729282e-13;  // 2^-40
+        const double least = fmin(fabs(own.x * da), fabs(own.x * db));
+        if (!(least >= lim)) form[0] = kFormShear;
+        if (!(least >= lim_grad)) form[3] = kFormShear;
     } else {
         const int col = 352 + 8 * u + h;
         shear[at(col + 0)] = p.z * sa;

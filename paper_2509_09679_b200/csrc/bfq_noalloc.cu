@@ -11,7 +11,7 @@
 //
 // The kernel is chosen by the rule of bfq_backward, so that dx is the same bits either way: calls it
 // takes to the n = 4096 kernel come here with the tables built in the array on every call and as many
-// CTAs as the rest of it holds partial sums for (72 at 96 KiB each).
+// CTAs as the rest of it holds partial sums for (69 at 96 KiB each).
 //
 // Consequences of the shared array: the row length is limited to BFQ_NOALLOC_MAX_N; all calls (from
 // any stream or thread) use the same bytes, so two calls that overlap on one GPU race; the array
@@ -52,7 +52,7 @@ static cudaError_t setup(int device, PerDevice** out) {
         e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device);
         int major = 0;
         if (e == cudaSuccess) e = cudaDeviceGetAttribute(&major, cudaDevAttrComputeCapabilityMajor, device);
-        if (e == cudaSuccess) e = bwd_short_prepare(device);
+        if (e == cudaSuccess) e = grad4096_prepare(device);
         if (e != cudaSuccess) return e;
         d.sm_count = sms, d.cc_major = major;
         d.base = p;
@@ -98,7 +98,7 @@ static cudaError_t launch(int device, const PerDevice& d, BackwardParams p, cons
     return cudaGetLastError();
 }
 
-// The array as a plan's tables and partial sums, as far as bwd_short_launch uses them.
+// The array as a plan's tables and partial sums, as far as grad4096_launch uses them.
 static cudaError_t launch_short(int device, const PerDevice& d, int log_n, const float* theta, const void* x, const void* g, int64_t rows, void* dx, bool f32,
                                 float* dtheta, cudaStream_t st, bool* taken) {
     bfq_plan view;
@@ -111,22 +111,20 @@ static cudaError_t launch_short(int device, const PerDevice& d, int log_n, const
     };
     view.tw = reinterpret_cast<float2*>(part(kTableBytes));
     view.prep4096 = part(fwdq4096_prep_bytes());
-    view.img_b4096 = reinterpret_cast<float*>(part(bwd4096_image_bytes()));
-    view.img_i4096 = reinterpret_cast<float*>(part(inv4096_image_bytes()));
-    view.dsign4096 = reinterpret_cast<int8_t*>(part(bwd4096_dsign_bytes()));
-    view.gsign4096 = reinterpret_cast<uint32_t*>(part(bwd4096_gsign_bytes()));
-    view.status_word = reinterpret_cast<int*>(part(4 * sizeof(int)));
+    view.img4096 = reinterpret_cast<float*>(part(fwdq4096_image_bytes()));
+    view.weight4096 = reinterpret_cast<float*>(part(grad4096_weight_bytes()));
+    view.slot_form = reinterpret_cast<int*>(part(sizeof(int) * d.sm_count));
+    view.status_word = reinterpret_cast<int*>(part(5 * sizeof(int)));
     view.form_flag = view.status_word + 1;
     view.partial = reinterpret_cast<float*>(at);
     const size_t left = kScratchBytes - size_t(at - static_cast<unsigned char*>(d.base));
     view.partial_floats = left / sizeof(float);
-    const int slots = int(left / bwd_short_partial_floats(1) / sizeof(float));
+    const int slots = int(left / grad4096_partial_floats(1) / sizeof(float));
     view.sm_count = slots < d.sm_count ? slots : d.sm_count;  // CTAs
-    *taken = view.sm_count > 0 && bwd_short_available(&view);
+    *taken = view.sm_count > 0 && grad4096_available(&view);
     if (!*taken) return cudaSuccess;
-    cudaError_t e = fwdq4096_prep_angles(&view, theta, st);
-    if (e == cudaSuccess) e = bwd4096_build_tables(&view, st);
-    if (e == cudaSuccess) e = bwd_short_launch(&view, x, g, rows, dx, dtheta, f32, st);
+    cudaError_t e = fwdq4096_build_forward(&view, theta, st);
+    if (e == cudaSuccess) e = grad4096_launch(&view, x, g, rows, view.n, dx, dtheta, f32, st);
     return e;
 }
 

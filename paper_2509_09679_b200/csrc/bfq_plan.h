@@ -21,11 +21,11 @@ struct bfq_plan {
     // these are built by bfq_set_angles
     float* img4096 = nullptr;    // [128][416] tensor-memory image of the rotation constants (n = 128 .. 4096)
     void* prep4096 = nullptr;    // staging for the image build: per-angle constants and negation flags (n = 128 .. 4096)
-    float* img_b4096 = nullptr;  // [128][384] (n < 4096: [96][128][4]) constants of the backward kernel (n = 128 .. 4096)
+    float* weight4096 = nullptr; // [2 forms][12][2048] what the backward kernel's sums are multiplied by (n = 128 .. 4096)
+    float* img_b4096 = nullptr;  // [128][384] (n < 4096: [96][128][4]) three-shear constants of the inverse kernel (n = 128 .. 4096)
     float* img_i4096 = nullptr;  // [104][128][4] scaled-form constants of the inverse kernel (n = 128 .. 4096)
-    int8_t* dsign4096 = nullptr; // [12][2048] sign applied to the accumulated d-theta (n = 128 .. 4096)
     uint32_t* gsign4096 = nullptr;  // [16 * 128] sign words applied to bf16 g rows (n = 128 .. 4096)
-    bool bwd_tables_valid = false;  // the three above match the current angles
+    bool bwd_tables_valid = false;  // the reverse tables match the current angles
     // n = 8192: backward tables of the two 4096-element halves (stages 0 .. 11), built on first use like the above
     float* img_b8192[2] = {nullptr, nullptr};
     float* img_i8192[2] = {nullptr, nullptr};  // scaled-form constants of the inverse kernel, per half
@@ -45,7 +45,9 @@ struct bfq_plan {
     int64_t partial_slots = 0;
     size_t partial_floats = 0;   // floats allocated behind `partial` (at n = 8192 the tuned backward may need more than the above)
     int* status_word = nullptr;  // device: non-zero when a bounded wait gave up
-    int* form_flag = nullptr;    // device (status_word + 1): stage form the table build selected for the tuned kernels
+    int* form_flag = nullptr;    // device (status_word + 1): stage form the table build selected for the forward kernels, the inverse
+                                 // (n = 8192: of the upper half in word 2) and, in word 3, the backward
+    int* slot_form = nullptr;    // device [sm_count]: form in which each CTA of the backward kernel took its sums (n = 128 .. 4096)
     // bfq_forward_quant_host: copy-in and copy-out streams and the events that order them with the caller's stream
     cudaStream_t host_in = nullptr, host_out = nullptr;
     cudaEvent_t host_ev[8] = {nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr};
