@@ -244,6 +244,7 @@ int bfq_plan_create(bfq_plan** out, int n, int64_t max_rows, int device) {
     if (n >= 128 && n <= 4096) {
         want(&plan->img4096, fwdq4096_image_bytes());
         want(&plan->prep4096, fwdq4096_prep_bytes());
+        if (n == 4096) want(&plan->flat4096, fwdq4096_image_bytes());
         want(&plan->weight4096, grad4096_weight_bytes());
         want(&plan->slot_form, sizeof(int) * plan->sm_count);
         want(&plan->img_b4096, bwd4096_image_bytes());
@@ -330,6 +331,10 @@ int bfq_set_angles(bfq_plan* plan, const float* theta, void* stream) {
 
 // bfq_forward after the checks, on the current device
 static int forward_rows(bfq_plan* plan, const void* x, int xt, int64_t rows, int64_t ldx, void* y, int yt, int64_t ldy, cudaStream_t st) {
+    if (xt == yt && x != y && forward_few_available(plan, rows) && !env_flag("BFQ_GENERIC_ONLY")) {
+        cudaError_t e = forward_few_launch(plan, x, xt == BFQ_F32, rows, ldx, 0, nullptr, nullptr, y, ldy, st);
+        return e == cudaSuccess ? BFQ_OK : cuda_fail(plan, e);
+    }
     if (xt == BFQ_BF16 && yt == BFQ_BF16 && x != y && rows < (int64_t(1) << 31) && !env_flag("BFQ_GENERIC_ONLY") &&
         fwdq4096_available(plan)) {
         cudaError_t e = fwdq4096_launch(plan, x, rows, ldx, false, nullptr, nullptr, y, ldy,
@@ -392,6 +397,10 @@ static int forward_quant_impl(bfq_plan* plan, const void* x, int xt, int64_t row
     DeviceGuard guard(plan->device);
     if (guard.err != cudaSuccess) return cuda_fail(plan, guard.err);
     cudaError_t e;
+    if (hist == nullptr && y == nullptr && forward_few_available(plan, rows) && !env_flag("BFQ_GENERIC_ONLY")) {
+        e = forward_few_launch(plan, x, xt == BFQ_F32, rows, ldx, bits, codes, scales, nullptr, 0, static_cast<cudaStream_t>(stream));
+        return e == cudaSuccess ? BFQ_OK : cuda_fail(plan, e);
+    }
     if (hist != nullptr) {  // statistics: the histogram starts at zero
         e = cudaMemsetAsync(hist, 0, sizeof(unsigned long long) << bits, static_cast<cudaStream_t>(stream));
         if (e != cudaSuccess) return cuda_fail(plan, e);

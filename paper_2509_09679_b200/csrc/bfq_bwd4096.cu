@@ -698,7 +698,7 @@ __global__ void __launch_bounds__(256) k_build_tables(const float4* __restrict__
     } else if (b < kTableBlocks) {
         build_gsign(256 * (b - 2 * kAngleBlocks) + threadIdx.x, flip, gsign);
     } else {
-        build_image_fwd(256 * (b - kTableBlocks) + threadIdx.x, prep, cs, img_fwd, form_fwd, weight);
+        build_image_fwd(256 * (b - kTableBlocks) + threadIdx.x, prep, cs, img_fwd, form_fwd, weight, nullptr);
     }
 }
 

@@ -29,6 +29,11 @@ cudaError_t fwdq4096_launch_f32(const bfq_plan* plan, const void* x, int64_t row
 cudaError_t fwdq4096_launch_stats(const bfq_plan* plan, const void* x, int64_t rows, int64_t ldx, uint8_t* codes,
                                   uint16_t* scales, unsigned long long* hist, float* rowstats, cudaStream_t st);
 
+// a few rows of n = 4096, a row to a cluster; bits as in fwdq_short_launch
+bool forward_few_available(const bfq_plan* plan, int64_t rows);
+cudaError_t forward_few_launch(const bfq_plan* plan, const void* x, bool f32, int64_t rows, int64_t ldx, int bits, uint8_t* codes, uint16_t* scales, void* y,
+                               int64_t ldy, cudaStream_t st);
+
 cudaError_t fwdq4096_build_forward(const bfq_plan* plan, const float* theta, cudaStream_t st);
 // rows of 128 .. 2048 elements: several as one of 4096 on the same kernel.  bits = 2, 4, 8: codes + scales, and
 // the rows if y is not null; bits = 0: the rows alone.  Rows are in the type of x, ldy apart (beside codes: contiguous)

@@ -68,10 +68,10 @@ __global__ void __launch_bounds__(256) k_prep_angles4096(const float* __restrict
 
 // Step 2 (one thread per angle): build_image_fwd in bfq_n4096.cuh
 __global__ void __launch_bounds__(256) k_build_image4096(const float4* __restrict__ prep, const double2* __restrict__ cs,
-                                                          float* __restrict__ img, int* __restrict__ form, float* __restrict__ weight) {
+                                                          float* __restrict__ img, int* __restrict__ form, float* __restrict__ weight, float* __restrict__ flat) {
     grid_dep_launch();
     grid_dep_wait();
-    build_image_fwd(blockIdx.x * blockDim.x + threadIdx.x, prep, cs, img, form, weight);
+    build_image_fwd(blockIdx.x * blockDim.x + threadIdx.x, prep, cs, img, form, weight, flat);
 }
 
 }  // namespace f4k
@@ -110,7 +110,7 @@ cudaError_t fwdq4096_build_forward(const bfq_plan* plan, const float* theta, cud
     float4* prep = reinterpret_cast<float4*>(plan->prep4096);
     double2* cs = reinterpret_cast<double2*>(prep + count);
     return launch_overlapped(f4k::k_build_image4096, dim3((count + 255) / 256), dim3(256), 0, st, prep, cs, plan->img4096,
-                             plan->form_flag, plan->weight4096);
+                             plan->form_flag, plan->weight4096, plan->flat4096);
 }
 
 // rows of 128 .. 2048 elements: several as one of 4096.  bits = 0: the rotated rows, in the type of x.

@@ -20,6 +20,8 @@ constexpr uint32_t kRowBytes = kN * 2;       // one bf16 row
 constexpr uint32_t kExWords = 4128;          // padded fp32 row (see the layouts below)
 constexpr uint32_t kExBytes = kExWords * 4;
 constexpr int kCols = 416;                   // tensor-memory columns in use
+constexpr int kFlatFloats = 11 * kN + 4 * (kN / 2);  // the same constants in the order of the angles: pairs of stages 0 .. 10, then fours
+constexpr int kFewRows = 16;                 // rows up to which k_forward_few takes a call: as many clusters of eight CTAs run at once
 
 __device__ __forceinline__ uint4 lds128(uint32_t a) {
     uint4 v;
@@ -199,9 +201,10 @@ __device__ __forceinline__ double factor_before(const double2* __restrict__ cs, 
 // One thread per angle: place the constants of pair (s, j) in both tensor-memory images
 // img[form][role][column], with the role / register / half of the pair's low element in its phase, and raise form[0]
 // when an element's factor leaves the range the scaled form is used in, form[3] when it leaves that of the backward kernel;
-// weight[form][angle] = the product of the factors with which the pair's elements enter the stage.
+// weight[form][angle] = the product of the factors with which the pair's elements enter the stage; flat (may be null): the
+// constants of each form once more in the order of the angles.
 __device__ __forceinline__ void build_image_fwd(int k, const float4* __restrict__ prep, const double2* __restrict__ cs, float* __restrict__ img,
-                                                int* __restrict__ form, float* __restrict__ weight) {
+                                                int* __restrict__ form, float* __restrict__ weight, float* __restrict__ flat) {
     if (k >= 12 * (kN / 2)) return;
     const int s = k / (kN / 2), j = k % (kN / 2);
     const int lo = ((j >> s) << (s + 1)) | (j & ((1 << s) - 1));
@@ -232,8 +235,13 @@ __device__ __forceinline__ void build_image_fwd(int k, const float4* __restrict_
         shear[at(32 * s + 4 * u + h + 2)] = sg * p.y;
         // k1 = -tan(theta) db/da, k2 = tan(theta) da/db, with one division
         const double w = own.y / (own.x * da * db);
-        scaled[at(32 * s + 4 * u + h)] = static_cast<float>(-w * db * db);
-        scaled[at(32 * s + 4 * u + h + 2)] = static_cast<float>(w * da * da);
+        const float k1 = static_cast<float>(-w * db * db), k2 = static_cast<float>(w * da * da);
+        scaled[at(32 * s + 4 * u + h)] = k1;
+        scaled[at(32 * s + 4 * u + h + 2)] = k2;
+        if (flat != nullptr) {
+            reinterpret_cast<float2*>(flat)[k] = make_float2(k1, k2);
+            reinterpret_cast<float2*>(flat + kFlatFloats)[k] = make_float2(sg * p.x, sg * p.y);
+        }
         const double lim = 5.421010862427522e-20;  // 2^-64
         const double lim_grad = 9.094947017729282e-13;  // 2^-40
         const double least = fmin(fabs(own.x * da), fabs(own.x * db));
@@ -249,6 +257,11 @@ __device__ __forceinline__ void build_image_fwd(int k, const float4* __restrict_
         scaled[at(col + 2)] = static_cast<float>(-own.y * db);
         scaled[at(col + 4)] = static_cast<float>(own.y * da);
         scaled[at(col + 6)] = static_cast<float>(own.x * db);
+        if (flat != nullptr) {
+            reinterpret_cast<float4*>(flat + 11 * kN)[j] = make_float4(static_cast<float>(own.x * da), static_cast<float>(-own.y * db),
+                                                                       static_cast<float>(own.y * da), static_cast<float>(own.x * db));
+            reinterpret_cast<float4*>(flat + kFlatFloats + 11 * kN)[j] = make_float4(p.z * sa, -p.w * sb, p.w * sa, p.z * sb);
+        }
     }
 }
 

@@ -21,6 +21,7 @@ struct bfq_plan {
     // these are built by bfq_set_angles
     float* img4096 = nullptr;    // [128][416] tensor-memory image of the rotation constants (n = 128 .. 4096)
     void* prep4096 = nullptr;    // staging for the image build: per-angle constants and negation flags (n = 128 .. 4096)
+    float* flat4096 = nullptr;   // [2 forms][53248] the constants of img4096 in the order of the angles (n = 4096)
     float* weight4096 = nullptr; // [2 forms][12][2048] what the backward kernel's sums are multiplied by (n = 128 .. 4096)
     float* img_b4096 = nullptr;  // [128][384] (n < 4096: [96][128][4]) three-shear constants of the inverse kernel (n = 128 .. 4096)
     float* img_i4096 = nullptr;  // [104][128][4] scaled-form constants of the inverse kernel (n = 128 .. 4096)

@@ -241,3 +241,29 @@ def test_bounded_wait_runs_out_and_the_plan_recovers():
     p.forward_quant(x.to(DEV), 4, codes=codes.view, scales=scales.view)
     check_quant(codes.view, scales.view, oracle.forward(to_f64(theta), to_f64(x)), 4, "after a timed-out call")
     assert p.device_status() == 0 and codes.intact() and scales.intact()
+
+
+@pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
+@pytest.mark.parametrize("kind", ["normal", "singular"])
+def test_a_few_rows_are_the_bits_of_many(dtype, kind):
+    """n = 4096: up to 16 rows go through the kernel that spreads a row over a cluster, more through the one that keeps the
+    constants in tensor memory; a row's codes, scales and numbers are the same bits (both rotation forms, rows with a stride)."""
+    n, many = 4096, 40
+    theta = synth.angles(n, "normal", 7)
+    if kind == "singular":
+        theta[3, ::5] = math.pi / 2
+    p = Plan(n, DEV)
+    p.set_angles(theta.to(DEV))
+    assert (p.stage_form() & 1) == (kind == "singular")
+    x = torch.zeros((many, n + 8), dtype=dtype, device=DEV)[:, :n]
+    x.copy_(synth.rows(many, n, "student_t3", 8, outliers=8, outlier_scale=50.0, dtype=dtype))
+    x[2] = 0
+    x[3] *= 1e-9
+    x[5] *= 1e9
+    whole = [p.forward(x)] + [t for bits in (2, 4, 8) for t in p.forward_quant(x, bits)]
+    for a, b in ((0, 1), (0, 16), (5, 8), (3, 20)):
+        part = [p.forward(x[a:b])] + [t for bits in (2, 4, 8) for t in p.forward_quant(x[a:b], bits)]
+        assert all(torch.equal(w[a:b], v) for w, v in zip(whole, part)), (a, b)
+    wide = torch.full((9, n + 24), 7.0, dtype=dtype, device=DEV)
+    p.forward(x[:9], out=wide[:, :n])
+    assert torch.equal(wide[:, :n], whole[0][:9]) and (wide[:, n:] == 7.0).all() and p.device_status() == 0
