@@ -1,4 +1,5 @@
-// Tuned backward pass for n = 4096 bf16 rows on sm_100a:  dx = Q^T g  and  d-theta summed over rows.
+// Tuned backward pass for n = 8192 bf16 rows on sm_100a, dx = Q^T g and d-theta summed over rows, on the two halves of 4096
+// elements (rows up to 4096: bfq_grad4096.cu); and the inverse of rows of 128 .. 8192 elements (further down).
 //
 // One persistent CTA per SM works on two rows at a time (row pair p of the CTA is rows 2p, 2p+1) with two
 // groups of 128 threads.  The upper group recomputes y for a pair and takes the reverse walk through stages 11, 10
@@ -7,7 +8,7 @@
 // pair.  The split balances the two groups' arithmetic (12 + 3 against 9 stage-equivalents of rotations, the lower
 // group also carrying both regroupings).  Each group owns the d-theta accumulators of its stages.  The thread roles,
 // phases and regrouping layouts are those of the forward kernel (bfq_n4096.cuh).  Per row pair:
-//   1. y = Q x with the three-shear constants, all 12 stages, in the tracked-sign basis sigma.
+//   1. y = Q x (the half's) with the three-shear constants, all 12 stages, in the tracked-sign basis sigma.
 //   2. y and g are moved to the basis sigma * (-1)^popcount(index).  Any two indices that a stage pairs
 //      differ in one bit, so in this basis the high element of every pair of every stage is negated
 //      relative to the low one, and there the inverse of a stage's rotation is the SAME three shears
@@ -32,7 +33,6 @@ using namespace ptx;
 using namespace f4k;
 
 constexpr int kCtaThreads = 2 * kThreads;
-constexpr int kSlots = 2;                    // TMA ring depth (row pairs), x and g rings separately
 constexpr int kBarRev = 1, kBarFwd = 2, kBarFull = 3, kBarEmpty = 4;  // named barriers
 constexpr int kConstCols = 384;              // 12 stages x 32 words
 constexpr int kAccCol = 384;                 // accumulators of stages 0..7: 16 columns each
@@ -42,15 +42,15 @@ constexpr int kWideCol = 416;  // wide inverse: (cos, +-sin) of the stage that j
 constexpr int kInvCols = 416;  // scaled inverse: stages 11..1 (32 columns each, stage s at 32 (s - 1)), then stage 0 (64)
 
 struct Smem {
-    static constexpr uint32_t kXOff = 0;                                   // [kSlots][2][kRowBytes]
-    static constexpr uint32_t kGOff = kXOff + kSlots * kPairBytes;         // [kSlots][2][kRowBytes]
-    static constexpr uint32_t kExFOff = kGOff + kSlots * kPairBytes;       // upper group, forward recompute: [2][kExBytes]
+    static constexpr uint32_t kXOff = 0;                                   // the halves of two x rows
+    static constexpr uint32_t kGOff = kXOff + 2 * kPairBytes;              // two whole g rows
+    static constexpr uint32_t kExFOff = kGOff + 2 * kPairBytes;            // upper group, forward recompute: [2][kExBytes]
     // y0, y1, g0, g1 of a row pair in the regrouping layouts: written by the upper group after stage 8 (this is both
     // the phase-3 -> phase-2 regrouping and the hand-off), re-used by the lower group for the regrouping after stage 4
     static constexpr uint32_t kExROff = kExFOff + 2 * kExBytes;            // [4][kExBytes]
     static constexpr uint32_t kAccOff = kExROff + 4 * kExBytes;            // [16][128] float4: stages 8..11
-    static constexpr uint32_t kBarOff = kAccOff + 16 * kThreads * 16;      // mbarriers, one per input slot
-    static constexpr uint32_t kTmemOff = kBarOff + 8 * 2 * kSlots;
+    static constexpr uint32_t kBarOff = kAccOff + 16 * kThreads * 16;      // mbarrier of the input slot
+    static constexpr uint32_t kTmemOff = kBarOff + 16;
     static constexpr uint32_t kUsed = kTmemOff + 16;
     static constexpr uint32_t kBytes = kUsed + 1024;
     // wide mode only: the upper group's sums of the stage that joins the halves, [16][128] packed pairs
@@ -80,21 +80,18 @@ struct Ctx {
     Addr a;
     uint32_t tlane;     // tensor-memory address of this thread's lane, column 0
     uint32_t acc_smem;  // this thread's first float4 of the shared-memory accumulators
-    int stages;         // SHORT: log2 of the row length, stages from there on are the identity and passed over
 };
 
 // ---- forward recompute: 24 chunks of 16 constants (two per stage), both rows ---------------------------
 // Chunk C is in Tcur; the next chunk is requested right after the wait.
-template <int C, bool SHORT>
+template <int C>
 __device__ __forceinline__ void fwd_chunks(u64 (&X0)[16], u64 (&X1)[16], uint32_t (&Tcur)[16], uint32_t (&Tnext)[16],
                                            const Ctx& cx) {
     constexpr int s = C / 2, K = s & 3, U0 = 4 * (C & 1);
     tmem_wait_ld16(Tcur);
     if constexpr (C + 1 < 24) tmem_ld16(cx.tlane + 16 * (C + 1), Tnext);
-    if (!SHORT || s < cx.stages) {
-        stage_lift<K, U0, 4, 16>(X0, Tcur);
-        stage_lift<K, U0, 4, 16>(X1, Tcur);
-    }
+    stage_lift<K, U0, 4, 16>(X0, Tcur);
+    stage_lift<K, U0, 4, 16>(X1, Tcur);
     if constexpr (C == 7) {  // inside each half-warp; the group-wide hand-off barrier of the previous row pair
                              // has put every other warp past its reads of these buffers
         fwd1_store(X0, cx.a.ex + 0 * kExBytes, cx.a);
@@ -111,7 +108,7 @@ __device__ __forceinline__ void fwd_chunks(u64 (&X0)[16], u64 (&X1)[16], uint32_
         fwd2_load(X0, cx.a.ex + 0 * kExBytes, cx.a);
         fwd2_load(X1, cx.a.ex + 1 * kExBytes, cx.a);
     }
-    if constexpr (C + 1 < 24) fwd_chunks<C + 1, SHORT>(X0, X1, Tnext, Tcur, cx);
+    if constexpr (C + 1 < 24) fwd_chunks<C + 1>(X0, X1, Tnext, Tcur, cx);
 }
 
 // ---- reverse walk: step I handles half c = I & 1 of stage s = 11 - I / 2 ---------------------------------
@@ -125,7 +122,7 @@ struct RevStep {
 };
 
 // steps I .. END-1 (END = 24: down to stage 0); hook(integral_constant<I>) runs after step I (regroupings, hand-off)
-template <int I, int END, bool SHORT, class F>
+template <int I, int END, class F>
 __device__ __forceinline__ void rev_steps(u64 (&Y0)[16], u64 (&Y1)[16], u64 (&G0)[16], u64 (&G1)[16],
                                           uint32_t (&Tcur)[16], uint32_t (&Tnext)[16], uint32_t (&Acur)[8],
                                           uint32_t (&Anext)[8], const Ctx& cx, F&& hook) {
@@ -143,43 +140,38 @@ __device__ __forceinline__ void rev_steps(u64 (&Y0)[16], u64 (&Y1)[16], u64 (&G0
         tmem_ld16(cx.tlane + N::kTCol, Tnext);
         if constexpr (N::kAccInTmem) tmem_ld8(cx.tlane + N::kAccCol, Anext);
     }
-    if (!SHORT || S::s < cx.stages) {
-        u64 A[4];
+    u64 A[4];
 #pragma unroll
-        for (int i = 0; i < 4; ++i) A[i] = pack2u(Acur[2 * i], Acur[2 * i + 1]);
-        dtheta4<S::K, S::U0>(A, Y0, Y1, G0, G1);
+    for (int i = 0; i < 4; ++i) A[i] = pack2u(Acur[2 * i], Acur[2 * i + 1]);
+    dtheta4<S::K, S::U0>(A, Y0, Y1, G0, G1);
 #pragma unroll
-        for (int i = 0; i < 4; ++i) unpack2u(A[i], Acur[2 * i], Acur[2 * i + 1]);
-    }
+    for (int i = 0; i < 4; ++i) unpack2u(A[i], Acur[2 * i], Acur[2 * i + 1]);
     if constexpr (S::kAccInTmem) {
         tmem_st8(cx.tlane + S::kAccCol, Acur);
     } else {
         sts128(cx.acc_smem + S::kAccSmem, make_uint4(Acur[0], Acur[1], Acur[2], Acur[3]));
         sts128(cx.acc_smem + S::kAccSmem + kThreads * 16, make_uint4(Acur[4], Acur[5], Acur[6], Acur[7]));
     }
-    if (!SHORT || S::s < cx.stages) {
-        if constexpr (S::s > 0) {  // y below stage 0 is x again: not needed
-            stage_lift<S::K, S::U0, 4, 16>(Y0, Tcur);
-            stage_lift<S::K, S::U0, 4, 16>(Y1, Tcur);
-        }
-        stage_lift<S::K, S::U0, 4, 16>(G0, Tcur);
-        stage_lift<S::K, S::U0, 4, 16>(G1, Tcur);
+    if constexpr (S::s > 0) {  // y below stage 0 is x again: not needed
+        stage_lift<S::K, S::U0, 4, 16>(Y0, Tcur);
+        stage_lift<S::K, S::U0, 4, 16>(Y1, Tcur);
     }
+    stage_lift<S::K, S::U0, 4, 16>(G0, Tcur);
+    stage_lift<S::K, S::U0, 4, 16>(G1, Tcur);
     hook(std::integral_constant<int, I>());
-    if constexpr (I + 1 < END) rev_steps<I + 1, END, SHORT>(Y0, Y1, G0, G1, Tnext, Tcur, Anext, Acur, cx, hook);
+    if constexpr (I + 1 < END) rev_steps<I + 1, END>(Y0, Y1, G0, G1, Tnext, Tcur, Anext, Acur, cx, hook);
 }
 
-// IN_F32: x, g and dx are fp32.  A row pair of x and of g then fills the whole input ring (one slot of 64 KB instead of
-// two of 32 KB): the next pair is requested as soon as the upper group has read g, behind a barrier of that group.
-// WIDE (bf16 rows): the launch handles half `half` of n = 8192 rows, i.e. stages 0 .. 11 of that half, whose tables it
+// A CTA handles half `half` of n = 8192 rows, i.e. stages 0 .. 11 of that half, whose tables it
 // is given.  x rows are the half's 4096 elements (the tensor map starts there); g rows are whole 8192-element rows (16 KB),
 // and the gradient that enters the half is the transposed stage-12 rotation of the two halves of g, formed as g is read:
 // g'_own = c g_own +- s g_other with (cos, sin) of stage 12 from `tw12`.  dx is written at column 4096 * half.  One input
-// slot, as for fp32 rows.  Stage 12's sums g_hi y_lo - g_lo y_hi are the same expression in g' and the halves' outputs
+// slot: the next pair is requested as soon as the upper group has read g, behind a barrier of that group.  Stage 12's sums
+// g_hi y_lo - g_lo y_hi are the same expression in g' and the halves' outputs
 // z before that stage (a rotation keeps the cross product of two vectors), so each launch adds its share while both are
 // in registers: half 0 has z_lo and forms g'_hi, half 1 has z_hi and forms g'_lo; the upper group keeps these sums in
 // shared memory and the CTA's slot of `partial` is kSlotFloatsWide long (sign of the share included).
-// what the CTAs of the upper half use in the wide mode instead of xmap, img, gsign, dsign
+// what the CTAs of the upper half use instead of xmap, img, gsign, dsign
 struct alignas(64) WideHalf {
     CUtensorMap xmap;
     const float* img;
@@ -187,24 +179,21 @@ struct alignas(64) WideHalf {
     const int8_t* dsign;
 };
 
-template <bool IN_F32, bool WIDE = false, bool SHORT = false>
 __global__ void __launch_bounds__(kCtaThreads, 1)
 k_bwd4096(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ CUtensorMap gmap,
           const float* __restrict__ img_lo, const uint32_t* __restrict__ gsign_lo, const int8_t* __restrict__ dsign_lo,
           void* __restrict__ dx_out, int64_t ld, float* __restrict__ partial, int rows, int* __restrict__ status,
-          const float2* __restrict__ tw12, const __grid_constant__ WideHalf upper, const ShortRows brief) {
-    static_assert(!(SHORT && WIDE), "one or the other");
-    static_assert(!(IN_F32 && WIDE), "the wide mode takes bf16 rows");
-    // wide mode: even CTAs work on the lower halves of the rows, odd CTAs on the upper halves (CTAs 2i and 2i + 1 take
+          const float2* __restrict__ tw12, const __grid_constant__ WideHalf upper) {
+    // even CTAs work on the lower halves of the rows, odd CTAs on the upper halves (CTAs 2i and 2i + 1 take
     // the same row pairs at about the same time, so the second read of a g row comes from L2)
-    const int ctas = WIDE ? int(gridDim.x >> 1) : int(gridDim.x);
-    const int half = WIDE ? int(blockIdx.x & 1u) : 0;
-    const CUtensorMap* const xm = (WIDE && half) ? &upper.xmap : &xmap;
-    const float* const img = (WIDE && half) ? upper.img : img_lo;
-    const uint32_t* const gsign = (WIDE && half) ? upper.gsign : gsign_lo;
-    const int8_t* const dsign = (WIDE && half) ? upper.dsign : dsign_lo;
+    const int ctas = int(gridDim.x >> 1);
+    const int half = int(blockIdx.x & 1u);
+    const CUtensorMap* const xm = half ? &upper.xmap : &xmap;
+    const float* const img = half ? upper.img : img_lo;
+    const uint32_t* const gsign = half ? upper.gsign : gsign_lo;
+    const int8_t* const dsign = half ? upper.dsign : dsign_lo;
     // (only dereferenced when dx_out is not null)
-    __nv_bfloat16* const dx = static_cast<__nv_bfloat16*>(dx_out) + (WIDE && dx_out != nullptr ? 4096 * half : 0);
+    __nv_bfloat16* const dx = static_cast<__nv_bfloat16*>(dx_out) + (dx_out != nullptr ? 4096 * half : 0);
     using S = Smem;
     extern __shared__ uint8_t smem_raw[];
     const uint32_t sbase = (smem_u32(smem_raw) + 1023u) & ~1023u;
@@ -214,8 +203,8 @@ k_bwd4096(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ CUte
     const int quarter = warp & 3;                    // tensor-memory lane quarter of this warp
 
     if (warp == 0) tmem_alloc512(sbase + S::kTmemOff);
-    if (threadIdx.x < 2 * kSlots) {
-        mbar_init(sbase + S::kBarOff + 8 * threadIdx.x, 1);
+    if (threadIdx.x == 0) {
+        mbar_init(sbase + S::kBarOff, 1);
         mbar_init_fence();
     }
     tmem_fence_before();
@@ -227,7 +216,6 @@ k_bwd4096(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ CUte
     Ctx cx;
     cx.tlane = tmem_base + (static_cast<uint32_t>(quarter * 32) << 16);
     cx.acc_smem = sbase + S::kAccOff + t * 16;
-    cx.stages = SHORT ? 12 - brief.log : 12;
     {
         const uint32_t t4 = (t >> 4) & 1, t5 = (t >> 5) & 1, t6 = (t >> 6) & 1;
         cx.a.ex = sbase + (is_fwd ? S::kExFOff : S::kExROff);  // the group's own regrouping buffers
@@ -239,44 +227,32 @@ k_bwd4096(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ CUte
     }
 
     const int pairs = (rows + 1) / 2;
-    const int first = WIDE ? int(blockIdx.x >> 1) : int(blockIdx.x);
+    const int first = int(blockIdx.x >> 1);
     const int stride = ctas;
     const int count = first < pairs ? (pairs - first + stride - 1) / stride : 0;
-    // both input rings belong to the upper group: one mbarrier per slot counts the x pair and the g pair
+    // the input slot belongs to the upper group: its mbarrier counts the x pair and the g pair
     const uint32_t xring = sbase + S::kXOff, gring = sbase + S::kGOff;
     const uint32_t bar_base = sbase + S::kBarOff;
 
     // a row index past the end is legal for the tensor map: the tile is filled with zeros
-    constexpr bool kOneSlot = IN_F32 || WIDE;
-    constexpr int kSlotsUsed = kOneSlot ? 1 : kSlots;
-    constexpr uint32_t kInRow = IN_F32 ? 2 * kRowBytes : kRowBytes;                // bytes of one x row
-    constexpr uint32_t kGRow = (IN_F32 || WIDE) ? 2 * kRowBytes : kRowBytes;       // bytes of one g row
-    static_assert(kSlots == 2, "an fp32 / wide row pair takes both bf16 slots of a ring");
+    constexpr uint32_t kGRow = 2 * kRowBytes;  // bytes of one g row
     auto request = [&](int k) {
-        const int slot = kOneSlot ? 0 : (k & 1);
         const int r0 = 2 * (first + k * stride);
-        const uint32_t bar = bar_base + 8 * slot;
-        mbar_expect_tx(bar, 2 * kInRow + 2 * kGRow);
-        const int at0 = SHORT ? r0 << brief.log : r0, at1 = SHORT ? (r0 + 1) << brief.log : r0 + 1;
-        tma_load_3d(xring + slot * kPairBytes, xm, 0, 0, at0, bar);
-        tma_load_3d(xring + slot * kPairBytes + kInRow, xm, 0, 0, at1, bar);
-        tma_load_3d(gring + slot * kPairBytes, &gmap, 0, 0, at0, bar);
-        tma_load_3d(gring + slot * kPairBytes + kGRow, &gmap, 0, 0, at1, bar);
+        mbar_expect_tx(bar_base, 2 * kRowBytes + 2 * kGRow);
+        tma_load_3d(xring, xm, 0, 0, r0, bar_base);
+        tma_load_3d(xring + kRowBytes, xm, 0, 0, r0 + 1, bar_base);
+        tma_load_3d(gring, &gmap, 0, 0, r0, bar_base);
+        tma_load_3d(gring + kGRow, &gmap, 0, 0, r0 + 1, bar_base);
     };
-    if (is_fwd && t == 0) {
-        for (int k = 0; k < kSlotsUsed && k < count; ++k) request(k);
-    }
+    if (is_fwd && t == 0 && count > 0) request(0);
     // constants into tensor memory (each group fills half of the columns), accumulators to zero
     {
-        // Short rows: the image is [column quad][role][4], so that a warp's load is 512 contiguous bytes (4 - 7 us less per call:
-        // 64.3 -> 58 us for 2048 rows of 4096).  The strip per role stays for the long batches of n = 4096: there the kernel
-        // built with the other fill ran 2 % slower (4.36 -> 4.45 ms for 262144 rows).
-        const float4* src = SHORT ? reinterpret_cast<const float4*>(img) + t : reinterpret_cast<const float4*>(img + t * kConstCols);
+        const float4* src = reinterpret_cast<const float4*>(img + t * kConstCols);
         for (int c = is_fwd ? 16 : 0; c < kConstCols; c += 32) {
             uint32_t v[16];
 #pragma unroll
             for (int i = 0; i < 4; ++i) {
-                const float4 f = __ldg(SHORT ? src + ((c >> 2) + i) * kThreads : src + (c >> 2) + i);
+                const float4 f = __ldg(src + (c >> 2) + i);
                 v[4 * i + 0] = __float_as_uint(f.x), v[4 * i + 1] = __float_as_uint(f.y);
                 v[4 * i + 2] = __float_as_uint(f.z), v[4 * i + 3] = __float_as_uint(f.w);
             }
@@ -288,7 +264,7 @@ k_bwd4096(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ CUte
             for (int i = 0; i < 16; ++i) z[i] = 0u;
             for (int c = kAccCol; c < 512; c += 16) tmem_st16(cx.tlane + c, z);
             for (int q = 0; q < 16; ++q) sts128(cx.acc_smem + q * kThreads * 16, make_uint4(0u, 0u, 0u, 0u));
-        } else if constexpr (WIDE) {
+        } else {
             for (int m = 0; m < 16; ++m) sts64(sbase + S::kAcc12Off + (m * kThreads + t) * 8, 0ull);
         }
         tmem_wait_st();
@@ -307,12 +283,7 @@ k_bwd4096(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ CUte
     if (is_fwd) {
         // ================= upper group: y = Q x, then d-theta and the reverse walk of stages 11, 10, 9 =================
         // x tile, phase-1 ownership (as in the forward kernel)
-        // (fp32: runs of 64 bytes at byte 64 (t & 15) + 2048 (t >> 4) + 1024 h: chunks 4 (t & 1) + c of line
-        // ((t & 15) >> 1) + 16 (t >> 4) + 8 h)
-        const uint32_t in_line = IN_F32 ? ((t & 15) >> 1) * 128u + (t >> 4) * 2048u : ((t >> 2) & 3) * 128u + (t >> 4) * 1024u;
-        const uint32_t in_x = IN_F32 ? ((((t & 1) << 2) ^ ((t >> 1) & 7)) << 4) : ((((t & 3) << 1) ^ ((t >> 2) & 3)) << 4);
-        // fp32 g: elements 2t + 256m, +1 are the 8-byte word t & 1 of chunk (t & 15) >> 1 of line (t >> 4) + 8m
-        const uint32_t f_a = (t >> 4) * 128u + ((((t & 15) >> 1) ^ (t >> 4)) << 4) + (t & 1) * 8u;
+        const uint32_t in_line = ((t >> 2) & 3) * 128u + (t >> 4) * 1024u, in_x = (((t & 3) << 1) ^ ((t >> 2) & 3)) << 4;
         // g tile, phase-3 ownership: the 32-bit word of elements 2t + 256m, 2t + 256m + 1 is word t & 3 of
         // 16-byte chunk (t & 31) >> 2 of 128-byte line (t >> 5) + 4m; the swizzle moves the chunk to
         // chunk ^ (line & 7)
@@ -321,31 +292,12 @@ k_bwd4096(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ CUte
         const uint32_t g_a1 = (t >> 5) * 128u + ((g_x ^ 4u) << 4) + (t & 3) * 4u;
         const uint4* gsv = reinterpret_cast<const uint4*>(gsign);
         for (int k = 0; k < count; ++k) {
-            const int slot = kOneSlot ? 0 : (k & 1);
-            // every thread of this group is past its reads of the other input slot (each iteration ends in a
-            // barrier with the lower group)
-            if (!kOneSlot && t == 0 && k >= 1 && k + 1 < count) request(k + 1);
             tmem_ld16(cx.tlane, T0);
-            mbar_wait_bounded(bar_base + 8 * slot, (kOneSlot ? k : (k >> 1)) & 1, status);
+            mbar_wait_bounded(bar_base, k & 1, status);
 #pragma unroll
             for (int r = 0; r < 2; ++r) {
                 u64(&X)[16] = r == 0 ? Y0 : Y1;
-                const uint32_t src = xring + slot * kPairBytes + r * kInRow + in_line;
-                if constexpr (IN_F32) {
-                    uint4 w[2][4];
-#pragma unroll
-                    for (int h = 0; h < 2; ++h)
-#pragma unroll
-                        for (int c = 0; c < 4; ++c) w[h][c] = lds128(src + 1024u * h + (in_x ^ (c << 4)));
-#pragma unroll
-                    for (int c = 0; c < 4; ++c) {
-                        X[4 * c + 0] = pack2u(w[0][c].x, w[1][c].x);
-                        X[4 * c + 1] = pack2u(w[0][c].y, w[1][c].y);
-                        X[4 * c + 2] = pack2u(w[0][c].z, w[1][c].z);
-                        X[4 * c + 3] = pack2u(w[0][c].w, w[1][c].w);
-                    }
-                    continue;
-                }
+                const uint32_t src = xring + r * kRowBytes + in_line;
                 uint4 w[2][2];
 #pragma unroll
                 for (int h = 0; h < 2; ++h)
@@ -362,7 +314,7 @@ k_bwd4096(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ CUte
                     }
                 }
             }
-            fwd_chunks<0, SHORT>(Y0, Y1, T0, T1, cx);
+            fwd_chunks<0>(Y0, Y1, T0, T1, cx);
             // y to the parity basis
 #pragma unroll
             for (int m = 0; m < 16; ++m) {
@@ -373,7 +325,7 @@ k_bwd4096(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ CUte
             }
             // g into the same basis
             tmem_ld16(cx.tlane + RevStep<0>::kTCol, T0);
-            if constexpr (WIDE) {
+            {
                 // elements 2t + 256m, +1 of both halves of the row (the upper half is 8192 bytes further on, the same
                 // line modulo 8) and (cos, sin) of the two stage-12 pairs they form; y carries the signs of the walk's basis
                 // here, the sign of each sum is put right when the sums are written out
@@ -406,33 +358,10 @@ k_bwd4096(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ CUte
                     }
                 }
             }
-#pragma unroll
-            for (int r = 0; r < (WIDE ? 0 : 2); ++r) {
-                u64(&G)[16] = r == 0 ? G0 : G1;
-                const uint32_t src = gring + slot * kPairBytes + r * kGRow;
-#pragma unroll
-                for (int qq = 0; qq < 4; ++qq) {
-                    const uint4 sw = __ldg(gsv + qq * kThreads + t);  // 2 KB in all: stays in L1
-                    const uint32_t s4[4] = {sw.x, sw.y, sw.z, sw.w};
-#pragma unroll
-                    for (int i = 0; i < 4; ++i) {
-                        const int m = 4 * qq + i;
-                        if constexpr (IN_F32) {
-                            uint32_t lo, hi;
-                            unpack2u(lds64(src + f_a + 1024u * m), lo, hi);
-                            G[m] = pack2u(lo ^ ((s4[i] & 0x8000u) << 16), hi ^ (s4[i] & 0x80000000u));
-                        } else {
-                            const uint32_t w = lds32(src + ((m & 1) ? g_a1 : g_a0) + 512u * m) ^ s4[i];
-                            G[m] = pack2u(bf16_lo(w), w & 0xFFFF0000u);
-                        }
-                    }
-                }
-            }
-            if constexpr (kOneSlot) {  // the one slot has been read by every thread of the group: next pair
-                bar_sync(cx.a.bar, kThreads);
-                if (t == 0 && k + 1 < count) request(k + 1);
-            }
-            rev_steps<0, kUpperSteps, SHORT>(Y0, Y1, G0, G1, T0, T1, A0, A1, cx, [](auto) {});
+            // the slot has been read by every thread of the group: next pair
+            bar_sync(cx.a.bar, kThreads);
+            if (t == 0 && k + 1 < count) request(k + 1);
+            rev_steps<0, kUpperSteps>(Y0, Y1, G0, G1, T0, T1, A0, A1, cx, [](auto) {});
             // phase 3 -> phase 2 regrouping = the hand-over: once the lower group is past its reads of the buffers for
             // the previous pair, store in the layout it reads
             bar_sync(kBarEmpty, kCtaThreads);
@@ -455,7 +384,7 @@ k_bwd4096(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ CUte
             rev2_load(Y1, exr + 1 * kExBytes, cx.a);
             rev2_load(G0, exr + 2 * kExBytes, cx.a);
             rev2_load(G1, exr + 3 * kExBytes, cx.a);
-            rev_steps<kUpperSteps, 24, SHORT>(Y0, Y1, G0, G1, T0, T1, A0, A1, cx, [&](auto step) {
+            rev_steps<kUpperSteps, 24>(Y0, Y1, G0, G1, T0, T1, A0, A1, cx, [&](auto step) {
                 constexpr int I = decltype(step)::value;
                 if constexpr (I == 15) {  // phase 2 -> phase 1, inside each half-warp, but the buffers were read across warps
                     bar_sync(cx.a.bar, kThreads);
@@ -480,33 +409,6 @@ k_bwd4096(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ CUte
                 for (int r = 0; r < 2; ++r) {
                     if (r0 + r < rows) {
                         const u64(&G)[16] = r == 0 ? G0 : G1;
-                        // SHORT: a run of 16 elements exists or not as a whole.  (Long rows are built without the test: with
-                        // one that is always true the same kernel took 0.7 to 1.6 % longer: 4.43 -> 4.50 ms for 262144 rows.)
-                        auto there = [&](int h) {
-                            return static_cast<int64_t>(r0 + r) * kN + 16 * (t & 15) + 512 * (t >> 4) + 256 * h < brief.elems;
-                        };
-                        if constexpr (IN_F32) {
-                            float* row = static_cast<float*>(dx_out) + static_cast<int64_t>(r0 + r) * ld + 16 * (t & 15) + 512 * (t >> 4);
-#pragma unroll
-                            for (int h = 0; h < 2; ++h) {
-                                uint32_t w[16];
-#pragma unroll
-                                for (int m = 0; m < 16; ++m) {
-                                    uint32_t lo, hi;
-                                    unpack2u(G[m], lo, hi);
-                                    // element m of half h: parity popcount(m) ^ h ^ popcount(t)
-                                    const bool odd_c = ((__builtin_popcount(m) + h) & 1) != 0;
-                                    w[m] = (h ? hi : lo) ^ (odd_c ? sgn_b : sgn_a);
-                                }
-                                if constexpr (SHORT) {
-                                    if (!there(h)) continue;
-                                }
-                                uint4* dst = reinterpret_cast<uint4*>(row + 256 * h);
-#pragma unroll
-                                for (int c = 0; c < 4; ++c) dst[c] = make_uint4(w[4 * c], w[4 * c + 1], w[4 * c + 2], w[4 * c + 3]);
-                            }
-                            continue;
-                        }
                         __nv_bfloat16* row = dx + static_cast<int64_t>(r0 + r) * ld + 16 * (t & 15) + 512 * (t >> 4);
 #pragma unroll
                         for (int h = 0; h < 2; ++h) {
@@ -523,9 +425,6 @@ k_bwd4096(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ CUte
                                 const uint32_t neg_hi = odd_c ? sgn_a : sgn_b;                  // bit 31: element 2j+1
                                 w[j] = cvt_bf16x2(e0, e1) ^ (neg_lo | neg_hi);
                             }
-                            if constexpr (SHORT) {
-                                if (!there(h)) continue;
-                            }
                             uint4* dst = reinterpret_cast<uint4*>(row + 256 * h);
                             dst[0] = make_uint4(w[0], w[1], w[2], w[3]);
                             dst[1] = make_uint4(w[4], w[5], w[6], w[7]);
@@ -539,19 +438,17 @@ k_bwd4096(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ CUte
 
     // ---- this CTA's sums -> its slot of the partial sums, with the sign of the basis undone ----
     __syncthreads();  // the upper group's sums of stages 9..11 (shared memory) are complete
-    float* const slot_out = partial + static_cast<int64_t>(blockIdx.x) * (WIDE ? kSlotFloatsWide : kSlotFloats);
-    if constexpr (WIDE) {
-        if (is_fwd) {
-            // this half's share of stage 12: pairs 2t + 256m, +1; y carried the signs of the basis g enters (the sign
-            // words), half 1's share is subtracted
-            const float sg = half ? -1.f : 1.f;
-            for (int m = 0; m < 16; ++m) {
-                float a0, a1;
-                unpack2(lds64(sbase + S::kAcc12Off + (m * kThreads + t) * 8), a0, a1);
-                const uint32_t sw = __ldg(gsign + (m >> 2) * 4 * kThreads + 4 * t + (m & 3));
-                *reinterpret_cast<float2*>(slot_out + kSlotFloats + 2 * t + 256 * m) =
-                    make_float2((sw & 0x8000u) ? -sg * a0 : sg * a0, (sw & 0x80000000u) ? -sg * a1 : sg * a1);
-            }
+    float* const slot_out = partial + static_cast<int64_t>(blockIdx.x) * kSlotFloatsWide;
+    if (is_fwd) {
+        // this half's share of stage 12: pairs 2t + 256m, +1; y carried the signs of the basis g enters (the sign
+        // words), half 1's share is subtracted
+        const float sg = half ? -1.f : 1.f;
+        for (int m = 0; m < 16; ++m) {
+            float a0, a1;
+            unpack2(lds64(sbase + S::kAcc12Off + (m * kThreads + t) * 8), a0, a1);
+            const uint32_t sw = __ldg(gsign + (m >> 2) * 4 * kThreads + 4 * t + (m & 3));
+            *reinterpret_cast<float2*>(slot_out + kSlotFloats + 2 * t + 256 * m) =
+                make_float2((sw & 0x8000u) ? -sg * a0 : sg * a0, (sw & 0x80000000u) ? -sg * a1 : sg * a1);
         }
     }
     if (!is_fwd) {
@@ -1148,7 +1045,7 @@ cudaError_t bwd8192_build_tables(const bfq_plan* plan, cudaStream_t st) {
 cudaError_t bwd8192_launch_halves(bfq_plan* plan, const void* x, const void* g, int64_t rows, int64_t ld, void* dx,
                                   float* dtheta, cudaStream_t st) {
     static bool attr_set[kMaxDevices] = {false};
-    auto kern = b4k::k_bwd4096<false, true>;
+    auto kern = b4k::k_bwd4096;
     if (!attr_set[plan->device]) {
         cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(b4k::Smem::kBytesWide));
         if (e != cudaSuccess) return e;
@@ -1175,7 +1072,7 @@ cudaError_t bwd8192_launch_halves(bfq_plan* plan, const void* x, const void* g, 
     upper.img = plan->img_b8192[1], upper.gsign = plan->gsign8192[1], upper.dsign = plan->dsign8192[1];
     kern<<<2 * grid, b4k::kCtaThreads, b4k::Smem::kBytesWide, st>>>(xmap, gmap, plan->img_b8192[0], plan->gsign8192[0],
                                                                   plan->dsign8192[0], dx, ld, plan->partial, int(rows),
-                                                                  plan->status_word, plan->tw + 12 * f4k::kN, upper, b4k::ShortRows{});
+                                                                  plan->status_word, plan->tw + 12 * f4k::kN, upper);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     b4k::k_reduce_wide<<<13 * f4k::kN / 32, 256, 0, st>>>(plan->partial, grid, dtheta);
