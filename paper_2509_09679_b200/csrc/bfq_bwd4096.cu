@@ -705,6 +705,7 @@ k_inv4096(const __grid_constant__ CUtensorMap ymap, const float* __restrict__ im
     const int q = warp & 3, g = warp >> 2;
     const int t = q * 32 + lane;
 
+    grid_dep_launch();
     if (warp == 0) tmem_alloc512(sbase + S::kTmemOff);
     if (threadIdx.x < G * kInSlots) {
         mbar_init(sbase + S::kBarOff + 8 * threadIdx.x, 1);
@@ -713,6 +714,8 @@ k_inv4096(const __grid_constant__ CUtensorMap ymap, const float* __restrict__ im
     if constexpr (SHORT) {
         if (threadIdx.x < G) sts32(sbase + S::kBadOff + 4 * threadIdx.x, 0u);
     }
+    // everything above overlaps the end of the kernel before this one; global memory is touched from here on
+    grid_dep_wait();
     tmem_fence_before();
     __syncthreads();
     tmem_fence_after();
@@ -1130,9 +1133,8 @@ cudaError_t inv_short_launch(bfq_plan* plan, const void* y, bool y_f32, int64_t 
     const b4k::ShortRows brief{12 - plan->log_n, rows * n, RowSource{y, ldy, plan->tw}, ldx};
     const int64_t joint = (brief.elems + f4k::kN - 1) / f4k::kN, want = (joint + G - 1) / G;
     const int grid = int(want < plan->sm_count ? want : plan->sm_count);
-    kern<<<grid, G * b4k::kThreads, S::kBytes, st>>>(ymap, plan->img_b4096, plan->img_i4096, plan->form_flag + 1, plan->gsign4096, x, ldx << (12 - plan->log_n),
+    return launch_overlapped(kern, dim3(grid), dim3(G * b4k::kThreads), S::kBytes, st, ymap, plan->img_b4096, plan->img_i4096, plan->form_flag + 1, plan->gsign4096, x, ldx << (12 - plan->log_n),
                                                     int(joint), plan->status_word, nullptr, b4k::InvUpper{}, brief);
-    return cudaGetLastError();
 }
 
 // fp32 rows in, fp32 rows out
@@ -1151,10 +1153,9 @@ cudaError_t inv4096_launch_f32(bfq_plan* plan, const void* y, int64_t rows, int6
     if (!encode_row_map_f32(&ymap, y, rows, ldy)) return cudaErrorInvalidValue;
     const int64_t want = (rows + G - 1) / G;
     const int grid = int(want < plan->sm_count ? want : plan->sm_count);
-    kern<<<grid, G * b4k::kThreads, S::kBytes, st>>>(ymap, plan->img_b4096, plan->img_i4096, plan->form_flag + 1,
+    return launch_overlapped(kern, dim3(grid), dim3(G * b4k::kThreads), S::kBytes, st, ymap, plan->img_b4096, plan->img_i4096, plan->form_flag + 1,
                                                     plan->gsign4096, x, ldx, int(rows), plan->status_word, nullptr,
                                                     b4k::InvUpper{}, b4k::ShortRows{});
-    return cudaGetLastError();
 }
 
 cudaError_t inv4096_launch(bfq_plan* plan, const void* y, int64_t rows, int64_t ldy, void* x, bool x_bf16, int64_t ldx,
@@ -1175,17 +1176,16 @@ cudaError_t inv4096_launch(bfq_plan* plan, const void* y, int64_t rows, int64_t 
     const int64_t want = (rows + G - 1) / G;
     const int grid = int(want < plan->sm_count ? want : plan->sm_count);
     if (x_bf16) {
-        b4k::k_inv4096<G, true><<<grid, G * b4k::kThreads, S::kBytes, st>>>(ymap, plan->img_b4096, plan->img_i4096,
+        return launch_overlapped(b4k::k_inv4096<G, true>, dim3(grid), dim3(G * b4k::kThreads), S::kBytes, st, ymap, plan->img_b4096, plan->img_i4096,
                                                                             plan->form_flag + 1, plan->gsign4096, x, ldx,
                                                                             int(rows), plan->status_word, nullptr,
                                                                             b4k::InvUpper{}, b4k::ShortRows{});
     } else {
-        b4k::k_inv4096<G, false><<<grid, G * b4k::kThreads, S::kBytes, st>>>(ymap, plan->img_b4096, plan->img_i4096,
+        return launch_overlapped(b4k::k_inv4096<G, false>, dim3(grid), dim3(G * b4k::kThreads), S::kBytes, st, ymap, plan->img_b4096, plan->img_i4096,
                                                                              plan->form_flag + 1, plan->gsign4096, x, ldx,
                                                                              int(rows), plan->status_word, nullptr,
                                                                              b4k::InvUpper{}, b4k::ShortRows{});
     }
-    return cudaGetLastError();
 }
 
 // n = 8192, bf16 rows in, bf16 or fp32 rows out: the inverse kernel's wide mode, even CTAs on the lower halves of x, odd
@@ -1221,15 +1221,14 @@ cudaError_t inv8192_launch(bfq_plan* plan, const void* y, int64_t rows, int64_t 
     const b4k::InvUpper upper{plan->img_b8192[1], plan->img_i8192[1], plan->form_flag + 2, plan->gsign8192[1]};
     const float2* tw12 = plan->tw + 12 * f4k::kN;
     if (x_bf16) {
-        b4k::k_inv4096<G, true, false, true><<<grid, G * b4k::kThreads, S::kBytes, st>>>(
+        return launch_overlapped(b4k::k_inv4096<G, true, false, true>, dim3(grid), dim3(G * b4k::kThreads), S::kBytes, st,
             ymap, plan->img_b8192[0], plan->img_i8192[0], plan->form_flag + 1, plan->gsign8192[0], x, ldx, int(rows),
             plan->status_word, tw12, upper, b4k::ShortRows{});
     } else {
-        b4k::k_inv4096<G, false, false, true><<<grid, G * b4k::kThreads, S::kBytes, st>>>(
+        return launch_overlapped(b4k::k_inv4096<G, false, false, true>, dim3(grid), dim3(G * b4k::kThreads), S::kBytes, st, 
             ymap, plan->img_b8192[0], plan->img_i8192[0], plan->form_flag + 1, plan->gsign8192[0], x, ldx, int(rows),
             plan->status_word, tw12, upper, b4k::ShortRows{});
     }
-    return cudaGetLastError();
 }
 
 }  // namespace bfq
