@@ -61,6 +61,17 @@ SIGNATURES = {
 _lib = None
 
 
+def _not_built(*args):
+    return None
+
+
+try:  # the plain forms of the smallest calls in C++: a result, a status, or None for "not plain, done below"
+    from . import fast_calls as _fast
+except ImportError:  # not built: every call is done below
+    class _fast:
+        attach = forward = forward_quant = inverse = _not_built
+
+
 class BfqError(RuntimeError):
     def __init__(self, status: int, where: str):
         self.status = status
@@ -80,6 +91,7 @@ def lib() -> ctypes.CDLL:
             fn = getattr(L, name)
             fn.restype, fn.argtypes = res, args
         _lib = L
+        _fast.attach(LIB_PATH)
     return _lib
 
 
@@ -163,6 +175,8 @@ class GemmOperand:
 class Plan:
     """Owns a bfq_plan for row length n on one CUDA device."""
 
+    _id, _index = 0, -1  # of the plan and its device, for fast_calls
+
     def __init__(self, n: int, device=None, max_rows: int = 0):
         dev = torch.device("cuda", torch.cuda.current_device()) if device is None else torch.device(device)
         if dev.type != "cuda":
@@ -174,9 +188,11 @@ class Plan:
         self._c = lib()
         _check(lib().bfq_plan_create(ctypes.byref(self._h), self.n, int(max_rows), self.device.index),
                "bfq_plan_create")
+        self._id, self._index = self._h.value, self.device.index
 
     def close(self):
         if getattr(self, "_h", None) is not None and self._h.value:
+            self._id = 0
             lib().bfq_plan_destroy(self._h)
             self._h = ctypes.c_void_p()
 
@@ -192,6 +208,10 @@ class Plan:
         _check(self._c.bfq_set_angles(self._h, theta.data_ptr(), _stream(theta)), "bfq_set_angles")
 
     def forward(self, x: torch.Tensor, out_dtype=None, out: torch.Tensor | None = None) -> torch.Tensor:
+        if out is None and out_dtype is None:
+            done = _fast.forward(self._id, self.n, self._index, x)
+            if done is not None:
+                return done if type(done) is not int else _check(done, "bfq_forward")
         n = self.n
         rows, ldx = _rows(x, n, self.device, what="x")
         y, ldy = self._row_output(x, rows, out_dtype, out)
@@ -220,6 +240,10 @@ class Plan:
         return codes, scales
 
     def forward_quant(self, x: torch.Tensor, bits: int, codes=None, scales=None):
+        if codes is None and scales is None:
+            done = _fast.forward_quant(self._id, self.n, self._index, x, bits)
+            if done is not None:
+                return done if type(done) is not int else _check(done, "bfq_forward_quant")
         rows, ldx = _rows(x, self.n, self.device, what="x")
         codes, scales = self._outputs(rows, self.n, bits, codes, scales)
         _check(self._c.bfq_forward_quant(self._h, x.data_ptr(), _dt(x), rows, ldx, int(bits), codes.data_ptr(),
@@ -325,6 +349,10 @@ class Plan:
         return codes, scales
 
     def inverse(self, y: torch.Tensor, out_dtype=None, out: torch.Tensor | None = None) -> torch.Tensor:
+        if out is None and out_dtype is None:
+            done = _fast.inverse(self._id, self.n, self._index, y)
+            if done is not None:
+                return done if type(done) is not int else _check(done, "bfq_inverse")
         rows, ldy = _rows(y, self.n, self.device, what="y")
         x, ldx = self._row_output(y, rows, out_dtype, out)
         _check(self._c.bfq_inverse(self._h, y.data_ptr(), _dt(y), rows, ldy, x.data_ptr(), _dt(x), ldx, _stream(y)),

@@ -1,10 +1,11 @@
-"""Builds the CUDA library in-tree: paper_2509_09679_b200/libbfq.so (sm_100a only)."""
+"""Builds the CUDA library in-tree, paper_2509_09679_b200/libbfq.so (sm_100a only), and the binding's C++ part beside it."""
 from __future__ import annotations
 
 import glob
 import os
 import subprocess
 import sys
+import sysconfig
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
@@ -12,6 +13,25 @@ LIB = os.path.join(HERE, "libbfq.so")
 NVCC = os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")
 FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-O3", "-lineinfo", "-std=c++17",
          "-Xcompiler", "-fPIC"]
+
+
+FAST = os.path.join(HERE, "fast_calls" + sysconfig.get_config_var("EXT_SUFFIX"))
+
+
+def build_fast_calls(force: bool = False) -> str:
+    """The extension module of csrc/fast_calls.cpp (the C ABI's header and torch's)."""
+    src = os.path.join(CSRC, "fast_calls.cpp")
+    newest = max(os.path.getmtime(p) for p in (src, os.path.join(os.path.dirname(HERE), "include", "bfq.h")))
+    if not force and os.path.exists(FAST) and os.path.getmtime(FAST) >= newest:
+        return FAST
+    import torch
+
+    at = os.path.dirname(torch.__file__)
+    cuda = os.path.dirname(os.path.dirname(NVCC))
+    subprocess.run([os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-fPIC", "-shared", f"-D_GLIBCXX_USE_CXX11_ABI={int(torch.compiled_with_cxx11_abi())}",
+                    f"-I{at}/include", f"-I{at}/include/torch/csrc/api/include", f"-I{sysconfig.get_paths()['include']}", f"-I{cuda}/include",
+                    src, "-o", FAST, f"-L{at}/lib", "-ltorch_python", "-ltorch", "-ltorch_cpu", "-lc10_cuda", "-lc10"], check=True)
+    return FAST
 
 
 def sources():
@@ -24,6 +44,7 @@ def _deps():
 
 
 def build(force: bool = False, verbose: bool = False) -> str:
+    build_fast_calls(force)
     newest = max(os.path.getmtime(p) for p in _deps())
     if not force and os.path.exists(LIB) and os.path.getmtime(LIB) >= newest:
         return LIB
