@@ -14,7 +14,7 @@
 //
 // A CTA per SM runs four groups of 128 threads as a pipeline, a row in each:
 //     D  g: stages 11 .. 8 down
-//     A  g: stages 7 .. 0 down, dx
+//     A  g: stages 7 .. 0 down, dx (or B: kDxByA)
 //     B  x and u: stages 0 .. 3 up
 //     C  x and u: stages 4 .. 7 up
 //     D  x and u: stages 8 .. 10 up, and the sums of 8 .. 11
@@ -44,6 +44,11 @@ constexpr int kAccCol = 384;                // sums of stages 0 .. 7: 16 columns
 constexpr int kLastCol = 352;               // constants of the last stage: half of them in tensor memory, the rest in shared memory
 constexpr int kSlotFloats = 12 * (kN / 2);  // a CTA's sums
 constexpr float kLift = 1048576.f;          // 2^20
+// Group A or group B scales u back and writes dx: whichever has the time.  us, written by A / by B: 65536 rows of 4096 bf16 846 / 879,
+// fp32 1016 / 932; 2^25 elements of n = 2048 bf16 125 / 116, fp32 152 / 138, n = 1024 119 / 115, 152 / 136, n = 256 117 / 119, 144 / 142,
+// n = 128 130 / 137, 166 / 156.
+template <bool IN_F32, int STAGES>
+constexpr bool kDxByA = !IN_F32 && (STAGES == 12 || STAGES <= 8);
 constexpr int kLag = 3;                     // rows between a row's two turns in group D
 enum : int { kFullDA = 1, kEmptyDA, kFullAB, kEmptyAB, kFullBC, kEmptyBC, kFullCD, kEmptyCD };
 
@@ -52,8 +57,10 @@ struct Smem {
     static constexpr uint32_t kRow = (IN_F32 ? 2 : 1) * kRowBytes;
     static constexpr uint32_t kXOff = 0;                             // [kSlots] rows
     static constexpr uint32_t kGOff = kXOff + kSlots * kRow;         // [kSlots] rows
-    static constexpr uint32_t kDAOff = kGOff + kSlots * kRow;        // g between phases 3 and 2
-    static constexpr uint32_t kAOff = kDAOff + kExBytes;             // g between phases 2 and 1
+    // g between phases 3 and 2, index bits i0 .. i11: word (i8 ^ i4) + 2 (i0 ^ i5) + 4 (i1 .. i3) + 32 (i4 .. i7) + 512 (i9 .. i11),
+    // so that D's scalar stores (lanes i1 .. i5) and A's 64-bit loads (lanes i0 .. i3) fall into different banks
+    static constexpr uint32_t kDAOff = kGOff + kSlots * kRow;
+    static constexpr uint32_t kAOff = kDAOff + 4 * kN;               // g between phases 2 and 1
     static constexpr uint32_t kABOff = kAOff + kExBytes;             // u, [8][128] of four numbers
     static constexpr uint32_t kBCOff = kABOff + 4 * kN;              // x, u
     static constexpr uint32_t kCDOff = kBCOff + 2 * kExBytes;        // x, u
@@ -258,6 +265,20 @@ __device__ __forceinline__ void store_dx(const Ctx& cx, const u64 (&U)[16], int 
     }
 }
 
+// u at its own size, and dx of the CTA's k-th row
+template <int FORM, bool IN_F32, int STAGES>
+__device__ __forceinline__ void write_dx(const Ctx& cx, u64 (&U)[16], int k) {
+    if constexpr (FORM == kFormScaled) {
+        const u64 back = pack2(1.f / kLift, 1.f / kLift);
+#pragma unroll
+        for (int m = 0; m < 16; ++m) U[m] = mul2(back, U[m]);
+    }
+    if (cx.dx == nullptr) return;
+    const int use = cx.done + k;
+    mbar_wait_bounded(cx.sbase + Smem<IN_F32>::kBarOff + 8 * (use & 1), (use >> 1) & 1, cx.status);  // x has arrived: dx may lie over it
+    store_dx<IN_F32, STAGES>(cx, U, cx.first + k * cx.stride);
+}
+
 // A thread's sixteen sums of one stage to the CTA's slot, in the order of the angles: consecutive lanes fill whole sectors
 template <int P>
 __device__ __forceinline__ bool write_sums(const Ctx& cx, int s, const uint32_t (&a)[16]) {
@@ -299,17 +320,22 @@ __device__ __forceinline__ void group_a(const Ctx& cx, const CUtensorMap* xmap) 
     using S = Smem<IN_F32>;
     const int t = cx.t;
     const uint32_t xbars = cx.sbase + S::kBarOff, xring = cx.sbase + S::kXOff;
-    const uint32_t from_d = cx.sbase + S::kDAOff, own = cx.sbase + S::kAOff, to_b = cx.sbase + S::kABOff + 16u * t;
+    const uint32_t from_d = cx.sbase + S::kDAOff + 16u * ((t >> 1) & 7) + 2048u * (t >> 4);
+    const uint32_t from_d0 = from_d + 8u * (t & 1), from_d1 = from_d + 8u * ((t & 1) ^ 1), own = cx.sbase + S::kAOff, to_b = cx.sbase + S::kABOff + 16u * t;
     if (t == 0) {
         for (int k = 0; k < kSlots && k < cx.count; ++k) request<IN_F32, STAGES>(cx, xmap, xring, xbars, k);
     }
     u64 G[16];
     uint32_t T0[16], T1[16];
     for (int k = 0; k < cx.count; ++k) {
-        const int use = cx.done + k;
         tmem_ld16(cx.tlane + first_col<6, STAGES>(), T0);
         bar_sync(kFullDA, 2 * kThreads);
-        rev2_load(G, from_d, cx.a);
+#pragma unroll
+        for (int m = 0; m < 16; ++m) {
+            uint32_t lo, hi;
+            unpack2u(lds64(((m >> 1) & 1 ? from_d1 : from_d0) + 128u * m), lo, hi);
+            G[m] = (m & 1) ? pack2u(hi, lo) : pack2u(lo, hi);
+        }
         if (k + 1 < cx.count) bar_arrive(kEmptyDA, 2 * kThreads);
         walk_down<FORM, 6, 22, STAGES>(G, T0, T1, cx.tlane, [&](auto step) {
             if constexpr (decltype(step)::value == 13) {  // below stage 4: phase 2 -> 1, inside each half-warp
@@ -319,15 +345,7 @@ __device__ __forceinline__ void group_a(const Ctx& cx, const CUtensorMap* xmap) 
                 rev1_load(G, own, cx.a);
             }
         });
-        if constexpr (FORM == kFormScaled) {
-            const u64 back = pack2(1.f / kLift, 1.f / kLift);
-#pragma unroll
-            for (int m = 0; m < 16; ++m) G[m] = mul2(back, G[m]);
-        }
-        if (cx.dx != nullptr) {
-            mbar_wait_bounded(xbars + 8 * (use & 1), (use >> 1) & 1, cx.status);  // x has arrived: dx may lie over it
-            store_dx<IN_F32, STAGES>(cx, G, cx.first + k * cx.stride);
-        }
+        if constexpr (kDxByA<IN_F32, STAGES>) write_dx<FORM, IN_F32, STAGES>(cx, G, k);
         if (k > 0) {
             bar_sync(kEmptyAB, 2 * kThreads);  // B has read the row before, x too
             if (t == 0 && k + 1 < cx.count) request<IN_F32, STAGES>(cx, xmap, xring, xbars, k + 1);
@@ -355,8 +373,15 @@ __device__ __forceinline__ bool group_b(const Ctx& cx) {
     uint32_t T0[16], T1[16], A0[8], A1[8];
     for (int k = 0; k < cx.count; ++k) {
         const int use = cx.done + k, slot = use & 1;
+        bar_sync(kFullAB, 2 * kThreads);
+#pragma unroll
+        for (int c = 0; c < 8; ++c) {
+            const uint4 w = lds128(from_a + c * kThreads * 16);
+            U[2 * c] = pack2u(w.x, w.y), U[2 * c + 1] = pack2u(w.z, w.w);
+        }
         tmem_ld16(cx.tlane, T0);
         tmem_ld8(cx.tlane + kAccCol, A0);
+        if constexpr (!kDxByA<IN_F32, STAGES>) write_dx<FORM, IN_F32, STAGES>(cx, U, k);
         mbar_wait_bounded(xbars + 8 * slot, (use >> 1) & 1, cx.status);
         const uint32_t src = cx.sbase + S::kXOff + slot * S::kRow + in_line;
         if constexpr (IN_F32) {
@@ -377,12 +402,6 @@ __device__ __forceinline__ bool group_b(const Ctx& cx) {
                     X[8 * c + 2 * j + 1] = pack2u(a[j] & 0xFFFF0000u, b[j] & 0xFFFF0000u);
                 }
             }
-        }
-        bar_sync(kFullAB, 2 * kThreads);
-#pragma unroll
-        for (int c = 0; c < 8; ++c) {
-            const uint4 w = lds128(from_a + c * kThreads * 16);
-            U[2 * c] = pack2u(w.x, w.y), U[2 * c + 1] = pack2u(w.z, w.w);
         }
         if (k + 1 < cx.count) bar_arrive(kEmptyAB, 2 * kThreads);
         walk_up<FORM, 0, 8, STAGES>(X, U, T0, T1, A0, A1, cx.tlane);
@@ -436,7 +455,9 @@ __device__ __forceinline__ bool group_d(const Ctx& cx, const CUtensorMap* gmap) 
     const uint32_t g_x = ((t & 31) >> 2) ^ (t >> 5);
     const uint32_t g_a0 = (t >> 5) * 128u + (g_x << 4) + (t & 3) * 4u, g_a1 = (t >> 5) * 128u + ((g_x ^ 4u) << 4) + (t & 3) * 4u;
     const uint32_t f_a = (t >> 4) * 128u + ((((t & 15) >> 1) ^ (t >> 4)) << 4) + (t & 1) * 8u;
-    const uint32_t last = cx.sbase + S::kLastOff + 16u * t, to_a = cx.sbase + S::kDAOff, from_c = cx.sbase + S::kCDOff;
+    const uint32_t last = cx.sbase + S::kLastOff + 16u * t, from_c = cx.sbase + S::kCDOff;
+    const uint32_t i4 = (t >> 3) & 1, i5 = (t >> 4) & 1, to_a0 = cx.sbase + S::kDAOff + 16u * (t & 7) + 128u * (t >> 3) + 8u * i5;
+    const uint32_t to_a[2] = {to_a0 + 4u * i4, to_a0 + 4u * (i4 ^ 1u)};
     constexpr bool kDiagonal = STAGES < 12, kUp = STAGES > 8;
     u64 X[16], U[16], A[4][2][4];
     uint32_t T0[16], T1[16];
@@ -479,7 +500,13 @@ __device__ __forceinline__ bool group_d(const Ctx& cx, const CUtensorMap* gmap) 
                 bar_sync(kEmptyDA, 2 * kThreads);  // A has read the row before, and every warp here is past its reads of g
                 if (t == 0 && i + 1 < cx.count) request<IN_F32, STAGES>(cx, gmap, gring, gbars, i + 1);
             }
-            rev2_store(U, to_a, cx.a);
+#pragma unroll
+            for (int m = 0; m < 16; ++m) {
+                uint32_t lo, hi;
+                unpack2u(U[m], lo, hi);
+                sts32(to_a[m & 1] + 2048u * (m >> 1), lo);
+                sts32((to_a[m & 1] ^ 8u) + 2048u * (m >> 1), hi);
+            }
             __threadfence_block();
             bar_arrive(kFullDA, 2 * kThreads);
         }

@@ -309,3 +309,35 @@ def test_statistics_count_the_codes_of_the_call_without_them(n, dtype, bits):
     assert torch.equal(codes, plain[0]) and torch.equal(scales, plain[1])
     assert np.array_equal(hist.cpu().numpy(), oracle.code_histogram(oracle.unpack(codes.cpu().numpy(), bits), bits))
     np.testing.assert_allclose(to_f64(moments), oracle.row_moments(oracle.forward(to_f64(theta), to_f64(x))), rtol=2e-5)
+
+
+@pytest.mark.parametrize("n,rows", [(128, 4096), (1024, 700), (4096, 300)])
+@pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
+def test_backward_where_the_scaled_sums_overflow(n, rows, dtype):
+    """Rows of x near the end of fp32's range: stored over a product of cosines they overflow, the sums of d-theta do not.  The
+    CTAs that meet them take their rows again; dx of the other rows is the same bits."""
+    p, theta, x, xd = inputs(n, rows, dtype)
+    g = synth.rows(rows, n, "normal", 5, dtype=dtype)
+    plain = p.backward(xd, g.to(DEV))[0]
+    for r in (3, rows // 2):
+        x[r] *= 2.0 ** 110
+        g[r] *= 2.0 ** -20
+    xd.copy_(x)
+    dx, dth = p.backward(xd, g.to(DEV))
+    dx_ref, dth_ref = oracle.backward(to_f64(theta), to_f64(x), to_f64(g))
+    check_rows_close(dx, dx_ref, np.abs(to_f64(g)).max(axis=1), "dx")
+    check_dtheta(dth, dth_ref, "dtheta")
+    keep = torch.ones(rows, dtype=torch.bool, device=DEV)
+    keep[3] = keep[rows // 2] = False
+    assert torch.equal(dx[keep], plain[keep]) and p.device_status() == 0
+
+
+@pytest.mark.parametrize("n,rows,over", [(4096, 301, "g"), (4096, 301, "x"), (512, 3001, "x")])
+def test_backward_into_its_own_input(n, rows, over):
+    """dx over g or x (no CTA may need its rows a second time then): the results of separate buffers, to rounding."""
+    p, theta, x, xd = inputs(n, rows, torch.float32)
+    gd = synth.rows(rows, n, "normal", 5).to(DEV)
+    dx, dth = p.backward(xd, gd)
+    dx2, dth2 = p.backward(xd, gd, dx=gd if over == "g" else xd)
+    assert (dx2 - dx).abs().max() <= 1e-5 * dx.abs().max() and (dth2 - dth).norm() <= 1e-5 * dth.norm()
+    assert p.device_status() == 0
