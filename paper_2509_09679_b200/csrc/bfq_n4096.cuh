@@ -21,7 +21,9 @@ constexpr uint32_t kExWords = 4128;          // padded fp32 row (see the layouts
 constexpr uint32_t kExBytes = kExWords * 4;
 constexpr int kCols = 416;                   // tensor-memory columns in use
 constexpr int kFlatFloats = 11 * kN + 4 * (kN / 2);  // the same constants in the order of the angles: pairs of stages 0 .. 10, then fours
-constexpr int kFewRows = 16;                 // rows up to which k_forward_few takes a call: as many clusters of eight CTAs run at once
+// Rows up to which k_forward_few takes a call.  us, that kernel / the one for many rows, bf16 rows out: 1 row 2.6 / 5.8, 16 2.9 / 5.8, 64 4.4 / 5.9,
+// 128 5.1 / 5.9; INT4 codes: 3.1, 3.5, 5.4, 6.2 / 6.1; from fp32 rows to codes 64 5.5 / 6.1, 128 6.4 / 6.0.
+constexpr int kFewRows = 64;
 
 __device__ __forceinline__ uint4 lds128(uint32_t a) {
     uint4 v;
