@@ -1,24 +1,30 @@
 // The dense factor of the composite transform (paper Sec. 3.3): Q1 = (I - A)(I + A)^{-1}, A skew-symmetric, from its strict
 // upper triangle, and the gradient of the parameters from the gradient of Q1.
 //
-// (I - A) and (I + A)^{-1} commute, so Q1 solves (I + A) Q1 = I - A: Gauss-Jordan with partial pivoting on the augmented
-// matrix [I + A | I - A], one CTA, float64 in shared memory (I + A has all singular values >= 1).  With M = (I + A)^{-1},
-// I + Q1 = 2 M and dQ1 = -(I + Q1) dA M, so dL/dA = -(I + Q1)^T (dL/dQ1) M^T = -2 M^T (dL/dQ1) M^T and the parameter (i < j)
-// receives dL/dA[i][j] - dL/dA[j][i].
+// With M = (I + A)^{-1}: Q1 = 2 M - I, and dQ1 = -(I + Q1) dA M = -2 M dA M, so dL/dA = -2 M^T (dL/dQ1) M^T and the parameter
+// (i < j) receives dL/dA[i][j] - dL/dA[j][i].
 //
-// A column step is a chain (find the pivot, divide, update), so its latency is what counts.  Two copies of the matrix take
-// turns: every thread reads the old one (the row exchange is only a matter of where a row is read) and writes the new one,
-// one block barrier per column; every warp finds the pivot by itself; a row is 2 n1 + 1 doubles, so that the lanes that read
-// down a column fall into different banks, and a thread's loads are all issued before its stores.  Four barriers and a serial
-// pivot search per column took 96 us for n1 = 40; now 35 us, and the gradient 24 us (76 with a solve of its own).
+// The inverse, one CTA, float64.  The symmetric part of I + A is I, and so is at least that of every Schur complement: pivots are
+// 1 and more wherever one eliminates, without a search, and entries grow by at most 1 + |A|^2 in all.  So the matrix is inverted
+// in place in registers (a 16 x 16 grid of threads, up to 4 x 4 entries each, cyclic), and a column step is one chain: the owners
+// of the pivot's row and column write them to shared memory, a barrier, every thread takes the reciprocal for itself and updates its
+// entries.  Parameters above 32, where that growth would show in fp32 results, take Gauss-Jordan with partial pivoting on
+// [I + A | I - A] (`solve`).  What bounds it is that chain.  n1 = 40: the
+// pivoted solve and its gradient took 35 and 24 us; a learning step of 2048 tokens of 40 x 128 went from 243 to 196 us with these
+// two and the backward on matrix instructions.
+//
+// The gradient: M to float64 from the Q1 the caller has, and two products, on 8 x 8 x 4 float64 matrix instructions: a product on
+// the plain pipe took 4 us, most of it operands from shared memory.
 #include "../../include/bfq.h"
 
 #include <cuda_runtime.h>
 
 #include "bfq_fast.h"
+#include "bfq_n4096.cuh"
 
 namespace bfq {
 namespace cay {
+using namespace ptx;
 
 constexpr int kThreads = 256;
 
@@ -79,93 +85,197 @@ __device__ __forceinline__ const double* solve(const float* __restrict__ params,
     return cur + n1;
 }
 
-__global__ void __launch_bounds__(kThreads) k_cayley(const float* __restrict__ params, int n1, float* __restrict__ q1) {
-    extern __shared__ double aug[];  // [2][n1][pitch]
-    const double* q = solve(params, n1, aug);
-    for (int e = threadIdx.x; e < n1 * n1; e += kThreads) q1[e] = static_cast<float>(q[(e / n1) * pitch(n1) + e % n1]);
+// 1 / p for 1 <= p < 2^100: the fp32 reciprocal and two Newton steps
+__device__ __forceinline__ double reciprocal(double p) {
+    double r = static_cast<double>(__frcp_rn(static_cast<float>(p)));
+    r = fma(r, fma(-p, r, 1.0), r);
+    return fma(r, fma(-p, r, 1.0), r);
 }
 
-// out = scale a b + add I (n1 x n1, row stride n1, all threads): four rows x two columns per thread, so that eight chains
-// overlap and a value that is read serves several of them
-__device__ __forceinline__ void product(double* out, const double* a, const double* b, int n1, double scale, double add) {
-    const int cols = (n1 + 1) / 2, items = ((n1 + 3) / 4) * cols;
-    for (int it = threadIdx.x; it < items; it += kThreads) {
-        const int i0 = 4 * (it / cols), j0 = 2 * (it % cols), j1 = min(j0 + 1, n1 - 1);
-        double s[4][2];
-        const double* row[4];
+// T = ceil(n1 / 16): entries (ty + 16 a, tx + 16 b) of thread (tx, ty); rows and columns from n1 on are never pivots
+template <int T>
+__device__ __forceinline__ void invert(double (&m)[T][T], int n1, double (&line)[2][2][64]) {
+    const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
+    auto publish = [&](int k) {  // row k and column k
+        double(&to)[2][64] = line[k & 1];
 #pragma unroll
-        for (int r = 0; r < 4; ++r) s[r][0] = s[r][1] = 0.0, row[r] = a + min(i0 + r, n1 - 1) * n1;
-#pragma unroll 4
-        for (int k = 0; k < n1; ++k) {
-            const double x = b[k * n1 + j0], y = b[k * n1 + j1];
+        for (int a = 0; a < T; ++a)
+            if (ty + 16 * a == k) {
 #pragma unroll
-            for (int r = 0; r < 4; ++r) s[r][0] = fma(row[r][k], x, s[r][0]), s[r][1] = fma(row[r][k], y, s[r][1]);
-        }
+                for (int b = 0; b < T; ++b) to[0][tx + 16 * b] = m[a][b];
+            }
 #pragma unroll
-        for (int r = 0; r < 4; ++r)
+        for (int b = 0; b < T; ++b)
+            if (tx + 16 * b == k) {
 #pragma unroll
-            for (int c = 0; c < 2; ++c)
-                if (i0 + r < n1 && j0 + c < n1) out[(i0 + r) * n1 + j0 + c] = scale * s[r][c] + (i0 + r == j0 + c ? add : 0.0);
+                for (int a = 0; a < T; ++a) to[1][ty + 16 * a] = m[a][b];
+            }
+        __syncthreads();
+    };
+    for (int k = 0; k < n1; ++k) {
+        publish(k);
+        const double(&at)[2][64] = line[k & 1];
+        double row[T], col[T];
+#pragma unroll
+        for (int a = 0; a < T; ++a) row[a] = at[0][tx + 16 * a], col[a] = at[1][ty + 16 * a];
+        const double inv = reciprocal(at[0][k]);
+#pragma unroll
+        for (int b = 0; b < T; ++b) row[b] *= inv;
+#pragma unroll
+        for (int a = 0; a < T; ++a)
+#pragma unroll
+            for (int b = 0; b < T; ++b) {
+                const bool in_row = ty + 16 * a == k, in_col = tx + 16 * b == k;
+                const double other = fma(-col[a], row[b], m[a][b]);
+                m[a][b] = in_row ? (in_col ? inv : row[b]) : (in_col ? -col[a] * inv : other);
+            }
     }
 }
 
-// M = (I + A)^{-1} in float64 from the Q1 the caller has: (I + Q1) / 2 is M to fp32 rounding, and each Newton step
-// M (2 I - (I + A) M) squares the error (residual of the first guess up to |A| 2^-24; two steps).  If Q1 is not the transform of
-// these parameters (the first residual is not small) the solve is done after all.  Six small products instead of a solve.
+__device__ __forceinline__ float parameter(const float* __restrict__ params, int n1, int i, int j) {  // A[i][j]
+    if (i == j) return 0.f;
+    const int lo = min(i, j), hi = max(i, j);
+    const float v = __ldg(params + lo * n1 - lo * (lo + 1) / 2 + (hi - lo - 1));
+    return i < j ? v : -v;
+}
+
+template <int T>
+__global__ void __launch_bounds__(kThreads) k_cayley(const float* __restrict__ params, int n1, float* __restrict__ q1) {
+    extern __shared__ double aug[];  // [2][n1][pitch], for `solve`
+    __shared__ double line[2][2][64];
+    const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
+    grid_dep_launch();
+    grid_dep_wait();
+    double m[T][T];
+    bool large = false;
+#pragma unroll
+    for (int a = 0; a < T; ++a)
+#pragma unroll
+        for (int b = 0; b < T; ++b) {
+            const int i = ty + 16 * a, j = tx + 16 * b;
+            const float v = i < n1 && j < n1 ? parameter(params, n1, i, j) : 0.f;
+            large |= !(fabsf(v) <= 32.f);
+            m[a][b] = static_cast<double>(v) + (i == j ? 1.0 : 0.0);
+        }
+    if (__syncthreads_or(large)) {
+        const double* q = solve(params, n1, aug);
+        for (int e = threadIdx.x; e < n1 * n1; e += kThreads) q1[e] = static_cast<float>(q[(e / n1) * pitch(n1) + e % n1]);
+        return;
+    }
+    invert<T>(m, n1, line);
+#pragma unroll
+    for (int a = 0; a < T; ++a)
+#pragma unroll
+        for (int b = 0; b < T; ++b) {
+            const int i = ty + 16 * a, j = tx + 16 * b;
+            if (i < n1 && j < n1) q1[i * n1 + j] = static_cast<float>(2.0 * m[a][b] - (i == j ? 1.0 : 0.0));
+        }
+}
+
+// matrices of the gradient: np = n1 rounded up to 8 rows of np + 4 numbers, zero from n1 on (the pitch spreads the eight rows of a
+// fragment over the banks)
+__host__ __device__ constexpr int padded(int n1) { return (n1 + 7) & ~7; }
+__host__ __device__ constexpr int row_of(int n1) { return padded(n1) + 4; }
+
+__device__ __forceinline__ void mma_884(double (&c)[2], double a, double b) {
+    asm volatile("mma.sync.aligned.m8n8k4.row.col.f64.f64.f64.f64 {%0,%1}, {%2}, {%3}, {%0,%1};" : "+d"(c[0]), "+d"(c[1]) : "d"(a), "d"(b));
+}
+
+// out = scale op(a) op(b) + add I: a warp takes 8 x 8 blocks, all its blocks' chains side by side.  AT / BT: the operand is stored
+// transposed.  Ends in a barrier.
+template <bool AT, bool BT>
+__device__ __forceinline__ void product(double* out, const double* a, const double* b, int n1, double scale, double add) {
+    constexpr int kWarps = kThreads / 32, kMost = 64 / kWarps;  // blocks of a warp at most
+    const int nb = padded(n1) / 8, blocks = nb * nb, w = row_of(n1), warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, q = lane & 3;
+    const int mine = (blocks - warp + kWarps - 1) / kWarps;
+    double acc[kMost][2];
+    const double *pa[kMost], *pb[kMost];
+#pragma unroll
+    for (int i = 0; i < kMost; ++i) {
+        const int blk = min(warp + i * kWarps, blocks - 1), bi = 8 * (blk / nb), bj = 8 * (blk % nb);
+        acc[i][0] = acc[i][1] = 0.0;
+        pa[i] = AT ? a + q * w + bi + g : a + (bi + g) * w + q;
+        pb[i] = BT ? b + (bj + g) * w + q : b + q * w + bj + g;
+    }
+    for (int k = 0; k < 2 * nb; ++k) {
+#pragma unroll
+        for (int i = 0; i < kMost; ++i)
+            if (i < mine) mma_884(acc[i], pa[i][AT ? 4 * k * w : 4 * k], pb[i][BT ? 4 * k : 4 * k * w]);
+    }
+#pragma unroll
+    for (int i = 0; i < kMost; ++i) {
+        if (i >= mine) continue;
+        const int blk = warp + i * kWarps, r = 8 * (blk / nb) + g, c = 8 * (blk % nb) + 2 * q;
+        out[r * w + c] = scale * acc[i][0] + (r == c ? add : 0.0);
+        out[r * w + c + 1] = scale * acc[i][1] + (r == c + 1 ? add : 0.0);
+    }
+    __syncthreads();
+}
+
+// M = (I + A)^{-1} in float64 from the Q1 the caller has: (I + Q1) / 2 is M to fp32 rounding (residual up to |A| 2^-24), and a
+// Newton step M (2 I - (I + A) M) squares the residual; a second one follows where the first residual's square is not far below
+// fp32 rounding.  If Q1 is not the transform of these parameters (the first residual is not small) the solve is done after all.
 __global__ void __launch_bounds__(kThreads) k_cayley_backward(const float* __restrict__ params, int n1, const float* __restrict__ q1,
                                                               const float* __restrict__ dq1, float* __restrict__ dparams) {
-    extern __shared__ double aug[];  // [2][n1][pitch] of the solve = four n1 x n1 matrices and more, then two
-    const int t = threadIdx.x, nn = n1 * n1;
-    double *ia = aug, *m = ia + nn, *r = m + nn, *next = r + nn;  // I + A, M, 2 I - (I + A) M, the next M
-    double* g = aug + 2 * n1 * pitch(n1);
-    double* left = g + nn;
-    __shared__ int far;
-    if (t == 0) far = 0;
-    for (int e = t; e < nn; e += kThreads) {
-        const int i = e / n1, j = e % n1;
-        double a = 0.0;
-        if (i < j) a = static_cast<double>(params[i * n1 - i * (i + 1) / 2 + (j - i - 1)]);
-        if (i > j) a = -static_cast<double>(params[j * n1 - j * (j + 1) / 2 + (i - j - 1)]);
+    extern __shared__ double aug[];  // [2][n1][pitch] of the solve, or I + A, M, 2 I - (I + A) M, the next M; then dQ1
+    const int t = threadIdx.x, np = padded(n1), w = row_of(n1), size = np * w;
+    double *ia = aug, *m = ia + size, *r = m + size, *next = r + size, *g = next + size;
+    grid_dep_launch();
+    grid_dep_wait();
+    for (int e = t; e < np * np; e += kThreads) {
+        const int i = e / np, j = e % np, at = i * w + j;
+        const bool in = i < n1 && j < n1;
         const double id = i == j ? 1.0 : 0.0;
-        ia[e] = id + a;
-        m[e] = 0.5 * (id + static_cast<double>(q1[e]));
-        g[e] = static_cast<double>(dq1[e]);
+        ia[at] = in ? id + static_cast<double>(parameter(params, n1, i, j)) : 0.0;
+        m[at] = in ? 0.5 * (id + static_cast<double>(__ldg(q1 + i * n1 + j))) : 0.0;
+        g[at] = in ? static_cast<double>(__ldg(dq1 + i * n1 + j)) : 0.0;
     }
     __syncthreads();
-    for (int step = 0; step < 2; ++step) {
-        product(r, ia, m, n1, -1.0, 2.0);
-        __syncthreads();
-        if (step == 0) {
-            for (int e = t; e < nn; e += kThreads)
-                if (!(fabs(r[e] - (e / n1 == e % n1 ? 1.0 : 0.0)) < 1e-4)) far = 1;
-            __syncthreads();
-            if (far != 0) break;
+    // whether an entry of I - (I + A) M is not below a limit (NaN is not); rows and columns from n1 on hold 2 I there
+    auto above = [&](double limit) {
+        bool far = false;
+        for (int e = t; e < n1 * n1; e += kThreads) {
+            const int i = e / n1, j = e % n1;
+            far |= !(fabs(r[i * w + j] - (i == j ? 1.0 : 0.0)) < limit);
         }
-        product(next, m, r, n1, 1.0, 0.0);
+        return __syncthreads_or(far) != 0;
+    };
+    product<false, false>(r, ia, m, n1, -1.0, 2.0);
+    if (!above(1e-4)) {
+        const bool twice = above(1e-6);  // else the residual's square, at most 64^2 1e-12, leaves M better than 4e-9
+        product<false, false>(next, m, r, n1, 1.0, 0.0);
+        double* done = next;
+        if (twice) {
+            product<false, false>(r, ia, next, n1, -1.0, 2.0);
+            product<false, false>(m, next, r, n1, 1.0, 0.0);
+            done = m;
+        }
+        m = done;
+    } else {
+        const double* q = solve(params, n1, aug);  // dQ1 lies behind its two buffers
         __syncthreads();
-        double* tmp = m;
-        m = next, next = tmp;
-    }
-    if (far != 0) {  // uniform
-        const double* q = solve(params, n1, aug);
-        // 2 M = I + Q1, kept in `left` while the solve's buffers turn back into matrices
-        for (int e = t; e < nn; e += kThreads) left[e] = 0.5 * (q[(e / n1) * pitch(n1) + e % n1] + (e / n1 == e % n1 ? 1.0 : 0.0));
+        double keep[64 * 64 / kThreads];
+#pragma unroll
+        for (int e = 0; e < 64 * 64 / kThreads; ++e) {  // 2 M = I + Q1, while the solve's buffers turn back into matrices
+            const int at = t + e * kThreads, i = at / np, j = at % np;
+            keep[e] = at < np * np && i < n1 && j < n1 ? 0.5 * (q[i * pitch(n1) + j] + (i == j ? 1.0 : 0.0)) : 0.0;
+        }
         __syncthreads();
         m = aug;
-        for (int e = t; e < nn; e += kThreads) m[e] = left[e];
+#pragma unroll
+        for (int e = 0; e < 64 * 64 / kThreads; ++e) {
+            const int at = t + e * kThreads;
+            if (at < np * np) m[(at / np) * w + at % np] = keep[e];
+        }
         __syncthreads();
-        r = aug + nn;
     }
-    // dL/dA = -2 M^T dQ1 M^T; M^T in r
-    for (int e = t; e < nn; e += kThreads) r[(e % n1) * n1 + e / n1] = m[e];
-    __syncthreads();
-    product(left, r, g, n1, 1.0, 0.0);
-    __syncthreads();
-    product(g, left, r, n1, -2.0, 0.0);
-    __syncthreads();
-    for (int e = t; e < nn; e += kThreads) {
+    // dL/dA = -2 M^T dQ1 M^T
+    double *left = m == ia ? r : ia, *both = r == left ? next : r;
+    product<true, false>(left, m, g, n1, 1.0, 0.0);
+    product<false, true>(both, left, m, n1, -2.0, 0.0);
+    for (int e = t; e < n1 * n1; e += kThreads) {
         const int i = e / n1, j = e % n1;
-        if (i < j) dparams[i * n1 - i * (i + 1) / 2 + (j - i - 1)] = static_cast<float>(g[i * n1 + j] - g[j * n1 + i]);
+        if (i < j) dparams[i * n1 - i * (i + 1) / 2 + (j - i - 1)] = static_cast<float>(both[i * w + j] - both[j * w + i]);
     }
 }
 
@@ -174,12 +284,22 @@ __global__ void __launch_bounds__(kThreads) k_cayley_backward(const float* __res
 // shared memory for n1 rows, and the limit of every n1: set once per device (a limit per call would be pulled away by another
 // thread's call with a smaller n1)
 static constexpr size_t cayley_smem(int n1) { return sizeof(double) * 2 * n1 * cay::pitch(n1); }
-static constexpr size_t cayley_backward_smem(int n1) { return cayley_smem(n1) + sizeof(double) * 2 * n1 * n1; }
+static constexpr size_t cayley_backward_smem(int n1) { return sizeof(double) * 5 * cay::padded(n1) * cay::row_of(n1); }
+static_assert(4 * cay::padded(64) * cay::row_of(64) >= 2 * 64 * cay::pitch(64) && cayley_backward_smem(64) <= 227 * 1024, "room for the solve, and in a CTA");
+template <class F>
+static cudaError_t for_tile(int n1, F&& f) {
+    if (n1 <= 16) return f(cay::k_cayley<1>);
+    if (n1 <= 32) return f(cay::k_cayley<2>);
+    if (n1 <= 48) return f(cay::k_cayley<3>);
+    return f(cay::k_cayley<4>);
+}
 static cudaError_t allow_smem(int device) {
     static bool allowed[kMaxDevices] = {false};
     if (allowed[device]) return cudaSuccess;
-    cudaError_t e = cudaFuncSetAttribute(cay::k_cayley, cudaFuncAttributeMaxDynamicSharedMemorySize, int(cayley_smem(BFQ_MAX_N1)));
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(cay::k_cayley_backward, cudaFuncAttributeMaxDynamicSharedMemorySize, int(cayley_backward_smem(BFQ_MAX_N1)));
+    cudaError_t e = cudaFuncSetAttribute(cay::k_cayley_backward, cudaFuncAttributeMaxDynamicSharedMemorySize, int(cayley_backward_smem(BFQ_MAX_N1)));
+    for (int n1 = 16; n1 <= 64; n1 += 16)
+        if (e == cudaSuccess)
+            e = for_tile(n1, [](auto kern) { return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(cayley_smem(BFQ_MAX_N1))); });
     allowed[device] = e == cudaSuccess;
     return e;
 }
@@ -187,15 +307,13 @@ static cudaError_t allow_smem(int device) {
 cudaError_t cayley_launch(const bfq_plan* plan, const float* params, int n1, float* q1, cudaStream_t st) {
     cudaError_t e = allow_smem(plan->device);
     if (e != cudaSuccess) return e;
-    cay::k_cayley<<<1, cay::kThreads, cayley_smem(n1), st>>>(params, n1, q1);
-    return cudaGetLastError();
+    return for_tile(n1, [&](auto kern) { return launch_overlapped(kern, dim3(1), dim3(cay::kThreads), cayley_smem(n1), st, params, n1, q1); });
 }
 
 cudaError_t cayley_backward_launch(const bfq_plan* plan, const float* params, int n1, const float* q1, const float* dq1, float* dparams, cudaStream_t st) {
     cudaError_t e = allow_smem(plan->device);
     if (e != cudaSuccess) return e;
-    cay::k_cayley_backward<<<1, cay::kThreads, cayley_backward_smem(n1), st>>>(params, n1, q1, dq1, dparams);
-    return cudaGetLastError();
+    return launch_overlapped(cay::k_cayley_backward, dim3(1), dim3(cay::kThreads), cayley_backward_smem(n1), st, params, n1, q1, dq1, dparams);
 }
 
 }  // namespace bfq
