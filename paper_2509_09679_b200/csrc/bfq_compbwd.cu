@@ -18,9 +18,10 @@
 // walks, and 20 KB of memory traffic in bf16, so the arithmetic bounds it (2048 tokens: 29 us at one multiply-add per lane and
 // cycle).  Composed from a dense product on permuted copies, the butterfly backward on 40 rows per token, a forward in fp32
 // and another dense product it took about 1000 us for 2048 tokens, and G' went through bf16 in between; this kernel
-// takes 145 us (191 us with scalar multiply-adds).
+// takes 145 us (191 us with scalar multiply-adds) where G is fp32; bf16 G: k_composite_backward_mma.
 #include "../../include/bfq.h"
 
+#include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
 #include "bfq_fast.h"
@@ -215,6 +216,182 @@ __global__ void __launch_bounds__(kThreads, 2) k_composite_backward(const Params
     }
 }
 
+// ---- bf16 gradients: the two dense products on the tensor cores ----------------------------------------------------
+// G in bf16 is an exact operand.  The other one, Q1 or X', goes in as three bf16 terms, 24 significant bits, so the products are those of
+// fp32 numbers and their sums are fp32 (m16n8k16; the small terms first or apart).  G stays in shared memory as bf16 rows, read as
+// matrices of 8 x 8 either way; Q1's terms are there as fragments; X' is split as it is read.
+// (a, b) = t[0] + t[1] + t[2], largest first: eight significant bits each, cut off, so that the sum is exact
+__device__ __forceinline__ void three_terms(float a, float b, uint32_t (&t)[3]) {
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+        t[i] = __byte_perm(__float_as_uint(a), __float_as_uint(b), 0x7632);
+        a -= __uint_as_float(__float_as_uint(a) & 0xFFFF0000u), b -= __uint_as_float(__float_as_uint(b) & 0xFFFF0000u);
+    }
+}
+__device__ __forceinline__ void mma_bf16(float (&c)[4], const uint4& a, uint32_t b0, uint32_t b1) {
+    asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
+                 : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
+                 : "r"(a.x), "r"(a.y), "r"(a.z), "r"(a.w), "r"(b0), "r"(b1));
+}
+__device__ __forceinline__ uint4 matrices(uint32_t at) {
+    uint4 v;
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(at) : "memory");
+    return v;
+}
+__device__ __forceinline__ uint4 matrices_transposed(uint32_t at) {
+    uint4 v;
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(at) : "memory");
+    return v;
+}
+
+constexpr int kWarps = kThreads / 32;
+// MT blocks of 16 runs.  dL/dQ1 is cut into tiles of 16 x 8, a warp has up to kTiles of them; with fewer tiles than warps, slices of the
+// positions go to different warps
+template <int L, int MT>
+struct Mma {
+    static constexpr int kTiles = MT <= 2 ? 1 : MT, kRow = (1 << L) + 8;  // bf16 of a row of G: 16 bytes off a multiple of 128
+    static constexpr int kFragments = 3 * MT * MT * 32;                   // uint4 of Q1
+    static size_t smem(int n1) { return size_t(16) * kFragments + size_t(2) * 16 * MT * kRow + sizeof(float) * 2 * n1 * Geo<L>::kPitch; }
+};
+
+template <int L, int MT>
+__global__ void __launch_bounds__(kThreads, 2) k_composite_backward_mma(const Params p) {
+    using Ge = Geo<L>;
+    using M = Mma<L, MT>;
+    extern __shared__ __align__(16) uint4 sm4[];
+    const int n1 = p.n1, t = threadIdx.x, warp = t >> 5, lane = t & 31, g8 = lane >> 2, q = lane & 3;
+    uint4* const frag = sm4;  // [term][block of k][block of rows][lane]: element [row][k] = Q1[k][row]
+    uint16_t* const Gb = reinterpret_cast<uint16_t*>(sm4 + M::kFragments);
+    float* const X = reinterpret_cast<float*>(Gb + 16 * MT * M::kRow);
+    float* const W = X + n1 * Ge::kPitch;
+    for (int e = t; e < MT * MT * 32; e += kThreads) {
+        const int l = e & 31, mt = (e >> 5) % MT, kt = (e >> 5) / MT;
+        uint32_t w[4][3];
+#pragma unroll
+        for (int r = 0; r < 4; ++r) {
+            const int row = 16 * mt + (l >> 2) + 8 * (r & 1), k = 16 * kt + 2 * (l & 3) + 8 * (r >> 1);
+            auto at = [&](int i) { return i < n1 && row < n1 ? p.q1[i * n1 + row] : 0.f; };
+            three_terms(at(k), at(k + 1), w[r]);
+        }
+#pragma unroll
+        for (int i = 0; i < 3; ++i) frag[i * MT * MT * 32 + e] = make_uint4(w[0][i], w[1][i], w[2][i], w[3][i]);
+    }
+    for (int e = n1 * M::kRow + t; e < 16 * MT * M::kRow; e += kThreads) Gb[e] = 0;  // runs that do not exist
+    const uint32_t gbase = smem_u32(Gb);
+    const int u = t % Ge::kU, r0 = t / Ge::kU;
+    const int nt = (n1 + 7) / 8, tiles = MT * nt;
+    const int slices = tiles >= kWarps ? 1 : kWarps / tiles, slice = tiles >= kWarps ? 0 : warp / tiles;
+    const int first_tile = tiles >= kWarps ? warp : (slice < slices ? warp % tiles : tiles);
+    float acc[4][3][4], dq[M::kTiles][4];
+#pragma unroll
+    for (int i = 0; i < 48; ++i) acc[i / 12][i / 4 % 3][i & 3] = 0.f;
+#pragma unroll
+    for (int i = 0; i < 4 * M::kTiles; ++i) dq[i >> 2][i & 3] = 0.f;
+
+    for (int64_t row = blockIdx.x; row < p.rows; row += gridDim.x) {
+        __syncthreads();  // the buffers' readers of the token before are done
+        load_token<L>(p.x, p.xt, row, p.ld, n1, X);
+        {
+            const uint4* src = reinterpret_cast<const uint4*>(static_cast<const __nv_bfloat16*>(p.g) + row * p.ld);
+            for (int c = t; c < n1 * (Ge::kN2 / 8); c += kThreads)
+                *reinterpret_cast<uint4*>(Gb + (c / (Ge::kN2 / 8)) * M::kRow + 8 * (c % (Ge::kN2 / 8))) = __ldg(src + c);
+        }
+        __syncthreads();
+        // G' = Q1^T G: a warp takes 16 positions at a time
+        for (int j0 = 16 * warp; j0 < Ge::kN2; j0 += 16 * kWarps) {
+            uint4 b[MT];
+            float s[MT][2][4];
+#pragma unroll
+            for (int kt = 0; kt < MT; ++kt) b[kt] = matrices_transposed(gbase + 2u * ((16 * kt + (lane & 15)) * M::kRow + j0 + 8 * (lane >> 4)));
+#pragma unroll
+            for (int i = 0; i < 8 * MT; ++i) s[i >> 3][(i >> 2) & 1][i & 3] = 0.f;
+#pragma unroll
+            for (int term = 2; term >= 0; --term)
+#pragma unroll
+                for (int kt = 0; kt < MT; ++kt)
+#pragma unroll
+                    for (int mt = 0; mt < MT; ++mt) {
+                        const uint4 a = frag[((term * MT + kt) * MT + mt) * 32 + lane];
+                        mma_bf16(s[mt][0], a, b[kt].x, b[kt].y);
+                        mma_bf16(s[mt][1], a, b[kt].z, b[kt].w);
+                    }
+#pragma unroll
+            for (int mt = 0; mt < MT; ++mt)
+#pragma unroll
+                for (int h = 0; h < 2; ++h)
+#pragma unroll
+                    for (int c = 0; c < 2; ++c) {
+                        const int r = 16 * mt + g8 + 8 * c;
+                        if (r < n1) *reinterpret_cast<float2*>(W + r * Ge::kPitch + place(j0 + 8 * h + 2 * q)) = make_float2(s[mt][h][2 * c], s[mt][h][2 * c + 1]);
+                    }
+        }
+        passes_up<L, 0>(X, p.tw, n1, u, r0);  // ends in a barrier
+        // dL/dQ1 += G X'^T
+#pragma unroll
+        for (int i = 0; i < M::kTiles; ++i) {
+            const int tile = first_tile + i * kWarps;
+            if (tile >= tiles) continue;
+            const int mt = tile % MT, run = min(8 * (tile / MT) + g8, n1 - 1);
+            const uint32_t arow = gbase + 2u * ((16 * mt + (lane & 15)) * M::kRow + 8 * (lane >> 4));
+            const float* xr = X + run * Ge::kPitch;
+            // a token's own sums, the large terms in two chains and the small ones in a third, then one rounded addition each: an MMA
+            // cuts its sum off where a multiply-add rounds it, which a chain over all tokens would collect
+            float part[3][4];
+#pragma unroll
+            for (int c = 0; c < 12; ++c) part[c >> 2][c & 3] = 0.f;
+#pragma unroll 4
+            for (int j = 16 * slice, k = 0; j < Ge::kN2; j += 16 * slices, k ^= 1) {
+                const uint4 a = matrices(arow + 2u * j);
+                const float2 lo = *reinterpret_cast<const float2*>(xr + place(j + 2 * q)), hi = *reinterpret_cast<const float2*>(xr + place(j + 8 + 2 * q));
+                uint32_t b0[3], b1[3];
+                three_terms(lo.x, lo.y, b0), three_terms(hi.x, hi.y, b1);
+                mma_bf16(part[2], a, b0[2], b1[2]);
+                mma_bf16(part[2], a, b0[1], b1[1]);
+                if (k == 0) mma_bf16(part[0], a, b0[0], b1[0]);
+                else mma_bf16(part[1], a, b0[0], b1[0]);
+            }
+#pragma unroll
+            for (int c = 0; c < 4; ++c) dq[i][c] += (part[0][c] + part[1][c]) + part[2][c];
+        }
+        __syncthreads();
+        passes_down<L, Ge::kPasses - 1>(X, W, p, row, u, r0, acc);
+    }
+
+    // ---- the CTA's sums, in the order of the run lanes and of the slices, to its slot ----
+    float* const sm = reinterpret_cast<float*>(sm4);
+    __syncthreads();
+    float* out = p.partial + static_cast<int64_t>(blockIdx.x) * (Ge::kAngles + n1 * n1);
+    for (int e = t; e < Ge::kAngles; e += kThreads) sm[e] = 0.f;
+    __syncthreads();
+    for (int r = 0; r < Ge::kRuns; ++r) {
+        if (r0 == r) add_angles<L, 0>(sm, u, acc);
+        __syncthreads();
+    }
+    for (int e = t; e < Ge::kAngles; e += kThreads) out[e] = sm[e];
+    __syncthreads();
+    if (slices > 1) {  // one tile per warp
+#pragma unroll
+        for (int c = 0; c < 4; ++c) sm[4 * t + c] = dq[0][c];
+        __syncthreads();
+        if (slice == 0)
+            for (int s = 1; s < slices; ++s)
+#pragma unroll
+                for (int c = 0; c < 4; ++c) dq[0][c] += sm[4 * (t + 32 * s * tiles) + c];
+    }
+    if (slice == 0) {
+#pragma unroll
+        for (int i = 0; i < M::kTiles; ++i) {
+            const int tile = first_tile + i * kWarps;
+            if (tile >= tiles) continue;
+#pragma unroll
+            for (int c = 0; c < 4; ++c) {
+                const int r = 16 * (tile % MT) + g8 + 8 * (c >> 1), k = 8 * (tile / MT) + 2 * q + (c & 1);
+                if (r < n1 && k < n1) out[Ge::kAngles + r * n1 + k] = dq[i][c];
+            }
+        }
+    }
+}
+
 // dtheta [angles], dq1 [count - angles]: the slots' entries added in a fixed order (a block = 32 slot lanes x 32 entries)
 __global__ void __launch_bounds__(1024) k_reduce_composite(const float* __restrict__ partial, int slots, int count, int angles,
                                                            float* __restrict__ dtheta, float* __restrict__ dq1) {
@@ -235,37 +412,45 @@ __global__ void __launch_bounds__(1024) k_reduce_composite(const float* __restri
     }
 }
 
-template <int L, int TILES>
-static cudaError_t launch(const bfq_plan* plan, Params p, float* dtheta, float* dq1, cudaStream_t st) {
-    using G = Geo<L>;
-    const int n1p = (p.n1 + 7) & ~7;
-    size_t floats = size_t(3) * p.n1 * G::kPitch + size_t(p.n1) * n1p;
-    if (floats < size_t(G::kAngles)) floats = G::kAngles;  // the sums at the end
-    if (floats < size_t(kThreads)) floats = kThreads;
-    const size_t smem = floats * sizeof(float);
-    auto kern = k_composite_backward<L, TILES>;
-    // as for the forward kernel: the limit of every n1, and CTAs per SM for each
-    static int8_t per_sm[kMaxDevices][BFQ_MAX_N1 + 1] = {{0}};
-    int8_t& occ = per_sm[plan->device][p.n1];
+// runs a kernel on as many CTAs as are resident (and have room for their sums), then adds the CTAs' sums; per_sm: CTAs per SM for
+// each n1, found on the first call.  The limit of shared memory is that of every n1 (one per call would be pulled away by another
+// thread's call).
+static cudaError_t run(const bfq_plan* plan, void (*kern)(Params), size_t smem, int8_t& per_sm, int angles, const Params& p, float* dtheta, float* dq1,
+                       cudaStream_t st) {
     cudaError_t e = cudaSuccess;
-    if (occ == 0) {
+    if (per_sm == 0) {
         e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kBackwardSmem);
         if (e != cudaSuccess) return e;
         int o = 0;
         e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o, kern, kThreads, smem);
         if (e != cudaSuccess) return e;
-        occ = static_cast<int8_t>(o > 0 ? o : 1);
+        per_sm = static_cast<int8_t>(o > 0 ? o : 1);
     }
-    const int count = G::kAngles + p.n1 * p.n1;
-    int64_t grid = int64_t(plan->sm_count) * occ;
+    const int count = angles + p.n1 * p.n1;
+    int64_t grid = int64_t(plan->sm_count) * per_sm;
     if (grid > p.rows) grid = p.rows;
     if (grid * count > int64_t(plan->partial_floats)) grid = int64_t(plan->partial_floats) / count;
     if (grid < 1) return cudaErrorInvalidValue;
     kern<<<int(grid), kThreads, smem, st>>>(p);
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    k_reduce_composite<<<(count + 31) / 32, 1024, 0, st>>>(p.partial, int(grid), count, G::kAngles, dtheta, dq1);
+    k_reduce_composite<<<(count + 31) / 32, 1024, 0, st>>>(p.partial, int(grid), count, angles, dtheta, dq1);
     return cudaGetLastError();
+}
+
+template <int L, int BLOCKS>  // blocks of 16 runs
+static cudaError_t launch(const bfq_plan* plan, const Params& p, float* dtheta, float* dq1, cudaStream_t st) {
+    using G = Geo<L>;
+    static int8_t per_sm[2][kMaxDevices][BFQ_MAX_N1 + 1] = {{{0}}};
+    const size_t at_end = sizeof(float) * (G::kAngles > 4 * kThreads ? G::kAngles : 4 * kThreads);  // the sums
+    if (p.gt == kBF16) {
+        const size_t smem = Mma<L, BLOCKS>::smem(p.n1);
+        if (smem <= kBackwardSmem)
+            return run(plan, k_composite_backward_mma<L, BLOCKS>, smem > at_end ? smem : at_end, per_sm[1][plan->device][p.n1], G::kAngles, p, dtheta, dq1, st);
+    }
+    const int n1p = (p.n1 + 7) & ~7;
+    const size_t smem = sizeof(float) * (size_t(3) * p.n1 * G::kPitch + size_t(p.n1) * n1p);
+    return run(plan, k_composite_backward<L, BLOCKS>, smem > at_end ? smem : at_end, per_sm[0][plan->device][p.n1], G::kAngles, p, dtheta, dq1, st);
 }
 
 template <int L>
