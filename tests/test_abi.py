@@ -107,3 +107,14 @@ def test_binding_rejects_bad_tensors_before_any_launch(monkeypatch):
         binding._rows(torch.zeros((4, 300)).as_strided((4, 256), (100, 1)), 256)   # overlapping rows
     with pytest.raises(ValueError, match="expected 4 rows"):
         binding._rows(torch.zeros((5, 256)), 256, None, 4, "out")
+
+
+def test_the_plain_forms_leave_everything_else_to_the_binding():
+    """fast_calls answers None to what is not plain rows on a plan's device: no plan, host tensors, other types and counts."""
+    import torch
+    fast = binding._fast
+    x = torch.zeros((2, 8))
+    for call in (fast.forward, fast.inverse):
+        assert call(0, 8, 0, x) is None and call(64, 8, 0, x) is None and call(64, 8, 0, [1.0]) is None and call(64, 8, 0) is None
+        assert call("plan", 8, 0, x) is None and call(64, 8.0, 0, x) is None
+    assert fast.forward_quant(64, 8, 0, x, 4) is None and fast.forward_quant(64, 8, 0, x, "4") is None
