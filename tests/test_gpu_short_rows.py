@@ -341,3 +341,33 @@ def test_backward_into_its_own_input(n, rows, over):
     dx2, dth2 = p.backward(xd, gd, dx=gd if over == "g" else xd)
     assert (dx2 - dx).abs().max() <= 1e-5 * dx.abs().max() and (dth2 - dth).norm() <= 1e-5 * dth.norm()
     assert p.device_status() == 0
+
+
+def test_backward_rounds_each_row_once_into_the_sums():
+    """d-theta against 64 bits (n = 4096).  A running sum of m rows with one rounding each is off by 2.5e-8 sqrt(m / 2) of the total (the
+    mean square of a rounding to 24 bits, the sum growing as a random walk), 4.3e-7 here with the 2e-7 that the rows' own rounding
+    gives; with two roundings per row it is 5.7e-7."""
+    n, rows = 4096, 65536
+    theta = synth.angles(n, "normal", 1)
+    p = Plan(n, DEV)
+    p.set_angles(theta.to(DEV))
+    x = synth.rows(rows, n, "student_t3", 3, outliers=8, outlier_scale=50.0, dtype=torch.bfloat16, device=DEV)
+    g = synth.rows(rows, n, "normal", 4, dtype=torch.bfloat16, device=DEV)
+    dth = p.backward(x, g)[1].double()
+    th = theta.to(DEV).double()
+    ref = torch.zeros_like(dth)
+    for r in range(0, rows, 16384):
+        u, v = x[r:r + 16384].double(), g[r:r + 16384].double()
+
+        def turn(w, s, back):
+            lo, hi = w.view(-1, n >> (s + 1), 2, 1 << s).unbind(2)
+            c, sn = torch.cos(th[s]).view(-1, 1 << s), torch.sin(th[s]).view(-1, 1 << s) * (-1 if back else 1)
+            return torch.stack((c * lo - sn * hi, sn * lo + c * hi), 2).view(-1, n)
+        for s in range(12):
+            u = turn(u, s, False)
+        for s in reversed(range(12)):
+            (ul, uh), (vl, vh) = (w.view(-1, n >> (s + 1), 2, 1 << s).unbind(2) for w in (u, v))
+            ref[s] += (vh * ul - vl * uh).sum(0).reshape(-1)
+            u, v = turn(u, s, True), turn(v, s, True)
+    assert (dth - ref).norm() <= 4.9e-7 * ref.norm()
+    assert p.device_status() == 0
