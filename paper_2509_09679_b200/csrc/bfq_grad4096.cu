@@ -22,9 +22,10 @@
 // exactly where it has to be regrouped.  B's and C's sums are in the tensor-memory columns that the constants leave free, D's
 // in registers (the groups' register shares differ); half of the last stage's constants are in shared memory instead.
 //
-// Range: factors of 2^-40 and more (else the three-shear form runs: `form`), and g comes down 2^20 times too large, so that 32
-// bits hold either end.  What overflows all the same leaves a sum that is not finite; the CTA then does its rows again
-// in the three-shear form, which has no factors, and rewrites only those pieces of dx that were not finite.
+// Range: factors of 2^-40 and more (else the three-shear form runs: `form`), and g comes down 2^40 times too large, so that nothing
+// is stored smaller than it is: however small g, no bits are lost.  What overflows instead (with the least factors g from about 2^80 on,
+// products of u and x from 2^48 on) leaves a sum that is not finite; the CTA then does its rows again in the three-shear form, which
+// has no factors, and rewrites only those pieces of dx that were not finite.
 #include <type_traits>
 
 #include "bfq_fast.h"
@@ -43,7 +44,7 @@ constexpr int kSlots = 2;                   // rows of x and of g on their way
 constexpr int kAccCol = 384;                // sums of stages 0 .. 7: 16 columns each
 constexpr int kLastCol = 352;               // constants of the last stage: half of them in tensor memory, the rest in shared memory
 constexpr int kSlotFloats = 12 * (kN / 2);  // a CTA's sums
-constexpr float kLift = 1048576.f;          // 2^20
+constexpr float kLift = 1099511627776.f;    // 2^40, the inverse of the least factor
 // Group A or group B scales u back and writes dx: whichever has the time.  us, written by A / by B: 65536 rows of 4096 bf16 846 / 879,
 // fp32 1016 / 932; 2^25 elements of n = 2048 bf16 125 / 116, fp32 152 / 138, n = 1024 119 / 115, 152 / 136, n = 256 117 / 119, 144 / 142,
 // n = 128 130 / 137, 166 / 156.

@@ -371,3 +371,23 @@ def test_backward_rounds_each_row_once_into_the_sums():
             u, v = turn(u, s, True), turn(v, s, True)
     assert (dth - ref).norm() <= 4.9e-7 * ref.norm()
     assert p.device_status() == 0
+
+
+@pytest.mark.parametrize("exponent", [-118, 0, 95])
+@pytest.mark.parametrize("n,rows", [(4096, 300), (1024, 700), (128, 4096)])
+def test_backward_at_either_end_of_the_range(n, rows, exponent):
+    """g at 2^exponent with angles whose cosines multiply to 2^-38, close to the least factor of the scaled form: g goes through the
+    stages times its factor, and must come out with all its bits where that product would be subnormal.  (At 2^95 it overflows on the
+    way and the rows are done again.)"""
+    log_n = n.bit_length() - 1
+    sign = torch.randint(0, 2, (log_n, n // 2), generator=torch.Generator().manual_seed(1)) * 2 - 1
+    theta = (sign * math.acos(2.0 ** (-38 / log_n))).float()
+    p = Plan(n, DEV)
+    p.set_angles(theta.to(DEV))
+    x = synth.rows(rows, n, "normal", 2)
+    g = synth.rows(rows, n, "normal", 3) * 2.0 ** exponent
+    dx, dth = p.backward(x.to(DEV), g.to(DEV))
+    dx_ref, dth_ref = oracle.backward(to_f64(theta), to_f64(x), to_f64(g))
+    check_rows_close(dx, dx_ref, np.abs(to_f64(g)).max(axis=1), "dx")
+    check_dtheta(dth, dth_ref, "dtheta")
+    assert p.device_status() == 0
