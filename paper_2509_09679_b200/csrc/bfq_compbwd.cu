@@ -220,6 +220,8 @@ __global__ void __launch_bounds__(kThreads, 2) k_composite_backward(const Params
 // G in bf16 is an exact operand.  The other one, Q1 or X', goes in as three bf16 terms, 24 significant bits, so the products are those of
 // fp32 numbers and their sums are fp32 (m16n8k16; the small terms first or apart).  G stays in shared memory as bf16 rows, read as
 // matrices of 8 x 8 either way; Q1's terms are there as fragments; X' is split as it is read.
+// An infinity has no such terms (infinity less itself, or times a term that is zero, is NaN): products that are not finite are formed
+// again in fp32, so that infinities stay infinities.
 // (a, b) = t[0] + t[1] + t[2], largest first: eight significant bits each, cut off, so that the sum is exact
 __device__ __forceinline__ void three_terms(float a, float b, uint32_t (&t)[3]) {
 #pragma unroll
@@ -243,6 +245,9 @@ __device__ __forceinline__ uint4 matrices_transposed(uint32_t at) {
     asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(at) : "memory");
     return v;
 }
+
+__device__ __forceinline__ bool finite(float v) { return fabsf(v) <= 3.402823466e38f; }
+__device__ __forceinline__ float bf16_at(const uint16_t* p) { return __uint_as_float(static_cast<uint32_t>(*p) << 16); }
 
 constexpr int kWarps = kThreads / 32;
 // MT blocks of 16 runs.  dL/dQ1 is cut into tiles of 16 x 8, a warp has up to kTiles of them; with fewer tiles than warps, slices of the
@@ -272,6 +277,8 @@ __global__ void __launch_bounds__(kThreads, 2) k_composite_backward_mma(const Pa
             const int row = 16 * mt + (l >> 2) + 8 * (r & 1), k = 16 * kt + 2 * (l & 3) + 8 * (r >> 1);
             auto at = [&](int i) { return i < n1 && row < n1 ? p.q1[i * n1 + row] : 0.f; };
             three_terms(at(k), at(k + 1), w[r]);
+            if (isinf(at(k))) w[r][1] &= 0xFFFF0000u, w[r][2] &= 0xFFFF0000u;
+            if (isinf(at(k + 1))) w[r][1] &= 0xFFFFu, w[r][2] &= 0xFFFFu;
         }
 #pragma unroll
         for (int i = 0; i < 3; ++i) frag[i * MT * MT * 32 + e] = make_uint4(w[0][i], w[1][i], w[2][i], w[3][i]);
@@ -315,6 +322,16 @@ __global__ void __launch_bounds__(kThreads, 2) k_composite_backward_mma(const Pa
                         mma_bf16(s[mt][0], a, b[kt].x, b[kt].y);
                         mma_bf16(s[mt][1], a, b[kt].z, b[kt].w);
                     }
+            if (!finite(s[0][0][0]) || !finite(s[0][0][1]) || !finite(s[0][1][0]) || !finite(s[0][1][1])) {
+                // an element of G that is not finite shows in every run at its position
+#pragma unroll
+                for (int i = 0; i < 8 * MT; ++i) {
+                    const int r = 16 * (i >> 3) + g8 + 4 * (i & 2), j = j0 + 2 * (i & 4) + 2 * q + (i & 1);
+                    float v = 0.f;
+                    for (int k = 0; k < n1 && r < n1; ++k) v = fmaf(p.q1[k * n1 + r], bf16_at(Gb + k * M::kRow + j), v);
+                    s[i >> 3][(i >> 2) & 1][i & 3] = v;
+                }
+            }
 #pragma unroll
             for (int mt = 0; mt < MT; ++mt)
 #pragma unroll
@@ -351,7 +368,16 @@ __global__ void __launch_bounds__(kThreads, 2) k_composite_backward_mma(const Pa
                 else mma_bf16(part[1], a, b0[0], b1[0]);
             }
 #pragma unroll
-            for (int c = 0; c < 4; ++c) dq[i][c] += (part[0][c] + part[1][c]) + part[2][c];
+            for (int c = 0; c < 4; ++c) {
+                float v = (part[0][c] + part[1][c]) + part[2][c];
+                const int r = 16 * mt + g8 + 8 * (c >> 1), k = 8 * (tile / MT) + 2 * q + (c & 1);
+                if (!finite(v) && r < n1 && k < n1) {
+                    v = 0.f;
+                    for (int j = 16 * slice; j < Ge::kN2; j += 16 * slices)
+                        for (int e = j; e < j + 16; ++e) v = fmaf(bf16_at(Gb + r * M::kRow + e), X[k * Ge::kPitch + place(e)], v);
+                }
+                dq[i][c] += v;
+            }
         }
         __syncthreads();
         passes_down<L, Ge::kPasses - 1>(X, W, p, row, u, r0, acc);

@@ -1,5 +1,7 @@
 """GPU parity of the composite transform Q1 (x) Q2 (paper Sec. 3.3) against the CPU oracle: the Cayley factor, the
 unquantized rows and the quantized rows, for several (n1, n2) including the paper's 40 x 128."""
+import math
+
 import numpy as np
 import pytest
 import torch
@@ -436,6 +438,25 @@ def test_composite_backward_takes_g_at_any_address_and_one_token_at_any_stride(d
     wide[:, :d] = x
     for a, b in zip(composite_backward(p, q1, params, x[:1], g[:1]), composite_backward(p, q1, params, wide[:1, :d], g[:1])):
         assert torch.equal(a, b)
+
+
+@pytest.mark.parametrize("n1,n2", [(40, 128), (12, 256), (2, 128), (7, 1024), (64, 128)])
+def test_composite_backward_keeps_infinities(n1, n2):
+    """Gradients in bf16 go through matrix instructions as sums of terms, which an infinity is not: what is infinite or NaN must be what
+    fp32 gradients of the same values give, in the tokens' dx, in d-theta and in dQ1."""
+    tokens, d = 40, n1 * n2
+    p = Plan(n2, DEV)
+    p.set_angles(synth.angles(n2, "normal", 3).to(DEV))
+    q1 = p.cayley(synth.cayley_params(n1, 3, 0.1).to(DEV), n1)
+    x, g = synth.rows(tokens, d, "normal", 4).to(DEV), synth.rows(tokens, d, "normal", 5, dtype=torch.bfloat16).to(DEV)
+    for where, row, at, value in ((g, 7, n2 + 5, math.inf), (g, 8, d - 1, -math.inf), (g, 9, 0, math.nan), (x, 10, n2 + 3, math.inf), (x, 11, 1, math.nan)):
+        kept = where[row, at].clone()
+        where[row, at] = value
+        for got, ref in zip(p.composite_backward(q1, x, g), p.composite_backward(q1, x, g.float())):
+            special = ~torch.isfinite(ref)
+            assert torch.equal(special, ~torch.isfinite(got)) and torch.equal(ref[special].nan_to_num(0.5), got[special].nan_to_num(0.5))
+        where[row, at] = kept
+    assert p.device_status() == 0
 
 
 @pytest.mark.parametrize("n1,scale", [(2, 1.0), (3, 50.0), (33, 0.5), (64, 5.0)])
