@@ -440,6 +440,26 @@ def test_composite_backward_takes_g_at_any_address_and_one_token_at_any_stride(d
         assert torch.equal(a, b)
 
 
+@pytest.mark.parametrize("n1,n2", [(40, 128), (12, 256), (2, 128), (3, 256), (7, 1024), (64, 128)])
+def test_composite_backward_of_fp32_rows_and_bf16_gradients(n1, n2):
+    """dx in fp32 is not hidden by a rounding to 16 bits: the products on matrix instructions (bf16 g) are as close to 64 bits as the fp32
+    multiply-adds that gradients of the same values in fp32 take.  Room for the spread of the two errors, the norms of N random numbers
+    each: 2 % for dx; twice the standard deviation of their ratio, 2 / sqrt(N), for dQ1 of N = n1^2 entries; 25 % for d-theta."""
+    tokens, d = 1000, n1 * n2
+    theta, params = synth.angles(n2, "normal", 3), synth.cayley_params(n1, 3, 0.1)
+    p = Plan(n2, DEV)
+    p.set_angles(theta.to(DEV))
+    q1 = p.cayley(params.to(DEV), n1)
+    x, g = synth.rows(tokens, d, "normal", 4), synth.rows(tokens, d, "normal", 5, dtype=torch.bfloat16)
+    th64, x64, g64, Q1 = to_f64(theta), to_f64(x).reshape(-1, n2), to_f64(g).reshape(tokens, n1, n2), to_f64(q1)
+    dx, dth = oracle.backward(th64, x64, np.einsum("ki,rkj->rij", Q1, g64).reshape(-1, n2))
+    dq1 = np.einsum("rij,rkj->ik", g64, oracle.forward(th64, x64).reshape(tokens, n1, n2))
+    error = [[np.linalg.norm(to_f64(a) - b.reshape(a.shape)) / np.linalg.norm(b) for a, b in zip(p.composite_backward(q1, x.to(DEV), gd), (dx, dth, dq1))]
+             for gd in (g.to(DEV), g.float().to(DEV))]
+    assert all(a <= more * b for a, b, more in zip(*error, (1.02, 1.25, 1 + 2 / n1))), error
+    assert error[0][0] <= 2e-7 and error[0][1] <= 5e-7 and error[0][2] <= 1e-6 and p.device_status() == 0
+
+
 @pytest.mark.parametrize("n1,n2", [(40, 128), (12, 256), (2, 128), (7, 1024), (64, 128)])
 def test_composite_backward_keeps_infinities(n1, n2):
     """Gradients in bf16 go through matrix instructions as sums of terms, which an infinity is not: what is infinite or NaN must be what
