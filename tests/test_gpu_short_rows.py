@@ -391,3 +391,27 @@ def test_backward_at_either_end_of_the_range(n, rows, exponent):
     check_rows_close(dx, dx_ref, np.abs(to_f64(g)).max(axis=1), "dx")
     check_dtheta(dth, dth_ref, "dtheta")
     assert p.device_status() == 0
+
+
+@pytest.mark.parametrize("n,rows", [(4096, 700), (1024, 3000), (128, 40000)])
+@pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
+def test_backward_with_an_infinity_in_g(n, rows, dtype):
+    """An infinity or NaN in a row of g leaves no angle's sum finite; beside it dx of a row that is only too large for the scaled form is
+    right, and dx of every other row the same bits."""
+    p, theta, x, xd = inputs(n, rows, dtype)
+    g = synth.rows(rows, n, "normal", 5, dtype=dtype)
+    plain = p.backward(xd, g.to(DEV))[0]
+    other = torch.ones(rows, dtype=torch.bool, device=DEV)
+    other[5] = other[rows - 2] = False
+    for large in (False, True):
+        g[5, 7], g[rows - 2, n - 1] = math.inf, math.nan
+        if large:
+            g[rows // 2] *= 2.0 ** 100
+            other[rows // 2] = False
+        dx, dth = p.backward(xd, g.to(DEV))
+        assert torch.equal(dx[other], plain[other]) and not torch.isfinite(dth).any()
+        assert not torch.isfinite(dx[5]).any() and torch.isnan(dx[rows - 2]).all()
+        if large:
+            row = g[rows // 2:rows // 2 + 1]
+            check_rows_close(dx[rows // 2:rows // 2 + 1], oracle.inverse(to_f64(theta), to_f64(row)), np.abs(to_f64(row)).max(axis=1), "dx")
+    assert p.device_status() == 0
