@@ -485,7 +485,7 @@ k_bwd4096(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ CUte
 // One thread per angle: the three-shear constants of pair (s, j), negated when its two elements carry
 // opposite signs, at the place the owning role reads them; and the sign that turns the accumulated
 // g_hi*y_lo - g_lo*y_hi of the parity basis into d-theta.
-__device__ __forceinline__ void build_image_bwd(int k, bool quads, const float4* __restrict__ prep, const uint8_t* __restrict__ flip,
+__device__ __forceinline__ void build_image_bwd(int k, bool quads, const float4* prep, const uint8_t* flip,
                                                 float* __restrict__ img, int8_t* __restrict__ dsign) {
     if (k >= 12 * (kN / 2)) return;
     const int s = k / (kN / 2), j = k % (kN / 2);
@@ -514,7 +514,7 @@ __device__ __forceinline__ void build_image_bwd(int k, bool quads, const float4*
 
 // One thread per 32-bit word of a bf16 g row in phase-3 ownership (role t, register m): bit 15 / bit 31 set
 // when element 2t + 256m / its neighbour must be negated to enter the basis sigma(after stage 11) * parity.
-__device__ __forceinline__ void build_gsign(int w, const uint8_t* __restrict__ flip, uint32_t* __restrict__ gsign) {
+__device__ __forceinline__ void build_gsign(int w, const uint8_t* flip, uint32_t* __restrict__ gsign) {
     if (w >= 16 * kThreads) return;
     const int m = (w / (4 * kThreads)) * 4 + (w & 3), t = (w >> 2) % kThreads;  // layout [m / 4][t][m % 4]
     const int e = 2 * t + 256 * m;
@@ -530,7 +530,7 @@ __device__ __forceinline__ void build_gsign(int w, const uint8_t* __restrict__ f
 // both factors are multiplied by cos(theta).  Stage 0 is a general 2x2 that absorbs the factors.  Image layout
 // [column quad][role][4]; stage s >= 1 at columns 32 (s - 1), stage 0 at 352.  *form is raised when a factor leaves
 // [2^-64, 1]: the kernel then walks in the three-shear form.
-__device__ __forceinline__ void build_image_inv(int k, const double2* __restrict__ cs, float* __restrict__ img, int* __restrict__ form) {
+__device__ __forceinline__ void build_image_inv(int k, const double2* cs, float* __restrict__ img, int* __restrict__ form) {
     if (k >= 12 * (kN / 2)) return;
     const int s = k / (kN / 2), j = k % (kN / 2);
     const int lo = ((j >> s) << (s + 1)) | (j & ((1 << s) - 1));
@@ -581,8 +581,8 @@ __device__ __forceinline__ void build_image_inv(int k, const double2* __restrict
 // *form_fwd must be kFormScaled before.
 constexpr int kAngleBlocks = 12 * (kN / 2) / 256, kSignBlocks = 16 * kThreads / 256;
 constexpr int kTableBlocks = 2 * kAngleBlocks + kSignBlocks;
-__global__ void __launch_bounds__(256) k_build_tables(const float4* __restrict__ prep, const uint8_t* __restrict__ flip,
-                                                       const double2* __restrict__ cs, float* __restrict__ img, int8_t* __restrict__ dsign,
+__global__ void __launch_bounds__(256) k_build_tables(const float4* prep, const uint8_t* flip,
+                                                       const double2* cs, float* __restrict__ img, int8_t* __restrict__ dsign,
                                                        float* __restrict__ img_inv, int* __restrict__ form, uint32_t* __restrict__ gsign, bool quads,
                                                        float* __restrict__ img_fwd, int* __restrict__ form_fwd, float* __restrict__ weight) {
     grid_dep_launch();
@@ -686,9 +686,9 @@ struct InvUpper {
 // STRIDED (SHORT): the short rows of x lie brief.ldx apart instead of one after the other.
 template <int G, bool OUT_BF16, bool IN_F32 = false, bool WIDE = false, bool SHORT = false, bool STRIDED = false>
 __global__ void __launch_bounds__(G * kThreads, 1)
-k_inv4096(const __grid_constant__ CUtensorMap ymap, const float* __restrict__ img_lo, const float* __restrict__ img_scaled_lo,
-          const int* __restrict__ form_lo, const uint32_t* __restrict__ gsign_lo, void* __restrict__ xout, int64_t ldx, int rows,
-          int* __restrict__ status, const float2* __restrict__ tw12, const InvUpper upper, const ShortRows brief) {
+k_inv4096(const __grid_constant__ CUtensorMap ymap, const float* img_lo, const float* img_scaled_lo,
+          const int* form_lo, const uint32_t* gsign_lo, void* __restrict__ xout, int64_t ldx, int rows,
+          int* __restrict__ status, const float2* tw12, const InvUpper upper, const ShortRows brief) {
     static_assert(!(SHORT && WIDE), "one or the other");
     static_assert(!(IN_F32 && WIDE), "the wide mode takes bf16 rows");
     const int half = WIDE ? int(blockIdx.x & 1u) : 0;
@@ -739,7 +739,7 @@ k_inv4096(const __grid_constant__ CUtensorMap ymap, const float* __restrict__ im
     }
     // constants: the scaled-form image ([column quad][role][4], coalesced, all loads in flight) unless the table build
     // flagged it out of range; then the three-shear image (strips per role, or the same layout for short rows)
-    const bool shear = __ldg(form) != 0;
+    const bool shear = load_plain(form) != 0;
     if (!shear) {
         constexpr int kFillBlocks = (kInvCols / 16 + G - 1) / G;
         float4 fill[kFillBlocks][4];
@@ -749,7 +749,7 @@ k_inv4096(const __grid_constant__ CUtensorMap ymap, const float* __restrict__ im
             const int b = g + j * G;
             if (b < kInvCols / 16) {
 #pragma unroll
-                for (int i = 0; i < 4; ++i) fill[j][i] = __ldg(base + (4 * b + i) * 128 + t);
+                for (int i = 0; i < 4; ++i) fill[j][i] = load_plain(base + (4 * b + i) * 128 + t);
             }
         }
 #pragma unroll
@@ -773,7 +773,7 @@ k_inv4096(const __grid_constant__ CUtensorMap ymap, const float* __restrict__ im
             uint32_t v[16];
 #pragma unroll
             for (int i = 0; i < 4; ++i) {
-                const float4 f = __ldg(src + ((c >> 2) + i) * kQuad);
+                const float4 f = load_plain(src + ((c >> 2) + i) * kQuad);
                 v[4 * i + 0] = __float_as_uint(f.x), v[4 * i + 1] = __float_as_uint(f.y);
                 v[4 * i + 2] = __float_as_uint(f.z), v[4 * i + 3] = __float_as_uint(f.w);
             }
@@ -792,7 +792,7 @@ k_inv4096(const __grid_constant__ CUtensorMap ymap, const float* __restrict__ im
                 uint32_t v[16];
 #pragma unroll
                 for (int i = 0; i < 4; ++i) {
-                    const float4 cs = __ldg(reinterpret_cast<const float4*>(tw12 + 2 * t + 256 * (4 * j + i)));
+                    const float4 cs = load_plain(reinterpret_cast<const float4*>(tw12 + 2 * t + 256 * (4 * j + i)));
                     v[4 * i + 0] = __float_as_uint(cs.x), v[4 * i + 1] = __float_as_uint(sg * cs.y);
                     v[4 * i + 2] = __float_as_uint(cs.z), v[4 * i + 3] = __float_as_uint(sg * cs.w);
                 }
@@ -844,7 +844,7 @@ k_inv4096(const __grid_constant__ CUtensorMap ymap, const float* __restrict__ im
                 tmem_ld32(tlane + kWideCol + 32 * hh, T1);
                 uint32_t s8[8] = {0u, 0u, 0u, 0u, 0u, 0u, 0u, 0u};
                 if constexpr (kSigns) {
-                    const uint4 sw0 = __ldg(gsv + (2 * hh) * kThreads + t), sw1 = __ldg(gsv + (2 * hh + 1) * kThreads + t);
+                    const uint4 sw0 = load_plain(gsv + (2 * hh) * kThreads + t), sw1 = load_plain(gsv + (2 * hh + 1) * kThreads + t);
                     s8[0] = sw0.x, s8[1] = sw0.y, s8[2] = sw0.z, s8[3] = sw0.w;
                     s8[4] = sw1.x, s8[5] = sw1.y, s8[6] = sw1.z, s8[7] = sw1.w;
                 }
@@ -873,7 +873,7 @@ k_inv4096(const __grid_constant__ CUtensorMap ymap, const float* __restrict__ im
                 // (t >> 4) + 8m; the swizzle moves the chunk to chunk ^ (line & 7)
                 uint32_t s4[4] = {0u, 0u, 0u, 0u};
                 if constexpr (kSigns) {
-                    const uint4 sw = __ldg(gsv + qq * kThreads + t);
+                    const uint4 sw = load_plain(gsv + qq * kThreads + t);
                     s4[0] = sw.x, s4[1] = sw.y, s4[2] = sw.z, s4[3] = sw.w;
                 }
 #pragma unroll
@@ -887,7 +887,7 @@ k_inv4096(const __grid_constant__ CUtensorMap ymap, const float* __restrict__ im
             }
             uint32_t s4[4] = {0u, 0u, 0u, 0u};
             if constexpr (kSigns) {
-                const uint4 sw = __ldg(gsv + qq * kThreads + t);  // 2 KB in all: stays in L1
+                const uint4 sw = load_plain(gsv + qq * kThreads + t);  // 2 KB in all: stays in L1
                 s4[0] = sw.x, s4[1] = sw.y, s4[2] = sw.z, s4[3] = sw.w;
             }
 #pragma unroll

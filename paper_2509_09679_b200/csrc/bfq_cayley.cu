@@ -32,7 +32,7 @@ constexpr int kMaxRows = 64 / (kThreads / 32);  // rows of a warp
 __host__ __device__ constexpr int pitch(int n1) { return 2 * n1 + 1; }
 
 // Q1 of the parameters, row-major with row stride pitch(n1), in one of the two buffers [n1][pitch] of `aug`
-__device__ __forceinline__ const double* solve(const float* __restrict__ params, int n1, double* aug) {
+__device__ __forceinline__ const double* solve(const float* params, int n1, double* aug) {
     const int t = threadIdx.x, lane = t & 31, w = pitch(n1), cols = 2 * n1;
     double* cur = aug;
     double* nxt = aug + n1 * w;
@@ -132,15 +132,15 @@ __device__ __forceinline__ void invert(double (&m)[T][T], int n1, double (&line)
     }
 }
 
-__device__ __forceinline__ float parameter(const float* __restrict__ params, int n1, int i, int j) {  // A[i][j]
+__device__ __forceinline__ float parameter(const float* params, int n1, int i, int j) {  // A[i][j]
     if (i == j) return 0.f;
     const int lo = min(i, j), hi = max(i, j);
-    const float v = __ldg(params + lo * n1 - lo * (lo + 1) / 2 + (hi - lo - 1));
+    const float v = params[lo * n1 - lo * (lo + 1) / 2 + (hi - lo - 1)];
     return i < j ? v : -v;
 }
 
 template <int T>
-__global__ void __launch_bounds__(kThreads) k_cayley(const float* __restrict__ params, int n1, float* __restrict__ q1) {
+__global__ void __launch_bounds__(kThreads) k_cayley(const float* params, int n1, float* __restrict__ q1) {
     extern __shared__ double aug[];  // [2][n1][pitch], for `solve`
     __shared__ double line[2][2][64];
     const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
@@ -215,8 +215,8 @@ __device__ __forceinline__ void product(double* out, const double* a, const doub
 // M = (I + A)^{-1} in float64 from the Q1 the caller has: (I + Q1) / 2 is M to fp32 rounding (residual up to |A| 2^-24), and a
 // Newton step M (2 I - (I + A) M) squares the residual; a second one follows where the first residual's square is not far below
 // fp32 rounding.  If Q1 is not the transform of these parameters (the first residual is not small) the solve is done after all.
-__global__ void __launch_bounds__(kThreads) k_cayley_backward(const float* __restrict__ params, int n1, const float* __restrict__ q1,
-                                                              const float* __restrict__ dq1, float* __restrict__ dparams) {
+__global__ void __launch_bounds__(kThreads) k_cayley_backward(const float* params, int n1, const float* q1,
+                                                              const float* dq1, float* __restrict__ dparams) {
     extern __shared__ double aug[];  // [2][n1][pitch] of the solve, or I + A, M, 2 I - (I + A) M, the next M; then dQ1
     const int t = threadIdx.x, np = padded(n1), w = row_of(n1), size = np * w;
     double *ia = aug, *m = ia + size, *r = m + size, *next = r + size, *g = next + size;
@@ -227,8 +227,8 @@ __global__ void __launch_bounds__(kThreads) k_cayley_backward(const float* __res
         const bool in = i < n1 && j < n1;
         const double id = i == j ? 1.0 : 0.0;
         ia[at] = in ? id + static_cast<double>(parameter(params, n1, i, j)) : 0.0;
-        m[at] = in ? 0.5 * (id + static_cast<double>(__ldg(q1 + i * n1 + j))) : 0.0;
-        g[at] = in ? static_cast<double>(__ldg(dq1 + i * n1 + j)) : 0.0;
+        m[at] = in ? 0.5 * (id + static_cast<double>(q1[i * n1 + j])) : 0.0;
+        g[at] = in ? static_cast<double>(dq1[i * n1 + j]) : 0.0;
     }
     __syncthreads();
     // whether an entry of I - (I + A) M is not below a limit (NaN is not); rows and columns from n1 on hold 2 I there

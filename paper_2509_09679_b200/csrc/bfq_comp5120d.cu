@@ -412,7 +412,7 @@ k_comp5120d(const __grid_constant__ Params P, const __grid_constant__ CUtensorMa
 // Between input c and output j there is one path through the butterfly (before stage s the index has the bits of j below s and
 // those of c from s on), so an entry is a product of seven numbers in double: one thread per entry.  (One thread per
 // column applying the stages took 77 us.)
-__global__ void __launch_bounds__(256) k_build_dense128(const float2* __restrict__ tw, __nv_bfloat16* __restrict__ img) {
+__global__ void __launch_bounds__(256) k_build_dense128(const float2* tw, __nv_bfloat16* __restrict__ img) {
     grid_dep_launch();
     grid_dep_wait();
     const int k = blockIdx.x * 256 + threadIdx.x, j = k >> 7, c = k & (kN2 - 1);
@@ -420,7 +420,7 @@ __global__ void __launch_bounds__(256) k_build_dense128(const float2* __restrict
 #pragma unroll
     for (int s = 0; s < 7; ++s) {
         const int i = (j & ((1 << s) - 1)) | (c & ~((1 << s) - 1));  // the index before stage s; bit s is c's, then j's
-        const float2 cs = __ldg(tw + s * (kN2 / 2) + (((i >> (s + 1)) << s) | (i & ((1 << s) - 1))));
+        const float2 cs = tw[s * (kN2 / 2) + (((i >> (s + 1)) << s) | (i & ((1 << s) - 1)))];
         const int from = (c >> s) & 1, to = (j >> s) & 1;
         v *= from == to ? double(cs.x) : (to ? double(cs.y) : -double(cs.y));
     }

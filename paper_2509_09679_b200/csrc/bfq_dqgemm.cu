@@ -497,7 +497,7 @@ __device__ __forceinline__ void produce(const Operand& op, int k_len, int g, int
     };
     constexpr int kScales = SCALED ? kPer : (kFold ? 4 : 1);
     float sc[kScales];
-    auto half_at = [](const uint16_t* q) { return __half2float(__ushort_as_half(__ldg(q))); };
+    auto half_at = [](const uint16_t* q) { return __half2float(__ushort_as_half(*q)); };
     auto load_scales = [&](const At& a) {
         if constexpr (SCALED) {
 #pragma unroll
@@ -748,8 +748,8 @@ k_dequant_gemm(const __grid_constant__ Params p, const __grid_constant__ CUtenso
 
     // scales that do not vary along k multiply the finished column / row of C
     const bool u_scales = is_codes(p.u.kind) && !p.u.transposed, v_scales = is_codes(p.v.kind) && !p.v.transposed;
-    auto u_scale = [&](int j) { return u_scales && j < p.u.rows ? p.alpha * __half2float(__ushort_as_half(__ldg(p.u.scales + j))) : p.alpha; };
-    auto v_scale = [&](int i) { return v_scales && i < p.v.rows ? __half2float(__ushort_as_half(__ldg(p.v.scales + i))) : 1.f; };
+    auto u_scale = [&](int j) { return u_scales && j < p.u.rows ? p.alpha * __half2float(__ushort_as_half(p.u.scales[j])) : p.alpha; };
+    auto v_scale = [&](int i) { return v_scales && i < p.v.rows ? __half2float(__ushort_as_half(p.v.scales[i])) : 1.f; };
 
     auto span_of = [&](bool u) {
         Span span;
@@ -992,7 +992,7 @@ __global__ void __launch_bounds__(32 * kFewWarps) k_few_rows(const Operand u, co
     Sum acc[4] = {0, 0, 0, 0};
     // a lane's kRound elements of each row start at a multiple of kRound: inside K as a whole, or cut at a 16-byte piece
     auto piece = [&](const uint8_t* row, bool yes, int at, int bits) {
-        return yes && at < k ? __ldg(reinterpret_cast<const uint4*>(row + int64_t(at) * bits / 8)) : make_uint4(0u, 0u, 0u, 0u);
+        return yes && at < k ? *reinterpret_cast<const uint4*>(row + int64_t(at) * bits / 8) : make_uint4(0u, 0u, 0u, 0u);
     };
     constexpr int kStride = kFewWarps * 4 * kRound;
     uint4 w[2][kULoads];
@@ -1049,8 +1049,8 @@ __global__ void __launch_bounds__(32 * kFewWarps) k_few_rows(const Operand u, co
         Sum sum = 0;
 #pragma unroll
         for (int x = 0; x < kFewWarps; ++x) sum += part[x][e >> 4][j];
-        float scale = alpha * __half2float(__ushort_as_half(__ldg(u.scales + j0 + j)));
-        if (is_codes(VK)) scale *= __half2float(__ushort_as_half(__ldg(v.scales + i)));
+        float scale = alpha * __half2float(__ushort_as_half(u.scales[j0 + j]));
+        if (is_codes(VK)) scale *= __half2float(__ushort_as_half(v.scales[i]));
         float value = sum;
         if constexpr (kInts) value = __int2float_rn(sum) * (1.f / float(1 << (Int8Chunk<UK>::kShift + Int8Chunk<VK>::kShift)));
         c[int64_t(i) * ldc + j0 + j] = value * scale;
@@ -1068,18 +1068,18 @@ static Operand make_operand(const void* data, const uint16_t* scales, int64_t ld
 // An fp32 operand as two bf16 matrices hi + lo of its stored rows (pitch: the row's length rounded up to 8), times the other
 // operand's scales where those vary along k: `row_scales` per stored row (stored [K][rows]), `col_scales` per element of a row.
 // The same arithmetic as in the tiles, so the products come out the same.  Bound by memory: 8 bytes per element.
-__global__ void __launch_bounds__(256) k_split_rows(const float* __restrict__ x, int64_t ld, int64_t rows, int width, const uint16_t* __restrict__ row_scales,
-                                                    const uint16_t* __restrict__ col_scales, uint16_t* __restrict__ hi, uint16_t* __restrict__ lo) {
+__global__ void __launch_bounds__(256) k_split_rows(const float* x, int64_t ld, int64_t rows, int width, const uint16_t* row_scales,
+                                                    const uint16_t* col_scales, uint16_t* __restrict__ hi, uint16_t* __restrict__ lo) {
     grid_dep_launch();
     grid_dep_wait();
     const int chunks = (width + 7) / 8;
     const int64_t total = rows * chunks, step = int64_t(gridDim.x) * blockDim.x;
-    auto half_at = [](const uint16_t* q) { return __half2float(__ushort_as_half(__ldg(q))); };
+    auto half_at = [](const uint16_t* q) { return __half2float(__ushort_as_half(*q)); };
     for (int64_t e = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; e < total; e += step) {
         const int64_t r = e / chunks;
         const int c = 8 * static_cast<int>(e - r * chunks);
         const float4* src = reinterpret_cast<const float4*>(x + r * ld + c);
-        const float4 none = make_float4(0.f, 0.f, 0.f, 0.f), a = __ldg(src), b = c + 4 < width ? __ldg(src + 1) : none;
+        const float4 none = make_float4(0.f, 0.f, 0.f, 0.f), a = *src, b = c + 4 < width ? src[1] : none;
         float v[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
         const float rs = row_scales != nullptr ? half_at(row_scales + r) : 1.f;
 #pragma unroll

@@ -21,18 +21,6 @@ constexpr int kRanks = 8, kThreads = 64, kBlock = kN / kRanks;  // elements of a
 __device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
 __device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
 
-// loads that stay where they are written: all of them are on their way before the first is waited for
-__device__ __forceinline__ float2 load2(const float2* p) {
-    float2 v;
-    asm volatile("ld.global.nc.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "l"(p));
-    return v;
-}
-__device__ __forceinline__ float4 load4(const float4* p) {
-    float4 v;
-    asm volatile("ld.global.nc.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "l"(p));
-    return v;
-}
-
 // where element i of a CTA's block lies between passes
 __device__ __forceinline__ int place(int i) { return i + (i >> 3); }
 // element e (three bits) of thread u in pass P: bits 3 P .. 3 P + 2 of its index are e
@@ -45,9 +33,9 @@ __device__ __forceinline__ constexpr int lo_of(int q) { return ((q >> K) << (K +
 __device__ __forceinline__ int angle_of(int lo, int s) { return s * (kN / 2) + (((lo >> (s + 1)) << s) | (lo & ((1 << s) - 1))); }
 
 template <int P, int K = 0>
-__device__ __forceinline__ void load_pass(const float2* __restrict__ flat, int rank, int u, float2 (&c)[3][4]) {
+__device__ __forceinline__ void load_pass(const float2* flat, int rank, int u, float2 (&c)[3][4]) {
 #pragma unroll
-    for (int q = 0; q < 4; ++q) c[K][q] = load2(flat + angle_of((rank << 9) | index_of<P>(u, lo_of<K>(q)), 3 * P + K));
+    for (int q = 0; q < 4; ++q) c[K][q] = load_plain(flat + angle_of((rank << 9) | index_of<P>(u, lo_of<K>(q)), 3 * P + K));
     if constexpr (K < 2) load_pass<P, K + 1>(flat, rank, u, c);
 }
 template <int K>
@@ -70,7 +58,7 @@ __device__ __forceinline__ void pass(float (&v)[8], const float2 (&c)[3][4], boo
 
 // BITS = 0: rows out, else codes and scales
 template <bool F32, int BITS>
-__global__ void __launch_bounds__(kThreads) k_forward_few(const void* __restrict__ x, int64_t ldx, const float* __restrict__ tables, const int* __restrict__ form,
+__global__ void __launch_bounds__(kThreads) k_forward_few(const void* x, int64_t ldx, const float* tables, const int* form,
                                                           uint8_t* __restrict__ codes, uint16_t* __restrict__ scales, void* __restrict__ y, int64_t ldy) {
     __shared__ float buf[kBlock + kBlock / 8];
     __shared__ float arrived[kBlock];       // [rank][64]
@@ -81,15 +69,16 @@ __global__ void __launch_bounds__(kThreads) k_forward_few(const void* __restrict
     cluster_arrive();  // the peers have started when this is over: waited for before the first store to one
     grid_dep_launch();
     grid_dep_wait();
-    const bool shear = __ldg(form) != 0;
-    // eight elements of the row, and the constants: (k1, k2) of stages 0 .. 10, then the four numbers of the last one
+    const bool shear = *form != 0;
+    // eight elements of the row, and the constants, by loads that stay where they are written: all of them are on their way before the
+    // first is waited for.  (k1, k2) of stages 0 .. 10, then the four numbers of the last one
     float v[8];
     if constexpr (F32) {
         const float4* src = reinterpret_cast<const float4*>(static_cast<const float*>(x) + row * ldx + rank * kBlock + 8 * u);
-        const float4 a = load4(src), b = load4(src + 1);
+        const float4 a = load_plain(src), b = load_plain(src + 1);
         v[0] = a.x, v[1] = a.y, v[2] = a.z, v[3] = a.w, v[4] = b.x, v[5] = b.y, v[6] = b.z, v[7] = b.w;
     } else {
-        const uint4 w = __ldg(reinterpret_cast<const uint4*>(static_cast<const __nv_bfloat16*>(x) + row * ldx + rank * kBlock + 8 * u));
+        const uint4 w = *reinterpret_cast<const uint4*>(static_cast<const __nv_bfloat16*>(x) + row * ldx + rank * kBlock + 8 * u);
         const uint32_t ws[4] = {w.x, w.y, w.z, w.w};
 #pragma unroll
         for (int i = 0; i < 4; ++i) v[2 * i] = __uint_as_float(ws[i] << 16), v[2 * i + 1] = __uint_as_float(ws[i] & 0xFFFF0000u);
@@ -105,9 +94,9 @@ __global__ void __launch_bounds__(kThreads) k_forward_few(const void* __restrict
     const int j = (rank << 6) | u;  // this thread's position in every block after the exchange
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
-        c9[q] = load2(flat + angle_of((lo_of<0>(q) << 9) | j, 9));
-        c10[q] = load2(flat + angle_of((lo_of<1>(q) << 9) | j, 10));
-        c11[q] = load4(last + ((q << 9) | j));
+        c9[q] = load_plain(flat + angle_of((lo_of<0>(q) << 9) | j, 9));
+        c10[q] = load_plain(flat + angle_of((lo_of<1>(q) << 9) | j, 10));
+        c11[q] = load_plain(last + ((q << 9) | j));
     }
     // the rotations start after all loads have been issued
     asm volatile("" : "+f"(v[0]), "+f"(v[1]), "+f"(v[2]), "+f"(v[3]), "+f"(v[4]), "+f"(v[5]), "+f"(v[6]), "+f"(v[7])::"memory");

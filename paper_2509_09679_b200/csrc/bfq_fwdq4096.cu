@@ -40,7 +40,7 @@ namespace f4k {
 // reduced-angle lifting constants and whether the reduction negates the pair.  The pair is negated iff
 // cos(theta) < 0, and phi = theta -+ pi in that case; tan(phi/2) and sin(phi) are odd in phi, so the constants for
 // the mirrored rotation G(-theta) are the negatives of the stored ones.
-__global__ void __launch_bounds__(256) k_prep_angles4096(const float* __restrict__ theta, float2* __restrict__ tw,
+__global__ void __launch_bounds__(256) k_prep_angles4096(const float* theta, float2* __restrict__ tw,
                                                           float4* __restrict__ prep, uint8_t* __restrict__ flip,
                                                           double2* __restrict__ cs, int* __restrict__ form, int levels) {
     const int k = blockIdx.x * blockDim.x + threadIdx.x;
@@ -67,7 +67,7 @@ __global__ void __launch_bounds__(256) k_prep_angles4096(const float* __restrict
 }
 
 // Step 2 (one thread per angle): build_image_fwd in bfq_n4096.cuh
-__global__ void __launch_bounds__(256) k_build_image4096(const float4* __restrict__ prep, const double2* __restrict__ cs,
+__global__ void __launch_bounds__(256) k_build_image4096(const float4* prep, const double2* cs,
                                                           float* __restrict__ img, int* __restrict__ form, float* __restrict__ weight, float* __restrict__ flat) {
     grid_dep_launch();
     grid_dep_wait();

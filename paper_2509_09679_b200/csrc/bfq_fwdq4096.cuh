@@ -171,7 +171,7 @@ enum : int { kOutInt4 = 0, kOutBf16 = 1, kOutInt4Stats = 2, kOutInt2 = 3, kOutIn
 // STRIDED (rows out alone): the short rows of the output lie ldy >> SUB apart instead of one after the other.
 template <int G, int CW, int XB, int TRANSFORM, int OUT, int STEP = 2, bool ROWS = false, bool IN_F32 = false, int SUB = 0, bool STRIDED = false>
 __global__ void __launch_bounds__(G * kGroupThreads, 1)
-k_fwdq4096(const __grid_constant__ CUtensorMap tmap, const float* __restrict__ img, const int* __restrict__ form,
+k_fwdq4096(const __grid_constant__ CUtensorMap tmap, const float* img, const int* form,
            uint8_t* __restrict__ codes,
            uint16_t* __restrict__ scales, __nv_bfloat16* __restrict__ yout, int64_t ldy, int rows,
            int* __restrict__ status, uint32_t tx_bytes, int wait_limit, unsigned long long* __restrict__ hist, int64_t elems,
@@ -190,13 +190,13 @@ k_fwdq4096(const __grid_constant__ CUtensorMap tmap, const float* __restrict__ i
     // image is fetched on the assumption that the table build selected it; the flag is checked below.
     constexpr int kFillBlocks = (kCols / 16 + G - 1) / G;
     float4 fill[kTmem ? kFillBlocks : 1][4];
-    auto fetch_image = [&](const float4* __restrict__ base) {
+    auto fetch_image = [&](const float4* base) {
 #pragma unroll
         for (int j = 0; j < kFillBlocks; ++j) {
             const int b = g + j * G;
             if (b < kCols / 16) {
 #pragma unroll
-                for (int i = 0; i < 4; ++i) fill[j][i] = __ldg(base + (4 * b + i) * 128 + t);
+                for (int i = 0; i < 4; ++i) fill[j][i] = load_plain(base + (4 * b + i) * 128 + t);
             }
         }
     };
@@ -219,7 +219,7 @@ k_fwdq4096(const __grid_constant__ CUtensorMap tmap, const float* __restrict__ i
     bool shear = false;
     if constexpr (kTmem) {
         fetch_image(reinterpret_cast<const float4*>(img));
-        shear = __ldg(form) != 0;
+        shear = load_plain(form) != 0;
     }
     if constexpr (kTmem) tmem_fence_before();
     __syncthreads();

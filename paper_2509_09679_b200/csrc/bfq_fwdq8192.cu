@@ -158,7 +158,7 @@ __device__ __forceinline__ uint32_t nibble_int2(u64 v, u64 inv2, float inv, bool
 template <int G, int BITS, int STEP = 2, bool ROWS = false, bool IN_F32 = false, bool HADAMARD = false>
 __global__ void __launch_bounds__(G * kGroupThreads, 1)
 k_fwdq8192(const __grid_constant__ CUtensorMap map_lo, const __grid_constant__ CUtensorMap map_hi,
-           const float* __restrict__ img, const int* __restrict__ form, uint8_t* __restrict__ codes,
+           const float* img, const int* form, uint8_t* __restrict__ codes,
            uint16_t* __restrict__ scales, int64_t ldy, int rows, int* __restrict__ status,
            __nv_bfloat16* __restrict__ yrows) {
     using S = Smem<G>;
@@ -228,12 +228,12 @@ k_fwdq8192(const __grid_constant__ CUtensorMap map_lo, const __grid_constant__ C
                 const int b = g + j * G;
                 if (b < kCols8 / 16) {
 #pragma unroll
-                    for (int i = 0; i < 4; ++i) fill[j][i] = __ldg(base + (4 * b + i) * 128 + t);
+                    for (int i = 0; i < 4; ++i) fill[j][i] = base[(4 * b + i) * 128 + t];
                 }
             }
         };
         fetch_image(kFormScaled);
-        shear = __ldg(form) != 0;
+        shear = *form != 0;
         if (shear) fetch_image(kFormShear);
 #pragma unroll
         for (int j = 0; j < kFillBlocks; ++j) {

@@ -539,7 +539,7 @@ __device__ __forceinline__ bool group_d(const Ctx& cx, const CUtensorMap* gmap) 
 // pass is possible (dx lies over x or g).
 template <bool IN_F32, int STAGES>
 __global__ void __launch_bounds__(kCta, 1)
-k_grad4096(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ CUtensorMap gmap, const float* __restrict__ img, const int* __restrict__ form,
+k_grad4096(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ CUtensorMap gmap, const float* img, const int* form,
            void* __restrict__ dx, int64_t ld, float* __restrict__ partial, int* __restrict__ slot_form, int rows, int* __restrict__ status, bool only_shear,
            int64_t elems) {
     using S = Smem<IN_F32>;
@@ -554,7 +554,7 @@ k_grad4096(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ CUt
     }
     if (threadIdx.x == 0) sts32(sbase + S::kBadOff, 0u);
     grid_dep_wait();
-    bool shear = only_shear || __ldg(form) != 0;
+    bool shear = only_shear || *form != 0;
     tmem_fence_before();
     __syncthreads();
     tmem_fence_after();
@@ -585,7 +585,7 @@ k_grad4096(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ CUt
                 const int b = group + kGroups * j;
                 if (b < kCols / 16) {
 #pragma unroll
-                    for (int i = 0; i < 4; ++i) f[j][i] = __ldg(base + (4 * b + i) * kThreads);
+                    for (int i = 0; i < 4; ++i) f[j][i] = load_plain(base + (4 * b + i) * kThreads);
                 }
             }
             const float lift = shear ? 1.f : kLift;
@@ -653,8 +653,8 @@ k_grad4096(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ CUt
 // angles (half is a multiple of 32): lane y adds terms y, y + 32, ... (term = slot * positions + r) in groups of four, then the
 // lanes are added as four sums, so that the roundings at the size of the whole sum are few.  (64 bits throughout were no closer, and
 // one row of 4096 took 1.3 us longer.)
-__global__ void __launch_bounds__(1024) k_reduce_grad(const float* __restrict__ partial, const int* __restrict__ slot_form, int slots, int half_log,
-                                                      const float* __restrict__ weight, float* __restrict__ out) {
+__global__ void __launch_bounds__(1024) k_reduce_grad(const float* partial, const int* slot_form, int slots, int half_log,
+                                                      const float* weight, float* __restrict__ out) {
     __shared__ float sh[32][33];
     const int x = threadIdx.x & 31, y = threadIdx.x >> 5;
     const int k = blockIdx.x * 32 + x, s = k >> half_log, j = k & ((1 << half_log) - 1);
@@ -665,7 +665,7 @@ __global__ void __launch_bounds__(1024) k_reduce_grad(const float* __restrict__ 
     auto weighted = [&](int i, float add) {
         const int slot = i >> pos_log;
         const float v = partial[static_cast<int64_t>(slot) * kSlotFloats + ((i & ((1 << pos_log) - 1)) << half_log) + at];
-        return fmaf(v, __ldg(slot_form + slot) != 0 ? w[1] : w[0], add);
+        return fmaf(v, slot_form[slot] != 0 ? w[1] : w[0], add);
     };
     float acc = 0.f;
     int i = y;

@@ -171,7 +171,7 @@ __device__ __forceinline__ void stage_scaled(u64 (&P)[16], const uint32_t (&T)[C
 
 // sign carried by element i when it enters stage s: the product of the negations (flip = 1) of the pairs
 // it belonged to in stages 0..s-1
-__device__ __forceinline__ int sign_before(const uint8_t* __restrict__ flip, int i, int s) {
+__device__ __forceinline__ int sign_before(const uint8_t* flip, int i, int s) {
     // all (at most twelve) flag loads are issued together: a loop with a run-time trip count would wait for each in turn
     int f = 0;
 #pragma unroll
@@ -187,7 +187,7 @@ enum : int { kFormScaled = 0, kFormShear = 1 };  // FORM: how the stages rotate 
 
 // factor carried by element i when it enters stage s: the product of the cosines of the pairs it belonged to in
 // stages 0..s-1 (its sign is the tracked sign of the three-shear form)
-__device__ __forceinline__ double factor_before(const double2* __restrict__ cs, int i, int s) {
+__device__ __forceinline__ double factor_before(const double2* cs, int i, int s) {
     double c[11];
 #pragma unroll
     for (int sp = 0; sp < 11; ++sp) {  // all loads issued together
@@ -205,7 +205,7 @@ __device__ __forceinline__ double factor_before(const double2* __restrict__ cs, 
 // when an element's factor leaves the range the scaled form is used in, form[3] when it leaves that of the backward kernel;
 // weight[form][angle] = the product of the factors with which the pair's elements enter the stage; flat (may be null): the
 // constants of each form once more in the order of the angles.
-__device__ __forceinline__ void build_image_fwd(int k, const float4* __restrict__ prep, const double2* __restrict__ cs, float* __restrict__ img,
+__device__ __forceinline__ void build_image_fwd(int k, const float4* prep, const double2* cs, float* __restrict__ img,
                                                 int* __restrict__ form, float* __restrict__ weight, float* __restrict__ flat) {
     if (k >= 12 * (kN / 2)) return;
     const int s = k / (kN / 2), j = k % (kN / 2);

@@ -58,8 +58,25 @@ __device__ __forceinline__ u64 mul2(u64 a, u64 b) {
 // stream is still running; grid_dep_wait() returns once that kernel has completed and its writes are visible
 // (at once for an ordinary launch).  grid_dep_launch() lets the next kernel of the stream start early under the
 // same rule.
+// Such a kernel lives while the one before it still writes, so it reads by plain loads: no __ldg and no const __restrict__
+// pointers (both allow ld.global.nc, which is for memory that nothing changes while the kernel lives, and which the compiler may
+// move across the wait).
 __device__ __forceinline__ void grid_dep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void grid_dep_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
+// such a load, where the scheduling around it matters
+template <class T>
+__device__ __forceinline__ T load_plain(const T* p) {
+    static_assert(sizeof(T) == 4 || sizeof(T) == 8 || sizeof(T) == 16, "one, two or four words");
+    union {
+        uint32_t w[sizeof(T) / 4];
+        T v;
+    } r;
+    if constexpr (sizeof(T) == 4) asm volatile("ld.global.u32 %0, [%1];" : "=r"(r.w[0]) : "l"(p));
+    else if constexpr (sizeof(T) == 8) asm volatile("ld.global.v2.u32 {%0, %1}, [%2];" : "=r"(r.w[0]), "=r"(r.w[1]) : "l"(p));
+    else asm volatile("ld.global.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(r.w[0]), "=r"(r.w[1]), "=r"(r.w[2]), "=r"(r.w[3]) : "l"(p));
+    return r.v;
+}
 
 // ---- named barriers (producer / consumer hand-off between warp teams) ---------------------------------
 __device__ __forceinline__ void bar_sync(int id, int nthreads) {

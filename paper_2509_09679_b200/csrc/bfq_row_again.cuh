@@ -88,7 +88,7 @@ __device__ __forceinline__ void row_again(const Again& p, int64_t row, uint32_t 
         const int s = p.inverse ? p.levels - 1 - i : i;
         for (int j = t; j < half; j += kGroupThreads) {
             const uint32_t lo = buf + 4 * (((j >> s) << (s + 1)) | (j & ((1 << s) - 1))), hi = lo + (4u << s);
-            const float2 cs = __ldg(p.from.tw + s * half + j);
+            const float2 cs = load_plain(p.from.tw + s * half + j);
             const float a = __uint_as_float(lds32(lo)), b = __uint_as_float(lds32(hi));
             sts32(lo, __float_as_uint(p.inverse ? cs.x * a + cs.y * b : cs.x * a - cs.y * b));
             sts32(hi, __float_as_uint(p.inverse ? cs.x * b - cs.y * a : cs.y * a + cs.x * b));
