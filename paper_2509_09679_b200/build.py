@@ -24,6 +24,8 @@ def build_fast_calls(force: bool = False) -> str:
     newest = max(os.path.getmtime(p) for p in (src, os.path.join(os.path.dirname(HERE), "include", "bfq.h")))
     if not force and os.path.exists(FAST) and os.path.getmtime(FAST) >= newest:
         return FAST
+    if os.path.exists(FAST):
+        os.remove(FAST)  # what is there is out of date, and stays so if the compiler fails
     import torch
 
     at = os.path.dirname(torch.__file__)
@@ -44,7 +46,15 @@ def _deps():
 
 
 def build(force: bool = False, verbose: bool = False) -> str:
-    build_fast_calls(force)
+    build_library(force, verbose)
+    try:
+        build_fast_calls(force)
+    except (ImportError, OSError, subprocess.CalledProcessError) as e:  # no C++ compiler, or no headers of Python or torch
+        print(f"warning: {FAST} was not built, every call goes through the interpreter: {e}", file=sys.stderr)
+    return LIB
+
+
+def build_library(force: bool = False, verbose: bool = False) -> str:
     newest = max(os.path.getmtime(p) for p in _deps())
     if not force and os.path.exists(LIB) and os.path.getmtime(LIB) >= newest:
         return LIB

@@ -118,3 +118,15 @@ def test_the_plain_forms_leave_everything_else_to_the_binding():
         assert call(0, 8, 0, x) is None and call(64, 8, 0, x) is None and call(64, 8, 0, [1.0]) is None and call(64, 8, 0) is None
         assert call("plan", 8, 0, x) is None and call(64, 8.0, 0, x) is None
     assert fast.forward_quant(64, 8, 0, x, 4) is None and fast.forward_quant(64, 8, 0, x, "4") is None
+
+
+def test_the_library_is_built_where_the_extension_cannot_be(monkeypatch, capsys):
+    """The C++ part of the binding is optional: without a compiler or headers for it the CUDA library is built all the same."""
+    from paper_2509_09679_b200 import build
+    done = []
+    monkeypatch.setattr(build, "build_library", lambda *a: done.append("library"))
+    for error in (FileNotFoundError("g++"), build.subprocess.CalledProcessError(1, "g++"), ModuleNotFoundError("torch")):
+        def fails(force, error=error):
+            raise error
+        monkeypatch.setattr(build, "build_fast_calls", fails)
+        assert build.build() == build.LIB and done.pop() == "library" and "was not built" in capsys.readouterr().err
