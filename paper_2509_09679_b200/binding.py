@@ -61,15 +61,29 @@ SIGNATURES = {
 _lib = None
 
 
-def _not_built(*args):
+def _not_native(*args):
     return None
 
 
-try:  # the plain forms of the smallest calls in C++: a result, a status, or None for "not plain, done below"
-    from . import fast_calls as _fast
-except ImportError:  # not built: every call is done below
-    class _fast:
-        attach = forward = forward_quant = inverse = _not_built
+class _Interpreted:
+    """In the place of fast_calls: every call is done by the methods below."""
+    forward = forward_quant = inverse = staticmethod(_not_native)
+
+
+_fast = _Interpreted  # set by lib()
+
+
+def _native_calls():
+    """fast_calls, the plain forms of the smallest calls in C++ (a result, a status, or None for "not plain, done below"), attached to
+    the library; or, where it is not built or built against another torch, what answers None to everything."""
+    try:
+        from . import fast_calls
+    except ImportError:
+        return _Interpreted
+    if getattr(fast_calls, "torch_version", None) != torch.__version__:  # its calls into torch could do anything
+        return _Interpreted
+    fast_calls.attach(LIB_PATH)
+    return fast_calls
 
 
 class BfqError(RuntimeError):
@@ -81,7 +95,7 @@ class BfqError(RuntimeError):
 
 def lib() -> ctypes.CDLL:
     """Loads libbfq.so (raises if it has not been built: there is no fallback)."""
-    global _lib
+    global _lib, _fast
     if _lib is None:
         if not os.path.exists(LIB_PATH):
             raise RuntimeError(f"{LIB_PATH} not found: run `python -m paper_2509_09679_b200.build` "
@@ -90,8 +104,8 @@ def lib() -> ctypes.CDLL:
         for name, (res, args) in SIGNATURES.items():
             fn = getattr(L, name)
             fn.restype, fn.argtypes = res, args
+        _fast = _native_calls()
         _lib = L
-        _fast.attach(LIB_PATH)
     return _lib
 
 

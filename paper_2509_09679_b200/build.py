@@ -16,23 +16,30 @@ FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-O3", "-lineinfo", "-std
 
 
 FAST = os.path.join(HERE, "fast_calls" + sysconfig.get_config_var("EXT_SUFFIX"))
+FAST_TORCH = os.path.join(HERE, "_build", "fast_calls.torch")  # the torch it was built against
 
 
 def build_fast_calls(force: bool = False) -> str:
     """The extension module of csrc/fast_calls.cpp (the C ABI's header and torch's)."""
-    src = os.path.join(CSRC, "fast_calls.cpp")
-    newest = max(os.path.getmtime(p) for p in (src, os.path.join(os.path.dirname(HERE), "include", "bfq.h")))
-    if not force and os.path.exists(FAST) and os.path.getmtime(FAST) >= newest:
-        return FAST
-    if os.path.exists(FAST):
-        os.remove(FAST)  # what is there is out of date, and stays so if the compiler fails
     import torch
 
+    src = os.path.join(CSRC, "fast_calls.cpp")
+    newest = max(os.path.getmtime(p) for p in (src, os.path.join(os.path.dirname(HERE), "include", "bfq.h")))
+    if not force and os.path.exists(FAST) and os.path.getmtime(FAST) >= newest and os.path.exists(FAST_TORCH):
+        with open(FAST_TORCH) as f:
+            if f.read() == torch.__version__:
+                return FAST
+    if os.path.exists(FAST):
+        os.remove(FAST)  # what is there is out of date, and stays so if the compiler fails
     at = os.path.dirname(torch.__file__)
     cuda = os.path.dirname(os.path.dirname(NVCC))
     subprocess.run([os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-fPIC", "-shared", f"-D_GLIBCXX_USE_CXX11_ABI={int(torch.compiled_with_cxx11_abi())}",
+                    f'-DBFQ_TORCH="{torch.__version__}"',
                     f"-I{at}/include", f"-I{at}/include/torch/csrc/api/include", f"-I{sysconfig.get_paths()['include']}", f"-I{cuda}/include",
                     src, "-o", FAST, f"-L{at}/lib", "-ltorch_python", "-ltorch", "-ltorch_cpu", "-lc10_cuda", "-lc10"], check=True)
+    os.makedirs(os.path.dirname(FAST_TORCH), exist_ok=True)
+    with open(FAST_TORCH, "w") as f:
+        f.write(torch.__version__)
     return FAST
 
 

@@ -110,11 +110,16 @@ PyObject* attach(PyObject*, PyObject* path) {
     const char* name = PyUnicode_AsUTF8(path);
     if (name == nullptr) return nullptr;
     void* lib = dlopen(name, RTLD_NOW | RTLD_LOCAL);
-    if (lib != nullptr) {
-        forward_quant_fn = reinterpret_cast<ForwardQuant>(dlsym(lib, "bfq_forward_quant"));
-        forward_fn = reinterpret_cast<Rows>(dlsym(lib, "bfq_forward"));
-        inverse_fn = reinterpret_cast<Rows>(dlsym(lib, "bfq_inverse"));
-    }
+    void* found[3] = {};
+    const char* names[3] = {"bfq_forward_quant", "bfq_forward", "bfq_inverse"};
+    for (int i = 0; i < 3; ++i)
+        if (lib == nullptr || (found[i] = dlsym(lib, names[i])) == nullptr) {
+            const char* why = dlerror();
+            PyErr_SetString(PyExc_OSError, why != nullptr ? why : names[i]);
+            return nullptr;
+        }
+    forward_quant_fn = reinterpret_cast<ForwardQuant>(found[0]);
+    forward_fn = reinterpret_cast<Rows>(found[1]), inverse_fn = reinterpret_cast<Rows>(found[2]);
     Py_RETURN_NONE;
 }
 
@@ -128,4 +133,9 @@ PyModuleDef module = {PyModuleDef_HEAD_INIT, "fast_calls", nullptr, -1, methods,
 
 }  // namespace
 
-PyMODINIT_FUNC PyInit_fast_calls() { return PyModule_Create(&module); }
+PyMODINIT_FUNC PyInit_fast_calls() {
+    PyObject* m = PyModule_Create(&module);
+    // calls nothing of torch's: the binding asks for this before it uses the module with the torch that is there
+    if (m != nullptr && PyModule_AddStringConstant(m, "torch_version", BFQ_TORCH) < 0) Py_CLEAR(m);
+    return m;
+}

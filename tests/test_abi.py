@@ -130,3 +130,39 @@ def test_the_library_is_built_where_the_extension_cannot_be(monkeypatch, capsys)
             raise error
         monkeypatch.setattr(build, "build_fast_calls", fails)
         assert build.build() == build.LIB and done.pop() == "library" and "was not built" in capsys.readouterr().err
+
+
+def test_the_extension_is_used_with_the_torch_it_was_built_against_only(monkeypatch, tmp_path):
+    """Another torch: the module that is there is not called, and the next build compiles it again."""
+    import sys
+    import torch
+    from paper_2509_09679_b200 import build
+    assert binding._native_calls() is sys.modules["paper_2509_09679_b200.fast_calls"]
+    commands = []
+    monkeypatch.setattr(build, "FAST", str(tmp_path / "fast_calls.so"))
+    monkeypatch.setattr(build, "FAST_TORCH", str(tmp_path / "fast_calls.torch"))
+
+    def compiler(command, check):
+        commands.append(command)
+        (tmp_path / "fast_calls.so").touch()
+    monkeypatch.setattr(build.subprocess, "run", compiler)
+    for _ in range(2):
+        build.build_fast_calls()
+    assert len(commands) == 1
+    monkeypatch.setattr(torch, "__version__", "0.1")
+    assert binding._native_calls() is binding._Interpreted and binding._Interpreted.forward(64, 8, 0, None) is None
+    for _ in range(2):
+        build.build_fast_calls()
+    assert len(commands) == 2 and '-DBFQ_TORCH="0.1"' in commands[1]
+
+
+def test_the_extension_says_what_it_does_not_find():
+    with pytest.raises(OSError):
+        binding._native_calls().attach("/nonexistent/libbfq.so")
+
+
+def test_importing_the_package_loads_no_compiled_code():
+    import subprocess
+    import sys
+    code = "import sys, paper_2509_09679_b200 as p; assert not any(m.endswith('fast_calls') for m in sys.modules) and p.binding._lib is None"
+    subprocess.run([sys.executable, "-c", code], check=True, cwd=os.path.dirname(os.path.dirname(os.path.abspath(__file__))))
