@@ -112,7 +112,9 @@ def test_binding_rejects_bad_tensors_before_any_launch(monkeypatch):
 def test_the_plain_forms_leave_everything_else_to_the_binding():
     """fast_calls answers None to what is not plain rows on a plan's device: no plan, host tensors, other types and counts."""
     import torch
+    binding.lib()
     fast = binding._fast
+    assert fast.__file__ == build.FAST  # the compiled module, not what answers None to everything
     x = torch.zeros((2, 8))
     for call in (fast.forward, fast.inverse):
         assert call(0, 8, 0, x) is None and call(64, 8, 0, x) is None and call(64, 8, 0, [1.0]) is None and call(64, 8, 0) is None

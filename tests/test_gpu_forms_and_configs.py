@@ -66,6 +66,29 @@ def test_rotation_forms_n4096(kind):
     assert p.device_status() == 0
 
 
+@pytest.mark.parametrize("kind", ["small", "steep", "singular", "hadamard", "uniform", "above", "below"])
+@pytest.mark.parametrize("n,rows", [(4096, 301), (512, 2000)])
+def test_rotation_forms_of_the_backward(n, rows, kind):
+    """The backward takes the scaled form down to factors of 2^-40 (the forward to 2^-64); no call says which it took.  "above" and
+    "below" are on either side of that, by the least product of an element's cosines."""
+    log_n = n.bit_length() - 1
+    if kind in ("above", "below"):
+        theta = torch.full((log_n, n // 2), math.acos(2.0 ** ((-39.5 if kind == "above" else -40.5) / log_n)))
+    else:
+        theta = angle_set(kind, n, 730)
+    theta = theta.float()
+    p = Plan(n, DEV)
+    p.set_angles(theta.to(DEV))
+    for dtype in (torch.float32, torch.bfloat16):
+        x = synth.rows(rows, n, "student_t3", 731, outliers=8, outlier_scale=50.0, dtype=dtype)
+        g = synth.rows(rows, n, "normal", 732, dtype=dtype)
+        dx, dth = p.backward(x.to(DEV), g.to(DEV))
+        dx_ref, dth_ref = oracle.backward(to_f64(theta), to_f64(x), to_f64(g))
+        check_rows_close(dx, dx_ref, absmax_rows(g), f"{kind} dx")
+        check_dtheta(dth, dth_ref, f"{kind} dtheta")
+    assert p.device_status() == 0
+
+
 @pytest.mark.parametrize("kind", ["small", "steep", "singular", "uniform"])
 def test_rotation_forms_n8192(kind):
     n, rows = 8192, 151
@@ -267,3 +290,41 @@ def test_a_few_rows_are_the_bits_of_many(dtype, kind):
     wide = torch.full((9, n + 24), 7.0, dtype=dtype, device=DEV)
     p.forward(x[:9], out=wide[:, :n])
     assert torch.equal(wide[:, :n], whole[0][:9]) and (wide[:, n:] == 7.0).all() and p.device_status() == 0
+
+
+@pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
+@pytest.mark.parametrize("n,rows", [(256, 33), (4096, 3), (8192, 5)])
+def test_native_calls_are_the_bindings(n, rows, dtype):
+    """Plain calls in C++ against the same calls with the caller's buffers, which the interpreter does: the same bits, contiguous and
+    strided rows, on a stream of its own behind work that is still running; and what either refuses."""
+    from paper_2509_09679_b200 import BfqError, binding
+    p = Plan(n, DEV)
+    with pytest.raises(BfqError, match="WORKSPACE"):  # angles not set
+        p.forward(torch.zeros((rows, n), dtype=dtype, device=DEV))
+    p.set_angles(synth.angles(n, "normal", 7).to(DEV))
+    fast, head = binding._fast, (p._id, n, p._index)
+    wide = torch.zeros((rows, n + 8), dtype=dtype, device=DEV)
+    source = synth.rows(rows, n + 8, "student_t3", 8, dtype=dtype).to(DEV)
+    torch.cuda.synchronize()
+    side = torch.cuda.Stream()
+    with torch.cuda.stream(side):
+        torch.cuda._sleep(20_000_000)  # the rows arrive late: a call on another stream would read zeros
+        wide.copy_(source)
+        native = [(fast.forward(*head, x), fast.inverse(*head, x)) + fast.forward_quant(*head, x, 4) for x in (wide[:, :n], wide[:1, :n], wide[:, :n].contiguous())]
+    side.synchronize()
+    for got, x in zip(native, (source[:, :n], source[:1, :n], source[:, :n])):
+        rows_out = [torch.empty((len(x), n), dtype=dtype, device=DEV) for _ in range(2)]
+        codes, scales = torch.empty((len(x), n // 2), dtype=torch.uint8, device=DEV), torch.empty(len(x), dtype=torch.float16, device=DEV)
+        ref = (p.forward(x, out=rows_out[0]), p.inverse(x, out=rows_out[1])) + p.forward_quant(x, 4, codes=codes, scales=scales)
+        assert all(isinstance(a, torch.Tensor) and a.dtype == b.dtype and torch.equal(a, b) for a, b in zip(got, ref))
+    # rows that overlap, as a single row may, are the binding's; an address between 16-byte lines is refused either way
+    one = source[0, :n].as_strided((1, n), (4, 1))
+    assert fast.forward(*head, one) is None and torch.equal(p.forward(one), p.forward(source[:1, :n]))
+    odd = torch.zeros(rows * n + 1, dtype=dtype, device=DEV)[1:].view(rows, n)
+    assert type(fast.forward(*head, odd)) is int
+    for call in (lambda: p.forward(odd), lambda: p.forward(odd, out=torch.empty((rows, n), dtype=dtype, device=DEV))):
+        with pytest.raises(BfqError, match="ALIGN"):
+            call()
+    # a closed plan, other types and no rows
+    assert fast.forward(0, n, 0, source[:, :n]) is None and fast.forward(*head, source[:, :n].half()) is None
+    assert p.forward(source[:0, :n]).shape == (0, n) and p.device_status() == 0

@@ -343,6 +343,20 @@ def test_backward_into_its_own_input(n, rows, over):
     assert p.device_status() == 0
 
 
+@pytest.mark.parametrize("n,rows", [(4096, 1001), (256, 20001), (128, 40000)])
+@pytest.mark.parametrize("over", ["g", "x"])
+def test_backward_into_its_own_bf16_input(n, rows, over):
+    """The same where the group of threads that brings g down writes dx, before another has read the row of x that may lie there:
+    several rows for each CTA.  (Both are fp32 results rounded to bf16: an ulp, 2^-7, apart at most.)"""
+    p, theta, x, xd = inputs(n, rows, torch.bfloat16)
+    gd = synth.rows(rows, n, "normal", 5, dtype=torch.bfloat16).to(DEV)
+    dx, dth = p.backward(xd, gd)
+    dx2, dth2 = p.backward(xd, gd, dx=gd if over == "g" else xd)
+    a, b = dx.float(), dx2.float()
+    assert ((a - b).abs() <= 2.0 ** -7 * a.abs() + 1e-5 * a.abs().max()).all() and (dth2 - dth).norm() <= 1e-5 * dth.norm()
+    assert p.device_status() == 0
+
+
 def test_backward_rounds_each_row_once_into_the_sums():
     """d-theta against 64 bits (n = 4096).  A running sum of m rows with one rounding each is off by 2.5e-8 sqrt(m / 2) of the total (the
     mean square of a rounding to 24 bits, the sum growing as a random walk), 4.3e-7 here with the 2e-7 that the rows' own rounding
