@@ -140,7 +140,9 @@ int bfq_inverse(bfq_plan* plan, const void* y, bfq_dtype yt, int64_t rows, int64
  * x, g: [rows][ld]; dx: [rows][ld] of dxt (may be NULL to skip); dtheta: device fp32
  * [log2 n][n/2], overwritten.  The sum over rows has a fixed order (per-CTA partial sums over a
  * static row assignment, then the CTAs' sums added in a fixed order): results are bit-identical run to run on the
- * same device.  The quantizer is not differentiated here; g is the caller's.
+ * same device.  The quantizer is not differentiated here; g is the caller's.  dx of a row depends on that row alone.  An infinity or NaN
+ * in g may leave every entry of dtheta not finite, also those of angles that its elements do not reach, and a call with such rows (or
+ * with finite ones that overflow in the scaled form, see bfq_stage_form) may take up to 2.7 times as long.
  */
 int bfq_backward(bfq_plan* plan, const void* x, bfq_dtype xt, const void* g, bfq_dtype gt,
                  int64_t rows, int64_t ld, void* dx, bfq_dtype dxt, float* dtheta, void* stream);
@@ -227,8 +229,10 @@ int bfq_last_cuda_error(const bfq_plan* plan);
  * cosines it has been through; when such a product leaves [2^-64, 1] (an angle within ~1e-19 .. of an odd multiple of
  * pi/2 along some path, e.g. angles that are exact multiples of pi/2) the table build selects the three-shear form
  * instead, which has no such limit.  Returns bit 0 = forward tables use the fallback, bit 1 = inverse tables (built by
- * the first bfq_inverse / bfq_backward after bfq_set_angles, for n < 4096 by bfq_set_angles; at n = 8192 the tables of either
- * half of the row) use the fallback; or a negative bfq_status.  Synchronises the device.  With the scaled form at n = 4096 and 8192, inputs must stay below about 2^56 in magnitude (intermediate values
+ * the first bfq_inverse after bfq_set_angles, at n = 8192 by the first bfq_inverse or bfq_backward, for n < 4096 by bfq_set_angles; at n =
+ * 8192 the tables of either half of the row) use the fallback; or a negative bfq_status.  bfq_backward on rows of up to 4096 elements
+ * takes the fallback from products below 2^-40 on, which is not reported; it needs no bound on its inputs: sums that are not finite are
+ * taken again without factors.  Synchronises the device.  With the scaled form at n = 4096 and 8192, inputs must stay below about 2^56 in magnitude (intermediate values
  * are the true values divided by the factor); rows of up to 2048 elements may hold any fp32 numbers: one whose results are not
  * finite there is computed again without factors.  (No counterpart in the paper; informational.)
  */

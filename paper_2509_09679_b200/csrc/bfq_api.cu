@@ -68,10 +68,11 @@ static bool use_short_rows(const bfq_plan* plan, int64_t rows, int64_t min_elems
     return rows < (int64_t(1) << 31) - 64 && rows * plan->n >= min_elems && !env_flag("BFQ_GENERIC_ONLY") && fwdq_short_available(plan);
 }
 static int64_t short_inverse_from(int n, bool f32) { return n == 128 && f32 ? int64_t(1) << 21 : 0; }
-// Backward: filling the tensor memory takes 27 - 29 us whatever the size, the generic kernel 22 - 25 us on a small batch.  Where
-// they meet (us, generic against short rows, fp32 / bf16; m = 2^16 elements): n = 128 at 2 m 30.8 : 30.6 / 30.8 : 28.8; n = 256
-// at 4 m 30.5 : 30.8 / 29.9 : 29.4; n = 512 at 5 m 28.8 : 28.7 / 28.7 : 28.2, at 6 m 30.8 : 28.7 / 30.8 : 27.7; n = 1024 at 9 m
-// 28.8 : 30.6 / 29.4 : 29.8, at 10 m 37.0 : 30.8 / 36.9 : 30.0; n = 2048 at 9 m 26.7 : 30.8 / 26.4 : 30.6, at 10 m 34.8 : 30.8 / 33.9 : 30.7.
+// Backward: lines at which the tuned kernel before k_grad4096, with 27 - 29 us on any small batch, met the generic one.  They are
+// on the safe side now: k_grad4096 takes less on either side of them (us, generic / k_grad4096, fp32 rows; the size just below the line):
+// n = 128 96 K elements 23.9 / 13.5; n = 256 192 K 23.6 / 13.8; n = 512 256 K 23.9 / 13.7; n = 1024 512 K 23.6 / 14.1; n = 2048 512 K
+// 21.8 / 14.4; bf16 rows 0.7 less.  It does down to a single row (n = 128: 1 K 14.9 / 9.5; n = 2048: 17.3 / 10.6), with a plan; without one
+// (bfq_backward_noalloc) every call builds the tables first, which has not been compared.
 static int64_t short_backward_from(int n) {
     const int64_t m = int64_t(1) << 16;
     return n == 128 ? 2 * m : (n == 256 ? 4 * m : (n == 512 ? 6 * m : 10 * m));
@@ -643,7 +644,7 @@ int bfq_inverse(bfq_plan* plan, const void* y, bfq_dtype yt, int64_t rows, int64
     if (yt == BFQ_BF16 && rows < (int64_t(1) << 31) && x != y && !env_flag("BFQ_GENERIC_ONLY") && bwd4096_available(plan)) {
         cudaStream_t st = static_cast<cudaStream_t>(stream);
         cudaError_t e = cudaSuccess;
-        if (!plan->bwd_tables_valid) {  // shared with bfq_backward: built on first use after bfq_set_angles
+        if (!plan->bwd_tables_valid) {  // built on first use after bfq_set_angles
             e = bwd4096_build_tables(plan, st);
             plan->bwd_tables_valid = (e == cudaSuccess);
         }

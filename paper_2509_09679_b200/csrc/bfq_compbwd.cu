@@ -18,7 +18,7 @@
 // walks, and 20 KB of memory traffic in bf16, so the arithmetic bounds it (2048 tokens: 29 us at one multiply-add per lane and
 // cycle).  Composed from a dense product on permuted copies, the butterfly backward on 40 rows per token, a forward in fp32
 // and another dense product it took about 1000 us for 2048 tokens, and G' went through bf16 in between; this kernel
-// takes 145 us (191 us with scalar multiply-adds) where G is fp32; bf16 G: k_composite_backward_mma.
+// takes 143 us (191 us with scalar multiply-adds) where G is fp32; bf16 G: k_composite_backward_mma, 112 us.
 #include "../../include/bfq.h"
 
 #include <cuda_bf16.h>

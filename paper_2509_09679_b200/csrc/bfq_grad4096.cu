@@ -9,8 +9,8 @@
 // d * true value, comes down through the transposed stages, lo = lo' + k2 * hi', hi = hi' + k1 * lo': the same constants, with lo
 // and hi changing places; so do the three-shear stages.  At the bottom d is 1: u is dx as it stands, and x and u go up with the
 // same factors, so that a pair's sum comes out times 1 / (d_lo * d_hi), one number per angle (`weight`), put right when the
-// CTAs' sums are added.  752 packed multiply-adds per row and thread, where recomputing y and walking y and g down in the
-// three-shear form (the only one in which one table served that) took 1056.
+// CTAs' sums are added.  560 packed multiply-adds of the rotations and 384 multiplications and additions of the sums per row and thread;
+// recomputing y and walking y and g down in the three-shear form (the only one in which one table served that) took 1056 in all.
 //
 // A CTA per SM runs four groups of 128 threads as a pipeline, a row in each:
 //     D  g: stages 11 .. 8 down
@@ -25,7 +25,10 @@
 // Range: factors of 2^-40 and more (else the three-shear form runs: `form`), and g comes down 2^40 times too large, so that nothing
 // is stored smaller than it is: however small g, no bits are lost.  What overflows instead (with the least factors g from about 2^80 on,
 // products of u and x from 2^48 on) leaves a sum that is not finite; the CTA then does its rows again in the three-shear form, which
-// has no factors, and rewrites only those pieces of dx that were not finite.
+// has no factors, and rewrites only those pieces of dx that were not finite.  The second pass takes 1.7 times as long as the first: 262144
+// x 4096 bf16 rows 9.1 ms in all as soon as one CTA meets one, 3.4 otherwise.  An infinity or NaN in g or x is such a row too (and leaves
+// no angle's sum finite where it is in g).  A look at g and dx between the passes that leaves the second one out for those cost every
+// call 8 %, in registers of the row loops.
 #include <type_traits>
 
 #include "bfq_fast.h"
@@ -214,7 +217,7 @@ struct Ctx {
     Addr a;
     uint32_t sbase, tlane;
     int t, count, done;  // done: rows of earlier passes, for the parity of the barriers
-    int first, stride, rows;
+    int first, stride;
     void* dx;
     int64_t ld, elems;
     int* status;
@@ -568,7 +571,7 @@ k_grad4096(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ CUt
     cx.a.r1 = 4u * (258u * (t & 15) + 32u * (t >> 4));
     cx.a.w2 = 4u * ((t & 15) + 2064u * ((t >> 4) & 1) + 512u * ((t >> 5) & 1) + 1024u * ((t >> 6) & 1));
     cx.a.r2 = 4u * (2u * (t & 15) + 32u * (t >> 4));
-    cx.first = blockIdx.x, cx.stride = gridDim.x, cx.rows = rows;
+    cx.first = blockIdx.x, cx.stride = gridDim.x;
     cx.count = cx.first < rows ? (rows - cx.first + cx.stride - 1) / cx.stride : 0;
     cx.dx = dx, cx.ld = ld, cx.elems = elems, cx.status = status;
     cx.out = partial + static_cast<int64_t>(blockIdx.x) * kSlotFloats;

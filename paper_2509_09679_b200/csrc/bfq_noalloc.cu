@@ -11,7 +11,7 @@
 //
 // The kernel is chosen by the rule of bfq_backward, so that dx is the same bits either way: calls it
 // takes to the n = 4096 kernel come here with the tables built in the array on every call and as many
-// CTAs as the rest of it holds partial sums for (69 at 96 KiB each).
+// CTAs as the rest of it holds partial sums for (70 at 96 KiB each on 148 SMs).
 //
 // Consequences of the shared array: the row length is limited to BFQ_NOALLOC_MAX_N; all calls (from
 // any stream or thread) use the same bytes, so two calls that overlap on one GPU race; the array
